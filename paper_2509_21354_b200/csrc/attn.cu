@@ -11,17 +11,21 @@
 //    without draining, every CTA moves nearly the same number of bytes whatever S is, and where a
 //    part begins follows from the launch arguments, the stored length and one keep count, so the
 //    first copies leave two dependent loads after the kernel starts.
-//  * Warp 8 (producer) turns tiles into addresses (page table; kept summary rows sit compacted in
-//    one contiguous run per sequence), merges rows that are contiguous in memory into runs with a
-//    ballot, and issues one bulk copy (TMA engine, global -> shared, mbarrier byte counting) per run
-//    into a 3-stage ring of 64-row K and V tiles.  The query row of a sequence travels with the
-//    first tile of that sequence.
-//  * Warps 0-7 (consumers) each take 8 rows of a tile: q.k partial sums per lane (4 head dims per
-//    lane), a butterfly transpose-reduce that leaves one row's logit per group of four lanes, online
-//    softmax with warp shuffles, then p.V with each lane owning 4 output dims.  When a CTA's run
-//    leaves a sequence, the consumers drop their (m, l, acc) into a double-buffered exchange area
-//    and carry on with the next sequence.
-//  * Warp 9 (merger) folds the eight consumer states of a finished sequence (or part of one), and
+//  * Warp 4 (producer) turns tiles into copies (TMA engine, global -> shared, mbarrier byte counting): one K and one V copy per
+//    chunk that a tile touches (kept summary rows sit compacted in one run per sequence: one copy), into a 3-stage ring
+//    of 64-row tiles.  The query row of a sequence travels with the first tile of that sequence.  Page ids of 32 chunks
+//    wait in the lanes' registers, so that a tile costs the warp shuffles and not a table look-up; before, every lane looked
+//    up the page of each of its rows and runs were found again with a ballot, which held the ring back: 512 sequences of
+//    1100 rows 56.7 us a step (5.0 TB/s), now 49.8 us (5.75 TB/s).
+//  * While the predecessor on the stream still runs, the producer goes through its first tile once on what the tables hold (a
+//    guess, repeated with the real values after the wait) and the consumers pull the guessed rows of two tiles into L2:
+//    8 layers of 128 sequences x 330 rows, one after the other, 12.7 -> 11.4 us a layer.
+//  * Warps 0-3 (consumers) each take 16 rows of a tile.  The logits q.k are eight warp-level MMAs (the rows are the M side, q
+//    fills the N side: bf16 products, fp32 sums), which leaves a group of four lanes with the logits of two rows; online
+//    softmax with warp shuffles, then p.V in fp32 with half a warp per row and 8 output dims per lane.  When a CTA's run
+//    leaves a sequence, the consumers drop their (m, l, acc) into a double-buffered exchange area and carry on with the
+//    next sequence.
+//  * Warp 5 (merger) folds the four consumer states of a finished sequence (or part of one), and
 //    either writes the output (this CTA had the whole sequence) or a partial record plus an atomic
 //    ticket; the CTA that draws a sequence's last ticket merges its records by log-sum-exp.  Nobody
 //    spins on another CTA.
@@ -52,12 +56,14 @@ __device__ __forceinline__ void stamp(int slot) {
 
 constexpr int AT_TILE = ATTN_TILE_ROWS;       // rows per stage
 constexpr int AT_STAGES = 3;
-constexpr int AT_CWARPS = 8;                  // consumer warps
-constexpr int AT_SUB = AT_TILE / AT_CWARPS;   // 8 rows per consumer warp per tile
+constexpr int AT_CWARPS = 4;                  // consumer warps
+constexpr int AT_SUB = AT_TILE / AT_CWARPS;   // 16 rows per consumer warp per tile: the rows of one m16n8k16 MMA
 constexpr int AT_PRODUCER = AT_CWARPS;        // warp ids
 constexpr int AT_THREADS = (AT_CWARPS + 2) * 32;
 constexpr int AT_STAGE_ELEMS = AT_TILE * D;   // bf16 elements of one K (or V) tile
-static_assert(AT_SUB == 8, "the transpose-reduce below is written for 8 rows per warp");
+constexpr int AT_MERGE_BELOW = 32;            // chunks shorter than this: copies of adjacent pages are merged
+constexpr int AT_PREFETCH_TILES = 2;          // most tiles a CTA pulls into L2 before its predecessor has finished
+static_assert(AT_SUB == 16, "the logits of a warp's rows are one m16n8k16 tile");
 
 // shared-memory carve-up (bytes)
 constexpr int AT_OFF_K = 0;
@@ -102,7 +108,6 @@ struct AttnGeo {
   int n;                       // tokens attended to (the new one included when one is being appended)
   int n_chunks;                // chunks the keep list covers (0 for full-cache attention)
   bool appending;              // the last tail row of every sequence is the new token, taken from k_new / v_new
-  uint32_t I, P;               // parts in the launch (S k); CTAs that get any (min(G, I): none of them is empty)
 };
 
 // CTA c of P takes parts [c I / P, (c + 1) I / P); CTAs c >= P take none.  32-bit arithmetic (64-bit division
@@ -112,6 +117,12 @@ __device__ __forceinline__ uint32_t piece_begin(uint32_t c, uint32_t I, uint32_t
 __device__ __forceinline__ uint32_t piece_of(uint32_t x, uint32_t I, uint32_t P) { return ((x + 1u) * P - 1u) / I; }
 
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+// bulk prefetch into L2 (16-byte aligned, a multiple of 16 bytes)
+__device__ __forceinline__ void prefetch_l2_bulk(const void* p, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+// read from L2 (never from a line that L1 may hold from before the predecessor finished)
+__device__ __forceinline__ int load_hint(const int32_t* p) { return *reinterpret_cast<const volatile int32_t*>(p); }
 
 // Pulls what the producer will look up for sequence s into L2 (fire and forget: the keep count, the page ids
 // of the raw tail, the head of the kept-chunk list), so that the dependent look-ups that follow cost an L2 hit each.
@@ -131,25 +142,72 @@ __device__ __forceinline__ int lead_rows_from(const AttnArgs& a, const AttnGeo& 
   if (a.mode == ATTN_DENSE || g.n_chunks <= 0) return 0;
   return min(max(keep_cnt, 0), g.n_chunks) * g.per;
 }
-__device__ __forceinline__ int lead_rows_of(const AttnArgs& a, const AttnGeo& g, int s) {
-  if (a.mode == ATTN_DENSE || g.n_chunks <= 0) return 0;
-  return lead_rows_from(a, g, a.v.keep_cnt[s]);
-}
-
-#define KVE_TR_ROUND(OFF, CNT)                                                        \
-  {                                                                                   \
-    const bool upper = (lane & (OFF)) != 0;                                           \
-    _Pragma("unroll") for (int j = 0; j < (CNT); ++j) {                               \
-      const float send = upper ? part[j] : part[j + (CNT)];                           \
-      const float keep = upper ? part[j + (CNT)] : part[j];                           \
-      part[j] = keep + __shfl_xor_sync(0xffffffffu, send, (OFF));                     \
-    }                                                                                 \
-  }
-
 // one tile of the CTA's work as the producer sees it
 struct TileDesc {
   int s, list, j, rows, flags;      // list 0: raw tail, 1: kept chunks; j: tile index inside the sequence's list
 };
+
+// The rows of a tile that lie in one chunk: `pos` is the chunk (raw tail) or the index in the keep list (kept chunks at full
+// resolution), `r` the first row inside it, `len` how many, `dst` where they go in the tile.
+struct TileSegment { int pos, r, len, dst; };
+__device__ __forceinline__ TileSegment tile_segment(int row0, int rows, int C, int pos) {
+  TileSegment g;
+  g.pos = pos;
+  const int lo = max(row0, g.pos * C), hi = min(row0 + rows, g.pos * C + C);
+  g.r = lo - g.pos * C;
+  g.len = max(hi - lo, 0);
+  g.dst = lo - row0;
+  return g;
+}
+
+__device__ __forceinline__ AttnGeo make_geometry(const AttnArgs& a, int n, int listed) {
+  AttnGeo g;
+  n = min(max(n, 0), a.v.max_tokens);
+  g.appending = a.k_new != nullptr && n < a.v.max_tokens;
+  if (g.appending) n += 1;
+  g.n = n;
+  g.n_chunks = (a.mode == ATTN_DENSE) ? 0 : min(max(listed, 0), a.v.max_chunks);
+  g.raw0 = g.n_chunks * a.v.C;
+  g.n_tail = max(0, n - g.raw0);
+  g.TT = (g.n_tail + AT_TILE - 1) / AT_TILE;
+  g.per = (a.mode == ATTN_RAW) ? a.v.C : 1;
+  return g;
+}
+
+// What the CTA will stream first, pulled into L2 while the predecessor on the stream is still running: lengths, keep lists and
+// page ids are read before they are final, but only to guess addresses (checked against the pools), and a prefetch returns
+// nothing - a wrong guess costs a few lines of L2, a right one (the decode loop: the same layer a token ago) takes the cold
+// look-ups and the first rows off the path.  Warp w takes every AT_CWARPS-th of the CTA's first tiles in its first sequence.
+__device__ __forceinline__ void prefetch_first_tiles(const AttnArgs& a, uint32_t i0, uint32_t i1, int warp, int lane) {
+  const LayerView& v = a.v;
+  const uint32_t uk = (uint32_t)a.k;
+  const int s = (int)(i0 / uk);
+  const AttnGeo g = make_geometry(a, load_hint(v.seq_len), a.mode == ATTN_DENSE ? 0 : load_hint(v.n_listed));
+  const int keep = a.mode == ATTN_DENSE ? 0 : load_hint(v.keep_cnt + s);
+  const int lead = min(max(keep, 0), g.n_chunks) * g.per;
+  const int tiles = g.TT + (lead + AT_TILE - 1) / AT_TILE;
+  const uint32_t p_lo = i0 - (uint32_t)s * uk, p_hi = min(i1 - (uint32_t)s * uk, uk);
+  const int j0 = (int)((p_lo * (uint32_t)tiles) / uk), j1 = min((int)((p_hi * (uint32_t)tiles) / uk), j0 + AT_PREFETCH_TILES);
+  const long long sb = (long long)s * v.max_chunks;
+  for (int j = j0 + warp; j < j1; j += AT_CWARPS) {
+    const bool tail = j < g.TT;
+    const int jj = tail ? j : j - g.TT, rows = min(AT_TILE, (tail ? g.n_tail : lead) - jj * AT_TILE);
+    if (!tail && a.mode == ATTN_SUMMARY) {
+      if (lane < 2) prefetch_l2_bulk((lane ? a.vkept : a.kkept) + (sb + jj * AT_TILE) * D, (uint32_t)rows * ROW_BYTES);
+      continue;
+    }
+    const int row0 = (tail ? g.raw0 : 0) + jj * AT_TILE;
+    const TileSegment sg = tile_segment(row0, rows, v.C, row0 / v.C + lane);
+    if (sg.len <= 0 || sg.pos >= v.max_chunks) continue;
+    const int chunk = tail ? sg.pos : load_hint(v.keep_idx + sb + sg.pos);
+    if (chunk < 0 || chunk >= v.max_chunks) continue;
+    const long long page = load_hint(v.page_table + sb + chunk);
+    if (page < 0 || page >= v.n_pages) continue;
+    const long long off = (page * v.C + sg.r) * D;
+    prefetch_l2_bulk(v.k_pages + off, (uint32_t)sg.len * ROW_BYTES);
+    prefetch_l2_bulk(v.v_pages + off, (uint32_t)sg.len * ROW_BYTES);
+  }
+}
 
 __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -168,13 +226,13 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
   const LayerView& v = a.v;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   KVE_STAMP(threadIdx.x == 0, 0);
-  if (warp == AT_PRODUCER) {
-    // where this CTA starts follows from the launch arguments alone: warm L2 with what the first look-ups need
-    // while the barriers are set up and the predecessor drains (prefetches return nothing, so they may run early)
-    const uint32_t I = (uint32_t)v.S * (uint32_t)a.k, P = min(gridDim.x, I);
-    if (blockIdx.x < P) prefetch_sequence_metadata(a, (int)(piece_begin(blockIdx.x, I, P) / (uint32_t)a.k), lane);
-    if (lane == 31) prefetch_l2(v.seq_len);
-    if (lane == 30) prefetch_l2(v.n_listed);
+  // this CTA's parts follow from the launch arguments alone
+  const uint32_t c = blockIdx.x, uk = (uint32_t)a.k;
+  const uint32_t n_items = (uint32_t)v.S * uk, n_pieces = min(gridDim.x, n_items);
+  const uint32_t i0 = piece_begin(c, n_items, n_pieces), i1 = piece_begin(c + 1, n_items, n_pieces);
+  if (i0 < i1) {
+    if (warp == AT_PRODUCER) prefetch_sequence_metadata(a, (int)(i0 / uk), lane);
+    else if (warp < AT_CWARPS) prefetch_first_tiles(a, i0, i1, warp, lane);
   }
   if (threadIdx.x == 0) {
     for (int i = 0; i < AT_STAGES; ++i) {
@@ -188,49 +246,17 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
     mbar_fence_init();
   }
   __syncthreads();
-  pdl_wait();      // lengths, keep lists, summaries and the new token come from earlier kernels
-  KVE_STAMP(threadIdx.x == 0, 1);
-
-  // this CTA's parts follow from the launch arguments; the producer asks for its first sequence's keep count at once,
-  // together with the length and the coverage below: three look-ups in flight instead of one after the other
-  const uint32_t c = blockIdx.x, uk = (uint32_t)a.k;
-  const uint32_t n_items = (uint32_t)v.S * uk, n_pieces = min(gridDim.x, n_items);
-  const uint32_t i0 = piece_begin(c, n_items, n_pieces), i1 = piece_begin(c + 1, n_items, n_pieces);
-  int keep_cnt_first = 0;
-  if (warp == AT_PRODUCER && i0 < i1 && a.mode != ATTN_DENSE) keep_cnt_first = v.keep_cnt[i0 / uk];
-
-  // ---- geometry (every thread) ---------------------------------------------------------------------------
-  AttnGeo g;
-  {
-    int n = v.seq_len[0];
-    // chunks the keep list covers: the device's own count, so that a launch replayed from a CUDA graph follows the
-    // gate triggers that happened since it was captured (the launch argument is only the host's view at capture time).
-    // Requested together with the length: nothing that could alias stands between the two loads.
-    const int listed = (a.mode == ATTN_DENSE) ? 0 : *v.n_listed;
-    n = min(max(n, 0), v.max_tokens);
-    g.appending = a.k_new != nullptr && n < v.max_tokens;
-    if (a.k_new != nullptr && !g.appending && blockIdx.x == 0 && threadIdx.x == 0) set_status(v.status, ERR_CAPACITY);   // cache full
-    if (g.appending) n += 1;
-    g.n = n;
-    g.n_chunks = min(max(listed, 0), v.max_chunks);
-    g.raw0 = g.n_chunks * v.C;
-    g.n_tail = max(0, n - g.raw0);
-    g.TT = (g.n_tail + AT_TILE - 1) / AT_TILE;
-    g.per = (a.mode == ATTN_RAW) ? v.C : 1;
-    g.I = n_items;
-    g.P = n_pieces;
-  }
-
   if (warp == AT_PRODUCER) {
     // ================= producer warp =================
     // walks the CTA's parts in order, sequence by sequence; within a sequence the tiles [j_lo, j_hi) that
     // its parts in this CTA cover (part p of a sequence with T tiles: tiles [p T / k, (p + 1) T / k))
-    const int s_first = (int)(i0 / uk), s_last = (int)((i1 - 1u) / uk);      // meaningful when i0 < i1
+    const int s_first = (int)(i0 / uk), s_last = i0 < i1 ? (int)((i1 - 1u) / uk) : s_first;
+    AttnGeo g;
     int s = s_first, j = 0, j_hi = 0, lt_rows = 0, tiles = 0;
     bool fresh = true;                      // the next tile is the first one of sequence s in this CTA
-    auto enter_sequence = [&]() {
-      if (s < s_last) prefetch_sequence_metadata(a, s + 1, lane);      // the next one's look-ups will hit L2
-      lt_rows = (s == s_first) ? lead_rows_from(a, g, keep_cnt_first) : lead_rows_of(a, g, s);
+    bool done = i0 >= i1;
+    auto enter_sequence = [&](int keep_cnt) {
+      lt_rows = lead_rows_from(a, g, keep_cnt);
       tiles = g.TT + (lt_rows + AT_TILE - 1) / AT_TILE;
       // part p of the sequence's tiles: [p tiles / k, (p + 1) tiles / k); p <= 32 and tiles < 2^20, so 32 bits do
       const uint32_t p_lo = (s == s_first) ? i0 - (uint32_t)s * uk : 0u;
@@ -239,8 +265,6 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
       j_hi = (int)((p_hi * (uint32_t)tiles) / uk);
       fresh = true;
     };
-    bool done = i0 >= i1;
-    if (!done) enter_sequence();
     auto next_tile = [&](TileDesc& t) {
       if (done) {
         t.s = -1; t.list = 0; t.j = 0; t.rows = 0; t.flags = TF_END;
@@ -262,51 +286,69 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
       }
       if (t.flags & TF_FLUSH) {
         if (s == s_last) done = true;
-        else { ++s; enter_sequence(); }
-      }
-    };
-    // addresses of the tile's rows: lane l resolves rows l and l + 32
-    struct TileAddr { const uint16_t *k[AT_TILE / 32], *v[AT_TILE / 32]; };
-    auto resolve = [&](const TileDesc& t, TileAddr& ta) {
-#pragma unroll
-      for (int half = 0; half < AT_TILE / 32; ++half) ta.k[half] = ta.v[half] = nullptr;
-      if (t.flags & TF_END) return;
-      const long long sb = (long long)t.s * v.max_chunks;
-#pragma unroll
-      for (int half = 0; half < AT_TILE / 32; ++half) {
-        const int rl = half * 32 + lane;
-        if (rl >= t.rows) continue;
-        const int L = t.j * AT_TILE + rl;              // row inside the sequence's list
-        int chunk, r;
-        if (t.list == 0) {
-          if (g.appending && L == g.n_tail - 1) {      // the token being appended: straight from the caller's buffers
-            ta.k[half] = a.k_new + (long long)t.s * D;
-            ta.v[half] = a.v_new + (long long)t.s * D;
-            continue;
-          }
-          const int p = g.raw0 + L;
-          chunk = p / v.C;
-          r = p - chunk * v.C;
-        } else if (a.mode == ATTN_SUMMARY) {
-          ta.k[half] = a.kkept + (sb + L) * D;
-          ta.v[half] = a.vkept + (sb + L) * D;
-          continue;
-        } else {                                       // RAW: row r of the (L / C)-th kept chunk
-          const int ci = L / v.C;
-          r = L - ci * v.C;
-          chunk = v.keep_idx[sb + ci];
-          if (chunk < 0 || chunk >= g.n_chunks) { set_status(v.status, ERR_CAPACITY); chunk = 0; }
+        else {
+          ++s;
+          if (s < s_last) prefetch_sequence_metadata(a, s + 1, lane);      // the next one's look-ups will hit L2
+          enter_sequence((a.mode == ATTN_DENSE || g.n_chunks <= 0) ? 0 : load_hint(v.keep_cnt + s));
         }
-        long long page = v.page_table[sb + chunk];
-        if (page < 0 || page >= v.n_pages) { set_status(v.status, ERR_CAPACITY); page = 0; }
-        const long long off = (page * v.C + r) * D;
-        ta.k[half] = v.k_pages + off;
-        ta.v[half] = v.v_pages + off;
       }
     };
-    // waits for the stage, publishes the tile's description, issues its copies; false on a timed-out wait
-    auto issue = [&](int i, const TileDesc& t, const TileAddr& ta) -> bool {
+    // Page ids of 32 consecutive entries of a sequence's chunk list (tail: chunk numbers, kept: positions in the keep list), one
+    // per lane: a tile spans two or three chunks, so the table is looked at once in 20 tiles or more instead of on
+    // every tile.  Entries that name nothing become -1 and are flagged when a tile uses them.
+    int pc_key = -1, pc_base = 0, pc_page = -1;
+    auto load_pages = [&](int seq, int list, int base) {
+      const long long sb = (long long)seq * v.max_chunks;
+      int chunk = base + lane;
+      if (list != 0) chunk = chunk < v.max_chunks ? load_hint(v.keep_idx + sb + chunk) : -1;
+      const bool named = chunk >= 0 && chunk < (list != 0 ? g.n_chunks : v.max_chunks);
+      pc_page = named ? load_hint(v.page_table + sb + chunk) : -1;
+      pc_key = seq * 2 + list;
+      pc_base = base;
+    };
+
+    // The first tile is worked out twice: once from what the tables hold while the predecessor still runs - only a guess at
+    // where to look, and a way to have the code at hand - and again from the real values, when the look-ups of the
+    // length, the coverage, the keep count and the guessed page ids go out together.
+    TileDesc d;
+    int guess_key = -1, guess_base = 0;
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+      if (pass == 1) {
+        pdl_wait();      // lengths, keep lists, summaries and the new token come from earlier kernels
+        KVE_STAMP(lane == 0, 1);
+      }
+      const int len_stored = load_hint(v.seq_len);
+      // chunks the keep list covers: the device's own count, so that a launch replayed from a CUDA graph follows the
+      // gate triggers that happened since it was captured (the launch argument is only the host's view at capture time)
+      const int listed = (a.mode == ATTN_DENSE) ? 0 : load_hint(v.n_listed);
+      const int keep_cnt = (a.mode == ATTN_DENSE || i0 >= i1) ? 0 : load_hint(v.keep_cnt + s_first);
+      if (guess_key >= 0 && (guess_key & 1) == 0) load_pages(guess_key >> 1, 0, guess_base);
+      g = make_geometry(a, len_stored, listed);
+      if (i0 >= i1) { next_tile(d); continue; }
+      s = s_first;
+      done = false;
+      enter_sequence(keep_cnt);
+      next_tile(d);
+      if (pass == 0) {
+        const int row0 = (d.list == 0 ? g.raw0 : 0) + d.j * AT_TILE;
+        if (d.rows > 0 && (d.list == 0 || a.mode == ATTN_RAW)) { guess_key = s_first * 2 + d.list; guess_base = row0 / v.C; }
+      }
+    }
+    if (a.k_new != nullptr && !g.appending && blockIdx.x == 0 && lane == 0) set_status(v.status, ERR_CAPACITY);   // cache full
+
+    // waits for the stage, publishes the tile's description, issues its copies; false on a timed-out wait.
+    // The END description takes a stage of its own (no copies): that is how the consumers learn that they are done.
+    auto issue = [&](int i, const TileDesc& t) -> bool {
       const int stage = i % AT_STAGES, round = i / AT_STAGES;
+      const long long sb = (long long)t.s * v.max_chunks;
+      const int row0 = (t.list == 0 ? g.raw0 : 0) + t.j * AT_TILE;
+      const int c0 = row0 / v.C;
+      const bool paged = t.rows > 0 && (t.list == 0 || a.mode == ATTN_RAW);
+      const int n_seg = paged ? (row0 + t.rows - 1) / v.C - c0 + 1 : 0;
+      // fused append: the last row of the tail is the new token, straight from the caller's buffers
+      const bool with_new = g.appending && t.list == 0 && t.rows > 0 && t.j * AT_TILE + t.rows == g.n_tail;
+      if (paged && (pc_key != t.s * 2 + t.list || c0 < pc_base || c0 + min(n_seg, 32) > pc_base + 32)) load_pages(t.s, t.list, c0);
       if (round > 0 && !mbar_wait_bounded(&empty[stage], (round - 1) & 1)) {
         if (lane == 0) set_status(v.status, ERR_TIMEOUT);
         return false;
@@ -319,61 +361,87 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
         if (with_q) bulk_g2s(Qs + stage * D, a.q + (long long)t.s * D, ROW_BYTES, &full[stage]);
       }
       __syncwarp();
-#pragma unroll
-      for (int half = 0; half < AT_TILE / 32; ++half) {
-        const int rl = half * 32 + lane;
-        const bool valid = rl < t.rows;
-        const uint16_t *kp = ta.k[half], *vp = ta.v[half];
-        const unsigned long long ka = (unsigned long long)kp, va = (unsigned long long)vp;
-        const unsigned long long kprev = __shfl_up_sync(0xffffffffu, ka, 1);
-        const unsigned long long vprev = __shfl_up_sync(0xffffffffu, va, 1);
-        const bool contiguous = valid && lane > 0 && ka == kprev + ROW_BYTES && va == vprev + ROW_BYTES;
-        const bool head = valid && !contiguous;
-        const unsigned headmask = __ballot_sync(0xffffffffu, head);
-        const unsigned validmask = __ballot_sync(0xffffffffu, valid);
+      uint16_t *kd = Ks + stage * AT_STAGE_ELEMS, *vd = Vs + stage * AT_STAGE_ELEMS;
+      if (!paged) {
+        if (t.rows > 0 && lane < 2)      // kept summary rows: one contiguous run per sequence
+          bulk_g2s(lane ? vd : kd, (lane ? a.vkept : a.kkept) + (sb + row0) * D, (uint32_t)t.rows * ROW_BYTES, &full[stage]);
+        return true;
+      }
+      int new_page = -1;
+      for (int x0 = 0; x0 < n_seg; x0 += 32) {
+        if (x0 > 0) load_pages(t.s, t.list, c0 + x0);
+        const TileSegment sg = tile_segment(row0, t.rows, v.C, c0 + x0 + lane);
+        const bool mine = x0 + lane < n_seg;
+        int page = __shfl_sync(0xffffffffu, pc_page, (sg.pos - pc_base) & 31);
+        if (mine && (page < 0 || page >= v.n_pages)) { set_status(v.status, ERR_CAPACITY); page = -1; }
+        // the segment with the row being appended ends one row earlier
+        const bool last = with_new && x0 + lane == n_seg - 1;
+        if (with_new && n_seg - 1 - x0 < 32) new_page = __shfl_sync(0xffffffffu, page, n_seg - 1 - x0);
+        const int len = mine ? sg.len - (last ? 1 : 0) : 0;
+        const long long off = ((long long)max(page, 0) * v.C + sg.r) * D;
+        uint32_t run = (uint32_t)len;
+        bool head = len > 0;
+        if (v.C < AT_MERGE_BELOW) {
+          // short chunks: pages that follow one another in memory travel as one copy
+          const long long end_prev = __shfl_up_sync(0xffffffffu, off + (long long)len * D, 1);
+          const int len_prev = __shfl_up_sync(0xffffffffu, len, 1);
+          head = len > 0 && !(lane > 0 && len_prev > 0 && off == end_prev);
+          const unsigned heads = __ballot_sync(0xffffffffu, head), live = __ballot_sync(0xffffffffu, len > 0);
+          const unsigned above = (lane == 31) ? 0u : (heads & ~((2u << lane) - 1u));
+          const int tail_lane = above ? __ffs(above) - 2 : 31 - __clz(live | 1u);      // last lane of the run (live lanes form a prefix)
+          const int run_end = __shfl_sync(0xffffffffu, sg.dst + len, tail_lane);
+          run = (uint32_t)(run_end - sg.dst);
+        }
         if (head) {
-          const unsigned above = (lane == 31) ? 0u : (headmask & ~((2u << lane) - 1u));
-          const int run_end = above ? (__ffs(above) - 1) : __popc(validmask);   // valid lanes form a prefix
-          const uint32_t bytes = (uint32_t)(run_end - lane) * ROW_BYTES;
-          bulk_g2s(Ks + stage * AT_STAGE_ELEMS + rl * D, kp, bytes, &full[stage]);
-          bulk_g2s(Vs + stage * AT_STAGE_ELEMS + rl * D, vp, bytes, &full[stage]);
+          bulk_g2s(kd + sg.dst * D, v.k_pages + off, run * ROW_BYTES, &full[stage]);
+          bulk_g2s(vd + sg.dst * D, v.v_pages + off, run * ROW_BYTES, &full[stage]);
+        }
+      }
+      if (with_new) {
+        if (lane < 2) bulk_g2s((lane ? vd : kd) + (t.rows - 1) * D, (lane ? a.v_new : a.k_new) + (long long)t.s * D, ROW_BYTES, &full[stage]);
+        // whoever streams the new row also stores it in its page (lanes 0-15 the K row, 16-31 the V row, 16 bytes each)
+        if (new_page >= 0) {
+          const int is_v = lane >> 4, l16 = lane & 15;
+          const uint4* src = reinterpret_cast<const uint4*>((is_v ? a.v_new : a.k_new) + (long long)t.s * D) + l16;
+          *(reinterpret_cast<uint4*>((is_v ? v.v_pages : v.k_pages) + ((long long)new_page * v.C + (g.n - 1) % v.C) * D) + l16) = __ldg(src);
         }
       }
       return true;
     };
-    // The first tiles go out as soon as each is resolved; from then on the addresses of tile i + 1 are
-    // looked up before the wait for its stage, i.e. while the consumers still work on the tiles in flight.
-    // The END description takes a stage of its own (no copies): that is how the consumers learn that they are done.
-    // fused append: whoever streams a sequence's last tail tile also stores the new token's row in its page
-    // (lanes 0-15 the K row, 16-31 the V row, 16 bytes each)
-    auto store_new_token = [&](const TileDesc& td) {
-      if (!g.appending || (td.flags & TF_END) || td.list != 0 || td.rows == 0 || td.j * AT_TILE + td.rows != g.n_tail) return;
-      const int pos = g.n - 1, chunk = pos / v.C, r = pos - chunk * v.C;
-      const long long page = v.page_table[(long long)td.s * v.max_chunks + chunk];
-      if (page < 0 || page >= v.n_pages) {
-        if (lane == 0) set_status(v.status, ERR_CAPACITY);
-        return;
-      }
-      const int is_v = lane >> 4, l16 = lane & 15;
-      const uint4* src = reinterpret_cast<const uint4*>((is_v ? a.v_new : a.k_new) + (long long)td.s * D) + l16;
-      uint4* dst = reinterpret_cast<uint4*>((is_v ? v.v_pages : v.k_pages) + (page * v.C + r) * D) + l16;
-      *dst = __ldg(src);
-    };
-    TileDesc d;
-    TileAddr t;
     for (int i = 0;; ++i) {
-      next_tile(d);
-      resolve(d, t);
-      store_new_token(d);
-      if (!issue(i, d, t) || (d.flags & TF_END)) break;
+      if (!issue(i, d) || (d.flags & TF_END)) break;
       KVE_STAMP(i == 0 && lane == 0, 2);
+      next_tile(d);
+    }
+    // Fused append: the length advances as soon as every CTA has read the old one, which is what the tickets count (nothing else
+    // in the launch reads it; later launches wait for this one to complete).
+    if (g.appending) {
+      __syncwarp();
+      int last = 0;
+      if (lane == 0) {
+        int arrived;
+        asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(arrived) : "l"(a.ticket) : "memory");
+        last = arrived == (int)gridDim.x - 1;
+      }
+      last = __shfl_sync(0xffffffffu, last, 0);
+      if (last) {
+        for (int b = lane; b < v.B; b += 32) v.seq_len[b] = g.n;
+        if (lane == 0) *a.ticket = 0;      // clean for the next launch
+      }
     }
     KVE_STAMP(lane == 0, 6);
   } else if (warp < AT_CWARPS) {
     // ================= consumer warps =================
+    pdl_wait();
     const float sl2 = a.scale * 1.44269504088896340736f;   // logits kept in log2 units
-    float qf[4] = {0.f, 0.f, 0.f, 0.f};
-    float m = -INFINITY, l = 0.f, acc[4] = {0.f, 0.f, 0.f, 0.f};
+    const int g8 = lane >> 2, tig = lane & 3;              // MMA fragment coordinates: rows g8 and g8 + 8 of the warp's 16
+    const int half = lane >> 4, l16 = lane & 15;           // p.V: rows 2 i + half, head dims 8 l16 .. + 7
+    uint4 qf[4];                                           // q as the B operand (the same in all eight columns): 8 dims from 8 (tig + 4 j)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) qf[j] = make_uint4(0u, 0u, 0u, 0u);
+    float m = -INFINITY, l = 0.f, acc[8];                  // l: this lane's rows only (replicated over tig), added up at the flush
+#pragma unroll
+    for (int x = 0; x < 8; ++x) acc[x] = 0.f;
     int n_flush = 0;
     for (int i = 0;; ++i) {
       const int stage = i % AT_STAGES, round = i / AT_STAGES;
@@ -397,46 +465,50 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
         break;
       }
       if (ti.z & TF_NEW) {
-        const uint2 qw = *reinterpret_cast<const uint2*>(Qs + stage * D + lane * 4);
-        qf[0] = bf16lo(qw.x); qf[1] = bf16hi(qw.x); qf[2] = bf16lo(qw.y); qf[3] = bf16hi(qw.y);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) qf[j] = *(reinterpret_cast<const uint4*>(Qs + stage * D) + tig + 4 * j);
         m = -INFINITY; l = 0.f;
-        acc[0] = acc[1] = acc[2] = acc[3] = 0.f;
+#pragma unroll
+        for (int x = 0; x < 8; ++x) acc[x] = 0.f;
       }
       const int nvalid = min(max(ti.y - warp * AT_SUB, 0), AT_SUB);
       if (nvalid > 0) {
-        const uint16_t* kt = Ks + stage * AT_STAGE_ELEMS + (warp * AT_SUB) * D + lane * 4;
-        const uint16_t* vt = Vs + stage * AT_STAGE_ELEMS + (warp * AT_SUB) * D + lane * 4;
-        float part[AT_SUB];
+        // ---- q.k of the warp's 16 rows: eight MMAs.  A lane fetches 8 consecutive head dims of a row at once; they feed the k
+        // positions of two MMAs, for K and q alike (a contraction does not notice the order).  All eight columns hold q, so
+        // every lane of a group of four ends up with the logits of its rows g8 and g8 + 8.
+        const uint4* kt = reinterpret_cast<const uint4*>(Ks + stage * AT_STAGE_ELEMS + (warp * AT_SUB) * D) + g8 * 16 + tig;
+        float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int r = 0; r < AT_SUB; ++r) {
-          const uint2 w = *reinterpret_cast<const uint2*>(kt + r * D);
-          part[r] = qf[0] * bf16lo(w.x);
-          part[r] = fmaf(qf[1], bf16hi(w.x), part[r]);
-          part[r] = fmaf(qf[2], bf16lo(w.y), part[r]);
-          part[r] = fmaf(qf[3], bf16hi(w.y), part[r]);
+        for (int j = 0; j < 4; ++j) {
+          const uint4 ra = kt[4 * j], rb = kt[4 * j + 8 * 16];
+          const uint32_t A0[4] = {ra.x, rb.x, ra.y, rb.y}, A1[4] = {ra.z, rb.z, ra.w, rb.w};
+          mma_bf16_16816(c0, A0, qf[j].x, qf[j].y);
+          mma_bf16_16816(c1, A1, qf[j].z, qf[j].w);
         }
-        KVE_TR_ROUND(16, 4)
-        KVE_TR_ROUND(8, 2)
-        KVE_TR_ROUND(4, 1)
-        float dot = part[0] + __shfl_xor_sync(0xffffffffu, part[0], 2);
-        dot += __shfl_xor_sync(0xffffffffu, dot, 1);                             // row (lane >> 2), full sum
-        const float logit = ((lane >> 2) < nvalid) ? dot * sl2 : -INFINITY;
-        const float m_new = fmaxf(m, warp_max(logit));
-        const float p = ex2_fast(logit - m_new);
+        // ---- online softmax ----
+        const float s0 = (g8 < nvalid) ? (c0[0] + c1[0]) * sl2 : -INFINITY;
+        const float s1 = (g8 + 8 < nvalid) ? (c0[2] + c1[2]) * sl2 : -INFINITY;
+        float mx = fmaxf(s0, s1);
+#pragma unroll
+        for (int o = 4; o <= 16; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        const float m_new = fmaxf(m, mx);
+        const float p0 = ex2_fast(s0 - m_new), p1 = ex2_fast(s1 - m_new);
         const float alpha = ex2_fast(m - m_new);
-        l = fmaf(l, alpha, 0.25f * warp_sum(p));    // every row sits on four lanes
+        l = fmaf(l, alpha, p0 + p1);
         m = m_new;
 #pragma unroll
-        for (int x = 0; x < 4; ++x) acc[x] *= alpha;
+        for (int x = 0; x < 8; ++x) acc[x] *= alpha;
+        // ---- p.V: half a warp per row, 16 bytes per lane ----
+        const uint4* vt = reinterpret_cast<const uint4*>(Vs + stage * AT_STAGE_ELEMS + (warp * AT_SUB) * D) + half * 16 + l16;
 #pragma unroll
-        for (int r = 0; r < AT_SUB; ++r) {
-          const float pr = __shfl_sync(0xffffffffu, p, 4 * r);
-          if (r < nvalid) {
-            const uint2 w = *reinterpret_cast<const uint2*>(vt + r * D);
-            acc[0] = fmaf(pr, bf16lo(w.x), acc[0]);
-            acc[1] = fmaf(pr, bf16hi(w.x), acc[1]);
-            acc[2] = fmaf(pr, bf16lo(w.y), acc[2]);
-            acc[3] = fmaf(pr, bf16hi(w.y), acc[3]);
+        for (int i2 = 0; i2 < 8; ++i2) {
+          const float pr = __shfl_sync(0xffffffffu, i2 < 4 ? p0 : p1, ((2 * i2 + half) & 7) * 4);
+          if (2 * i2 + half < nvalid) {            // rows beyond the tile's last one hold stale bytes
+            const uint4 w = vt[i2 * 32];
+            acc[0] = fmaf(pr, bf16lo(w.x), acc[0]); acc[1] = fmaf(pr, bf16hi(w.x), acc[1]);
+            acc[2] = fmaf(pr, bf16lo(w.y), acc[2]); acc[3] = fmaf(pr, bf16hi(w.y), acc[3]);
+            acc[4] = fmaf(pr, bf16lo(w.z), acc[4]); acc[5] = fmaf(pr, bf16hi(w.z), acc[5]);
+            acc[6] = fmaf(pr, bf16lo(w.w), acc[6]); acc[7] = fmaf(pr, bf16hi(w.w), acc[7]);
           }
         }
       }
@@ -450,8 +522,13 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
           break;
         }
         float* cw = comb + (fb * AT_CWARPS + warp) * ATTN_PARTIAL_FLOATS;
-        *reinterpret_cast<float4*>(cw + lane * 4) = make_float4(acc[0], acc[1], acc[2], acc[3]);
-        if (lane == 0) { cw[128] = m; cw[129] = l; }
+        float tot[8], lt = l;
+#pragma unroll
+        for (int x = 0; x < 8; ++x) tot[x] = acc[x] + __shfl_xor_sync(0xffffffffu, acc[x], 16);      // even + odd rows
+#pragma unroll
+        for (int o = 4; o <= 16; o <<= 1) lt += __shfl_xor_sync(0xffffffffu, lt, o);
+        *reinterpret_cast<float4*>(cw + l16 * 8 + half * 4) = half ? make_float4(tot[4], tot[5], tot[6], tot[7]) : make_float4(tot[0], tot[1], tot[2], tot[3]);
+        if (lane == 0) { cw[128] = m; cw[129] = lt; }
         if (warp == 0 && lane == 0) finfo[fb] = make_int4(ti.x, ti.w, 0, 0);
         __syncwarp();
         if (lane == 0) mbar_arrive(&ffull[fb]);      // release
@@ -460,6 +537,7 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
     }
   } else {
     // ================= merger warp =================
+    pdl_wait();
     for (int f = 0;; ++f) {
       const int fb = f & 1;
       if (!mbar_wait_bounded(&ffull[fb], (f >> 1) & 1)) {
@@ -469,7 +547,7 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
       const int4 fi = finfo[fb];                   // (sequence, -, -, -); sequence < 0: no more work
       const int s = fi.x;
       if (s < 0) break;
-      // ---- the eight consumer states -> one ----
+      // ---- the consumer states -> one ----
       const float* cb = comb + fb * AT_CWARPS * ATTN_PARTIAL_FLOATS;
       float mC = -INFINITY;
 #pragma unroll
@@ -488,7 +566,7 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
       if (lane == 0) mbar_arrive(&fempty[fb]);     // the exchange buffer may be refilled
 
       // ---- which CTAs hold parts of sequence s ----
-      const uint32_t c0 = piece_of((uint32_t)s * uk, g.I, g.P), c1 = piece_of((uint32_t)(s + 1) * uk - 1u, g.I, g.P);
+      const uint32_t c0 = piece_of((uint32_t)s * uk, n_items, n_pieces), c1 = piece_of((uint32_t)(s + 1) * uk - 1u, n_items, n_pieces);
       const int n_parts = (int)(c1 - c0 + 1u);
       if (n_parts > 1) {
         float* mine = a.partials + (long long)(s + c) * ATTN_PARTIAL_FLOATS;
@@ -535,21 +613,6 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
       o.y = pack_bf16x2(accC[2] * inv, accC[3] * inv);
       *reinterpret_cast<uint2*>(a.out + (long long)s * D + lane * 4) = o;
       if (a.lse && lane == 0) a.lse[s] = (lC > 0.f) ? (mC + log2f(lC)) * 0.69314718055994530942f : -INFINITY;
-    }
-    // fused append: every CTA read the old length when it started; the last one to get here publishes the new one
-    if (g.appending) {
-      __syncwarp();
-      int last = 0;
-      if (lane == 0) {
-        int arrived;
-        asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(arrived) : "l"(a.ticket) : "memory");
-        last = arrived == (int)gridDim.x - 1;
-      }
-      last = __shfl_sync(0xffffffffu, last, 0);
-      if (last) {
-        for (int b = lane; b < v.B; b += 32) v.seq_len[b] = g.n;
-        if (lane == 0) *a.ticket = 0;      // clean for the next launch
-      }
     }
     KVE_STAMP(lane == 0, 5);
   }

@@ -1257,3 +1257,25 @@ def test_whole_path_random_geometries(seed):
                         agg=agg, d_sum=d_sum, seed=60 + seed)
     pieces = tuple(sorted(rng.random(int(rng.integers(0, 3))).tolist())) + (1.0,)
     full_check(wl, str(rng.choice(["summary", "raw"])), pieces=pieces, keep=float(rng.choice([0.25, 0.5, 0.75])))
+
+
+@pytest.mark.parametrize("pages", [None, "random"])
+@pytest.mark.parametrize("C", [1, 8, 31, 32, 48, 200])
+def test_decode_step_over_tiles_of_many_and_of_broken_chunks(C, pages):
+    """A 64-row tile is copied chunk by chunk (chunks below 32 tokens: adjacent pages together): tiles of 64 chunks, of chunks
+    that straddle tiles, a new token that opens a tile, a page or both; every step against the oracle, pages byte-exact."""
+    b = _binding()
+    n0, steps = 126, 5
+    wl = wlm.Workload("tiles", B=1, H=3, n=n0, C=C, W=n0 + steps, d_g=64, n_append=steps, seed=90 + C)
+    K, V = wlm.gen_kv(wl, n=n0 + steps)
+    st = b.Store(B=1, H=3, C_=C, W=wl.W, max_tokens=n0 + steps, d_g=64, agg="mean", page_perm=pages, seed=C)
+    load_kv(st, 0, K[:, :n0], V[:, :n0])
+    oracle = kvo.Oracle("f64")
+    for n in range(n0, n0 + steps):
+        q = wlm.gen_q(wl, 0, n)
+        out = st.decode_step(0, b.bits_to_bf16(np.ascontiguousarray(K[:, n])), b.bits_to_bf16(np.ascontiguousarray(V[:, n])), b.bits_to_bf16(q))
+        want, _, _ = oracle.attn_dense(q, np.ascontiguousarray(K[:, :n + 1]), np.ascontiguousarray(V[:, :n + 1]), hz.SCALE)
+        hz.check_output(b.bf16_to_bits(out), want, f"C {C}, {n + 1} tokens")
+    assert st.poll_status() == 0
+    Kd, Vd = pages_to_plain(st, 0, n0 + steps)
+    assert np.array_equal(Kd, K) and np.array_equal(Vd, V)
