@@ -190,11 +190,16 @@ bool wrong_device(const kvE_store* st) {
 
 // How an attention launch is cut up.  Every sequence is cut into k equal parts and CTA c of G takes the contiguous
 // run of parts [c S k / G, (c + 1) S k / G), which it streams as one piece (no break between parts of one sequence).
-// G is one resident wave at most (two CTAs per SM).  k is chosen by a small cost model in microseconds, fitted to
-// measurements: a CTA takes about 1.4 us per 64-row tile whether it shares its SM or not (its eight consumer warps set
-// that pace; two CTAs per SM are what saturates HBM), so the launch lasts as long as the busiest CTA's tiles, plus its
-// end: about 0.5 us when every CTA owns whole sequences (k = 1), about 3.5 us and growing with the number of records
-// when sequences are shared and the last ones go through global memory (record, fence, ticket, merge).
+// G is one resident wave at most (two CTAs per SM).  k is chosen by a cost model in microseconds, fitted to
+// chains of kvE_decode_step launches (8 to 512 sequences of 64 to 16000 rows, every k on 148 and on 296 CTAs):
+//   the busiest CTA's 64-row tiles, 0.9 us each while every CTA has an SM to itself and 1.25 us in pairs;
+//   k > 1: a sequence's parts meet in global memory (record, ticket, merge): 1.7 us + 0.05 k;
+//   k > 1 and CTAs that hold pieces of several sequences: several such ends one after the other, 1.8 us more;
+//   never less than the bytes at 6.4 TB/s, under which the ends hide, plus 0.35 us for every tile that the busiest CTA
+//   has above the average (it runs on when the others have stopped).
+// The smallest k within 0.3 us of the best is taken.  What the lines separate, microseconds per launch: 128 sequences of 330 rows:
+// whole sequences 9.6, halves 9.9, thirds 12.3 (two kinds of CTA); 64: whole 9.6, thirds 8.6; 8: whole 9.1, sixths 7.7;
+// 256 of 330: whole 11.4, fifths 13.9; 60 of 2000: quarters 16.2, whole 35.9; 512 of 1090: quarters 49.7, halves 53.5; 512 of 4096: quarters 164, whole 168.
 struct AttnCut { int k, grid; };
 AttnCut attention_cut(const kvE_store* st, AttnMode mode, const LayerState& ls) {
   const long long n_upper = ls.reserve_upper > ls.n_tokens ? ls.reserve_upper : ls.n_tokens;
@@ -208,22 +213,23 @@ AttnCut attention_cut(const kvE_store* st, AttnMode mode, const LayerState& ls) 
   if (tiles < 1) tiles = 1;
   const long long G = st->attn_grid_max, S = st->S;
   const long long k_max = tiles < MAX_SPLITS ? tiles : MAX_SPLITS;
-  auto cost_of = [&](long long k, long long* grid_out) {
+  const double hbm_us = (double)S * (double)(tail + lead) * 512.0 / 6.4e6;
+  auto cost_of = [&](long long k) {
     const long long parts = S * k, grid = parts < G ? parts : G;
     const long long rounds = (parts + grid - 1) / grid;                 // parts of the busiest CTA
-    if (grid_out) *grid_out = grid;
-    return (double)rounds * (double)tiles / (double)k * 1.4 + (k > 1 ? 4.5 + 0.06 * (double)k : 0.5);
+    const double busiest = rounds == 1 ? (double)((tiles + k - 1) / k) : (double)rounds * (double)tiles / (double)k;
+    const double ends = k == 1 ? 0.0 : 1.7 + 0.05 * (double)k + (rounds > 1 ? 1.8 : 0.0);
+    const double us = busiest * (2 * grid <= G ? 0.9 : 1.25) + ends;
+    const double stream = hbm_us + 0.35 * (busiest - (double)(S * tiles) / (double)grid);
+    return us > stream ? us : stream;
   };
   // the kernel cuts the parts up in 32-bit arithmetic: S k (G + 1) must stay below 2^32
   double best = 1e30;
   for (long long k = 1; k <= k_max && S * k * (G + 1) < (1LL << 32); ++k)
-    if (cost_of(k, nullptr) < best) best = cost_of(k, nullptr);
-  long long k_pick = 1;      // whole sequences only when that is the cheapest; else near-ties go to the finer cut (evener bytes per CTA)
-  for (long long k = 2; k <= k_max && S * k * (G + 1) < (1LL << 32); ++k)
-    if (cost_of(k, nullptr) <= best + 0.3 && cost_of(1, nullptr) > best + 1e-9) k_pick = k;
-  long long grid = 1;
-  cost_of(k_pick, &grid);
-  return AttnCut{(int)k_pick, (int)grid};
+    if (cost_of(k) < best) best = cost_of(k);
+  long long k_pick = 1;
+  while (cost_of(k_pick) > best + 0.3) ++k_pick;
+  return AttnCut{(int)k_pick, (int)(S * k_pick < G ? S * k_pick : G)};
 }
 
 struct KeptRows { void *k, *v; };      // kept summary rows of a layer, compacted by kvE_compact
