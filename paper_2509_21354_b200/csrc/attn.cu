@@ -11,21 +11,25 @@
 //    without draining, every CTA moves nearly the same number of bytes whatever S is, and where a
 //    part begins follows from the launch arguments, the stored length and one keep count, so the
 //    first copies leave two dependent loads after the kernel starts.
-//  * Warp 4 (producer) turns tiles into copies (TMA engine, global -> shared, mbarrier byte counting): one K and one V copy per
+//  * Warp 8 (producer) turns tiles into copies (TMA engine, global -> shared, mbarrier byte counting): one K and one V copy per
 //    chunk that a tile touches (kept summary rows sit compacted in one run per sequence: one copy), into a 3-stage ring
-//    of 64-row tiles.  The query row of a sequence travels with the first tile of that sequence.  Page ids of 32 chunks
-//    wait in the lanes' registers, so that a tile costs the warp shuffles and not a table look-up; before, every lane looked
-//    up the page of each of its rows and runs were found again with a ballot, which held the ring back: 512 sequences of
-//    1100 rows 56.7 us a step (5.0 TB/s), now 49.8 us (5.75 TB/s).
-//  * While the predecessor on the stream still runs, the producer goes through its first tile once on what the tables hold (a
+//    of 64-row tiles.  The query row of a sequence travels with the first tile of that sequence.  Up to 32 tiles are worked
+//    out side by side, one per lane (page ids included), and the lanes take turns at issuing theirs: a tile costs the
+//    waits and the copies.  With the work done tile by tile the warp needed 1700 cycles a tile (divisions by the chunk
+//    size, shuffles, 64-bit addresses) and held everything back: 8 layers of 128 sequences x 330 rows 9.75 us a
+//    layer, 8.75 us so.  (With the page of every ROW looked up, 512 sequences x 1100 rows took 56.7 us, 5.0 TB/s;
+//    49.8 us now.)
+//  * While the predecessor on the stream still runs, the producer goes through its first tiles once on what the tables hold (a
 //    guess, repeated with the real values after the wait) and the consumers pull the guessed rows of two tiles into L2:
-//    8 layers of 128 sequences x 330 rows, one after the other, 12.7 -> 11.4 us a layer.
-//  * Warps 0-3 (consumers) each take 16 rows of a tile.  The logits q.k are eight warp-level MMAs (the rows are the M side, q
-//    fills the N side: bf16 products, fp32 sums), which leaves a group of four lanes with the logits of two rows; online
+//    12.7 -> 11.4 us a layer in that setting.
+//  * Warps 0-7 (consumers) are two groups of four that take tiles in turn, 16 rows per warp.  (One group: 8.75 us a layer, two:
+//    8.2 us - a tile is ~1400 cycles of dependent steps, and two of them now run at a time.)  The logits q.k are eight
+//    warp-level MMAs (the rows are the M side, q fills the N side: bf16 products, fp32 sums), which leaves a group of
+//    four lanes with the logits of two rows; online
 //    softmax with warp shuffles, then p.V in fp32 with half a warp per row and 8 output dims per lane.  When a CTA's run
 //    leaves a sequence, the consumers drop their (m, l, acc) into a double-buffered exchange area and carry on with the
 //    next sequence.
-//  * Warp 5 (merger) folds the four consumer states of a finished sequence (or part of one), and
+//  * Warp 9 (merger) folds the eight consumer states of a finished sequence (or part of one), and
 //    either writes the output (this CTA had the whole sequence) or a partial record plus an atomic
 //    ticket; the CTA that draws a sequence's last ticket merges its records by log-sum-exp.  Nobody
 //    spins on another CTA.
@@ -56,12 +60,14 @@ __device__ __forceinline__ void stamp(int slot) {
 
 constexpr int AT_TILE = ATTN_TILE_ROWS;       // rows per stage
 constexpr int AT_STAGES = 3;
-constexpr int AT_CWARPS = 4;                  // consumer warps
-constexpr int AT_SUB = AT_TILE / AT_CWARPS;   // 16 rows per consumer warp per tile: the rows of one m16n8k16 MMA
+constexpr int AT_CGROUPS = 2;                 // consumer groups, which take tiles in turn
+constexpr int AT_GWARPS = 4;                  // warps of a group
+constexpr int AT_CWARPS = AT_CGROUPS * AT_GWARPS;
+constexpr int AT_SUB = AT_TILE / AT_GWARPS;   // 16 rows per warp per tile: the rows of one m16n8k16 MMA
 constexpr int AT_PRODUCER = AT_CWARPS;        // warp ids
 constexpr int AT_THREADS = (AT_CWARPS + 2) * 32;
 constexpr int AT_STAGE_ELEMS = AT_TILE * D;   // bf16 elements of one K (or V) tile
-constexpr int AT_MERGE_BELOW = 32;            // chunks shorter than this: copies of adjacent pages are merged
+constexpr int AT_LANE_SEGS = 3;               // chunks a tile may touch for one lane to issue its copies: chunks of 32 tokens and more
 constexpr int AT_PREFETCH_TILES = 2;          // most tiles a CTA pulls into L2 before its predecessor has finished
 static_assert(AT_SUB == 16, "the logits of a warp's rows are one m16n8k16 tile");
 
@@ -83,8 +89,23 @@ constexpr int TF_NEW = 1;      // first tile of a (sequence, list) in this CTA: 
 constexpr int TF_FLUSH = 2;    // last tile of a (sequence, list) in this CTA: hand the state to the merger afterwards
 constexpr int TF_END = 4;      // no tile: the CTA's work is done
 
+// x / d for x < 2^31 as a multiplication (a runtime divisor costs the producer a chain of some twenty instructions)
+struct FastDiv {
+  uint32_t mul, shift;
+  __device__ __forceinline__ uint32_t div(uint32_t x) const { return (uint32_t)(((uint64_t)x * mul) >> shift); }
+};
+static FastDiv fast_div(uint32_t d) {      // mul = ceil(2^shift / d) with 2^(shift - 31) >= d: exact below 2^31
+  FastDiv f;
+  uint32_t log2_up = 0;
+  while ((1u << log2_up) < d) ++log2_up;
+  f.shift = 31 + log2_up;
+  f.mul = (uint32_t)(((1ull << f.shift) + d - 1) / d);
+  return f;
+}
+
 struct AttnArgs {
   LayerView v;
+  FastDiv by_c, by_k;          // by the chunk size, by k
   int mode;
   int n_chunks;                // the host's count of chunks under the keep list: a prefetch hint; the kernel reads the device's
   int k;                       // parts per sequence
@@ -142,9 +163,14 @@ __device__ __forceinline__ int lead_rows_from(const AttnArgs& a, const AttnGeo& 
   if (a.mode == ATTN_DENSE || g.n_chunks <= 0) return 0;
   return min(max(keep_cnt, 0), g.n_chunks) * g.per;
 }
-// one tile of the CTA's work as the producer sees it
-struct TileDesc {
-  int s, list, j, rows, flags;      // list 0: raw tail, 1: kept chunks; j: tile index inside the sequence's list
+// up to 32 tiles of one sequence as the producer sees them, one per lane
+struct TilePlan {
+  int n, s;                         // tiles of the batch, their sequence (the same in every lane)
+  int list, rows, flags;            // list 0: raw tail, 1: kept chunks
+  int row0, c0, n_seg;              // first row in the list; its chunk (kept chunks: position in the keep list); chunks the tile touches
+  int page[AT_LANE_SEGS];           // their pages (-1: none), when there are no more than that
+  int i_new, new_page;              // the tile that ends with the token being appended (-1: none), that token's page
+  uint4 new_row;                    // this lane's 16 bytes of it
 };
 
 // The rows of a tile that lie in one chunk: `pos` is the chunk (raw tail) or the index in the keep list (kept chunks at full
@@ -197,7 +223,7 @@ __device__ __forceinline__ void prefetch_first_tiles(const AttnArgs& a, uint32_t
       continue;
     }
     const int row0 = (tail ? g.raw0 : 0) + jj * AT_TILE;
-    const TileSegment sg = tile_segment(row0, rows, v.C, row0 / v.C + lane);
+    const TileSegment sg = tile_segment(row0, rows, v.C, (int)a.by_c.div((uint32_t)row0) + lane);
     if (sg.len <= 0 || sg.pos >= v.max_chunks) continue;
     const int chunk = tail ? sg.pos : load_hint(v.keep_idx + sb + sg.pos);
     if (chunk < 0 || chunk >= v.max_chunks) continue;
@@ -248,70 +274,74 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
   __syncthreads();
   if (warp == AT_PRODUCER) {
     // ================= producer warp =================
-    // walks the CTA's parts in order, sequence by sequence; within a sequence the tiles [j_lo, j_hi) that
-    // its parts in this CTA cover (part p of a sequence with T tiles: tiles [p T / k, (p + 1) T / k))
+    // walks the CTA's parts in order, sequence by sequence; within a sequence the tiles [j, j_hi) that its parts in this CTA
+    // cover (part p of a sequence with T tiles: tiles [p T / k, (p + 1) T / k))
     const int s_first = (int)(i0 / uk), s_last = i0 < i1 ? (int)((i1 - 1u) / uk) : s_first;
     AttnGeo g;
-    int s = s_first, j = 0, j_hi = 0, lt_rows = 0, tiles = 0;
-    bool fresh = true;                      // the next tile is the first one of sequence s in this CTA
-    bool done = i0 >= i1;
+    int s = s_first, j = 0, j_hi = 0, lt_rows = 0, keep_next = 0;
+    bool fresh = true, done = i0 >= i1;
     auto enter_sequence = [&](int keep_cnt) {
       lt_rows = lead_rows_from(a, g, keep_cnt);
-      tiles = g.TT + (lt_rows + AT_TILE - 1) / AT_TILE;
+      const uint32_t tiles = (uint32_t)(g.TT + (lt_rows + AT_TILE - 1) / AT_TILE);
       // part p of the sequence's tiles: [p tiles / k, (p + 1) tiles / k); p <= 32 and tiles < 2^20, so 32 bits do
       const uint32_t p_lo = (s == s_first) ? i0 - (uint32_t)s * uk : 0u;
       const uint32_t p_hi = (s == s_last) ? i1 - (uint32_t)s * uk : uk;
-      j = (int)((p_lo * (uint32_t)tiles) / uk);
-      j_hi = (int)((p_hi * (uint32_t)tiles) / uk);
+      j = (int)a.by_k.div(p_lo * tiles);
+      j_hi = (int)a.by_k.div(p_hi * tiles);
       fresh = true;
-    };
-    auto next_tile = [&](TileDesc& t) {
-      if (done) {
-        t.s = -1; t.list = 0; t.j = 0; t.rows = 0; t.flags = TF_END;
-        return;
-      }
-      t.s = s;
-      if (j >= j_hi) {
-        // parts without a tile (fewer tiles than parts, or a sequence without a retained row): an empty tile keeps
-        // the bookkeeping uniform - the merger still gets this CTA's (empty) share of the sequence
-        t.list = 0; t.j = 0; t.rows = 0;
-        t.flags = TF_NEW | TF_FLUSH;
-      } else {
-        t.list = j >= g.TT ? 1 : 0;
-        t.j = t.list ? j - g.TT : j;
-        t.rows = min(AT_TILE, (t.list ? lt_rows : g.n_tail) - t.j * AT_TILE);
-        t.flags = (fresh ? TF_NEW : 0) | (j + 1 >= j_hi ? TF_FLUSH : 0);
-        fresh = false;
-        ++j;
-      }
-      if (t.flags & TF_FLUSH) {
-        if (s == s_last) done = true;
-        else {
-          ++s;
-          if (s < s_last) prefetch_sequence_metadata(a, s + 1, lane);      // the next one's look-ups will hit L2
-          enter_sequence((a.mode == ATTN_DENSE || g.n_chunks <= 0) ? 0 : load_hint(v.keep_cnt + s));
-        }
+      if (s < s_last) {      // the next one's look-ups: its keep count now, the rest into L2
+        keep_next = (a.mode == ATTN_DENSE) ? 0 : load_hint(v.keep_cnt + s + 1);
+        prefetch_sequence_metadata(a, s + 1, lane);
       }
     };
-    // Page ids of 32 consecutive entries of a sequence's chunk list (tail: chunk numbers, kept: positions in the keep list), one
-    // per lane: a tile spans two or three chunks, so the table is looked at once in 20 tiles or more instead of on
-    // every tile.  Entries that name nothing become -1 and are flagged when a tile uses them.
-    int pc_key = -1, pc_base = 0, pc_page = -1;
-    auto load_pages = [&](int seq, int list, int base) {
+    auto page_of = [&](int seq, int list, int pos) -> int {      // -1: names nothing
       const long long sb = (long long)seq * v.max_chunks;
-      int chunk = base + lane;
-      if (list != 0) chunk = chunk < v.max_chunks ? load_hint(v.keep_idx + sb + chunk) : -1;
-      const bool named = chunk >= 0 && chunk < (list != 0 ? g.n_chunks : v.max_chunks);
-      pc_page = named ? load_hint(v.page_table + sb + chunk) : -1;
-      pc_key = seq * 2 + list;
-      pc_base = base;
+      int chunk = pos;
+      if (list != 0) chunk = pos < v.max_chunks ? load_hint(v.keep_idx + sb + pos) : -1;
+      return (chunk >= 0 && chunk < (list != 0 ? g.n_chunks : v.max_chunks)) ? load_hint(v.page_table + sb + chunk) : -1;
+    };
+    // The next tiles of a sequence, up to 32, worked out side by side: lane i holds tile i and will issue its copies.  `guess`: a
+    // plan whose page ids are taken over where it looked at the same tail chunks.
+    auto make_plan = [&](TilePlan& p, const TilePlan* guess) {
+      p.n = 0;
+      p.i_new = -1;
+      if (done) return;
+      const int left = j_hi - j, idx = j + lane;
+      p.n = min(32, max(left, 1));       // parts without a tile: an empty one keeps the bookkeeping uniform
+      p.s = s;
+      p.list = idx >= g.TT ? 1 : 0;
+      const int jj = p.list ? idx - g.TT : idx;
+      p.rows = lane < left ? min(AT_TILE, (p.list ? lt_rows : g.n_tail) - jj * AT_TILE) : 0;
+      p.flags = (fresh && lane == 0 ? TF_NEW : 0) | (idx + 1 >= j_hi ? TF_FLUSH : 0);
+      p.row0 = (p.list ? 0 : g.raw0) + jj * AT_TILE;
+      p.c0 = (int)a.by_c.div((uint32_t)p.row0);
+      p.n_seg = (p.rows > 0 && (p.list == 0 || a.mode == ATTN_RAW)) ? (int)a.by_c.div((uint32_t)(p.row0 + p.rows - 1)) - p.c0 + 1 : 0;
+      if (p.n_seg <= AT_LANE_SEGS) {
+        const bool known = guess != nullptr && p.list == 0 && guess->list == 0 && guess->c0 == p.c0 && guess->n_seg >= p.n_seg;
+#pragma unroll
+        for (int x = 0; x < AT_LANE_SEGS; ++x) p.page[x] = known ? guess->page[x] : (x < p.n_seg ? page_of(s, p.list, p.c0 + x) : -1);
+      }
+      // fused append: the last row of the tail is the new token; whoever streams it also stores it in its page (lanes 0-15 the K
+      // row, 16-31 the V row, 16 bytes each)
+      const int i_new = g.TT - 1 - j;
+      if (g.appending && i_new >= 0 && i_new < min(32, left)) {
+        p.i_new = i_new;
+        p.new_page = page_of(s, 0, (int)a.by_c.div((uint32_t)(g.n - 1)));
+        p.new_row = __ldcg(reinterpret_cast<const uint4*>((lane >> 4 ? a.v_new : a.k_new) + (long long)s * D) + (lane & 15));
+      }
+      j += p.n;
+      fresh = false;
+      if (j >= j_hi) {
+        if (s == s_last) done = true;
+        else { ++s; enter_sequence(keep_next); }
+      }
     };
 
-    // The first tile is worked out twice: once from what the tables hold while the predecessor still runs - only a guess at
+    // The first tiles are worked out twice: once from what the tables hold while the predecessor still runs - only a guess at
     // where to look, and a way to have the code at hand - and again from the real values, when the look-ups of the
     // length, the coverage, the keep count and the guessed page ids go out together.
-    TileDesc d;
-    int guess_key = -1, guess_base = 0;
+    TilePlan cur, nxt;
+    nxt.n = 0;
 #pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {
       if (pass == 1) {
@@ -323,95 +353,106 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
       // gate triggers that happened since it was captured (the launch argument is only the host's view at capture time)
       const int listed = (a.mode == ATTN_DENSE) ? 0 : load_hint(v.n_listed);
       const int keep_cnt = (a.mode == ATTN_DENSE || i0 >= i1) ? 0 : load_hint(v.keep_cnt + s_first);
-      if (guess_key >= 0 && (guess_key & 1) == 0) load_pages(guess_key >> 1, 0, guess_base);
-      g = make_geometry(a, len_stored, listed);
-      if (i0 >= i1) { next_tile(d); continue; }
-      s = s_first;
-      done = false;
-      enter_sequence(keep_cnt);
-      next_tile(d);
-      if (pass == 0) {
-        const int row0 = (d.list == 0 ? g.raw0 : 0) + d.j * AT_TILE;
-        if (d.rows > 0 && (d.list == 0 || a.mode == ATTN_RAW)) { guess_key = s_first * 2 + d.list; guess_base = row0 / v.C; }
+      if (pass == 1 && cur.n > 0) {
+        nxt = cur;
+#pragma unroll
+        for (int x = 0; x < AT_LANE_SEGS; ++x) nxt.page[x] = (nxt.list == 0 && x < nxt.n_seg) ? page_of(s_first, 0, nxt.c0 + x) : -1;
       }
+      g = make_geometry(a, len_stored, listed);
+      s = s_first;
+      done = i0 >= i1;
+      if (!done) enter_sequence(keep_cnt);
+      make_plan(cur, pass == 1 && nxt.n > 0 ? &nxt : nullptr);
     }
     if (a.k_new != nullptr && !g.appending && blockIdx.x == 0 && lane == 0) set_status(v.status, ERR_CAPACITY);   // cache full
 
-    // waits for the stage, publishes the tile's description, issues its copies; false on a timed-out wait.
-    // The END description takes a stage of its own (no copies): that is how the consumers learn that they are done.
-    auto issue = [&](int i, const TileDesc& t) -> bool {
-      const int stage = i % AT_STAGES, round = i / AT_STAGES;
-      const long long sb = (long long)t.s * v.max_chunks;
-      const int row0 = (t.list == 0 ? g.raw0 : 0) + t.j * AT_TILE;
-      const int c0 = row0 / v.C;
-      const bool paged = t.rows > 0 && (t.list == 0 || a.mode == ATTN_RAW);
-      const int n_seg = paged ? (row0 + t.rows - 1) / v.C - c0 + 1 : 0;
-      // fused append: the last row of the tail is the new token, straight from the caller's buffers
-      const bool with_new = g.appending && t.list == 0 && t.rows > 0 && t.j * AT_TILE + t.rows == g.n_tail;
-      if (paged && (pc_key != t.s * 2 + t.list || c0 < pc_base || c0 + min(n_seg, 32) > pc_base + 32)) load_pages(t.s, t.list, c0);
-      if (round > 0 && !mbar_wait_bounded(&empty[stage], (round - 1) & 1)) {
-        if (lane == 0) set_status(v.status, ERR_TIMEOUT);
-        return false;
-      }
-      if (lane == 0) {
-        info[stage] = make_int4(t.s, t.rows, t.flags, t.list);
-        const bool with_q = (t.flags & TF_NEW) != 0;
-        const uint32_t bytes = (uint32_t)t.rows * 2u * ROW_BYTES + (with_q ? (uint32_t)ROW_BYTES : 0u);
-        mbar_arrive_expect_tx(&full[stage], bytes);      // release: the description is visible to whoever sees the phase
-        if (with_q) bulk_g2s(Qs + stage * D, a.q + (long long)t.s * D, ROW_BYTES, &full[stage]);
-      }
-      __syncwarp();
+    // The copies of tile i of the batch: lane i waits for the stage, publishes the tile's description and issues one K and one V
+    // copy per chunk the tile touches, all from its own registers; the lanes take turns.  Chunks so short that a tile
+    // has more than AT_LANE_SEGS of them: the whole warp, 32 chunks at a time.  False on a timed-out wait.
+    int it = 0;
+    auto issue = [&](const TilePlan& p, int i) -> bool {
+      const int stage = it % AT_STAGES, round = it / AT_STAGES;
+      ++it;
       uint16_t *kd = Ks + stage * AT_STAGE_ELEMS, *vd = Vs + stage * AT_STAGE_ELEMS;
-      if (!paged) {
-        if (t.rows > 0 && lane < 2)      // kept summary rows: one contiguous run per sequence
-          bulk_g2s(lane ? vd : kd, (lane ? a.vkept : a.kkept) + (sb + row0) * D, (uint32_t)t.rows * ROW_BYTES, &full[stage]);
-        return true;
-      }
-      int new_page = -1;
-      for (int x0 = 0; x0 < n_seg; x0 += 32) {
-        if (x0 > 0) load_pages(t.s, t.list, c0 + x0);
-        const TileSegment sg = tile_segment(row0, t.rows, v.C, c0 + x0 + lane);
-        const bool mine = x0 + lane < n_seg;
-        int page = __shfl_sync(0xffffffffu, pc_page, (sg.pos - pc_base) & 31);
-        if (mine && (page < 0 || page >= v.n_pages)) { set_status(v.status, ERR_CAPACITY); page = -1; }
-        // the segment with the row being appended ends one row earlier
-        const bool last = with_new && x0 + lane == n_seg - 1;
-        if (with_new && n_seg - 1 - x0 < 32) new_page = __shfl_sync(0xffffffffu, page, n_seg - 1 - x0);
-        const int len = mine ? sg.len - (last ? 1 : 0) : 0;
-        const long long off = ((long long)max(page, 0) * v.C + sg.r) * D;
-        uint32_t run = (uint32_t)len;
-        bool head = len > 0;
-        if (v.C < AT_MERGE_BELOW) {
-          // short chunks: pages that follow one another in memory travel as one copy
-          const long long end_prev = __shfl_up_sync(0xffffffffu, off + (long long)len * D, 1);
-          const int len_prev = __shfl_up_sync(0xffffffffu, len, 1);
-          head = len > 0 && !(lane > 0 && len_prev > 0 && off == end_prev);
-          const unsigned heads = __ballot_sync(0xffffffffu, head), live = __ballot_sync(0xffffffffu, len > 0);
-          const unsigned above = (lane == 31) ? 0u : (heads & ~((2u << lane) - 1u));
-          const int tail_lane = above ? __ffs(above) - 2 : 31 - __clz(live | 1u);      // last lane of the run (live lanes form a prefix)
-          const int run_end = __shfl_sync(0xffffffffu, sg.dst + len, tail_lane);
-          run = (uint32_t)(run_end - sg.dst);
-        }
-        if (head) {
-          bulk_g2s(kd + sg.dst * D, v.k_pages + off, run * ROW_BYTES, &full[stage]);
-          bulk_g2s(vd + sg.dst * D, v.v_pages + off, run * ROW_BYTES, &full[stage]);
-        }
-      }
-      if (with_new) {
-        if (lane < 2) bulk_g2s((lane ? vd : kd) + (t.rows - 1) * D, (lane ? a.v_new : a.k_new) + (long long)t.s * D, ROW_BYTES, &full[stage]);
-        // whoever streams the new row also stores it in its page (lanes 0-15 the K row, 16-31 the V row, 16 bytes each)
-        if (new_page >= 0) {
-          const int is_v = lane >> 4, l16 = lane & 15;
-          const uint4* src = reinterpret_cast<const uint4*>((is_v ? a.v_new : a.k_new) + (long long)t.s * D) + l16;
-          *(reinterpret_cast<uint4*>((is_v ? v.v_pages : v.k_pages) + ((long long)new_page * v.C + (g.n - 1) % v.C) * D) + l16) = __ldg(src);
+      const bool with_new = i == p.i_new;
+      bool ok = true;
+      if (lane == i) {
+        ok = round == 0 || mbar_wait_bounded(&empty[stage], (round - 1) & 1);
+        if (ok) {
+          info[stage] = make_int4(p.s, p.rows, p.flags, p.list);
+          const bool with_q = (p.flags & TF_NEW) != 0;
+          mbar_arrive_expect_tx(&full[stage], (uint32_t)p.rows * 2u * ROW_BYTES + (with_q ? (uint32_t)ROW_BYTES : 0u));      // release: whoever sees the phase sees the description
+          if (p.n_seg > 0 && p.n_seg <= AT_LANE_SEGS) {
+            int r = p.row0 - p.c0 * v.C, dst = 0, rest = p.rows - (with_new ? 1 : 0);
+#pragma unroll
+            for (int x = 0; x < AT_LANE_SEGS; ++x) {
+              const int len = min(v.C - r, rest);
+              if (len > 0) {
+                int page = p.page[x];
+                if (page < 0 || page >= v.n_pages) { set_status(v.status, ERR_CAPACITY); page = 0; }
+                const long long off = ((long long)page * v.C + r) * D;
+                bulk_g2s(kd + dst * D, v.k_pages + off, (uint32_t)len * ROW_BYTES, &full[stage]);
+                bulk_g2s(vd + dst * D, v.v_pages + off, (uint32_t)len * ROW_BYTES, &full[stage]);
+              }
+              dst += len; rest -= len; r = 0;
+            }
+          } else if (p.n_seg == 0 && p.rows > 0) {      // kept summary rows: one contiguous run per sequence
+            const long long off = ((long long)p.s * v.max_chunks + p.row0) * D;
+            bulk_g2s(kd, a.kkept + off, (uint32_t)p.rows * ROW_BYTES, &full[stage]);
+            bulk_g2s(vd, a.vkept + off, (uint32_t)p.rows * ROW_BYTES, &full[stage]);
+          }
+          if (with_new) {
+            bulk_g2s(kd + (p.rows - 1) * D, a.k_new + (long long)p.s * D, ROW_BYTES, &full[stage]);
+            bulk_g2s(vd + (p.rows - 1) * D, a.v_new + (long long)p.s * D, ROW_BYTES, &full[stage]);
+          }
+          if (with_q) bulk_g2s(Qs + stage * D, a.q + (long long)p.s * D, ROW_BYTES, &full[stage]);
+        } else {
+          set_status(v.status, ERR_TIMEOUT);
         }
       }
-      return true;
+      ok = __shfl_sync(0xffffffffu, (int)ok, i) != 0;
+      if (v.C < AT_TILE / (AT_LANE_SEGS - 1)) {
+        const int n_seg = __shfl_sync(0xffffffffu, p.n_seg, i);
+        if (ok && n_seg > AT_LANE_SEGS) {
+          const int row0 = __shfl_sync(0xffffffffu, p.row0, i), c0 = __shfl_sync(0xffffffffu, p.c0, i);
+          const int rows = __shfl_sync(0xffffffffu, p.rows, i) - (with_new ? 1 : 0), list = __shfl_sync(0xffffffffu, p.list, i);
+          for (int x = lane; x < n_seg; x += 32) {
+            const TileSegment sg = tile_segment(row0, rows, v.C, c0 + x);
+            if (sg.len <= 0) continue;
+            int page = page_of(p.s, list, sg.pos);
+            if (page < 0 || page >= v.n_pages) { set_status(v.status, ERR_CAPACITY); page = 0; }
+            const long long off = ((long long)page * v.C + sg.r) * D;
+            bulk_g2s(kd + sg.dst * D, v.k_pages + off, (uint32_t)sg.len * ROW_BYTES, &full[stage]);
+            bulk_g2s(vd + sg.dst * D, v.v_pages + off, (uint32_t)sg.len * ROW_BYTES, &full[stage]);
+          }
+          __syncwarp();
+        }
+      }
+      return ok;
     };
-    for (int i = 0;; ++i) {
-      if (!issue(i, d) || (d.flags & TF_END)) break;
-      KVE_STAMP(i == 0 && lane == 0, 2);
-      next_tile(d);
+    bool ok = true;
+    while (ok && cur.n > 0) {
+      for (int i = 0; ok && i < cur.n; ++i) {
+        if (i == cur.n - 1) make_plan(nxt, nullptr);      // its look-ups run while this batch's last copies are issued
+        ok = issue(cur, i);
+        KVE_STAMP(it == 1 && lane == 0, 2);
+      }
+      if (cur.i_new >= 0) {
+        if (cur.new_page >= 0 && cur.new_page < v.n_pages)
+          *(reinterpret_cast<uint4*>((lane >> 4 ? v.v_pages : v.k_pages) + ((long long)cur.new_page * v.C + (g.n - 1 - (int)a.by_c.div((uint32_t)(g.n - 1)) * v.C)) * D) + (lane & 15)) = cur.new_row;
+        else if (lane == 0) set_status(v.status, ERR_CAPACITY);
+      }
+      cur = nxt;
+    }
+    // a description without a tile takes a stage of its own (no copies): that is how the consumers learn that they are done
+    if (ok && lane == 0) {
+      const int stage = it % AT_STAGES, round = it / AT_STAGES;
+      if (round == 0 || mbar_wait_bounded(&empty[stage], (round - 1) & 1)) {
+        info[stage] = make_int4(-1, 0, TF_END, 0);
+        mbar_arrive(&full[stage]);
+      } else {
+        set_status(v.status, ERR_TIMEOUT);
+      }
     }
     // Fused append: the length advances as soon as every CTA has read the old one, which is what the tickets count (nothing else
     // in the launch reads it; later launches wait for this one to complete).
@@ -434,6 +475,7 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
     // ================= consumer warps =================
     pdl_wait();
     const float sl2 = a.scale * 1.44269504088896340736f;   // logits kept in log2 units
+    const int gwarp = warp % AT_GWARPS;
     const int g8 = lane >> 2, tig = lane & 3;              // MMA fragment coordinates: rows g8 and g8 + 8 of the warp's 16
     const int half = lane >> 4, l16 = lane & 15;           // p.V: rows 2 i + half, head dims 8 l16 .. + 7
     uint4 qf[4];                                           // q as the B operand (the same in all eight columns): 8 dims from 8 (tig + 4 j)
@@ -471,12 +513,12 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
 #pragma unroll
         for (int x = 0; x < 8; ++x) acc[x] = 0.f;
       }
-      const int nvalid = min(max(ti.y - warp * AT_SUB, 0), AT_SUB);
+      const int nvalid = i % AT_CGROUPS == warp / AT_GWARPS ? min(max(ti.y - gwarp * AT_SUB, 0), AT_SUB) : 0;      // the other groups' tiles: only their flags
       if (nvalid > 0) {
         // ---- q.k of the warp's 16 rows: eight MMAs.  A lane fetches 8 consecutive head dims of a row at once; they feed the k
         // positions of two MMAs, for K and q alike (a contraction does not notice the order).  All eight columns hold q, so
         // every lane of a group of four ends up with the logits of its rows g8 and g8 + 8.
-        const uint4* kt = reinterpret_cast<const uint4*>(Ks + stage * AT_STAGE_ELEMS + (warp * AT_SUB) * D) + g8 * 16 + tig;
+        const uint4* kt = reinterpret_cast<const uint4*>(Ks + stage * AT_STAGE_ELEMS + (gwarp * AT_SUB) * D) + g8 * 16 + tig;
         float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
@@ -499,7 +541,7 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
 #pragma unroll
         for (int x = 0; x < 8; ++x) acc[x] *= alpha;
         // ---- p.V: half a warp per row, 16 bytes per lane ----
-        const uint4* vt = reinterpret_cast<const uint4*>(Vs + stage * AT_STAGE_ELEMS + (warp * AT_SUB) * D) + half * 16 + l16;
+        const uint4* vt = reinterpret_cast<const uint4*>(Vs + stage * AT_STAGE_ELEMS + (gwarp * AT_SUB) * D) + half * 16 + l16;
 #pragma unroll
         for (int i2 = 0; i2 < 8; ++i2) {
           const float pr = __shfl_sync(0xffffffffu, i2 < 4 ? p0 : p1, ((2 * i2 + half) & 7) * 4);
@@ -628,6 +670,7 @@ cudaError_t launch_attn(const LayerView& v, AttnMode mode, int n_chunks, int par
     if (e != cudaSuccess) return e;
   }
   AttnArgs a;
+  a.by_c = fast_div((uint32_t)v.C); a.by_k = fast_div((uint32_t)(parts_per_seq < 1 ? 1 : parts_per_seq));
   a.v = v; a.mode = (int)mode; a.n_chunks = n_chunks; a.k = parts_per_seq < 1 ? 1 : parts_per_seq;
   a.q = static_cast<const uint16_t*>(q); a.out = static_cast<uint16_t*>(out); a.lse = lse; a.scale = scale;
   a.kkept = static_cast<const uint16_t*>(kkept); a.vkept = static_cast<const uint16_t*>(vkept);
