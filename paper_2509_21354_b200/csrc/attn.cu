@@ -476,14 +476,15 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
     pdl_wait();
     const float sl2 = a.scale * 1.44269504088896340736f;   // logits kept in log2 units
     const int gwarp = warp % AT_GWARPS;
-    const int g8 = lane >> 2, tig = lane & 3;              // MMA fragment coordinates: rows g8 and g8 + 8 of the warp's 16
+    const int g8 = lane >> 2, tig = lane & 3, odd = g8 & 1;              // MMA fragment coordinates: rows g8 and g8 + 8 of the warp's 16
     const int half = lane >> 4, l16 = lane & 15;           // p.V: rows 2 i + half, head dims 8 l16 .. + 7
     uint4 qf[4];                                           // q as the B operand (the same in all eight columns): 8 dims from 8 (tig + 4 j)
 #pragma unroll
     for (int j = 0; j < 4; ++j) qf[j] = make_uint4(0u, 0u, 0u, 0u);
-    float m = -INFINITY, l = 0.f, acc[8];                  // l: this lane's rows only (replicated over tig), added up at the flush
+    float2 acc[4];
+    float m = -INFINITY, l = 0.f;                          // l: this lane's rows only (replicated over tig), added up at the flush
 #pragma unroll
-    for (int x = 0; x < 8; ++x) acc[x] = 0.f;
+    for (int x = 0; x < 4; ++x) acc[x] = make_float2(0.f, 0.f);
     int n_flush = 0;
     for (int i = 0;; ++i) {
       const int stage = i % AT_STAGES, round = i / AT_STAGES;
@@ -508,28 +509,29 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
       }
       if (ti.z & TF_NEW) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) qf[j] = *(reinterpret_cast<const uint4*>(Qs + stage * D) + tig + 4 * j);
+        for (int j = 0; j < 4; ++j) qf[j] = *(reinterpret_cast<const uint4*>(Qs + stage * D) + tig + 4 * (j ^ odd));
         m = -INFINITY; l = 0.f;
 #pragma unroll
-        for (int x = 0; x < 8; ++x) acc[x] = 0.f;
+        for (int x = 0; x < 4; ++x) acc[x] = make_float2(0.f, 0.f);
       }
       const int nvalid = i % AT_CGROUPS == warp / AT_GWARPS ? min(max(ti.y - gwarp * AT_SUB, 0), AT_SUB) : 0;      // the other groups' tiles: only their flags
       if (nvalid > 0) {
         // ---- q.k of the warp's 16 rows: eight MMAs.  A lane fetches 8 consecutive head dims of a row at once; they feed the k
-        // positions of two MMAs, for K and q alike (a contraction does not notice the order).  All eight columns hold q, so
-        // every lane of a group of four ends up with the logits of its rows g8 and g8 + 8.
+        // positions of two MMAs, for K and q alike (a contraction does not notice the order).  Odd rows and odd columns go through
+        // the dims in another order than even ones, so that a quarter warp's two rows (256 bytes apart) lie in different banks:
+        // of the eight columns, all of which hold q, those of the row's own parity are its logit.
         const uint4* kt = reinterpret_cast<const uint4*>(Ks + stage * AT_STAGE_ELEMS + (gwarp * AT_SUB) * D) + g8 * 16 + tig;
         float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const uint4 ra = kt[4 * j], rb = kt[4 * j + 8 * 16];
+          const uint4 ra = kt[4 * (j ^ odd)], rb = kt[4 * (j ^ odd) + 8 * 16];
           const uint32_t A0[4] = {ra.x, rb.x, ra.y, rb.y}, A1[4] = {ra.z, rb.z, ra.w, rb.w};
           mma_bf16_16816(c0, A0, qf[j].x, qf[j].y);
           mma_bf16_16816(c1, A1, qf[j].z, qf[j].w);
         }
         // ---- online softmax ----
-        const float s0 = (g8 < nvalid) ? (c0[0] + c1[0]) * sl2 : -INFINITY;
-        const float s1 = (g8 + 8 < nvalid) ? (c0[2] + c1[2]) * sl2 : -INFINITY;
+        const float s0 = (g8 < nvalid) ? (odd ? c0[1] + c1[1] : c0[0] + c1[0]) * sl2 : -INFINITY;
+        const float s1 = (g8 + 8 < nvalid) ? (odd ? c0[3] + c1[3] : c0[2] + c1[2]) * sl2 : -INFINITY;
         float mx = fmaxf(s0, s1);
 #pragma unroll
         for (int o = 4; o <= 16; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -539,7 +541,7 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
         l = fmaf(l, alpha, p0 + p1);
         m = m_new;
 #pragma unroll
-        for (int x = 0; x < 8; ++x) acc[x] *= alpha;
+        for (int x = 0; x < 4; ++x) acc[x] = mul2(acc[x], make_float2(alpha, alpha));
         // ---- p.V: half a warp per row, 16 bytes per lane ----
         const uint4* vt = reinterpret_cast<const uint4*>(Vs + stage * AT_STAGE_ELEMS + (gwarp * AT_SUB) * D) + half * 16 + l16;
 #pragma unroll
@@ -547,10 +549,11 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
           const float pr = __shfl_sync(0xffffffffu, i2 < 4 ? p0 : p1, ((2 * i2 + half) & 7) * 4);
           if (2 * i2 + half < nvalid) {            // rows beyond the tile's last one hold stale bytes
             const uint4 w = vt[i2 * 32];
-            acc[0] = fmaf(pr, bf16lo(w.x), acc[0]); acc[1] = fmaf(pr, bf16hi(w.x), acc[1]);
-            acc[2] = fmaf(pr, bf16lo(w.y), acc[2]); acc[3] = fmaf(pr, bf16hi(w.y), acc[3]);
-            acc[4] = fmaf(pr, bf16lo(w.z), acc[4]); acc[5] = fmaf(pr, bf16hi(w.z), acc[5]);
-            acc[6] = fmaf(pr, bf16lo(w.w), acc[6]); acc[7] = fmaf(pr, bf16hi(w.w), acc[7]);
+            const float2 pp = make_float2(pr, pr);
+            acc[0] = fma2(pp, make_float2(bf16lo(w.x), bf16hi(w.x)), acc[0]);
+            acc[1] = fma2(pp, make_float2(bf16lo(w.y), bf16hi(w.y)), acc[1]);
+            acc[2] = fma2(pp, make_float2(bf16lo(w.z), bf16hi(w.z)), acc[2]);
+            acc[3] = fma2(pp, make_float2(bf16lo(w.w), bf16hi(w.w)), acc[3]);
           }
         }
       }
@@ -566,7 +569,10 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
         float* cw = comb + (fb * AT_CWARPS + warp) * ATTN_PARTIAL_FLOATS;
         float tot[8], lt = l;
 #pragma unroll
-        for (int x = 0; x < 8; ++x) tot[x] = acc[x] + __shfl_xor_sync(0xffffffffu, acc[x], 16);      // even + odd rows
+        for (int x = 0; x < 4; ++x) {      // even + odd rows
+          tot[2 * x] = acc[x].x + __shfl_xor_sync(0xffffffffu, acc[x].x, 16);
+          tot[2 * x + 1] = acc[x].y + __shfl_xor_sync(0xffffffffu, acc[x].y, 16);
+        }
 #pragma unroll
         for (int o = 4; o <= 16; o <<= 1) lt += __shfl_xor_sync(0xffffffffu, lt, o);
         *reinterpret_cast<float4*>(cw + l16 * 8 + half * 4) = half ? make_float4(tot[4], tot[5], tot[6], tot[7]) : make_float4(tot[0], tot[1], tot[2], tot[3]);
