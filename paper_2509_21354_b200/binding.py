@@ -115,16 +115,29 @@ def load_library(build_if_missing: bool = True) -> C.CDLL:
     return lib
 
 
-def _stream(stream=None) -> C.c_void_p:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+# Marshalling is on the path of every decode step (a token of a small cache takes the GPU 7 us), so it passes plain integers and
+# floats (argtypes converts them), asks torch for the raw stream handle and compares shapes as tuples: set_len and 7 decode
+# steps issued call by call 172 us with ctypes objects, stream objects and numpy scalars, 119 us so.
+_BF16 = torch.bfloat16
+_DEFAULT_SCALE = 1.0 / 128.0 ** 0.5
 
 
-def _p(t) -> C.c_void_p:
+def _stream(st, stream=None) -> int:
+    """the handle of `stream`, or of the current stream on the store's device"""
+    return torch._C._cuda_getCurrentRawStream(st.device_index) if stream is None else stream.cuda_stream
+
+
+def _p(t) -> int:
     if t is None:
-        return C.c_void_p(0)
+        return 0
     assert t.is_cuda and t.is_contiguous()
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+def _rows(t, shape) -> int:
+    """address of a contiguous bf16 device tensor of the given shape"""
+    assert t.dtype is _BF16 and t.shape == shape and t.is_cuda and t.is_contiguous()
+    return t.data_ptr()
 
 
 def _check(fn, rc, handle=None):
@@ -192,6 +205,8 @@ class Store:
                               max_query_tokens=max_query_tokens)
         self.B, self.H, self.S, self.C, self.W, self.d_g = B, H, B * H, C_, W, d_g
         self.n_layers, self.max_tokens = n_layers, max_tokens
+        self.row_shape = (self.S, 128)
+        self.device_index = torch.cuda.current_device() if self.device.index is None else self.device.index
         self.max_chunks = -(-max_tokens // C_)
         S, mc, L, dev = self.S, self.max_chunks, n_layers, self.device
         n_pages = L * S * mc
@@ -271,11 +286,11 @@ class Store:
     def refresh_next(self, layer, agg_weights, lstm_weights, tau, stream=None):
         """the trigger with its position taken from the device at execution time (replayable from a CUDA graph)"""
         aw = C.byref(agg_weights.c) if agg_weights is not None else None
-        _check("kvE_refresh_next", self.lib.kvE_refresh_next(self.handle, layer, aw, C.byref(lstm_weights.c), C.c_float(tau),
-                                                             _stream(stream)), self.handle)
+        _check("kvE_refresh_next", self.lib.kvE_refresh_next(self.handle, layer, aw, C.byref(lstm_weights.c), tau,
+                                                             _stream(self, stream)), self.handle)
 
     def adopt_device_state(self, layer, stream=None):
-        _check("kvE_adopt_device_state", self.lib.kvE_adopt_device_state(self.handle, layer, _stream(stream)), self.handle)
+        _check("kvE_adopt_device_state", self.lib.kvE_adopt_device_state(self.handle, layer, _stream(self, stream)), self.handle)
 
     def compact(self, layer, tau, stream=None):
         kvE_compact(self, layer, tau, stream)
@@ -283,7 +298,7 @@ class Store:
     def refresh(self, layer, agg_weights, lstm_weights, tau, stream=None):
         """summaries of all stale chunks, gate from scratch, keep list, in one call"""
         aw = C.byref(agg_weights.c) if agg_weights is not None else None
-        _check("kvE_refresh", self.lib.kvE_refresh(self.handle, layer, aw, C.byref(lstm_weights.c), C.c_float(tau), _stream(stream)),
+        _check("kvE_refresh", self.lib.kvE_refresh(self.handle, layer, aw, C.byref(lstm_weights.c), tau, _stream(self, stream)),
                self.handle)
 
     def compact_topk(self, layer, k, stream=None):
@@ -294,13 +309,13 @@ class Store:
 
     def decode_step(self, layer, k_new, v_new, q, out=None, lse=None, scale=None, n_reserve=0, stream=None):
         """append one token per sequence (k_new, v_new: bf16 [S, 128]) at the device-held length and attend, one launch"""
-        for t in (k_new, v_new, q):
-            assert t.dtype == torch.bfloat16 and tuple(t.shape) == (self.S, 128)
+        shape = self.row_shape
         if out is None:
             out = torch.empty_like(q)
-        scale = 1.0 / np.sqrt(128.0) if scale is None else scale
-        _check("kvE_decode_step", self.lib.kvE_decode_step(self.handle, layer, _p(k_new), _p(v_new), _p(q), _p(out), _p(lse),
-                                                           C.c_float(scale), int(n_reserve), _stream(stream)), self.handle)
+        rc = self.lib.kvE_decode_step(self.handle, layer, _rows(k_new, shape), _rows(v_new, shape), _rows(q, shape), _p(out), _p(lse),
+                                      _DEFAULT_SCALE if scale is None else scale, n_reserve, _stream(self, stream))
+        if rc:
+            _check("kvE_decode_step", rc, self.handle)
         return out
 
     def decode_attn_dense(self, layer, q, out=None, lse=None, scale=None, stream=None):
@@ -313,7 +328,7 @@ class Store:
         n_new = k_new.numel() // (self.S * 128)
         assert n_new * self.S * 128 == k_new.numel()
         _check("kvE_append_next", self.lib.kvE_append_next(self.handle, layer, _p(k_new), _p(v_new), n_new, int(n_reserve),
-                                                           _stream(stream)), self.handle)
+                                                           _stream(self, stream)), self.handle)
 
     def decode_attn_block(self, layer, q, dense=False, out=None, lse=None, scale=None, stream=None, causal=False):
         return kvE_decode_attn_block(self, layer, q, dense, out, lse, scale, stream, causal)
@@ -333,7 +348,7 @@ class Store:
 
     def selftest_timeout(self, which: int, stream=None):
         """launches the kernel whose bounded wait runs out (which: 0 = CTA-scope wait, 1 = cluster-scope wait)"""
-        _check("kvE_selftest_timeout", self.lib.kvE_selftest_timeout(self.handle, int(which), _stream(stream)), self.handle)
+        _check("kvE_selftest_timeout", self.lib.kvE_selftest_timeout(self.handle, int(which), _stream(self, stream)), self.handle)
 
     def layer_state(self, layer=0) -> dict:
         return kvE_layer_state(self, layer)
@@ -350,45 +365,45 @@ def kvE_append(st: Store, layer, k_new, v_new, stream=None) -> int:
     assert k_new.dtype == torch.bfloat16 and k_new.shape == v_new.shape and k_new.shape[0] == st.S and k_new.shape[2] == 128
     ready = C.c_int(0)
     _check("kvE_append", st.lib.kvE_append(st.handle, layer, _p(k_new), _p(v_new), int(k_new.shape[1]),
-                                           C.byref(ready), _stream(stream)), st.handle)
+                                           C.byref(ready), _stream(st, stream)), st.handle)
     return ready.value
 
 
 def kvE_set_len(st: Store, layer, n, stream=None):
-    _check("kvE_set_len", st.lib.kvE_set_len(st.handle, layer, int(n), _stream(stream)), st.handle)
+    _check("kvE_set_len", st.lib.kvE_set_len(st.handle, layer, int(n), _stream(st, stream)), st.handle)
 
 
 def kvE_summarize_chunks(st: Store, layer, chunk_begin, chunk_end, agg_weights=None, stream=None):
     w = C.byref(agg_weights.c) if agg_weights is not None else None
     _check("kvE_summarize_chunks", st.lib.kvE_summarize_chunks(st.handle, layer, int(chunk_begin), int(chunk_end), w,
-                                                               _stream(stream)), st.handle)
+                                                               _stream(st, stream)), st.handle)
 
 
 def kvE_gate(st: Store, layer, chunk_begin, chunk_end, lstm_weights, stream=None):
     _check("kvE_gate", st.lib.kvE_gate(st.handle, layer, int(chunk_begin), int(chunk_end), C.byref(lstm_weights.c),
-                                       _stream(stream)), st.handle)
+                                       _stream(st, stream)), st.handle)
 
 
 def kvE_gate_next(st: Store, layer, lstm_weights, tau, stream=None):
-    _check("kvE_gate_next", st.lib.kvE_gate_next(st.handle, layer, C.byref(lstm_weights.c), C.c_float(tau), _stream(stream)),
+    _check("kvE_gate_next", st.lib.kvE_gate_next(st.handle, layer, C.byref(lstm_weights.c), tau, _stream(st, stream)),
            st.handle)
 
 
 def kvE_compact(st: Store, layer, tau, stream=None):
-    _check("kvE_compact", st.lib.kvE_compact(st.handle, layer, C.c_float(tau), _stream(stream)), st.handle)
+    _check("kvE_compact", st.lib.kvE_compact(st.handle, layer, tau, _stream(st, stream)), st.handle)
 
 
 def kvE_compact_topk(st: Store, layer, k, stream=None):
-    _check("kvE_compact_topk", st.lib.kvE_compact_topk(st.handle, layer, int(k), _stream(stream)), st.handle)
+    _check("kvE_compact_topk", st.lib.kvE_compact_topk(st.handle, layer, int(k), _stream(st, stream)), st.handle)
 
 
 def _attn(fn_name, st, layer, q, out, lse, scale, stream):
-    assert q.dtype == torch.bfloat16 and tuple(q.shape) == (st.S, 128)
+    q_ptr = _rows(q, st.row_shape)
     if out is None:
         out = torch.empty_like(q)
-    scale = 1.0 / np.sqrt(128.0) if scale is None else scale
-    _check(fn_name, getattr(st.lib, fn_name)(st.handle, layer, _p(q), _p(out), _p(lse), C.c_float(scale),
-                                              _stream(stream)), st.handle)
+    rc = getattr(st.lib, fn_name)(st.handle, layer, q_ptr, _p(out), _p(lse), _DEFAULT_SCALE if scale is None else scale, _stream(st, stream))
+    if rc:
+        _check(fn_name, rc, st.handle)
     return out
 
 
@@ -409,9 +424,9 @@ def kvE_decode_attn_block(st: Store, layer, q, dense=False, out=None, lse=None, 
     assert out.shape == q.shape and out.dtype == torch.bfloat16
     if lse is not None:
         assert lse.dtype == torch.float32 and tuple(lse.shape) == tuple(q.shape[:3])
-    scale = (1.0 / 128.0 ** 0.5) if scale is None else scale
+    scale = _DEFAULT_SCALE if scale is None else scale
     _check("kvE_decode_attn_block", st.lib.kvE_decode_attn_block(st.handle, layer, _p(q), int(q.shape[1]), int(bool(dense)),
-                                                                 int(bool(causal)), _p(out), _p(lse), C.c_float(scale), _stream(stream)), st.handle)
+                                                                 int(bool(causal)), _p(out), _p(lse), scale, _stream(st, stream)), st.handle)
     return out
 
 
@@ -428,8 +443,8 @@ def kvE_reclaim_pages(st: Store, layer, chunk_begin, chunk_end, mode="discarded"
         free_count = torch.zeros((1,), dtype=torch.int32, device=st.device)
     assert free_list.dtype == torch.int32 and free_count.dtype == torch.int32
     _check("kvE_reclaim_pages", st.lib.kvE_reclaim_pages(st.handle, layer, int(chunk_begin), int(chunk_end), RECLAIM[mode],
-                                                        _p(free_list), C.c_int64(free_list.numel()), _p(free_count),
-                                                        _stream(stream)), st.handle)
+                                                        _p(free_list), free_list.numel(), _p(free_count),
+                                                        _stream(st, stream)), st.handle)
     return free_list, free_count
 
 
@@ -446,16 +461,16 @@ def kvE_decode_step_host(st: Store, layer, k_new, v_new, q, out, agg_weights, ls
     wait=False calls kvE_decode_step_host_async: the step is only enqueued (pinned buffers required)."""
     for t in (k_new, v_new, q, out):
         assert not t.is_cuda and t.dtype == torch.bfloat16 and tuple(t.shape) == (st.S, 128) and t.is_contiguous()
-    scale = 1.0 / np.sqrt(128.0) if scale is None else scale
+    scale = _DEFAULT_SCALE if scale is None else scale
     aw = C.byref(agg_weights.c) if agg_weights is not None else None
     if not wait:
         assert all(t.is_pinned() for t in (k_new, v_new, q, out))
     fn = st.lib.kvE_decode_step_host if wait else st.lib.kvE_decode_step_host_async
     _check("kvE_decode_step_host",
-           fn(st.handle, layer, C.c_void_p(k_new.data_ptr()), C.c_void_p(v_new.data_ptr()),
-                                       C.c_void_p(q.data_ptr()), C.c_void_p(out.data_ptr()), aw,
-                                       C.byref(lstm_weights.c), C.c_float(tau), C.c_float(scale),
-                                       1 if from_scratch else 0, _stream(stream)), st.handle)
+           fn(st.handle, layer, k_new.data_ptr(), v_new.data_ptr(),
+                                       q.data_ptr(), out.data_ptr(), aw,
+                                       C.byref(lstm_weights.c), tau, scale,
+                                       1 if from_scratch else 0, _stream(st, stream)), st.handle)
 
 
 def kvE_poll_status(st: Store) -> int:

@@ -215,21 +215,23 @@ AttnCut attention_cut(const kvE_store* st, AttnMode mode, const LayerState& ls) 
   const long long k_max = tiles < MAX_SPLITS ? tiles : MAX_SPLITS;
   const double hbm_us = (double)S * (double)(tail + lead) * 512.0 / 6.4e6;
   auto cost_of = [&](long long k) {
-    const long long parts = S * k, grid = parts < G ? parts : G;
-    const long long rounds = (parts + grid - 1) / grid;                 // parts of the busiest CTA
-    const double busiest = rounds == 1 ? (double)((tiles + k - 1) / k) : (double)rounds * (double)tiles / (double)k;
+    const unsigned parts = (unsigned)(S * k), grid = parts < (unsigned)G ? parts : (unsigned)G;
+    const unsigned rounds = (parts + grid - 1) / grid;                 // parts of the busiest CTA
+    const double busiest = rounds == 1 ? (double)(((unsigned)tiles + (unsigned)k - 1) / (unsigned)k) : (double)rounds * (double)tiles / (double)k;
     const double ends = k == 1 ? 0.0 : 1.7 + 0.05 * (double)k + (rounds > 1 ? 1.8 : 0.0);
-    const double us = busiest * (2 * grid <= G ? 0.9 : 1.25) + ends;
+    const double us = busiest * (2 * grid <= (unsigned)G ? 0.9 : 1.25) + ends;
     const double stream = hbm_us + 0.35 * (busiest - (double)(S * tiles) / (double)grid);
     return us > stream ? us : stream;
   };
   // the kernel cuts the parts up in 32-bit arithmetic: S k (G + 1) must stay below 2^32
-  double best = 1e30;
-  for (long long k = 1; k <= k_max && S * k * (G + 1) < (1LL << 32); ++k)
-    if (cost_of(k) < best) best = cost_of(k);
-  long long k_pick = 1;
-  while (cost_of(k_pick) > best + 0.3) ++k_pick;
-  return AttnCut{(int)k_pick, (int)(S * k_pick < G ? S * k_pick : G)};
+  double best = 1e30, cost[MAX_SPLITS + 1];
+  for (long long k = 1; k <= k_max && S * k * (G + 1) < (1LL << 32); ++k) {
+    cost[k] = cost_of(k);
+    if (cost[k] < best) best = cost[k];
+  }
+  int k_pick = 1;
+  while (cost[k_pick] > best + 0.3) ++k_pick;
+  return AttnCut{k_pick, (int)(S * k_pick < G ? S * k_pick : G)};
 }
 
 struct KeptRows { void *k, *v; };      // kept summary rows of a layer, compacted by kvE_compact
