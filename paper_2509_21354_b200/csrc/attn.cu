@@ -89,20 +89,6 @@ constexpr int TF_NEW = 1;      // first tile of a (sequence, list) in this CTA: 
 constexpr int TF_FLUSH = 2;    // last tile of a (sequence, list) in this CTA: hand the state to the merger afterwards
 constexpr int TF_END = 4;      // no tile: the CTA's work is done
 
-// x / d for x < 2^31 as a multiplication (a runtime divisor costs the producer a chain of some twenty instructions)
-struct FastDiv {
-  uint32_t mul, shift;
-  __device__ __forceinline__ uint32_t div(uint32_t x) const { return (uint32_t)(((uint64_t)x * mul) >> shift); }
-};
-static FastDiv fast_div(uint32_t d) {      // mul = ceil(2^shift / d) with 2^(shift - 31) >= d: exact below 2^31
-  FastDiv f;
-  uint32_t log2_up = 0;
-  while ((1u << log2_up) < d) ++log2_up;
-  f.shift = 31 + log2_up;
-  f.mul = (uint32_t)(((1ull << f.shift) + d - 1) / d);
-  return f;
-}
-
 struct AttnArgs {
   LayerView v;
   FastDiv by_c, by_k;          // by the chunk size, by k

@@ -184,6 +184,20 @@ __device__ __forceinline__ NextChunk next_chunk(const int32_t* n_listed, const i
   return nx;
 }
 
+// x / d for x < 2^31 as a multiplication (a runtime divisor costs a chain of some twenty instructions)
+struct FastDiv {
+  uint32_t mul, shift;
+  __device__ __forceinline__ uint32_t div(uint32_t x) const { return (uint32_t)(((uint64_t)x * mul) >> shift); }
+};
+inline FastDiv fast_div(uint32_t d) {      // mul = ceil(2^shift / d) with 2^(shift - 31) >= d: exact below 2^31
+  FastDiv f;
+  uint32_t log2_up = 0;
+  while ((1u << log2_up) < d) ++log2_up;
+  f.shift = 31 + log2_up;
+  f.mul = (uint32_t)(((1ull << f.shift) + d - 1) / d);
+  return f;
+}
+
 // host side: launch with the programmatic-serialisation attribute
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {

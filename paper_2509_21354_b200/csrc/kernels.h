@@ -75,6 +75,8 @@ cudaError_t launch_append_next(const LayerView& v, const void* k_new, const void
 // else the launch does nothing (a trigger that is replayed from a CUDA graph)
 cudaError_t launch_chunk_mean(const LayerView& v, int t0, int t1, bool final_output, bool pool_max, cudaStream_t st, int dev_window);
 cudaError_t launch_chunk_mlp(const LayerView& v, int t0, int t1, const MlpWeights& w, int d_sum, cudaStream_t st, int dev_window);
+// the MLP's second layer on pooled activations hid [2][S * (t1 - t0)][d_sum]: Kbar = W2 hid + b2 (d_sum 128 or 256)
+cudaError_t launch_pooled_out(const LayerView& v, int t0, int t1, const MlpWeights& w, int d_sum, const float* hid, cudaStream_t st);
 // per-token MLP aggregator: hid = scratch of 2 * S * (t1 - t0) * d_sum floats
 bool token_mlp_supported(int C, int d_sum);
 cudaError_t launch_chunk_token_mlp(const LayerView& v, int t0, int t1, const MlpWeights& w, int d_sum, float* hid, cudaStream_t st);

@@ -268,8 +268,11 @@ __device__ __forceinline__ void store_split8(const float (&x)[8], unsigned char*
     *reinterpret_cast<uint4*>(dst + pl * plane_stride) = make_uint4(w[0][pl], w[1][pl], w[2][pl], w[3][pl]);
 }
 
+// POOLED: the second layer alone, on the pooled activations hid [2][n_units][d_sum] of the per-token aggregator
+template <bool POOLED>
 __global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerView v, int t0, int n_range, long long n_units,
-                                                                         MlpWeights w, int d_sum, int dev_window) {
+                                                                         MlpWeights w, int d_sum, int dev_window,
+                                                                         const float* __restrict__ hid) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   unsigned char* As = smem + MT_SMEM_A;
@@ -294,7 +297,7 @@ __global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerVi
   const long long n_tiles = (n_units + MT_M - 1) / MT_M;
 
   // ---- one-time set-up -----------------------------------------------------------------------------
-  for (int i = tid; i < d_sum * 16; i += MT_THREADS) {              // W1 [d_sum][128]: rows of 16 pieces, 2 K-blocks
+  for (int i = tid; !POOLED && i < d_sum * 16; i += MT_THREADS) {   // W1 [d_sum][128]: rows of 16 pieces, 2 K-blocks
     const int r = i >> 4, p = i & 15;
     cp_async16(W1s + (p >> 3) * (d_sum * umma::KBLOCK_ROW_BYTES) + umma::piece_offset(r, p & 7),
                reinterpret_cast<const uint4*>(W1 + (long long)r * D) + p, true);
@@ -305,7 +308,7 @@ __global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerVi
     cp_async16(W2s + (p >> 3) * MT_PLANE_KB_BYTES + umma::piece_offset(r, p & 7),
                reinterpret_cast<const uint4*>(W2 + (long long)r * d_sum) + p, true);
   }
-  for (int i = tid; i < d_sum; i += MT_THREADS) b1s[i] = b1[i];
+  for (int i = tid; !POOLED && i < d_sum; i += MT_THREADS) b1s[i] = b1[i];
   for (int i = tid; i < D; i += MT_THREADS) b2s[i] = b2[i];
   if (warp == 0) umma::tmem_alloc(tmem_slot, MT_TMEM_COLS);
   if (tid == 0) {
@@ -336,6 +339,7 @@ __global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerVi
   }
   for (long long tile = blockIdx.x; tile < n_tiles && !failed && due; tile += gridDim.x) {
     const long long unit0 = tile * MT_M;
+    if constexpr (!POOLED) {
     // ---- chunk means -> three bf16 planes (layer-1 A operand) ------------------------------------------
     {
       // a thread keeps its 32-byte column pc and walks down 4 rows: all 8 loads first, then the splits
@@ -386,6 +390,7 @@ __global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerVi
       if (__syncthreads_or(!ok)) { failed = true; break; }
     }
     umma::fence_after_sync();
+    }
 
     // ---- layer 2 in slices of 64 hidden units ------------------------------------------------------------
     for (int j = 0; j < n_slices; ++j) {
@@ -396,13 +401,27 @@ __global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerVi
         if (__syncthreads_or(!ok)) { failed = true; break; }
       }
       float h[16];
-      umma::tmem_ld16(tmem_h + tmem_lane + (uint32_t)(j * 64 + part * 16), h);
+      if constexpr (POOLED) {
+        const long long unit = unit0 + row_in_tile;
+        const float4* src = reinterpret_cast<const float4*>(hid + ((long long)side * n_units + unit) * d_sum + j * 64 + part * 16);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float4 x = unit < n_units ? src[e] : make_float4(0.f, 0.f, 0.f, 0.f);
+          h[4 * e] = x.x; h[4 * e + 1] = x.y; h[4 * e + 2] = x.z; h[4 * e + 3] = x.w;
+        }
+      } else {
+        umma::tmem_ld16(tmem_h + tmem_lane + (uint32_t)(j * 64 + part * 16), h);
+      }
       unsigned char* abuf = As + buf * 3 * MT_PLANE_KB_BYTES;
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         float g[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) g[e] = gelu_tc(h[q * 8 + e] + b1s[j * 64 + part * 16 + q * 8 + e]);
+        for (int e = 0; e < 8; e += 2) {
+          float2 y = make_float2(h[q * 8 + e], h[q * 8 + e + 1]);
+          if constexpr (!POOLED) y = gelu2(add2(y, *reinterpret_cast<const float2*>(b1s + j * 64 + part * 16 + q * 8 + e)));
+          g[e] = y.x; g[e + 1] = y.y;
+        }
         store_split8(g, abuf + umma::piece_offset(row_in_tile, part * 2 + q), MT_PLANE_KB_BYTES);
       }
       umma::fence_smem_to_async();
@@ -487,6 +506,19 @@ __global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerVi
   if (warp == 0) umma::tmem_dealloc(tmem_h, MT_TMEM_COLS);
 }
 
+cudaError_t launch_pooled_out(const LayerView& v, int t0, int t1, const MlpWeights& w, int d_sum, const float* hid, cudaStream_t st) {
+  const int n_range = t1 - t0;
+  const long long n_units = (long long)v.S * n_range;
+  if (d_sum % 64 != 0 || d_sum > MT_MAX_DSUM || n_units + MT_M >= (1LL << 31) || (long long)v.S * v.max_chunks >= (1LL << 31))
+    return cudaErrorInvalidValue;
+  static DeviceFlags opted;
+  const cudaError_t e = smem_opt_in(opted, kve_chunk_mlp_tc_kernel<true>, MT_SMEM_BYTES);
+  if (e != cudaSuccess) return e;
+  const long long n_tiles = (n_units + MT_M - 1) / MT_M, half = sm_count() / 2;
+  return launch_pdl(kve_chunk_mlp_tc_kernel<true>, dim3((unsigned)(n_tiles < half ? n_tiles : half), 2), dim3(MT_THREADS), MT_SMEM_BYTES, st, v,
+                    t0, n_range, n_units, w, d_sum, -1, hid);
+}
+
 cudaError_t launch_chunk_mlp(const LayerView& v, int t0, int t1, const MlpWeights& w, int d_sum, cudaStream_t st, int dev_window) {
   const int n_range = dev_window >= 0 ? 1 : t1 - t0;
   const long long n_units = (long long)v.S * n_range;
@@ -495,14 +527,14 @@ cudaError_t launch_chunk_mlp(const LayerView& v, int t0, int t1, const MlpWeight
       (long long)v.S * v.max_chunks < (1LL << 31)) {
     static DeviceFlags opted_tc;
     {
-      cudaError_t e = smem_opt_in(opted_tc, kve_chunk_mlp_tc_kernel, MT_SMEM_BYTES);
+      cudaError_t e = smem_opt_in(opted_tc, kve_chunk_mlp_tc_kernel<false>, MT_SMEM_BYTES);
       if (e != cudaSuccess) return e;
     }
     const long long n_tiles = (n_units + MT_M - 1) / MT_M;
     const long long half = sm_count() / 2;
     const long long per_side = n_tiles < half ? n_tiles : half;  // one CTA per SM: half of the SMs per side
     dim3 grid((unsigned)per_side, 2);
-    return launch_pdl(kve_chunk_mlp_tc_kernel, grid, dim3(MT_THREADS), MT_SMEM_BYTES, st, v, t0, n_range, n_units, w, d_sum, dev_window);
+    return launch_pdl(kve_chunk_mlp_tc_kernel<false>, grid, dim3(MT_THREADS), MT_SMEM_BYTES, st, v, t0, n_range, n_units, w, d_sum, dev_window, nullptr);
   }
   const size_t smem = sizeof(float) * (size_t)MLP_ROWS * (D + d_sum);
   static DeviceFlags opted;
