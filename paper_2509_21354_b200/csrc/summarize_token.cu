@@ -29,14 +29,17 @@ namespace kve {
 
 constexpr int TM_N = 128;                                   // tokens per tile
 constexpr int TM_SLAB = 128;                                // hidden units per MMA
-constexpr int TM_THREADS = 512;                             // 16 warps: four per scheduler hide the latency of the activation chains
+constexpr int TM_EPI_WARPS = 16;                            // four per scheduler hide the latency of the activation chains
+constexpr int TM_COPY_WARPS = 4;
+constexpr int TM_MMA_WARP = TM_EPI_WARPS + TM_COPY_WARPS;
+constexpr int TM_THREADS = (TM_MMA_WARP + 1) * 32;
 constexpr int TM_MAX_DSUM = 256;
 constexpr int TM_KB_BYTES = TM_N * umma::KBLOCK_ROW_BYTES;  // 16 KB: 128 rows x 64 head dims
 constexpr int TM_SMEM_W1 = 0;                               // 2 K-blocks of [d_sum rows][64]: up to 64 KB
 constexpr int TM_SMEM_X = TM_SMEM_W1 + 2 * TM_MAX_DSUM * umma::KBLOCK_ROW_BYTES;   // 2 buffers x 2 K-blocks: 64 KB
 constexpr int TM_SMEM_POOL = TM_SMEM_X + 2 * 2 * TM_KB_BYTES;          // [2 tile parities][4 groups of 32 tokens][d_sum] sums
 constexpr int TM_SMEM_BAR = TM_SMEM_POOL + 2 * 4 * TM_MAX_DSUM * 4;
-constexpr int TM_SMEM_BYTES = TM_SMEM_BAR + 32 + 1024;      // + slack to reach a 1024-byte boundary
+constexpr int TM_SMEM_BYTES = TM_SMEM_BAR + 64 + 1024;      // + slack to reach a 1024-byte boundary
 constexpr int TM_TMEM_COLS = 512;                           // two accumulators of up to two slabs x 128 columns
 static_assert(TM_SMEM_BYTES > 116 * 1024, "one CTA per SM: each allocates all of tensor memory");
 
@@ -54,169 +57,212 @@ struct TokenMlpArgs {
 template <int DSUM>
 __global__ void __launch_bounds__(TM_THREADS, 1) kve_token_mlp_pool_kernel(TokenMlpArgs a) {
   constexpr int SLABS = DSUM / TM_SLAB;
-  constexpr int COLS = TM_N * SLABS / 4;       // tokens a thread goes through per tile: 64 or 32
+  constexpr int COLS = TM_N * SLABS / 4;       // tokens an epilogue thread goes through per tile: 64 or 32
   constexpr int GROUPS = COLS / 32;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   unsigned char* W1s = smem + TM_SMEM_W1;
   unsigned char* Xs = smem + TM_SMEM_X;
   float* pool = reinterpret_cast<float*>(smem + TM_SMEM_POOL);
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + TM_SMEM_BAR);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + TM_SMEM_BAR + 8);
+  uint64_t* x_full = reinterpret_cast<uint64_t*>(smem + TM_SMEM_BAR);      // [2] token buffer filled by the copy warps
+  uint64_t* acc_full = x_full + 2;                                          // [2] accumulator written, token buffer read (MMA commit)
+  uint64_t* acc_free = acc_full + 2;                                        // [2] accumulator read by the epilogue warps
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_free + 2);
 
   pdl_launch_dependents();
   const LayerView& v = a.v;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int side = blockIdx.y;
-  const uint16_t* W1 = side ? a.w.W1V : a.w.W1K;
-  const uint16_t* pages = side ? v.v_pages : v.k_pages;
 
-  // ---- one-time set-up: W1 of this side, tensor memory, barrier --------------------------------------------
+  // ---- one-time set-up: W1 of this side, tensor memory, barriers -------------------------------------------
+  const uint16_t* W1 = side ? a.w.W1V : a.w.W1K;
   for (int i = tid; i < DSUM * 16; i += TM_THREADS) {              // W1 [DSUM][128]: rows of 16 pieces, 2 K-blocks
     const int r = i >> 4, p = i & 15;
     cp_async16(W1s + (p >> 3) * (DSUM * umma::KBLOCK_ROW_BYTES) + umma::piece_offset(r, p & 7),
                reinterpret_cast<const uint4*>(W1 + (long long)r * D) + p, true);
   }
-  if (warp == 0) umma::tmem_alloc(tmem_slot, TM_TMEM_COLS);
+  if (warp == TM_MMA_WARP) umma::tmem_alloc(tmem_slot, TM_TMEM_COLS);
   if (tid == 0) {
-    mbar_init(bar, 1);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&x_full[i], TM_COPY_WARPS * 32);
+      mbar_init(&acc_full[i], 1);
+      mbar_init(&acc_free[i], TM_EPI_WARPS);
+    }
     mbar_fence_init();
   }
-  const uint32_t x_base = smem_u32(Xs), w1_base = smem_u32(W1s);
-  constexpr uint32_t idesc = umma::instr_desc_bf16(TM_SLAB, TM_N);
-
-  // this thread's hidden unit and tokens: tensor-memory lane 32 (warp & 3) + lane of slab `slab`, columns [col0, col0 + COLS)
-  const int lg = warp & 3, quarter = warp >> 2;
-  const int slab = SLABS == 2 ? quarter >> 1 : 0, col0 = (SLABS == 2 ? quarter & 1 : quarter) * COLS;
-  const int unit = slab * TM_SLAB + lg * 32 + lane;
-  const float b1_scaled = (side ? a.w.b1V : a.w.b1K)[unit] * GELU_SCALE;
-  const uint32_t tmem_off = (uint32_t)(slab * TM_N + col0) + ((uint32_t)(lg * 32) << 16);
-
-  // A CTA walks whole items (a chunk longer than a tile keeps all its 128-token slices on one CTA, in a row).  What this
-  // thread copies of a tile: the 16-byte piece p of the rows r0 + 32 i.
-  const int p16 = tid & 15, r0 = tid >> 4;
-  int src_item = blockIdx.x, src_slice = 0;                         // the tile the next look-up is for
-  int page[TM_N / 32], page_slice = 0;                              // its pages (-1: no row) and slice
-  auto look_up = [&]() {
-#pragma unroll
-    for (int i = 0; i < TM_N / 32; ++i) {
-      const int r = r0 + 32 * i;
-      const int u_in = a.units_per_item > 1 ? r / v.C : 0;
-      const int u = src_item * a.units_per_item + u_in;
-      page[i] = -1;
-      if (src_item < a.n_items && u < a.n_units) {
-        const int s = (int)a.by_range.div((uint32_t)u);
-        const int t = a.t0 + (u - s * a.n_range);
-        page[i] = max(v.page_table[(long long)s * v.max_chunks + t], -2);      // below -1: a bad entry, flagged when it is used
-        if (page[i] == -1) page[i] = -2;
-      }
-    }
-    page_slice = src_slice;
-    if (++src_slice == a.tiles_per_item) { src_slice = 0; src_item += gridDim.x; }
-  };
-  // copies of the tile looked up last, zeros where there is no row
-  auto gather = [&](int buf) {
-    unsigned char* dst0 = Xs + buf * 2 * TM_KB_BYTES + (p16 >> 3) * TM_KB_BYTES;
-#pragma unroll
-    for (int i = 0; i < TM_N / 32; ++i) {
-      const int r = r0 + 32 * i;
-      const bool live = page[i] >= 0 && page[i] < v.n_pages;
-      if (!live && page[i] != -1) set_status(v.status, ERR_CAPACITY);
-      const int r_in = (a.units_per_item > 1 ? r % v.C : r) + page_slice * TM_N;
-      cp_async16(dst0 + umma::piece_offset(r, p16 & 7), pages + (live ? ((long long)page[i] * v.C + r_in) * D : 0) + p16 * 8, live);
-    }
-  };
-  auto issue_mma = [&](uint32_t tmem_acc, int buf) {
-    umma::fence_after_sync();
-#pragma unroll
-    for (int sl = 0; sl < SLABS; ++sl)
-#pragma unroll
-      for (int kb = 0; kb < 2; ++kb)
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          umma::mma_bf16(tmem_acc + sl * TM_N, umma::smem_desc(w1_base + kb * (DSUM * umma::KBLOCK_ROW_BYTES) + sl * (TM_SLAB * umma::KBLOCK_ROW_BYTES) + k * 32),
-                         umma::smem_desc(x_base + (buf * 2 + kb) * TM_KB_BYTES + k * 32), idesc, (kb | k) != 0);
-    umma::commit(bar);
-  };
-  // the finished sums of a tile (its last slice): pooled activations out
-  const float inv_c = 1.f / (float)v.C;
-  const int groups_per_chunk = (v.C < TM_N ? v.C : TM_N) / 32;
-  auto write_pooled = [&](int item, int parity) {
-    const float* pl = pool + parity * 4 * TM_MAX_DSUM;
-    for (int i = tid; i < a.units_per_item * DSUM; i += TM_THREADS) {
-      const int u_in = i / DSUM, col = i - u_in * DSUM, u = item * a.units_per_item + u_in;
-      float sum = 0.f;
-      for (int g = 0; g < groups_per_chunk; ++g) sum += pl[(u_in * groups_per_chunk + g) * TM_MAX_DSUM + col];
-      if (u < a.n_units) a.hid[((long long)side * a.n_units + u) * DSUM + col] = sum * inv_c;
-    }
-  };
-
-  pdl_wait();      // W1 is on its way; the pages come from earlier kernels
-  const int my_items = a.n_items > (int)blockIdx.x ? (a.n_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
-  const long long n_tiles = (long long)my_items * a.tiles_per_item;      // of this CTA
-  look_up();
-  if (n_tiles > 0) gather(0);
-  look_up();
   cp_async_wait_all();
   umma::fence_smem_to_async();
   umma::fence_before_sync();
   __syncthreads();
   umma::fence_after_sync();
   const uint32_t tmem_d = *tmem_slot;
-  if (n_tiles > 0 && tid == 0) issue_mma(tmem_d, 0);
-  if (n_tiles > 1) gather(1);
-  look_up();
+  pdl_wait();      // the pages come from earlier kernels
 
-  float2 relu_sum[GROUPS], tail_sum[GROUPS];      // per 32 tokens: sum of max(u, 0) and of the tails
+  // A CTA walks whole items (a chunk longer than a tile keeps all its 128-token slices on one CTA, in a row)
+  const int my_items = a.n_items > (int)blockIdx.x ? (a.n_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
+  const int n_tiles = my_items * a.tiles_per_item;      // of this CTA
+  const int chunk_shift = v.C >= TM_N ? 7 : (v.C == 64 ? 6 : 5);      // row r of a tile: chunk r >> chunk_shift
+
+  if (warp >= TM_EPI_WARPS && warp < TM_MMA_WARP) {
+    // ================= copy warps: the tile's rows into the swizzled layout =================
+    const int ct = tid - TM_EPI_WARPS * 32, p16 = ct & 15, r0 = ct >> 4;      // the 16-byte piece p16 of the rows r0 + 8 i
+    const uint16_t* pages = (side ? v.v_pages : v.k_pages) + p16 * 8;
+    unsigned char* dst0 = Xs + (p16 >> 3) * TM_KB_BYTES;
+    int item = blockIdx.x, slice = 0;
+    int page[4];                                       // of the (up to four) chunks of the tile to come, looked up a tile ahead
+    auto look_up = [&]() {
 #pragma unroll
-  for (int g = 0; g < GROUPS; ++g) relu_sum[g] = tail_sum[g] = make_float2(0.f, 0.f);
-  int item = blockIdx.x, slice = 0, done_item = -1;      // done_item: its sums wait in the other parity's pool
-  for (long long tile = 0; tile < n_tiles; ++tile) {
-    const int sel = (int)(tile & 1);
-    const bool ok = mbar_wait_bounded(bar, (uint32_t)sel);      // this tile's MMAs are done: its token buffer is free
-    cp_async_wait_all();                                        // the next tile's rows are in place
-    umma::fence_smem_to_async();
-    umma::fence_before_sync();
-    if (__syncthreads_or(!ok)) {      // also: the other accumulator and the other pool were left a tile ago
-      if (tid == 0) set_status(v.status, ERR_TIMEOUT);
-      break;
-    }
-    umma::fence_after_sync();
-    if (tile + 1 < n_tiles && tid == 0) issue_mma(tmem_d + (uint32_t)(sel ^ 1) * (SLABS * TM_N), sel ^ 1);
-    if (tile + 2 < n_tiles) {
-      gather(sel);
-      look_up();      // the page ids arrive while this tile is worked through
-    }
-    if (done_item >= 0) write_pooled(done_item, sel ^ 1);
-    done_item = -1;
+      for (int x = 0; x < 4; ++x) {
+        const int u = item * a.units_per_item + x;
+        page[x] = -1;
+        if (x < a.units_per_item && item < a.n_items && u < a.n_units) {
+          const int s = (int)a.by_range.div((uint32_t)u);
+          page[x] = v.page_table[(long long)s * v.max_chunks + a.t0 + (u - s * a.n_range)];
+        }
+      }
+    };
+    look_up();
+    bool ok = true;
+    for (int tile = 0; tile <= n_tiles && ok; ++tile) {
+      if (tile < n_tiles) {
+        const int buf = tile & 1;
+        // the products of two tiles ago have read this buffer
+        if (tile >= 2) ok = mbar_wait_bounded(&acc_full[buf], (uint32_t)(((tile >> 1) - 1) & 1));
+        long long src[4];                              // element offset of the first row taken from each chunk; -1: zeros
 #pragma unroll
-    for (int g = 0; g < GROUPS; ++g) {
-      float h[32];
-      umma::tmem_ld32(tmem_d + (uint32_t)sel * (SLABS * TM_N) + tmem_off + (uint32_t)(g * 32), h);
+        for (int x = 0; x < 4; ++x) {
+          const bool live = page[x] >= 0 && page[x] < v.n_pages;
+          if (!live && x < a.units_per_item && item * a.units_per_item + x < a.n_units) set_status(v.status, ERR_CAPACITY);
+          src[x] = live ? ((long long)page[x] * v.C + slice * TM_N) * D : -1;
+        }
+        if (++slice == a.tiles_per_item) { slice = 0; item += gridDim.x; }
+        look_up();
 #pragma unroll
-      for (int e = 0; e < 32; e += 2) {
-        float2 relu, ea;
-        const float2 u = fma2(make_float2(h[e], h[e + 1]), make_float2(GELU_SCALE, GELU_SCALE), make_float2(b1_scaled, b1_scaled));
-        const float2 p = gelu_tail2(u, relu, ea);
-        tail_sum[g] = fma2(ea, p, tail_sum[g]);
-        relu_sum[g] = add2(relu_sum[g], relu);
+        for (int i = 0; i < TM_N / 8; ++i) {
+          const long long base = chunk_shift == 7 ? src[0] : (chunk_shift == 6 ? src[i >> 3] : src[i >> 2]);
+          const int r = r0 + 8 * i, r_in = r & ((1 << chunk_shift) - 1);
+          cp_async16(dst0 + buf * 2 * TM_KB_BYTES + umma::piece_offset(r, p16 & 7), pages + (base < 0 ? 0 : base + r_in * D), base >= 0);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+      }
+      if (tile > 0) {      // the tile before has arrived
+        if (tile < n_tiles) asm volatile("cp.async.wait_group 1;" ::: "memory");
+        else asm volatile("cp.async.wait_group 0;" ::: "memory");
+        umma::fence_smem_to_async();
+        mbar_arrive(&x_full[(tile - 1) & 1]);
       }
     }
-    if (++slice == a.tiles_per_item) {      // the chunk(s) of this item are complete
+    if (!ok) set_status(v.status, ERR_TIMEOUT);
+    cp_async_wait_all();
+  } else if (warp == TM_MMA_WARP) {
+    // ================= MMA issue (one thread) =================
+    if (lane == 0) {
+      constexpr uint32_t idesc = umma::instr_desc_bf16(TM_SLAB, TM_N);
+      const uint32_t x_base = smem_u32(Xs), w1_base = smem_u32(W1s);
+      for (int tile = 0; tile < n_tiles; ++tile) {
+        const int buf = tile & 1;
+        if (!mbar_wait_bounded(&x_full[buf], (uint32_t)((tile >> 1) & 1)) ||
+            (tile >= 2 && !mbar_wait_bounded(&acc_free[buf], (uint32_t)(((tile >> 1) - 1) & 1)))) {
+          set_status(v.status, ERR_TIMEOUT);
+          break;
+        }
+        umma::fence_after_sync();
+#pragma unroll
+        for (int sl = 0; sl < SLABS; ++sl)
+#pragma unroll
+          for (int kb = 0; kb < 2; ++kb)
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              umma::mma_bf16(tmem_d + (uint32_t)(buf * SLABS + sl) * TM_N,
+                             umma::smem_desc(w1_base + kb * (DSUM * umma::KBLOCK_ROW_BYTES) + sl * (TM_SLAB * umma::KBLOCK_ROW_BYTES) + k * 32),
+                             umma::smem_desc(x_base + (buf * 2 + kb) * TM_KB_BYTES + k * 32), idesc, (kb | k) != 0);
+        umma::commit(&acc_full[buf]);
+      }
+    }
+  } else {
+    // ================= epilogue warps =================
+    // this thread's hidden unit and tokens: tensor-memory lane 32 (warp & 3) + lane of slab `slab`, columns [col0, col0 + COLS)
+    const int lg = warp & 3, quarter = warp >> 2;
+    const int slab = SLABS == 2 ? quarter >> 1 : 0, col0 = (SLABS == 2 ? quarter & 1 : quarter) * COLS;
+    const int unit = slab * TM_SLAB + lg * 32 + lane;
+    const float b1_scaled = (side ? a.w.b1V : a.w.b1K)[unit] * GELU_SCALE;
+    const uint32_t tmem_t = tmem_d + (uint32_t)(slab * TM_N + col0) + ((uint32_t)(lg * 32) << 16);
+    const float inv_c = 1.f / (float)v.C;
+    float* hid = a.hid + (long long)side * a.n_units * DSUM;
+    // chunks no longer than this thread's tokens are summed by it alone; longer ones meet in shared memory
+    const int chunk_groups = (1 << chunk_shift) / 32;
+    float sum[GROUPS];                                  // per 32 tokens (of all slices of a long chunk)
+#pragma unroll
+    for (int g = 0; g < GROUPS; ++g) sum[g] = 0.f;
+    int item = blockIdx.x, slice = 0, item_parity = 0;
+    bool alive = true;      // a warp whose wait ran out goes on without waiting: the others meet it at the barrier below
+    for (int tile = 0; tile < n_tiles; ++tile) {
+      const int buf = tile & 1;
+      if (alive && !__all_sync(0xffffffffu, mbar_wait_bounded(&acc_full[buf], (uint32_t)((tile >> 1) & 1)))) {
+        alive = false;
+        if (lane == 0) set_status(v.status, ERR_TIMEOUT);
+      }
+      umma::fence_after_sync();
+      const uint32_t cols = tmem_t + (uint32_t)(buf * SLABS * TM_N);
+      uint32_t h[2][16];                                // 16 columns in work, 16 on their way
+      umma::tmem_ld16_nowait(cols, h[0]);
 #pragma unroll
       for (int g = 0; g < GROUPS; ++g) {
-        pool[(sel * 4 + col0 / 32 + g) * TM_MAX_DSUM + unit] = (relu_sum[g].x + relu_sum[g].y) * (1.f / GELU_SCALE) - (tail_sum[g].x + tail_sum[g].y);
-        relu_sum[g] = tail_sum[g] = make_float2(0.f, 0.f);
+        float2 relu_sum = make_float2(0.f, 0.f), tail_sum = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          umma::tmem_ld_wait16(h[q]);
+          if (2 * g + q + 1 < 2 * GROUPS) umma::tmem_ld16_nowait(cols + (uint32_t)((2 * g + q + 1) * 16), h[(q + 1) & 1]);
+          else {
+            umma::fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&acc_free[buf]);
+          }
+#pragma unroll
+          for (int e = 0; e < 16; e += 2) {
+            float2 relu, ea;
+            const float2 u = fma2(make_float2(__uint_as_float(h[q][e]), __uint_as_float(h[q][e + 1])), make_float2(GELU_SCALE, GELU_SCALE),
+                                  make_float2(b1_scaled, b1_scaled));
+            const float2 p = gelu_tail2(u, relu, ea);
+            tail_sum = fma2(ea, p, tail_sum);
+            relu_sum = add2(relu_sum, relu);
+          }
+        }
+        sum[g] += (relu_sum.x + relu_sum.y) * (1.f / GELU_SCALE) - (tail_sum.x + tail_sum.y);
       }
-      done_item = item;
+      if (++slice < a.tiles_per_item) continue;
+      // the chunk(s) of this item are complete
+      if (chunk_groups <= GROUPS) {
+        const int first = item * a.units_per_item + col0 / 32 / chunk_groups;
+        if (GROUPS == 2 && chunk_groups == 2) {
+          if (first < a.n_units) hid[(long long)first * DSUM + unit] = (sum[0] + sum[GROUPS - 1]) * inv_c;
+        } else {
+#pragma unroll
+          for (int g = 0; g < GROUPS; ++g)
+            if (first + g < a.n_units) hid[(long long)(first + g) * DSUM + unit] = sum[g] * inv_c;
+        }
+      } else {
+        float* pl = pool + (item_parity & 1) * 4 * TM_MAX_DSUM;
+#pragma unroll
+        for (int g = 0; g < GROUPS; ++g) pl[(col0 / 32 + g) * TM_MAX_DSUM + unit] = sum[g];
+        asm volatile("bar.sync 1, %0;" ::"n"(TM_EPI_WARPS * 32) : "memory");      // the other parity keeps the next item apart
+        for (int i = tid; i < a.units_per_item * DSUM; i += TM_EPI_WARPS * 32) {
+          const int u_in = i / DSUM, col = i - u_in * DSUM, u = item * a.units_per_item + u_in;
+          float s = 0.f;
+          for (int g = 0; g < chunk_groups; ++g) s += pl[(u_in * chunk_groups + g) * TM_MAX_DSUM + col];
+          if (u < a.n_units) hid[(long long)u * DSUM + col] = s * inv_c;
+        }
+        ++item_parity;
+      }
+#pragma unroll
+      for (int g = 0; g < GROUPS; ++g) sum[g] = 0.f;
       slice = 0;
       item += gridDim.x;
     }
   }
   umma::fence_before_sync();
   __syncthreads();
-  if (done_item >= 0) write_pooled(done_item, (int)((n_tiles - 1) & 1));
-  if (warp == 0) umma::tmem_dealloc(tmem_d, TM_TMEM_COLS);
+  if (warp == TM_MMA_WARP) umma::tmem_dealloc(tmem_d, TM_TMEM_COLS);
 }
 
 bool token_mlp_supported(int C, int d_sum) {
