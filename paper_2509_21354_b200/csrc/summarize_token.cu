@@ -36,10 +36,12 @@ constexpr int TM_THREADS = (TM_MMA_WARP + 1) * 32;
 constexpr int TM_MAX_DSUM = 256;
 constexpr int TM_KB_BYTES = TM_N * umma::KBLOCK_ROW_BYTES;  // 16 KB: 128 rows x 64 head dims
 constexpr int TM_SMEM_W1 = 0;                               // 2 K-blocks of [d_sum rows][64]: up to 64 KB
-constexpr int TM_SMEM_X = TM_SMEM_W1 + 2 * TM_MAX_DSUM * umma::KBLOCK_ROW_BYTES;   // 2 buffers x 2 K-blocks: 64 KB
-constexpr int TM_SMEM_POOL = TM_SMEM_X + 2 * 2 * TM_KB_BYTES;          // [2 tile parities][4 groups of 32 tokens][d_sum] sums
+constexpr int TM_XBUFS = 4;                                  // token buffers
+constexpr int TM_LAG = 2;                                    // tiles whose copies are under way behind the newest
+constexpr int TM_SMEM_X = TM_SMEM_W1 + 2 * TM_MAX_DSUM * umma::KBLOCK_ROW_BYTES;   // 4 buffers x 2 K-blocks: 128 KB
+constexpr int TM_SMEM_POOL = TM_SMEM_X + TM_XBUFS * 2 * TM_KB_BYTES;          // [2 tile parities][4 groups of 32 tokens][d_sum] sums
 constexpr int TM_SMEM_BAR = TM_SMEM_POOL + 2 * 4 * TM_MAX_DSUM * 4;
-constexpr int TM_SMEM_BYTES = TM_SMEM_BAR + 64 + 1024;      // + slack to reach a 1024-byte boundary
+constexpr int TM_SMEM_BYTES = TM_SMEM_BAR + 128 + 1024;      // + slack to reach a 1024-byte boundary
 constexpr int TM_TMEM_COLS = 512;                           // two accumulators of up to two slabs x 128 columns
 static_assert(TM_SMEM_BYTES > 116 * 1024, "one CTA per SM: each allocates all of tensor memory");
 
@@ -64,8 +66,9 @@ __global__ void __launch_bounds__(TM_THREADS, 1) kve_token_mlp_pool_kernel(Token
   unsigned char* W1s = smem + TM_SMEM_W1;
   unsigned char* Xs = smem + TM_SMEM_X;
   float* pool = reinterpret_cast<float*>(smem + TM_SMEM_POOL);
-  uint64_t* x_full = reinterpret_cast<uint64_t*>(smem + TM_SMEM_BAR);      // [2] token buffer filled by the copy warps
-  uint64_t* acc_full = x_full + 2;                                          // [2] accumulator written, token buffer read (MMA commit)
+  uint64_t* x_full = reinterpret_cast<uint64_t*>(smem + TM_SMEM_BAR);      // [4] token buffer filled by the copy warps
+  uint64_t* x_free = x_full + TM_XBUFS;                                     // [4] token buffer read (MMA commit)
+  uint64_t* acc_full = x_free + TM_XBUFS;                                   // [2] accumulator written (MMA commit)
   uint64_t* acc_free = acc_full + 2;                                        // [2] accumulator read by the epilogue warps
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_free + 2);
 
@@ -83,8 +86,11 @@ __global__ void __launch_bounds__(TM_THREADS, 1) kve_token_mlp_pool_kernel(Token
   }
   if (warp == TM_MMA_WARP) umma::tmem_alloc(tmem_slot, TM_TMEM_COLS);
   if (tid == 0) {
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < TM_XBUFS; ++i) {
       mbar_init(&x_full[i], TM_COPY_WARPS * 32);
+      mbar_init(&x_free[i], 1);
+    }
+    for (int i = 0; i < 2; ++i) {
       mbar_init(&acc_full[i], 1);
       mbar_init(&acc_free[i], TM_EPI_WARPS);
     }
@@ -123,11 +129,10 @@ __global__ void __launch_bounds__(TM_THREADS, 1) kve_token_mlp_pool_kernel(Token
     };
     look_up();
     bool ok = true;
-    for (int tile = 0; tile <= n_tiles && ok; ++tile) {
+    for (int tile = 0; tile < n_tiles + TM_LAG && ok; ++tile) {
       if (tile < n_tiles) {
-        const int buf = tile & 1;
-        // the products of two tiles ago have read this buffer
-        if (tile >= 2) ok = mbar_wait_bounded(&acc_full[buf], (uint32_t)(((tile >> 1) - 1) & 1));
+        const int buf = tile % TM_XBUFS;
+        if (tile >= TM_XBUFS) ok = mbar_wait_bounded(&x_free[buf], (uint32_t)((tile / TM_XBUFS - 1) & 1));
         long long src[4];                              // element offset of the first row taken from each chunk; -1: zeros
 #pragma unroll
         for (int x = 0; x < 4; ++x) {
@@ -143,13 +148,12 @@ __global__ void __launch_bounds__(TM_THREADS, 1) kve_token_mlp_pool_kernel(Token
           const int r = r0 + 8 * i, r_in = r & ((1 << chunk_shift) - 1);
           cp_async16(dst0 + buf * 2 * TM_KB_BYTES + umma::piece_offset(r, p16 & 7), pages + (base < 0 ? 0 : base + r_in * D), base >= 0);
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
       }
-      if (tile > 0) {      // the tile before has arrived
-        if (tile < n_tiles) asm volatile("cp.async.wait_group 1;" ::: "memory");
-        else asm volatile("cp.async.wait_group 0;" ::: "memory");
+      asm volatile("cp.async.commit_group;" ::: "memory");      // (an empty group at the end keeps the count)
+      if (tile >= TM_LAG) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(TM_LAG) : "memory");
         umma::fence_smem_to_async();
-        mbar_arrive(&x_full[(tile - 1) & 1]);
+        mbar_arrive(&x_full[(tile - TM_LAG) % TM_XBUFS]);
       }
     }
     if (!ok) set_status(v.status, ERR_TIMEOUT);
@@ -160,8 +164,8 @@ __global__ void __launch_bounds__(TM_THREADS, 1) kve_token_mlp_pool_kernel(Token
       constexpr uint32_t idesc = umma::instr_desc_bf16(TM_SLAB, TM_N);
       const uint32_t x_base = smem_u32(Xs), w1_base = smem_u32(W1s);
       for (int tile = 0; tile < n_tiles; ++tile) {
-        const int buf = tile & 1;
-        if (!mbar_wait_bounded(&x_full[buf], (uint32_t)((tile >> 1) & 1)) ||
+        const int buf = tile & 1, xb = tile % TM_XBUFS;
+        if (!mbar_wait_bounded(&x_full[xb], (uint32_t)((tile / TM_XBUFS) & 1)) ||
             (tile >= 2 && !mbar_wait_bounded(&acc_free[buf], (uint32_t)(((tile >> 1) - 1) & 1)))) {
           set_status(v.status, ERR_TIMEOUT);
           break;
@@ -175,7 +179,8 @@ __global__ void __launch_bounds__(TM_THREADS, 1) kve_token_mlp_pool_kernel(Token
             for (int k = 0; k < 4; ++k)
               umma::mma_bf16(tmem_d + (uint32_t)(buf * SLABS + sl) * TM_N,
                              umma::smem_desc(w1_base + kb * (DSUM * umma::KBLOCK_ROW_BYTES) + sl * (TM_SLAB * umma::KBLOCK_ROW_BYTES) + k * 32),
-                             umma::smem_desc(x_base + (buf * 2 + kb) * TM_KB_BYTES + k * 32), idesc, (kb | k) != 0);
+                             umma::smem_desc(x_base + (xb * 2 + kb) * TM_KB_BYTES + k * 32), idesc, (kb | k) != 0);
+        umma::commit(&x_free[xb]);
         umma::commit(&acc_full[buf]);
       }
     }
@@ -185,7 +190,7 @@ __global__ void __launch_bounds__(TM_THREADS, 1) kve_token_mlp_pool_kernel(Token
     const int lg = warp & 3, quarter = warp >> 2;
     const int slab = SLABS == 2 ? quarter >> 1 : 0, col0 = (SLABS == 2 ? quarter & 1 : quarter) * COLS;
     const int unit = slab * TM_SLAB + lg * 32 + lane;
-    const float b1_scaled = (side ? a.w.b1V : a.w.b1K)[unit] * GELU_SCALE;
+    const float b1 = (side ? a.w.b1V : a.w.b1K)[unit];
     const uint32_t tmem_t = tmem_d + (uint32_t)(slab * TM_N + col0) + ((uint32_t)(lg * 32) << 16);
     const float inv_c = 1.f / (float)v.C;
     float* hid = a.hid + (long long)side * a.n_units * DSUM;
@@ -220,15 +225,14 @@ __global__ void __launch_bounds__(TM_THREADS, 1) kve_token_mlp_pool_kernel(Token
           }
 #pragma unroll
           for (int e = 0; e < 16; e += 2) {
-            float2 relu, ea;
-            const float2 u = fma2(make_float2(__uint_as_float(h[q][e]), __uint_as_float(h[q][e + 1])), make_float2(GELU_SCALE, GELU_SCALE),
-                                  make_float2(b1_scaled, b1_scaled));
-            const float2 p = gelu_tail2(u, relu, ea);
-            tail_sum = fma2(ea, p, tail_sum);
+            float2 relu, abs_x;
+            const float2 x = add2(make_float2(__uint_as_float(h[q][e]), __uint_as_float(h[q][e + 1])), make_float2(b1, b1));
+            const float2 tail = gelu_tail2(x, relu, abs_x);
+            tail_sum = fma2(abs_x, tail, tail_sum);
             relu_sum = add2(relu_sum, relu);
           }
         }
-        sum[g] += (relu_sum.x + relu_sum.y) * (1.f / GELU_SCALE) - (tail_sum.x + tail_sum.y);
+        sum[g] += (relu_sum.x + relu_sum.y) - (tail_sum.x + tail_sum.y);
       }
       if (++slice < a.tiles_per_item) continue;
       // the chunk(s) of this item are complete
