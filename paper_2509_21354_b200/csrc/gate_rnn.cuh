@@ -12,9 +12,9 @@ constexpr int RNN_THREADS = RNN_WARPS * 32;
 
 struct RnnArgs {
   const float* P;          // [S * n_range][4 d_g], column 4 u + gate: the pre-activations W_ih x + b of unit u
-  float* H;                // [S * n_range][d_g]: h_t for the score kernel
+  float* H;                // [S * n_range][d_g / 8]: partial sums of w_s . h_t for the score kernel
   const uint16_t* W_hh;    // bf16 [4 d_g][d_g]
-  const float* w_s;        // [d_g] (score kernel)
+  const float* w_s;        // [d_g]
   float b_s;
   float* scores;           // [S][max_chunks]
   float* lstm_h;           // [S][d_g]
@@ -82,6 +82,23 @@ __device__ __forceinline__ void cluster_sync_all() {
 
 __device__ __forceinline__ float fast_sigmoid(float x) { return __fdividef(1.f, 1.f + __expf(-x)); }
 __device__ __forceinline__ float fast_tanh(float x) { return 2.f * fast_sigmoid(2.f * x) - 1.f; }
+// One LSTM cell: pre-activations in the order i, f, g, o; updates c, returns h.  With E(x) = 2^(-x log2 e):
+//   c = f c + i g = [c (1 + E_i)(1 + E_2g) + (1 - E_2g)(1 + E_f)] / [(1 + E_f)(1 + E_i)(1 + E_2g)],  h = (1 - E_2c) / [(1 + E_o)(1 + E_2c)]
+// five exponentials and two reciprocals.  The exponents stop at 40 (a sigmoid of 1e-12), which keeps the products finite.
+__device__ __forceinline__ float exp2_neg_capped(float x, float scale) {      // 2^(-x scale), at most 2^40; NaN stays NaN
+  float y;
+  asm("min.NaN.f32 %0, %1, 0f42200000;" : "=f"(y) : "f"(-x * scale));
+  return ex2_fast(y);
+}
+__device__ __forceinline__ float lstm_cell(const float (&pre)[4], float& c) {
+  constexpr float L2E = 1.44269504088896340736f;
+  const float ei = 1.f + exp2_neg_capped(pre[0], L2E), ef = 1.f + exp2_neg_capped(pre[1], L2E);
+  const float g2 = exp2_neg_capped(pre[2], 2.f * L2E), eo = 1.f + exp2_neg_capped(pre[3], L2E);
+  const float eg = 1.f + g2, ig = ei * eg;
+  c = __fdividef(fmaf(c, ig, (1.f - g2) * ef), ef * ig);
+  const float c2 = exp2_neg_capped(c, 2.f * L2E);
+  return __fdividef(1.f - c2, eo * (1.f + c2));
+}
 // four 8 x 8 b16 blocks of shared memory as mma fragments (lane l gives the address of row l & 7 of block l >> 3)
 __device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], uint32_t addr) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
