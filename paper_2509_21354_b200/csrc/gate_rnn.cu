@@ -247,7 +247,11 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RNN_THREADS, 1) kve
       }
       KVE_RNN_MARK(1);
 
-      if (NG > 1) load_p((gi + 1) % NG, step + (gi + 1) / NG, pv);
+      if (NG > 1) {
+        // (the vote is a scheduling fence: without it the compiler spreads the loads' address arithmetic over the MMA chain)
+        if (!__all_sync(0xffffffffu, alive)) break;
+        load_p((gi + 1) % NG, step + (gi + 1) / NG, pv);
+      }
       // ---- cell update (thread-local), planes of h_t into the warp's staging area ---------------------
       if (CL > 1) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
       __syncwarp();      // earlier copies have read the staging area
