@@ -237,27 +237,50 @@ __global__ void __launch_bounds__(MLP_THREADS) kve_chunk_mlp_kernel(LayerView v,
 // core forms is exact and the result differs from a plain fp32 loop only in summation order.
 //  * A CTA serves one side (keys or values) and keeps that side's W1 and W2 (64 KB each, K-major,
 //    128-byte swizzle) in shared memory for all its tiles.
-//  * Layer 1: 24 tcgen05.mma (3 planes x K/16) of shape 128 x d_sum accumulate H in tensor memory.
-//  * Layer 2 runs in slices of 64 hidden units: the eight warps read a slice of H from tensor
-//    memory, add b1, apply the erf GELU, split into planes and store them as the next A operand
-//    (double-buffered, 48 KB per slice, in the space the layer-1 planes have left); one thread
-//    issues the slice's 12 MMAs into the second accumulator while the warps prepare the next slice.
-//  * Epilogue: Y + b2 -> fp32 summary and its bf16 rounding.
+//  * Warps 8-15 load the means of a tile, split them and store the planes as the A operand of layer 1 (96 KB); later they take
+//    Y of the tile before out of tensor memory, add b2 and write the fp32 summary and its bf16 rounding.
+//  * Warp 16 (one thread) issues the MMAs: layer 1 in halves of 128 hidden units into two accumulators, layer 2 in slices of
+//    32 units into Y - whichever has its inputs ready.
+//  * Warps 0-7, two groups of four, take the slices in turn: 32 hidden units of a row per thread out of tensor memory, b1, GELU,
+//    split, and back into TENSOR memory as the A operand of layer 2 (shared memory is full).  One group's slice is
+//    multiplied while the other's is worked out.
+// So layer 1 of a tile, its activations, layer 2 and the output of the tile before overlap.  Per tile the MMAs now take
+// ~13000 cycles (the ones with their left operand in tensor memory 130 to 180 each, the others 85) and the activations
+// ~9000 per warp; with all sixteen warps going through the phases together a tile took 22500 cycles.  512 x 121 chunks:
+// 96 -> 88 us; the second layer alone on 256 x 56 chunks 25 -> 15 us; small launches (256 x 56 chunks: 33 us) are the weights'
+// way into shared memory and the latency of one or two tiles, and did not change.
+// POOLED: the second layer alone, on the pooled activations hid [2][n_units][d_sum] of the per-token aggregator.
 // Every mbarrier wait is bounded; on give-up the status word gets KVE_ERR_TIMEOUT.
 constexpr int MT_M = 128;
-constexpr int MT_THREADS = 512;   // 16 warps: four per scheduler, to hide the latency of the GELU / split phases
+constexpr int MT_GELU_WARPS = 8, MT_IO_WARPS = 8;
+constexpr int MT_MMA_WARP = MT_GELU_WARPS + MT_IO_WARPS;
+constexpr int MT_THREADS = (MT_MMA_WARP + 1) * 32;
 constexpr int MT_MAX_DSUM = 256;
+constexpr int MT_SLICE = 32;                                              // hidden units per layer-2 slice
 constexpr int MT_PLANE_KB_BYTES = MT_M * umma::KBLOCK_ROW_BYTES;          // 16 KB: one plane, one K-block of 64
-constexpr int MT_SMEM_A = 0;                                              // 96 KB: 3 planes x 2 K-blocks, later 2 x (3 planes x 1)
+constexpr int MT_SMEM_A = 0;                                              // 96 KB: 3 planes x 2 K-blocks
 constexpr int MT_SMEM_W1 = MT_SMEM_A + 6 * MT_PLANE_KB_BYTES;
 constexpr int MT_SMEM_W2 = MT_SMEM_W1 + MT_MAX_DSUM * D * 2;
 constexpr int MT_SMEM_B1 = MT_SMEM_W2 + D * MT_MAX_DSUM * 2;
 constexpr int MT_SMEM_B2 = MT_SMEM_B1 + MT_MAX_DSUM * 4;
 constexpr int MT_SMEM_BAR = MT_SMEM_B2 + D * 4;
-constexpr int MT_SMEM_BYTES = MT_SMEM_BAR + 64 + 1024;                    // + slack to reach a 1024-byte boundary
-constexpr int MT_TMEM_COLS = 512;                                         // H: columns [0, d_sum), Y: columns [256, 384)
-constexpr int MT_TMEM_Y = 256;
+constexpr int MT_SMEM_BYTES = MT_SMEM_BAR + 128 + 1024;                   // + slack to reach a 1024-byte boundary
+static_assert(MT_SMEM_BYTES <= 227 * 1024, "shared memory of one CTA");
+constexpr int MT_TMEM_COLS = 512;      // H halves: columns 0 and 128; Y: 256; activations of the two groups: 384, 432 (3 planes x 16)
+constexpr int MT_TMEM_Y = 256, MT_TMEM_ACT = 384, MT_ACT_COLS = 3 * MT_SLICE / 2;
 
+// 8 consecutive floats with one 32-byte access (a whole sector)
+__device__ __forceinline__ void load8(const float* p, float (&x)[8]) {
+  asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]), "=f"(x[4]), "=f"(x[5]), "=f"(x[6]), "=f"(x[7])
+               : "l"(p)
+               : "memory");
+}
+__device__ __forceinline__ void store8(float* p, const float (&x)[8]) {
+  asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]), "f"(x[4]),
+               "f"(x[5]), "f"(x[6]), "f"(x[7])
+               : "memory");
+}
 // splits 8 consecutive fp32 values and stores the three 16-byte pieces at dst + pl * plane_stride
 __device__ __forceinline__ void store_split8(const float (&x)[8], unsigned char* dst, int plane_stride) {
   uint32_t w[4][3];
@@ -268,9 +291,8 @@ __device__ __forceinline__ void store_split8(const float (&x)[8], unsigned char*
     *reinterpret_cast<uint4*>(dst + pl * plane_stride) = make_uint4(w[0][pl], w[1][pl], w[2][pl], w[3][pl]);
 }
 
-// POOLED: the second layer alone, on the pooled activations hid [2][n_units][d_sum] of the per-token aggregator
 template <bool POOLED>
-__global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerView v, int t0, int n_range, long long n_units,
+__global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerView v, int t0, int n_range, FastDiv by_range, int n_units,
                                                                          MlpWeights w, int d_sum, int dev_window,
                                                                          const float* __restrict__ hid) {
   extern __shared__ unsigned char smem_raw[];
@@ -280,21 +302,23 @@ __global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerVi
   unsigned char* W2s = smem + MT_SMEM_W2;
   float* b1s = reinterpret_cast<float*>(smem + MT_SMEM_B1);
   float* b2s = reinterpret_cast<float*>(smem + MT_SMEM_B2);
-  uint64_t* bar_h = reinterpret_cast<uint64_t*>(smem + MT_SMEM_BAR);       // layer-1 MMAs done
-  uint64_t* bar_buf = bar_h + 1;                                            // [2]: slice MMAs that read buffer b done
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + MT_SMEM_BAR + 32);
+  uint64_t* a_full = reinterpret_cast<uint64_t*>(smem + MT_SMEM_BAR);      // planes of a tile's means stored
+  uint64_t* a_free = a_full + 1;                                            // ... read (layer 1 done)
+  uint64_t* h_full = a_free + 1;                                            // [2] accumulator of a half written
+  uint64_t* h_free = h_full + 2;                                            // [2] ... read
+  uint64_t* act_full = h_free + 2;                                          // [2] a group's slice of activations stored
+  uint64_t* act_free = act_full + 2;                                        // [2] ... multiplied
+  uint64_t* y_full = act_free + 2;                                          // Y of a tile complete
+  uint64_t* y_free = y_full + 1;                                            // ... read
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(y_free + 1);
 
   pdl_launch_dependents();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int side = blockIdx.y;
   const uint16_t* W1 = side ? w.W1V : w.W1K;
   const uint16_t* W2 = side ? w.W2V : w.W2K;
-  const float* b1 = side ? w.b1V : w.b1K;
-  const float* b2 = side ? w.b2V : w.b2K;
   float* sum_f32 = side ? v.vsum_f32 : v.ksum_f32;
   uint16_t* sum_b16 = side ? v.vsum_bf16 : v.ksum_bf16;
-  const int n_slices = d_sum / 64;
-  const long long n_tiles = (n_units + MT_M - 1) / MT_M;
 
   // ---- one-time set-up -----------------------------------------------------------------------------
   for (int i = tid; !POOLED && i < d_sum * 16; i += MT_THREADS) {   // W1 [d_sum][128]: rows of 16 pieces, 2 K-blocks
@@ -303,18 +327,25 @@ __global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerVi
                reinterpret_cast<const uint4*>(W1 + (long long)r * D) + p, true);
   }
   const int w2_pieces = d_sum / 8;
-  for (int i = tid; i < D * w2_pieces; i += MT_THREADS) {           // W2 [128][d_sum]: n_slices K-blocks of 16 KB
+  for (int i = tid; i < D * w2_pieces; i += MT_THREADS) {           // W2 [128][d_sum]: K-blocks of 16 KB
     const int r = i / w2_pieces, p = i - r * w2_pieces;
     cp_async16(W2s + (p >> 3) * MT_PLANE_KB_BYTES + umma::piece_offset(r, p & 7),
                reinterpret_cast<const uint4*>(W2 + (long long)r * d_sum) + p, true);
   }
-  for (int i = tid; !POOLED && i < d_sum; i += MT_THREADS) b1s[i] = b1[i];
-  for (int i = tid; i < D; i += MT_THREADS) b2s[i] = b2[i];
-  if (warp == 0) umma::tmem_alloc(tmem_slot, MT_TMEM_COLS);
+  for (int i = tid; !POOLED && i < d_sum; i += MT_THREADS) b1s[i] = (side ? w.b1V : w.b1K)[i];
+  for (int i = tid; i < D; i += MT_THREADS) b2s[i] = (side ? w.b2V : w.b2K)[i];
+  if (warp == MT_MMA_WARP) umma::tmem_alloc(tmem_slot, MT_TMEM_COLS);
   if (tid == 0) {
-    mbar_init(bar_h, 1);
-    mbar_init(&bar_buf[0], 1);
-    mbar_init(&bar_buf[1], 1);
+    mbar_init(a_full, MT_IO_WARPS);
+    mbar_init(a_free, 1);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&h_full[i], 1);
+      mbar_init(&h_free[i], MT_GELU_WARPS);
+      mbar_init(&act_full[i], MT_GELU_WARPS / 2);
+      mbar_init(&act_free[i], 1);
+    }
+    mbar_init(y_full, 1);
+    mbar_init(y_free, MT_IO_WARPS);
     mbar_fence_init();
   }
   cp_async_wait_all();
@@ -322,188 +353,189 @@ __global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerVi
   umma::fence_before_sync();
   __syncthreads();
   umma::fence_after_sync();
-  const uint32_t tmem_h = *tmem_slot, tmem_y = tmem_h + MT_TMEM_Y;
-  const uint32_t idesc1 = umma::instr_desc_bf16(MT_M, d_sum), idesc2 = umma::instr_desc_bf16(MT_M, D);
-  const uint32_t a_base = smem_u32(As), w1_base = smem_u32(W1s), w2_base = smem_u32(W2s);
-  const int lg = warp & 3, part = warp >> 2;      // tensor-memory lanes 32 lg .., column part (0..3) of whatever is read
-  const int row_in_tile = lg * 32 + lane;
-  const uint32_t tmem_lane = (uint32_t)(lg * 32) << 16;
+  const uint32_t tmem = *tmem_slot;
 
   pdl_wait();      // weights, barriers and tensor memory are set up; the chunk means come from the previous kernel
-  uint32_t ph_h = 0, ph_buf[2] = {0, 0};
-  bool failed = false, due = true;
+  int n_tiles = (n_units + MT_M - 1) / MT_M;
   if (dev_window >= 0) {      // one chunk per sequence, found on the device
     const NextChunk nx = next_chunk(v.n_listed, v.seq_len, v.C, dev_window, v.max_chunks);
-    due = nx.due;
+    if (!nx.due) n_tiles = 0;
     t0 = nx.t;
   }
-  for (long long tile = blockIdx.x; tile < n_tiles && !failed && due; tile += gridDim.x) {
-    const long long unit0 = tile * MT_M;
-    if constexpr (!POOLED) {
-    // ---- chunk means -> three bf16 planes (layer-1 A operand) ------------------------------------------
-    {
-      // a thread keeps its 32-byte column pc and walks down 4 rows: all 8 loads first, then the splits
-      // (32-bit index arithmetic, one division per row; the host checks the ranges)
-      const int pc = tid & 15;
-      const uint32_t u0 = (uint32_t)unit0, nr = (uint32_t)n_range, total = (uint32_t)n_units;
-      float4 lo[4], hi[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const uint32_t unit = u0 + (tid >> 4) + 32 * i;
-        lo[i] = hi[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (unit < total) {
-          const uint32_t s = unit / nr;
-          const uint32_t t = (uint32_t)t0 + (unit - s * nr);
-          const float4* src = reinterpret_cast<const float4*>(sum_f32 + (size_t)(s * (uint32_t)v.max_chunks + t) * D + pc * 8);
-          lo[i] = src[0];
-          hi[i] = src[1];
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int r = (tid >> 4) + 32 * i;
-        const float x[8] = {lo[i].x, lo[i].y, lo[i].z, lo[i].w, hi[i].x, hi[i].y, hi[i].z, hi[i].w};
-        // plane pl, K-block kb at (pl * 2 + kb) * 16 KB
-        store_split8(x, As + (pc >> 3) * MT_PLANE_KB_BYTES + umma::piece_offset(r, pc & 7), 2 * MT_PLANE_KB_BYTES);
-      }
-    }
-    umma::fence_smem_to_async();
-    __syncthreads();
-    if (tid == 0) {
-      umma::fence_after_sync();
-      bool acc = false;
-#pragma unroll 1
-      for (int pl = 2; pl >= 0; --pl)                 // smallest plane first
-#pragma unroll
-        for (int kb = 0; kb < 2; ++kb)
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            umma::mma_bf16(tmem_h, umma::smem_desc(a_base + (pl * 2 + kb) * MT_PLANE_KB_BYTES + k * 32),
-                           umma::smem_desc(w1_base + kb * (d_sum * umma::KBLOCK_ROW_BYTES) + k * 32), idesc1, acc);
-            acc = true;
-          }
-      umma::commit(bar_h);
-    }
-    {
-      const bool ok = mbar_wait_bounded(bar_h, ph_h);
-      ph_h ^= 1;
-      if (__syncthreads_or(!ok)) { failed = true; break; }
-    }
-    umma::fence_after_sync();
-    }
+  const int my_tiles = n_tiles > (int)blockIdx.x ? (n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
+  const int n_halves = (d_sum + 127) / 128, n_slices = d_sum / MT_SLICE;
+  auto summary_row = [&](int unit) -> long long {
+    const int s = (int)by_range.div((uint32_t)unit);
+    return (long long)s * v.max_chunks + t0 + (unit - s * n_range);
+  };
+  const uint32_t lane_bits = (uint32_t)((warp & 3) * 32) << 16;      // the tensor-memory lanes of this warp
+  const int row = (warp & 3) * 32 + lane;                             // row of the tile = tensor-memory lane
+  bool ok = true;
 
-    // ---- layer 2 in slices of 64 hidden units ------------------------------------------------------------
-    for (int j = 0; j < n_slices; ++j) {
-      const int buf = j & 1;
-      if (j >= 2) {        // the MMAs of slice j - 2 still read this buffer
-        const bool ok = mbar_wait_bounded(&bar_buf[buf], ph_buf[buf]);
-        ph_buf[buf] ^= 1;
-        if (__syncthreads_or(!ok)) { failed = true; break; }
-      }
-      float h[16];
-      if constexpr (POOLED) {
-        const long long unit = unit0 + row_in_tile;
-        const float4* src = reinterpret_cast<const float4*>(hid + ((long long)side * n_units + unit) * d_sum + j * 64 + part * 16);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float4 x = unit < n_units ? src[e] : make_float4(0.f, 0.f, 0.f, 0.f);
-          h[4 * e] = x.x; h[4 * e + 1] = x.y; h[4 * e + 2] = x.z; h[4 * e + 3] = x.w;
+  if (warp < MT_GELU_WARPS) {
+    // ================= activations =================
+    const int group = warp >> 2;
+    const uint32_t act = tmem + MT_TMEM_ACT + group * MT_ACT_COLS + lane_bits;
+    int n_act = 0;                                        // slices of this group so far
+    for (int k = 0; k < my_tiles && ok; ++k) {
+      const int unit = (blockIdx.x + k * gridDim.x) * MT_M + row;
+      for (int j = group; j < n_slices && ok; j += 2, ++n_act) {
+        const int half = k * n_halves + (j >> 2), hb = half & 1;      // running number of the half, its accumulator
+        if constexpr (!POOLED) {
+          if ((j & 3) == group) ok = __all_sync(0xffffffffu, mbar_wait_bounded(&h_full[hb], (uint32_t)((half >> 1) & 1)));
+          if (!ok) break;
+          umma::fence_after_sync();
         }
-      } else {
-        umma::tmem_ld16(tmem_h + tmem_lane + (uint32_t)(j * 64 + part * 16), h);
-      }
-      unsigned char* abuf = As + buf * 3 * MT_PLANE_KB_BYTES;
+        uint32_t p[3][16];
 #pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        float g[8];
+        for (int q = 0; q < 2; ++q) {
+          float h[16];
+          if constexpr (POOLED) {
+            const float* src = hid + ((long long)side * n_units + unit) * d_sum + j * MT_SLICE + q * 16;
 #pragma unroll
-        for (int e = 0; e < 8; e += 2) {
-          float2 y = make_float2(h[q * 8 + e], h[q * 8 + e + 1]);
-          if constexpr (!POOLED) y = gelu2(add2(y, *reinterpret_cast<const float2*>(b1s + j * 64 + part * 16 + q * 8 + e)));
-          g[e] = y.x; g[e + 1] = y.y;
+            for (int e = 0; e < 16; ++e) h[e] = 0.f;
+            if (unit < n_units) {
+              load8(src, reinterpret_cast<float(&)[8]>(h[0]));
+              load8(src + 8, reinterpret_cast<float(&)[8]>(h[8]));
+            }
+          } else {
+            umma::tmem_ld16(tmem + hb * 128 + (j & 3) * MT_SLICE + q * 16 + lane_bits, h);
+          }
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            float2 y = make_float2(h[2 * e], h[2 * e + 1]);
+            if constexpr (!POOLED) y = gelu2(add2(y, *reinterpret_cast<const float2*>(b1s + j * MT_SLICE + q * 16 + 2 * e)));
+            uint32_t s3[3];
+            split3_pair(y.x, y.y, s3);
+#pragma unroll
+            for (int pl = 0; pl < 3; ++pl) p[pl][q * 8 + e] = s3[pl];
+          }
         }
-        store_split8(g, abuf + umma::piece_offset(row_in_tile, part * 2 + q), MT_PLANE_KB_BYTES);
-      }
-      umma::fence_smem_to_async();
-      umma::fence_before_sync();
-      __syncthreads();
-      if (tid == 0) {
+        if (!POOLED && (j + 2 >= n_slices || (j & 3) >= 2)) {      // this group's last slice of the half
+          umma::fence_before_sync();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&h_free[hb]);
+        }
+        // the group's slice before has been multiplied
+        if (n_act > 0) ok = __all_sync(0xffffffffu, mbar_wait_bounded(&act_free[group], (uint32_t)((n_act - 1) & 1)));
+        if (!ok) break;
         umma::fence_after_sync();
-        const uint32_t ab = a_base + buf * 3 * MT_PLANE_KB_BYTES;
+#pragma unroll
+        for (int pl = 0; pl < 3; ++pl) umma::tmem_st16_nowait(act + pl * (MT_SLICE / 2), p[pl]);
+        umma::tmem_st_wait();
+        umma::fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&act_full[group]);
+      }
+    }
+    if (!ok && lane == 0) set_status(v.status, ERR_TIMEOUT);
+  } else if (warp < MT_MMA_WARP) {
+    // ================= means in, summaries out =================
+    const int c0 = ((warp - MT_GELU_WARPS) >> 2) * 64;      // this thread's 64 columns of its row: K-block c0 / 64
+    // a thread keeps its 32-byte column and walks down 8 rows, so that a warp's load covers whole rows
+    const int io = tid - MT_GELU_WARPS * 32, pc = io & 15;
+    for (int k = POOLED ? 0 : -1; k < my_tiles && ok; ++k) {      // round k: the means of tile k + 1 in, then the summaries of tile k out
+      if (!POOLED && k + 1 < my_tiles) {
+        const int unit0 = (blockIdx.x + (k + 1) * gridDim.x) * MT_M + (io >> 4);
+        float x[8][8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int unit = unit0 + 16 * i;
+#pragma unroll
+          for (int e = 0; e < 8; ++e) x[i][e] = 0.f;
+          if (unit < n_units) load8(sum_f32 + summary_row(unit) * D + pc * 8, x[i]);
+        }
+        if (k >= 0) ok = __all_sync(0xffffffffu, mbar_wait_bounded(a_free, (uint32_t)(k & 1)));
+        if (!ok) break;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)      // plane pl, K-block kb at (pl * 2 + kb) * 16 KB
+          store_split8(x[i], As + (pc >> 3) * MT_PLANE_KB_BYTES + umma::piece_offset((io >> 4) + 16 * i, pc & 7), 2 * MT_PLANE_KB_BYTES);
+        umma::fence_smem_to_async();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(a_full);
+      }
+      if (k < 0) continue;
+      ok = __all_sync(0xffffffffu, mbar_wait_bounded(y_full, (uint32_t)(k & 1)));
+      if (!ok) break;
+      umma::fence_after_sync();
+      float y[2][32];
+      umma::tmem_ld32(tmem + MT_TMEM_Y + c0 + lane_bits, y[0]);
+      umma::tmem_ld32(tmem + MT_TMEM_Y + c0 + 32 + lane_bits, y[1]);
+      umma::fence_before_sync();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(y_free);
+      const int unit = (blockIdx.x + k * gridDim.x) * MT_M + row;
+      if (unit < n_units) {
+        const long long o = summary_row(unit) * D + c0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          float z[8];
+#pragma unroll
+          for (int e = 0; e < 8; ++e) z[e] = y[q >> 2][(q & 3) * 8 + e] + b2s[c0 + q * 8 + e];
+          store8(sum_f32 + o + q * 8, z);
+          *reinterpret_cast<uint4*>(sum_b16 + o + q * 8) =
+              make_uint4(pack_bf16x2(z[0], z[1]), pack_bf16x2(z[2], z[3]), pack_bf16x2(z[4], z[5]), pack_bf16x2(z[6], z[7]));
+        }
+      }
+    }
+    if (!ok && lane == 0) set_status(v.status, ERR_TIMEOUT);
+  } else if (lane == 0) {
+    // ================= MMA issue (one thread) =================
+    const uint32_t a_base = smem_u32(As), w1_base = smem_u32(W1s), w2_base = smem_u32(W2s);
+    constexpr uint32_t idesc2 = umma::instr_desc_bf16(MT_M, D);
+    const int n_l1 = POOLED ? 0 : my_tiles * n_halves, n_l2 = my_tiles * n_slices;
+    int l1 = 0, l2 = 0, l1_tile = 0, l1_half = 0, l2_tile = 0, l2_slice = 0;
+    uint32_t idle = 0;
+    while (l2 < n_l2) {
+      bool progress = false;
+      // layer 1: a half of a tile's hidden units into accumulator l1 & 1, once that has been read
+      if (l1 < n_l1 && mbar_test_wait(a_full, (uint32_t)(l1_tile & 1)) &&
+          (l1 < 2 || mbar_test_wait(&h_free[l1 & 1], (uint32_t)(((l1 >> 1) - 1) & 1)))) {
+        umma::fence_after_sync();
+        const int width = d_sum - l1_half * 128 < 128 ? 64 : 128;
+        const uint32_t idesc1 = umma::instr_desc_bf16(MT_M, width);
+        bool acc = false;
+#pragma unroll 1
+        for (int pl = 2; pl >= 0; --pl)                 // smallest plane first
+#pragma unroll 1
+          for (int kb = 0; kb < 2; ++kb)
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+              umma::mma_bf16(tmem + (l1 & 1) * 128, umma::smem_desc(a_base + (pl * 2 + kb) * MT_PLANE_KB_BYTES + s * 32),
+                             umma::smem_desc(w1_base + kb * (d_sum * umma::KBLOCK_ROW_BYTES) + l1_half * 128 * umma::KBLOCK_ROW_BYTES + s * 32), idesc1, acc);
+              acc = true;
+            }
+        umma::commit(&h_full[l1 & 1]);
+        ++l1;
+        if (++l1_half == n_halves) { l1_half = 0; ++l1_tile; umma::commit(a_free); }
+        progress = true;
+      }
+      // layer 2: 32 hidden units; the first slice of a tile overwrites Y, once that has been read
+      if (mbar_test_wait(&act_full[l2_slice & 1], (uint32_t)(((l2_tile * n_slices + l2_slice) >> 1) & 1)) &&
+          (l2_slice > 0 || l2_tile == 0 || mbar_test_wait(y_free, (uint32_t)((l2_tile - 1) & 1)))) {
+        umma::fence_after_sync();
+        const uint32_t act = tmem + MT_TMEM_ACT + (l2_slice & 1) * MT_ACT_COLS;
+        const uint32_t wb = w2_base + (l2_slice >> 1) * MT_PLANE_KB_BYTES + (l2_slice & 1) * 64;
 #pragma unroll 1
         for (int pl = 2; pl >= 0; --pl)
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
-            umma::mma_bf16(tmem_y, umma::smem_desc(ab + pl * MT_PLANE_KB_BYTES + k * 32),
-                           umma::smem_desc(w2_base + j * MT_PLANE_KB_BYTES + k * 32), idesc2, !(j == 0 && pl == 2 && k == 0));
-        umma::commit(&bar_buf[buf]);
+          for (int s = 0; s < 2; ++s)
+            umma::mma_bf16_ts(tmem + MT_TMEM_Y, act + pl * (MT_SLICE / 2) + s * 8, umma::smem_desc(wb + s * 32), idesc2,
+                              !(l2_slice == 0 && pl == 2 && s == 0));
+        umma::commit(&act_free[l2_slice & 1]);
+        ++l2;
+        if (++l2_slice == n_slices) { l2_slice = 0; ++l2_tile; umma::commit(y_full); }
+        progress = true;
       }
+      if (progress) idle = 0;
+      else if (++idle > (1u << 24)) { set_status(v.status, ERR_TIMEOUT); break; }
+      else if (idle > 4096) __nanosleep(64);
     }
-    if (failed) break;
-    // drain: one outstanding commit per buffer that was used (the later one covers every MMA before it)
-    {
-      bool ok = true;
-      const int first = (n_slices >= 2) ? (n_slices & 1) : 0;     // older buffer first
-      for (int u = 0; u < (n_slices >= 2 ? 2 : 1); ++u) {
-        const int b = (first + u) & 1;
-        ok = mbar_wait_bounded(&bar_buf[b], ph_buf[b]) && ok;
-        ph_buf[b] ^= 1;
-      }
-      if (__syncthreads_or(!ok)) { failed = true; break; }
-    }
-    umma::fence_after_sync();
-
-    // ---- epilogue: Y + b2 -> fp32 summary and its bf16 rounding ----------------------------------------------
-    // The operand space is idle now: it holds the output row table and, per warp, a 32 x 32 block on
-    // its way out.  tcgen05.ld hands a thread one row; the block is turned through shared memory
-    // (16-byte groups, group q of row r at position q ^ (r & 7)) so that every store instruction
-    // writes whole 128-byte (fp32) / 64-byte (bf16) row segments.
-    {
-      int* row_tab = reinterpret_cast<int*>(As + (MT_THREADS / 32) * 4096);       // [128] summary row, -1 beyond the end
-      float* stg = reinterpret_cast<float*>(As) + warp * 1024;
-      if (tid < MT_M) {
-        const long long unit = unit0 + tid;
-        int o = -1;
-        if (unit < n_units) {
-          const uint32_t s = (uint32_t)unit / (uint32_t)n_range;
-          o = (int)(s * (uint32_t)v.max_chunks + (uint32_t)t0 + ((uint32_t)unit - s * (uint32_t)n_range));
-        }
-        row_tab[tid] = o;
-      }
-      __syncthreads();
-      {
-        const int c = part * 32;
-        float y[32];
-        umma::tmem_ld32(tmem_y + tmem_lane + (uint32_t)c, y);
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-          *reinterpret_cast<float4*>(stg + lane * 32 + ((q ^ (lane & 7)) << 2)) =
-              make_float4(y[4 * q] + b2s[c + 4 * q], y[4 * q + 1] + b2s[c + 4 * q + 1], y[4 * q + 2] + b2s[c + 4 * q + 2],
-                          y[4 * q + 3] + b2s[c + 4 * q + 3]);
-        __syncwarp();
-        const int q = lane & 7;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int rr = i * 4 + (lane >> 3);
-          const float4 val = *reinterpret_cast<const float4*>(stg + rr * 32 + ((q ^ (rr & 7)) << 2));
-          const int orow = row_tab[lg * 32 + rr];
-          if (orow >= 0) {
-            const size_t o = (size_t)orow * D + c + q * 4;
-            *reinterpret_cast<float4*>(sum_f32 + o) = val;
-            *reinterpret_cast<uint2*>(sum_b16 + o) = make_uint2(pack_bf16x2(val.x, val.y), pack_bf16x2(val.z, val.w));
-          }
-        }
-        __syncwarp();
-      }
-    }
-    umma::fence_before_sync();
-    __syncthreads();     // accumulators and operand space are free for the next tile
   }
-  if (failed && tid == 0) set_status(v.status, ERR_TIMEOUT);
 
   umma::fence_before_sync();
   __syncthreads();
-  if (warp == 0) umma::tmem_dealloc(tmem_h, MT_TMEM_COLS);
+  if (warp == MT_MMA_WARP) umma::tmem_dealloc(tmem, MT_TMEM_COLS);
 }
 
 cudaError_t launch_pooled_out(const LayerView& v, int t0, int t1, const MlpWeights& w, int d_sum, const float* hid, cudaStream_t st) {
@@ -516,7 +548,7 @@ cudaError_t launch_pooled_out(const LayerView& v, int t0, int t1, const MlpWeigh
   if (e != cudaSuccess) return e;
   const long long n_tiles = (n_units + MT_M - 1) / MT_M, half = sm_count() / 2;
   return launch_pdl(kve_chunk_mlp_tc_kernel<true>, dim3((unsigned)(n_tiles < half ? n_tiles : half), 2), dim3(MT_THREADS), MT_SMEM_BYTES, st, v,
-                    t0, n_range, n_units, w, d_sum, -1, hid);
+                    t0, n_range, fast_div((uint32_t)n_range), (int)n_units, w, d_sum, -1, hid);
 }
 
 cudaError_t launch_chunk_mlp(const LayerView& v, int t0, int t1, const MlpWeights& w, int d_sum, cudaStream_t st, int dev_window) {
@@ -534,7 +566,8 @@ cudaError_t launch_chunk_mlp(const LayerView& v, int t0, int t1, const MlpWeight
     const long long half = sm_count() / 2;
     const long long per_side = n_tiles < half ? n_tiles : half;  // one CTA per SM: half of the SMs per side
     dim3 grid((unsigned)per_side, 2);
-    return launch_pdl(kve_chunk_mlp_tc_kernel<false>, grid, dim3(MT_THREADS), MT_SMEM_BYTES, st, v, t0, n_range, n_units, w, d_sum, dev_window, nullptr);
+    return launch_pdl(kve_chunk_mlp_tc_kernel<false>, grid, dim3(MT_THREADS), MT_SMEM_BYTES, st, v, t0, n_range, fast_div((uint32_t)n_range), (int)n_units, w, d_sum, dev_window,
+                      nullptr);
   }
   const size_t smem = sizeof(float) * (size_t)MLP_ROWS * (D + d_sum);
   static DeviceFlags opted;
