@@ -45,8 +45,8 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 SCALE = 1.0 / math.sqrt(128.0)
 def kernels_per_step(wl, Nc):
     """kernel launches of one from-scratch step: set_len, append, chunk mean [+ chunk MLP], gate projection,
-    recurrence, score head, keep list, kept-row gather, attention"""
-    return 9 + (1 if wl.agg == "mlp" else 0)
+    recurrence with its score head, keep list with its gather, attention"""
+    return 7 + (1 if wl.agg == "mlp" else 0)
 
 
 def load_peaks():

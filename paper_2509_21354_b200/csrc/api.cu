@@ -265,13 +265,12 @@ void release_host_objects(kvE_store* st) {
     for (cudaEvent_t e : st->ev) cudaEventDestroy(e);
 }
 
-// the keep list no longer covers chunks from `value` on (their summaries or scores changed): host count and device count
-int lower_listed(kvE_store* st, int layer, int value, cudaStream_t stream) {
-  LayerState& ls = st->layers[layer];
-  if (ls.n_compacted <= value) return KVE_OK;
+// The keep list no longer covers chunks from `value` on (their summaries or scores change): the host count, and what the
+// kernel about to be launched makes the device count (-1: it stands)
+int lower_listed(LayerState& ls, int value) {
+  if (ls.n_compacted <= value) return -1;
   ls.n_compacted = value;
-  cudaError_t e = launch_set_listed(view(st, layer), value, stream);
-  return e == cudaSuccess ? KVE_OK : cuda_fail(st, e);
+  return value;
 }
 
 }  // namespace
@@ -427,9 +426,10 @@ int kvE_summarize_chunks(kvE_store* st, int layer, int chunk_begin, int chunk_en
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const LayerView v = view(st, layer);
   cudaError_t e = cudaSuccess;
+  const int list_cut = lower_listed(ls, chunk_begin);      // the compacted copies of these summaries are stale
   if (!token_mlp) {
     Prof prof(st, KVE_K_CHUNK_MEAN, s);
-    e = launch_chunk_mean(v, chunk_begin, chunk_end, !mlp, st->cfg.agg == KVE_AGG_MAX, s, -1);
+    e = launch_chunk_mean(v, chunk_begin, chunk_end, !mlp, st->cfg.agg == KVE_AGG_MAX, s, -1, list_cut);
   } else {
     Prof prof(st, KVE_K_CHUNK_MLP, s);
     MlpWeights mw;
@@ -437,7 +437,7 @@ int kvE_summarize_chunks(kvE_store* st, int layer, int chunk_begin, int chunk_en
     mw.W1V = static_cast<const uint16_t*>(w->W1V); mw.W2V = static_cast<const uint16_t*>(w->W2V);
     mw.b1K = w->b1K; mw.b2K = w->b2K; mw.b1V = w->b1V; mw.b2V = w->b2V;
     e = launch_chunk_token_mlp(v, chunk_begin, chunk_end, mw, st->cfg.d_sum,
-                               reinterpret_cast<float*>(static_cast<char*>(st->buf.workspace) + st->off_P), s);
+                               reinterpret_cast<float*>(static_cast<char*>(st->buf.workspace) + st->off_P), list_cut, s);
   }
   if (e == cudaSuccess && mlp) {
     Prof prof(st, KVE_K_CHUNK_MLP, s);
@@ -449,7 +449,7 @@ int kvE_summarize_chunks(kvE_store* st, int layer, int chunk_begin, int chunk_en
   }
   if (e != cudaSuccess) return cuda_fail(st, e);
   if (chunk_begin <= ls.n_summarised && chunk_end > ls.n_summarised) ls.n_summarised = chunk_end;
-  return lower_listed(st, layer, chunk_begin, s);                   // the compacted copies of these summaries are stale
+  return KVE_OK;
 }
 
 int kvE_gate(kvE_store* st, int layer, int chunk_begin, int chunk_end, const kvE_lstm_weights* w, void* stream) {
@@ -470,7 +470,7 @@ int kvE_gate(kvE_store* st, int layer, int chunk_begin, int chunk_end, const kvE
   {
     Prof prof(st, KVE_K_GATE_PROJ, s);
     e = launch_gate_proj(v, chunk_begin, chunk_end, static_cast<const uint16_t*>(w->W_ih), w->b_ih, w->b_hh,
-                         st->cfg.d_g, P, s);
+                         st->cfg.d_g, P, lower_listed(ls, chunk_begin), s);      // scores change under the keep list
   }
   if (e == cudaSuccess) {
     Prof prof(st, KVE_K_GATE_RNN, s);
@@ -480,7 +480,7 @@ int kvE_gate(kvE_store* st, int layer, int chunk_begin, int chunk_end, const kvE
   }
   if (e != cudaSuccess) return cuda_fail(st, e);
   ls.n_gated = chunk_end;
-  return lower_listed(st, layer, chunk_begin, s);                   // scores changed under the keep list
+  return KVE_OK;
 }
 
 int kvE_compact(kvE_store* st, int layer, float tau, void* stream) {
@@ -539,7 +539,7 @@ int kvE_refresh_next(kvE_store* st, int layer, const kvE_agg_weights* aw, const 
   cudaError_t e;
   {
     Prof prof(st, KVE_K_CHUNK_MEAN, s);
-    e = launch_chunk_mean(v, 0, 1, !mlp, st->cfg.agg == KVE_AGG_MAX, s, W);
+    e = launch_chunk_mean(v, 0, 1, !mlp, st->cfg.agg == KVE_AGG_MAX, s, W, -1);
   }
   if (e == cudaSuccess && mlp) {
     Prof prof(st, KVE_K_CHUNK_MLP, s);

@@ -99,16 +99,6 @@ cudaError_t launch_append_next(const LayerView& v, const void* k_new, const void
                     static_cast<const uint4*>(v_new), n_new, ticket);
 }
 
-__global__ void kve_set_listed_kernel(int32_t* n_listed, int listed) {
-  pdl_launch_dependents();
-  pdl_wait();
-  if (threadIdx.x == 0) *n_listed = listed;
-}
-
-cudaError_t launch_set_listed(const LayerView& v, int n_listed, cudaStream_t st) {
-  return launch_pdl(kve_set_listed_kernel, dim3(1), dim3(32), 0, st, v.n_listed, n_listed);
-}
-
 cudaError_t launch_set_len(const LayerView& v, int n, int n_listed, cudaStream_t st) {
   return launch_pdl(kve_set_len_kernel, dim3((v.B + 127) / 128), dim3(128), 0, st, v.seq_len, v.B, n, v.n_listed, n_listed);
 }

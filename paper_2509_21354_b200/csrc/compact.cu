@@ -1,6 +1,5 @@
 // kvE_compact kernel: the retention rule of Sec. 3.2, "keep chunk t iff s_t >= tau", turned into an
-// ascending list of kept chunk ids per sequence.  One warp per sequence: 32 scores per round, a
-// ballot gives the keep mask, popcount of the lower lanes gives each kept chunk its slot.
+// ascending list of kept chunk ids per sequence, and the kept chunks' summary rows copied into one run.
 #include "common.cuh"
 #include "kernels.h"
 
@@ -8,34 +7,60 @@ namespace kve {
 
 constexpr int COMPACT_WARPS = 4;
 
-__global__ void __launch_bounds__(COMPACT_WARPS * 32) kve_compact_kernel(LayerView v, int n_chunks, float tau) {
+// One CTA per sequence.  Every warp goes through the scores, 32 a round: a ballot gives the keep mask, popcount of the lower
+// lanes gives each kept chunk its slot.  The rounds' results are written by the warps in turn: the ids, and the kept summary
+// rows ("compacted chunk tokens", Sec. 3.3: attention then fetches them with one bulk copy per 64 rows), lanes 0-15 the
+// K row, lanes 16-31 the V row, 16 bytes each, GATHER_ROWS loads in flight.  (As two kernels, one warp per sequence and then
+// one per 8 kept rows, a second launch and a round trip of the list through memory: 2.2 us more in a chain of small launches.)
+constexpr int GATHER_ROWS = 8;
+
+__global__ void __launch_bounds__(COMPACT_WARPS * 32) kve_compact_kernel(LayerView v, int n_chunks, float tau, uint4* __restrict__ kkept,
+                                                                        uint4* __restrict__ vkept) {
   pdl_launch_dependents();
   pdl_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int s = blockIdx.x * COMPACT_WARPS + warp;
-  if (s >= v.S) return;
-  const float* sc = v.scores + (long long)s * v.max_chunks;
-  int32_t* idx = v.keep_idx + (long long)s * v.max_chunks;
+  const int s = blockIdx.x;
+  const long long sb = (long long)s * v.max_chunks;
+  const int is_v = lane >> 4, l16 = lane & 15;
+  const uint4* src = reinterpret_cast<const uint4*>(is_v ? v.vsum_bf16 : v.ksum_bf16) + l16;
+  uint4* dst = (is_v ? vkept : kkept) + l16;
   int base = 0;
-  for (int t0 = 0; t0 < n_chunks; t0 += 32) {
+  for (int t0 = 0, round = 0; t0 < n_chunks; t0 += 32, ++round) {
     const int t = t0 + lane;
-    const bool keep = (t < n_chunks) && (sc[t] >= tau);
-    const unsigned mask = __ballot_sync(0xffffffffu, keep);
-    if (keep) idx[base + __popc(mask & ((1u << lane) - 1u))] = t;
-    base += __popc(mask);
+    const bool keep = (t < n_chunks) && (v.scores[sb + t] >= tau);
+    unsigned mask = __ballot_sync(0xffffffffu, keep);
+    const int kept = __popc(mask);
+    if (round % COMPACT_WARPS == warp) {
+      if (keep) v.keep_idx[sb + base + __popc(mask & ((1u << lane) - 1u))] = t;
+      for (int i = 0; i < kept; i += GATHER_ROWS) {
+        uint4 w[GATHER_ROWS];
+        unsigned m = mask;
+#pragma unroll
+        for (int r = 0; r < GATHER_ROWS; ++r) {
+          if (i + r < kept) w[r] = __ldg(src + (sb + t0 + __ffs(m) - 1) * 16);
+          m &= m - 1;
+        }
+        mask = m;
+#pragma unroll
+        for (int r = 0; r < GATHER_ROWS; ++r)
+          if (i + r < kept) dst[(sb + base + i + r) * 16] = w[r];
+      }
+    }
+    base += kept;
   }
-  for (int t = base + lane; t < v.max_chunks; t += 32) idx[t] = -1;
-  if (lane == 0) v.keep_cnt[s] = base;
-  if (s == 0 && lane == 0) *v.n_listed = n_chunks;      // what the attention kernel reads: the list covers chunks [0, n_chunks)
+  for (int t = base + (int)threadIdx.x; t < v.max_chunks; t += COMPACT_WARPS * 32) v.keep_idx[sb + t] = -1;
+  if (threadIdx.x == 0) {
+    v.keep_cnt[s] = base;
+    if (s == 0) *v.n_listed = n_chunks;      // what the attention kernel reads: the list covers chunks [0, n_chunks)
+  }
 }
 
-// ---- what attention wants from a fresh keep list ---------------------------------------------------------
-// The kept chunks' summary rows, copied into one contiguous run per sequence ("compacted chunk tokens",
-// Sec. 3.3): attention then fetches a sequence's kept rows with one bulk copy per 64 rows instead of one
-// per row, on every decode step until the next trigger.  One warp moves 8 kept rows: lanes 0-15 the K
-// row, lanes 16-31 the V row, 16 bytes each, all 8 loads in flight.
-constexpr int GATHER_ROWS = 8;
+cudaError_t launch_compact(const LayerView& v, int n_chunks, float tau, void* kkept, void* vkept, cudaStream_t st) {
+  return launch_pdl(kve_compact_kernel, dim3((unsigned)v.S), dim3(COMPACT_WARPS * 32), 0, st, v, n_chunks, tau, static_cast<uint4*>(kkept),
+                    static_cast<uint4*>(vkept));
+}
 
+// ---- the kept rows of a list that is in memory already (top-k), compacted: one warp moves 8 kept rows --------------------
 __global__ void __launch_bounds__(COMPACT_WARPS * 32) kve_keep_gather_kernel(LayerView v, int n_chunks, int groups,
                                                                             uint4* __restrict__ kkept, uint4* __restrict__ vkept) {
   pdl_launch_dependents();
@@ -66,19 +91,12 @@ __global__ void __launch_bounds__(COMPACT_WARPS * 32) kve_keep_gather_kernel(Lay
     if (t[r] >= 0) dst[(sb + i0 + r) * 16 + l16] = w[r];
 }
 
-// after either retention rule: the kept rows, compacted
 static cudaError_t launch_keep_gather(const LayerView& v, int n_chunks, void* kkept, void* vkept, cudaStream_t st) {
   if (n_chunks <= 0) return cudaSuccess;
   const int groups = (n_chunks + GATHER_ROWS - 1) / GATHER_ROWS;
   const long long units = (long long)v.S * groups;
   return launch_pdl(kve_keep_gather_kernel, dim3((unsigned)((units + COMPACT_WARPS - 1) / COMPACT_WARPS)), dim3(COMPACT_WARPS * 32), 0, st,
                     v, n_chunks, groups, static_cast<uint4*>(kkept), static_cast<uint4*>(vkept));
-}
-
-cudaError_t launch_compact(const LayerView& v, int n_chunks, float tau, void* kkept, void* vkept, cudaStream_t st) {
-  cudaError_t e = launch_pdl(kve_compact_kernel, dim3((v.S + COMPACT_WARPS - 1) / COMPACT_WARPS), dim3(COMPACT_WARPS * 32), 0, st, v,
-                             n_chunks, tau);
-  return e == cudaSuccess ? launch_keep_gather(v, n_chunks, kkept, vkept, st) : e;
 }
 
 // ---- kvE_compact_topk kernel: keep the k highest-scoring chunks of every sequence --------------------------

@@ -38,7 +38,7 @@ __global__ void __launch_bounds__(PJ_THREADS, 1) kve_gate_proj_kernel(LayerView 
                                                                       const uint16_t* __restrict__ W_ih,
                                                                       const float* __restrict__ b_ih,
                                                                       const float* __restrict__ b_hh, int n_cols,
-                                                                      float* __restrict__ P) {
+                                                                      float* __restrict__ P, int list_cut) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   unsigned char* Bs = smem + PJ_SMEM_B;
@@ -136,6 +136,7 @@ __global__ void __launch_bounds__(PJ_THREADS, 1) kve_gate_proj_kernel(LayerView 
   };
 
   pdl_wait();      // the weight slice is on its way; the summaries come from the previous kernel
+  if (list_cut >= 0 && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *v.n_listed = list_cut;
   long long tile = blockIdx.y;
   if (tile < n_tiles) gather_a(tile);
   cp_async_wait_all();
@@ -175,7 +176,7 @@ __global__ void __launch_bounds__(PJ_THREADS, 1) kve_gate_proj_kernel(LayerView 
 }
 
 cudaError_t launch_gate_proj(const LayerView& v, int t0, int t1, const uint16_t* W_ih, const float* b_ih,
-                             const float* b_hh, int d_g, float* P, cudaStream_t st) {
+                             const float* b_hh, int d_g, float* P, int list_cut, cudaStream_t st) {
   const int n_range = t1 - t0;
   const long long n_rows = (long long)v.S * n_range;
   if (n_rows <= 0) return cudaSuccess;
@@ -193,7 +194,7 @@ cudaError_t launch_gate_proj(const LayerView& v, int t0, int t1, const uint16_t*
   if (row_ctas > n_tiles) row_ctas = n_tiles;
   if (row_ctas < 1) row_ctas = 1;
   dim3 grid((unsigned)col_slices, (unsigned)row_ctas);
-  return launch_pdl(kve_gate_proj_kernel, grid, dim3(PJ_THREADS), PJ_SMEM_BYTES, st, v, t0, n_range, n_rows, W_ih, b_ih, b_hh, n_cols, P);
+  return launch_pdl(kve_gate_proj_kernel, grid, dim3(PJ_THREADS), PJ_SMEM_BYTES, st, v, t0, n_range, n_rows, W_ih, b_ih, b_hh, n_cols, P, list_cut);
 }
 
 }  // namespace kve

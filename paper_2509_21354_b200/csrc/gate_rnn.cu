@@ -28,7 +28,7 @@
 //  * P_{t+1} is fetched a round ahead: the projection kernel stores the four pre-activations of a hidden unit side by side, so a
 //    thread takes them with one 16-byte load.
 //  * The score head is not part of the chain: a warp leaves its 8 units' share of w_s . h_t per sequence (d_g / 8 partial sums
-//    per (s, t)), and a second, fully parallel kernel adds them up in a fixed order (an eighth of the bytes of h_t).
+//    per (s, t): an eighth of the bytes of h_t), and when the chain is through the cluster adds them up in a fixed order.
 //  Measured, recurrence and score head: 512 sequences x 121 chunks 314 -> RNN_NG2 us, 256 x 56 92.5 -> RNN_NG1 us, 8 x 28 at
 //  d_g = 128 51.6 -> 33 us (there a cluster of two CTAs halves the MMA chain: one CTA held all of W_hh).  Slower: waiting for the
 //  CTA's own planes and the peers' apart, with the own units' MMAs in between (255 -> 261 us a step on 256 sequences), and
@@ -326,44 +326,21 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RNN_THREADS, 1) kve
         a.lstm_h[(long long)s * DG + ug] = hlast[gi][e];
       }
     }
-  // nobody leaves while a peer may still be sending into its shared memory
+  // nobody leaves while a peer may still be sending into its shared memory; the partial sums of all CTAs are in place behind it
   cluster_sync_all();
   KVE_RNN_ONCE(6);
-}
-
-// ---- score head: s_t = sigmoid(w_s . h_t + b_s) from the warps' partial sums, one thread per (sequence, chunk) row -------
-// A row's d_g / 8 partial sums lie side by side and are added in order.
-constexpr int SCORE_THREADS = 256;
-
-template <int PARTS>
-__global__ void __launch_bounds__(SCORE_THREADS) kve_gate_score_kernel(const float* __restrict__ parts, float b_s, float* __restrict__ scores,
-                                                                      long long n_rows, int n_range, int t0, int max_chunks) {
-  pdl_launch_dependents();
-  pdl_wait();
-  const long long row = (long long)blockIdx.x * SCORE_THREADS + threadIdx.x;
-  if (row >= n_rows) return;
-  const float4* src = reinterpret_cast<const float4*>(parts + row * PARTS);
-  float4 x[PARTS / 4];
+  // ---- score head: s_t = sigmoid(w_s . h_t + b_s); a row's d_g / 8 partial sums lie side by side and are added in order -----------
+  const int n_seq = min(NS * NG, a.S - seq0);
+  for (int i = (int)rank * RNN_THREADS + tid; i < n_seq * a.n_range; i += CL * RNN_THREADS) {
+    const float4* src = reinterpret_cast<const float4*>(a.H + ((long long)seq0 * a.n_range + i) * (DG / 8));
+    float sum = 0.f;
 #pragma unroll
-  for (int i = 0; i < PARTS / 4; ++i) x[i] = __ldcs(src + i);
-  float acc = 0.f;
-#pragma unroll
-  for (int i = 0; i < PARTS / 4; ++i) {
-    acc += x[i].x; acc += x[i].y; acc += x[i].z; acc += x[i].w;
-  }
-  const int s = (int)(row / n_range);
-  const int t = t0 + (int)(row - (long long)s * n_range);
-  scores[(long long)s * max_chunks + t] = 1.f / (1.f + expf(-(acc + b_s)));
-}
-
-static cudaError_t launch_score(const float* parts, float b_s, float* scores, long long n_rows, int n_range, int t0, int max_chunks, int d_g,
-                                cudaStream_t st) {
-  const dim3 grid((unsigned)((n_rows + SCORE_THREADS - 1) / SCORE_THREADS)), block(SCORE_THREADS);
-  switch (d_g) {
-    case 256: return launch_pdl(kve_gate_score_kernel<32>, grid, block, 0, st, parts, b_s, scores, n_rows, n_range, t0, max_chunks);
-    case 128: return launch_pdl(kve_gate_score_kernel<16>, grid, block, 0, st, parts, b_s, scores, n_rows, n_range, t0, max_chunks);
-    case 64:  return launch_pdl(kve_gate_score_kernel<8>, grid, block, 0, st, parts, b_s, scores, n_rows, n_range, t0, max_chunks);
-    default:  return cudaErrorInvalidValue;
+    for (int q = 0; q < DG / 32; ++q) {
+      const float4 x = __ldcg(src + q);
+      sum += x.x; sum += x.y; sum += x.z; sum += x.w;
+    }
+    const int s = i / a.n_range;
+    a.scores[(long long)(seq0 + s) * a.max_chunks + a.t0 + (i - s * a.n_range)] = 1.f / (1.f + expf(-(sum + a.b_s)));
   }
 }
 
@@ -399,10 +376,7 @@ cudaError_t launch_gate_rnn(const LayerView& v, int t0, int t1, const uint16_t* 
   a.P = P; a.H = H; a.W_hh = W_hh; a.w_s = w_s; a.b_s = b_s;
   a.scores = v.scores; a.lstm_h = v.lstm_h; a.lstm_c = v.lstm_c; a.status = v.status;
   a.S = v.S; a.max_chunks = v.max_chunks; a.t0 = t0; a.n_range = t1 - t0; a.reset = reset_state ? 1 : 0;
-  const cudaError_t e = planes == 3 ? launch_rnn_planes<3>(a, d_g, st) : launch_rnn_planes<2>(a, d_g, st);
-  if (e != cudaSuccess) return e;
-  const long long n_rows = (long long)v.S * a.n_range;
-  return launch_score(H, b_s, v.scores, n_rows, a.n_range, t0, v.max_chunks, d_g, st);
+  return planes == 3 ? launch_rnn_planes<3>(a, d_g, st) : launch_rnn_planes<2>(a, d_g, st);
 }
 
 }  // namespace kve

@@ -12,7 +12,7 @@ constexpr int RNN_THREADS = RNN_WARPS * 32;
 
 struct RnnArgs {
   const float* P;          // [S * n_range][4 d_g], column 4 u + gate: the pre-activations W_ih x + b of unit u
-  float* H;                // [S * n_range][d_g / 8]: partial sums of w_s . h_t for the score kernel
+  float* H;                // [S * n_range][d_g / 8]: partial sums of w_s . h_t
   const uint16_t* W_hh;    // bf16 [4 d_g][d_g]
   const float* w_s;        // [d_g]
   float b_s;

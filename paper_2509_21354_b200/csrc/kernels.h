@@ -65,7 +65,6 @@ constexpr int ATTN_TILE_ROWS = 64;
 constexpr int ATTN_PARTIAL_FLOATS = 132;       // acc[128], m, l, 2 pad: keeps every record 16-byte aligned
 
 cudaError_t launch_append(const LayerView& v, const void* k_new, const void* v_new, int n_new, int pos0, cudaStream_t st);
-cudaError_t launch_set_listed(const LayerView& v, int n_listed, cudaStream_t st);      // the device copy of the keep list's coverage
 // n_listed >= 0: also set the device copy of the keep list's coverage to it
 cudaError_t launch_set_len(const LayerView& v, int n, int n_listed, cudaStream_t st);
 cudaError_t launch_append_next(const LayerView& v, const void* k_new, const void* v_new, int n_new, int32_t* ticket,
@@ -73,15 +72,16 @@ cudaError_t launch_append_next(const LayerView& v, const void* k_new, const void
 // dev_window < 0: chunks [t0, t1).  dev_window >= 0 (the window size W): ONE chunk per sequence whose index the kernel
 // finds on the device - the chunk behind the keep list's coverage, if the stored length says it has left the window,
 // else the launch does nothing (a trigger that is replayed from a CUDA graph)
-cudaError_t launch_chunk_mean(const LayerView& v, int t0, int t1, bool final_output, bool pool_max, cudaStream_t st, int dev_window);
+// list_cut >= 0 (here, launch_chunk_token_mlp, launch_gate_proj): the keep list covers no more than that many chunks from now on
+cudaError_t launch_chunk_mean(const LayerView& v, int t0, int t1, bool final_output, bool pool_max, cudaStream_t st, int dev_window, int list_cut);
 cudaError_t launch_chunk_mlp(const LayerView& v, int t0, int t1, const MlpWeights& w, int d_sum, cudaStream_t st, int dev_window);
 // the MLP's second layer on pooled activations hid [2][S * (t1 - t0)][d_sum]: Kbar = W2 hid + b2 (d_sum 128 or 256)
 cudaError_t launch_pooled_out(const LayerView& v, int t0, int t1, const MlpWeights& w, int d_sum, const float* hid, cudaStream_t st);
 // per-token MLP aggregator: hid = scratch of 2 * S * (t1 - t0) * d_sum floats
 bool token_mlp_supported(int C, int d_sum);
-cudaError_t launch_chunk_token_mlp(const LayerView& v, int t0, int t1, const MlpWeights& w, int d_sum, float* hid, cudaStream_t st);
+cudaError_t launch_chunk_token_mlp(const LayerView& v, int t0, int t1, const MlpWeights& w, int d_sum, float* hid, int list_cut, cudaStream_t st);
 cudaError_t launch_gate_proj(const LayerView& v, int t0, int t1, const uint16_t* W_ih, const float* b_ih,
-                             const float* b_hh, int d_g, float* P, cudaStream_t st);
+                             const float* b_hh, int d_g, float* P, int list_cut, cudaStream_t st);
 // planes: bf16 planes of the fp32 state h that enter the recurrent product (2, or 3 = exact products)
 cudaError_t launch_gate_rnn(const LayerView& v, int t0, int t1, const uint16_t* W_hh, const float* w_s, float b_s,
                             int d_g, const float* P, float* H, bool reset_state, int planes, cudaStream_t st);

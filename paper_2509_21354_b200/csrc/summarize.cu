@@ -31,9 +31,10 @@ __device__ __forceinline__ void max_row(float (&acc)[8], const uint4& w) {
 // POOL_MAX: element-wise maximum of the chunk instead of its mean (the "pooling" aggregator of Sec. 3.1)
 template <bool POOL_MAX>
 __global__ void __launch_bounds__(MEAN_WARPS * 32) kve_chunk_mean_kernel(LayerView v, int t0, int n_range,
-                                                                        long long n_units, int final_output, int dev_window) {
+                                                                        long long n_units, int final_output, int dev_window, int list_cut) {
   pdl_launch_dependents();
   pdl_wait();
+  if (list_cut >= 0 && blockIdx.x == 0 && threadIdx.x == 0) *v.n_listed = list_cut;
   if (dev_window >= 0) {      // one chunk per sequence, found on the device
     const NextChunk nx = next_chunk(v.n_listed, v.seq_len, v.C, dev_window, v.max_chunks);
     if (!nx.due) return;
@@ -106,15 +107,15 @@ static int mean_ctas_per_sm() {
 // That only holds if the CTAs land on an empty GPU: the kernel is therefore launched WITHOUT the programmatic edge the
 // other kernels use.  (Launched early, beside the tail of its predecessor, its CTAs spread unevenly over the SMs
 // and the static striding turns that into a tail: measured +25 % on 4 GB of stale KV.)
-cudaError_t launch_chunk_mean(const LayerView& v, int t0, int t1, bool final_output, bool pool_max, cudaStream_t st, int dev_window) {
+cudaError_t launch_chunk_mean(const LayerView& v, int t0, int t1, bool final_output, bool pool_max, cudaStream_t st, int dev_window, int list_cut) {
   const int n_range = dev_window >= 0 ? 1 : t1 - t0;
   const long long n_units = (long long)v.S * n_range;
   if (n_units <= 0) return cudaSuccess;
   long long blocks = (n_units + MEAN_WARPS - 1) / MEAN_WARPS;
   const long long wave = (long long)sm_count() * (pool_max ? mean_ctas_per_sm<true>() : mean_ctas_per_sm<false>());
   if (blocks > wave) blocks = wave;
-  if (pool_max) kve_chunk_mean_kernel<true><<<dim3((unsigned)blocks), dim3(MEAN_WARPS * 32), 0, st>>>(v, t0, n_range, n_units, 1, dev_window);
-  else kve_chunk_mean_kernel<false><<<dim3((unsigned)blocks), dim3(MEAN_WARPS * 32), 0, st>>>(v, t0, n_range, n_units, final_output ? 1 : 0, dev_window);
+  if (pool_max) kve_chunk_mean_kernel<true><<<dim3((unsigned)blocks), dim3(MEAN_WARPS * 32), 0, st>>>(v, t0, n_range, n_units, 1, dev_window, list_cut);
+  else kve_chunk_mean_kernel<false><<<dim3((unsigned)blocks), dim3(MEAN_WARPS * 32), 0, st>>>(v, t0, n_range, n_units, final_output ? 1 : 0, dev_window, list_cut);
   return cudaGetLastError();
 }
 

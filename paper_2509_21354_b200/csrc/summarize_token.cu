@@ -52,6 +52,7 @@ struct TokenMlpArgs {
   int tiles_per_item;        // max(1, C / 128): 128-token tiles of one chunk
   int units_per_item;        // max(1, 128 / C): chunks in one tile
   int n_units, n_items;
+  int list_cut;              // >= 0: the keep list covers no more than that from now on
   MlpWeights w;
   float* hid;                // [2][n_units][d_sum] pooled activations (side, unit = s * n_range + (t - t0))
 };
@@ -103,6 +104,7 @@ __global__ void __launch_bounds__(TM_THREADS, 1) kve_token_mlp_pool_kernel(Token
   umma::fence_after_sync();
   const uint32_t tmem_d = *tmem_slot;
   pdl_wait();      // the pages come from earlier kernels
+  if (a.list_cut >= 0 && blockIdx.x == 0 && side == 0 && tid == 0) *v.n_listed = a.list_cut;
 
   // A CTA walks whole items (a chunk longer than a tile keeps all its 128-token slices on one CTA, in a row)
   const int my_items = a.n_items > (int)blockIdx.x ? (a.n_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
@@ -282,7 +284,7 @@ static cudaError_t launch_pool(const TokenMlpArgs& a, dim3 grid, cudaStream_t st
   return e == cudaSuccess ? launch_pdl(kve_token_mlp_pool_kernel<DSUM>, grid, dim3(TM_THREADS), TM_SMEM_BYTES, st, a) : e;
 }
 
-cudaError_t launch_chunk_token_mlp(const LayerView& v, int t0, int t1, const MlpWeights& w, int d_sum, float* hid, cudaStream_t st) {
+cudaError_t launch_chunk_token_mlp(const LayerView& v, int t0, int t1, const MlpWeights& w, int d_sum, float* hid, int list_cut, cudaStream_t st) {
   const int n_range = t1 - t0;
   const long long n_units = (long long)v.S * n_range;
   if (n_units <= 0) return cudaSuccess;
@@ -293,7 +295,7 @@ cudaError_t launch_chunk_token_mlp(const LayerView& v, int t0, int t1, const Mlp
   a.units_per_item = v.C < TM_N ? TM_N / v.C : 1;
   a.n_units = (int)n_units;
   a.n_items = (a.n_units + a.units_per_item - 1) / a.units_per_item;
-  a.w = w; a.hid = hid;
+  a.w = w; a.hid = hid; a.list_cut = list_cut;
   // one CTA per SM, half of the SMs per side; a CTA walks whole items (all 128-token slices of a chunk in a row)
   long long per_side = sm_count() / 2;
   if (per_side > a.n_items) per_side = a.n_items;
