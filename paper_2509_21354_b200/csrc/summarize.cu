@@ -1,9 +1,15 @@
 // kvE_summarize_chunks kernels (Eq. 2): per (sequence, chunk) the mean of the chunk's C key rows and
 // of its C value rows, then (AGG_MLP) a 2-layer GELU MLP on each mean.
 //
-// chunk_mean: HBM-bound.  One warp per (sequence, chunk): lanes 0-15 stream the K page, lanes 16-31 the
-// V page, 16 bytes per lane per row, rows added in temporal order in fp32 (so the sum has the same
-// rounding as a plain sequential loop), divided by C with an IEEE division.
+// chunk_mean: HBM-bound.  One warp per page (K or V of a (sequence, chunk) unit): 8 bytes per lane and row, 32 rows in flight,
+// added in temporal order in fp32 (so the sum has the same rounding as a plain sequential loop), divided by C with an
+// IEEE division.  Two-warp CTAs, dealt out by the hardware: a few units spread over all SMs, and many need no common wave.
+//   Measured (chains of launches, DRAM): 8 sequences x 28 chunks of 64 tokens 12.3 -> 3.3 us, 128 x 1 (one trigger) 10.3 -> 3.0,
+//   512 x 12 of 128 tokens 95 -> 62 us (6.5 TB/s), 512 x 121 of 128 tokens 672 -> 614 us (6.6 TB/s).  (Before: a warp per
+//   unit, 16 bytes per lane, 8 rows in flight, one resident wave striding over the units, launched behind a drained GPU.)
+// The kernel wants the L1 that attention, with its 200 KB of shared memory per SM, takes away: CTAs that land beside it keep
+// the SM in that split for as long as any of them is there, and 32 rows in flight per lane do not fit (4 GB: 720 us).  Large
+// launches therefore ask for the large L1 (an SM drains before its first CTA); small ones start at once.
 #include "common.cuh"
 #include "kernels.h"
 #include "umma.cuh"
@@ -11,27 +17,14 @@
 
 namespace kve {
 
-constexpr int MEAN_WARPS = 8;
-constexpr int MEAN_UNROLL = 8;
-
-__device__ __forceinline__ void add_row(float (&acc)[8], const uint4& w) {
-  acc[0] += bf16lo(w.x); acc[1] += bf16hi(w.x);
-  acc[2] += bf16lo(w.y); acc[3] += bf16hi(w.y);
-  acc[4] += bf16lo(w.z); acc[5] += bf16hi(w.z);
-  acc[6] += bf16lo(w.w); acc[7] += bf16hi(w.w);
-}
-
-__device__ __forceinline__ void max_row(float (&acc)[8], const uint4& w) {
-  acc[0] = fmaxf(acc[0], bf16lo(w.x)); acc[1] = fmaxf(acc[1], bf16hi(w.x));
-  acc[2] = fmaxf(acc[2], bf16lo(w.y)); acc[3] = fmaxf(acc[3], bf16hi(w.y));
-  acc[4] = fmaxf(acc[4], bf16lo(w.z)); acc[5] = fmaxf(acc[5], bf16hi(w.z));
-  acc[6] = fmaxf(acc[6], bf16lo(w.w)); acc[7] = fmaxf(acc[7], bf16hi(w.w));
-}
+constexpr int MEAN_WARPS = 2;
+constexpr int MEAN_UNROLL = 32;                       // rows in flight
+constexpr long long MEAN_LARGE_ROWS = 1LL << 16;      // K (or V) rows from which a launch asks for the large L1: 32 MB
 
 // POOL_MAX: element-wise maximum of the chunk instead of its mean (the "pooling" aggregator of Sec. 3.1)
 template <bool POOL_MAX>
-__global__ void __launch_bounds__(MEAN_WARPS * 32) kve_chunk_mean_kernel(LayerView v, int t0, int n_range,
-                                                                        long long n_units, int final_output, int dev_window, int list_cut) {
+__global__ void __launch_bounds__(MEAN_WARPS * 32) kve_chunk_mean_kernel(LayerView v, int t0, int n_range, FastDiv by_range,
+                                                                        int final_output, int dev_window, int list_cut) {
   pdl_launch_dependents();
   pdl_wait();
   if (list_cut >= 0 && blockIdx.x == 0 && threadIdx.x == 0) *v.n_listed = list_cut;
@@ -40,83 +33,69 @@ __global__ void __launch_bounds__(MEAN_WARPS * 32) kve_chunk_mean_kernel(LayerVi
     if (!nx.due) return;
     t0 = nx.t;
   }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // persistent warps: unit = global warp id, then strides of the whole grid
-  for (long long unit = (long long)blockIdx.x * MEAN_WARPS + warp; unit < n_units; unit += (long long)gridDim.x * MEAN_WARPS) {
-  const int s = (int)(unit / n_range);
-  const int t = t0 + (int)(unit - (long long)s * n_range);
-  const int is_v = lane >> 4, l16 = lane & 15;
+  const int lane = threadIdx.x & 31, is_v = threadIdx.x >> 5, unit = (int)blockIdx.x;
+  const int s = (int)by_range.div((uint32_t)unit), t = t0 + (unit - s * n_range);
   const long long page = v.page_table[(long long)s * v.max_chunks + t];
   if (page < 0 || page >= v.n_pages) {
     if (lane == 0) set_status(v.status, ERR_CAPACITY);
-    continue;
+    return;
   }
-  const uint4* src = reinterpret_cast<const uint4*>((is_v ? v.v_pages : v.k_pages) + page * v.C * D) + l16;
-  float acc[8];
+  const uint2* src = reinterpret_cast<const uint2*>((is_v ? v.v_pages : v.k_pages) + page * v.C * D) + lane;
+  float acc[4];
 #pragma unroll
-  for (int x = 0; x < 8; ++x) acc[x] = POOL_MAX ? -INFINITY : 0.f;
+  for (int x = 0; x < 4; ++x) acc[x] = POOL_MAX ? -INFINITY : 0.f;
+  auto take = [&](const uint2& w) {      // the next row
+    const float f[4] = {bf16lo(w.x), bf16hi(w.x), bf16lo(w.y), bf16hi(w.y)};
+#pragma unroll
+    for (int x = 0; x < 4; ++x) acc[x] = POOL_MAX ? fmaxf(acc[x], f[x]) : acc[x] + f[x];
+  };
   int j = 0;
   for (; j + MEAN_UNROLL <= v.C; j += MEAN_UNROLL) {
-    uint4 w[MEAN_UNROLL];
+    uint2 w[MEAN_UNROLL];
 #pragma unroll
-    for (int u = 0; u < MEAN_UNROLL; ++u) w[u] = __ldcs(src + (long long)(j + u) * 16);
+    for (int u = 0; u < MEAN_UNROLL; ++u) w[u] = __ldcs(src + (j + u) * (D / 4));
 #pragma unroll
-    for (int u = 0; u < MEAN_UNROLL; ++u) {
-      if (POOL_MAX) max_row(acc, w[u]); else add_row(acc, w[u]);
-    }
+    for (int u = 0; u < MEAN_UNROLL; ++u) take(w[u]);
   }
-  for (; j < v.C; ++j) {
-    const uint4 w1 = __ldcs(src + (long long)j * 16);
-    if (POOL_MAX) max_row(acc, w1); else add_row(acc, w1);
+  if (j < v.C) {      // the rest of the chunk, in flight together too
+    uint2 w[MEAN_UNROLL];
+#pragma unroll
+    for (int u = 0; u < MEAN_UNROLL; ++u)
+      if (j + u < v.C) w[u] = __ldcs(src + (j + u) * (D / 4));
+#pragma unroll
+    for (int u = 0; u < MEAN_UNROLL; ++u)
+      if (j + u < v.C) take(w[u]);
   }
   if (!POOL_MAX) {
     const float fc = (float)v.C;
 #pragma unroll
-    for (int x = 0; x < 8; ++x) acc[x] = __fdiv_rn(acc[x], fc);
+    for (int x = 0; x < 4; ++x) acc[x] = __fdiv_rn(acc[x], fc);
   }
-
-  const long long o = ((long long)s * v.max_chunks + t) * D + l16 * 8;
-  float4* of = reinterpret_cast<float4*>((is_v ? v.vsum_f32 : v.ksum_f32) + o);
-  of[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
-  of[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
-  if (final_output) {
-    uint4 b;
-    b.x = pack_bf16x2(acc[0], acc[1]);
-    b.y = pack_bf16x2(acc[2], acc[3]);
-    b.z = pack_bf16x2(acc[4], acc[5]);
-    b.w = pack_bf16x2(acc[6], acc[7]);
-    *reinterpret_cast<uint4*>((is_v ? v.vsum_bf16 : v.ksum_bf16) + o) = b;
-  }
-  }
+  const long long o = ((long long)s * v.max_chunks + t) * D + lane * 4;
+  *reinterpret_cast<float4*>((is_v ? v.vsum_f32 : v.ksum_f32) + o) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+  if (final_output)
+    *reinterpret_cast<uint2*>((is_v ? v.vsum_bf16 : v.ksum_bf16) + o) = make_uint2(pack_bf16x2(acc[0], acc[1]), pack_bf16x2(acc[2], acc[3]));
 }
 
-// CTAs of the mean kernel that are resident per SM (registers decide), looked up once per device
-template <bool POOL_MAX>
-static int mean_ctas_per_sm() {
-  static std::atomic<int> cached[MAX_DEVICES];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) return 4;
-  int n = cached[dev].load(std::memory_order_acquire);
-  if (n > 0) return n;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kve_chunk_mean_kernel<POOL_MAX>, MEAN_WARPS * 32, 0) != cudaSuccess || n <= 0) n = 4;
-  cached[dev].store(n, std::memory_order_release);
-  return n;
-}
-
-// The grid is exactly one resident wave and every warp strides over the units, so all SMs carry the same share.
-// That only holds if the CTAs land on an empty GPU: the kernel is therefore launched WITHOUT the programmatic edge the
-// other kernels use.  (Launched early, beside the tail of its predecessor, its CTAs spread unevenly over the SMs
-// and the static striding turns that into a tail: measured +25 % on 4 GB of stale KV.)
 cudaError_t launch_chunk_mean(const LayerView& v, int t0, int t1, bool final_output, bool pool_max, cudaStream_t st, int dev_window, int list_cut) {
   const int n_range = dev_window >= 0 ? 1 : t1 - t0;
   const long long n_units = (long long)v.S * n_range;
   if (n_units <= 0) return cudaSuccess;
-  long long blocks = (n_units + MEAN_WARPS - 1) / MEAN_WARPS;
-  const long long wave = (long long)sm_count() * (pool_max ? mean_ctas_per_sm<true>() : mean_ctas_per_sm<false>());
-  if (blocks > wave) blocks = wave;
-  if (pool_max) kve_chunk_mean_kernel<true><<<dim3((unsigned)blocks), dim3(MEAN_WARPS * 32), 0, st>>>(v, t0, n_range, n_units, 1, dev_window, list_cut);
-  else kve_chunk_mean_kernel<false><<<dim3((unsigned)blocks), dim3(MEAN_WARPS * 32), 0, st>>>(v, t0, n_range, n_units, final_output ? 1 : 0, dev_window, list_cut);
-  return cudaGetLastError();
+  if (n_units >= (1LL << 31)) return cudaErrorInvalidValue;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  attr[1].val.sharedMemCarveout = cudaSharedmemCarveoutMaxL1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)n_units);
+  cfg.blockDim = dim3(MEAN_WARPS * 32);
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = n_units * v.C >= MEAN_LARGE_ROWS ? 2 : 1;
+  const FastDiv by_range = fast_div((uint32_t)n_range);
+  return pool_max ? cudaLaunchKernelEx(&cfg, kve_chunk_mean_kernel<true>, v, t0, n_range, by_range, 1, dev_window, list_cut)
+                  : cudaLaunchKernelEx(&cfg, kve_chunk_mean_kernel<false>, v, t0, n_range, by_range, final_output ? 1 : 0, dev_window, list_cut);
 }
 
 // ---- aggregator MLP (Eq. 2 read as mean -> d_sum -> d, exact-erf GELU), fp32 FMA ------------------
