@@ -123,7 +123,6 @@ __device__ __forceinline__ uint32_t piece_begin(uint32_t c, uint32_t I, uint32_t
 // the CTA that holds part x
 __device__ __forceinline__ uint32_t piece_of(uint32_t x, uint32_t I, uint32_t P) { return ((x + 1u) * P - 1u) / I; }
 
-__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 // bulk prefetch into L2 (16-byte aligned, a multiple of 16 bytes)
 __device__ __forceinline__ void prefetch_l2_bulk(const void* p, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");

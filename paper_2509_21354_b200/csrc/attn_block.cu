@@ -58,6 +58,7 @@ cudaError_t launch_attn_block(const LayerView& v, const void* maps, AttnMode mod
   if (R > ATTN_BLOCK_MAX_ROWS || hp < 8) return cudaErrorInvalidValue;
   BlockArgs a;
   a.v = v; a.mode = (int)mode; a.n_chunks = n_chunks;
+  a.by_c = fast_div((uint32_t)v.C); a.by_h = fast_div((uint32_t)v.H); a.by_g = fast_div((uint32_t)G); a.by_split = fast_div((uint32_t)plan.rows_per_split);
   a.rows_per_split = plan.rows_per_split; a.max_splits = plan.max_splits;
   a.T = T; a.G = G; a.R = R; a.rec_rows = (R + 15) / 16 * 16; a.causal = causal; a.hp = hp; a.sum_row0 = sum_row0;
   a.q = static_cast<const uint16_t*>(q); a.out = static_cast<uint16_t*>(out); a.lse = lse; a.scale = scale;

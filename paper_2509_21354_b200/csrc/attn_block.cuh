@@ -23,6 +23,7 @@ constexpr int BK_REC = ATTN_PARTIAL_FLOATS;     // floats per (query row) record
 
 struct BlockArgs {
   LayerView v;
+  FastDiv by_c, by_h, by_g, by_split;      // by the chunk size, KV heads, query heads per KV head, rows per split
   int mode, n_chunks, rows_per_split, max_splits;
   int T, G, R;              // query tokens, query heads per KV head, T * G
   int rec_rows;             // query-row records per (sequence, split) in `partials`
@@ -49,7 +50,7 @@ struct BlockGeom {
 __device__ __forceinline__ BlockGeom block_geometry(const BlockArgs& a, int s, int split) {
   const LayerView& v = a.v;
   BlockGeom g;
-  int n = v.seq_len[s / v.H];
+  int n = v.seq_len[a.by_h.div((uint32_t)s)];
   n = min(max(n, 0), v.max_tokens);
   const int M = (a.mode == ATTN_DENSE) ? 0 : min(max(v.keep_cnt[s], 0), a.n_chunks);
   g.raw0 = (a.mode == ATTN_DENSE) ? 0 : a.n_chunks * v.C;
@@ -57,7 +58,7 @@ __device__ __forceinline__ BlockGeom block_geometry(const BlockArgs& a, int s, i
   g.n_tail = max(0, n - g.raw0);
   g.tail_pad = (g.n_tail + BK_TILE - 1) / BK_TILE * BK_TILE;
   g.n_rows = g.tail_pad + n_lead;
-  g.n_splits = max(1, (g.n_rows + a.rows_per_split - 1) / a.rows_per_split);
+  g.n_splits = max(1, (int)a.by_split.div((uint32_t)(g.n_rows + a.rows_per_split - 1)));
   // a replayed launch the sequence has outgrown: the splits that exist still merge and the ticket
   // counter still returns to zero; the caller learns about the dropped rows from the status word
   g.outgrown = g.n_splits > (int)gridDim.x;
@@ -83,9 +84,23 @@ __device__ __forceinline__ uint32_t tile_piece(int row, int p16) {
 
 // element offset of query / output row r of KV sequence s in the [B][T][Hq][128] layout
 __device__ __forceinline__ long long q_row_offset(const BlockArgs& a, int s, int r) {
-  const int b = s / a.v.H, h = s - b * a.v.H;
-  const int t = r / a.G, g = r - t * a.G;
+  const int b = (int)a.by_h.div((uint32_t)s), h = s - b * a.v.H;
+  const int t = (int)a.by_g.div((uint32_t)r), g = r - t * a.G;
   return ((((long long)b * a.T + t) * (a.G * a.v.H)) + h * a.G + g) * D;
+}
+
+// Page ids of the first three tiles of a split, looked up as if they were raw-tail tiles: where those begin follows from the
+// launch arguments, so the look-ups need not wait for the stored length (lane j: the page of box j)
+struct FirstPages { int page[3]; };
+__device__ __forceinline__ FirstPages first_pages(const BlockArgs& a, int s, int split, int lane) {
+  FirstPages f;
+  const int raw0 = (a.mode == ATTN_DENSE) ? 0 : a.n_chunks * a.v.C;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const int chunk = (int)a.by_c.div((uint32_t)(raw0 + split * a.rows_per_split + i * BK_TILE + lane * a.hp));
+    f.page[i] = (lane * a.hp < BK_TILE && chunk < a.v.max_chunks) ? a.v.page_table[(long long)s * a.v.max_chunks + chunk] : -1;
+  }
+  return f;
 }
 
 // Producer warp: resolves page ids three tiles ahead and fetches the CTA's tiles with 2-D tensor
@@ -97,17 +112,16 @@ __device__ __forceinline__ long long q_row_offset(const BlockArgs& a, int s, int
 template <int STAGES>
 __device__ __forceinline__ void block_producer(const BlockArgs& a, const BlockGeom& gm, int s, int lane,
                                                const CUtensorMap* tmK, const CUtensorMap* tmV, const CUtensorMap* tmKs,
-                                               const CUtensorMap* tmVs, unsigned char* ring, uint64_t* full,
+                                               const CUtensorMap* tmVs, const FirstPages& first, unsigned char* ring, uint64_t* full,
                                                uint64_t* empty) {
   const LayerView& v = a.v;
   struct TileSrc { int src[2]; };
   const long long sb = (long long)s * v.max_chunks;
-  auto page_row = [&](int chunk, int r) -> int {
-    long long page = v.page_table[sb + chunk];
+  auto page_row = [&](long long page, int r) -> int {
     if (page < 0 || page >= v.n_pages) { set_status(v.status, ERR_CAPACITY); page = 0; }
     return (int)(page * v.C + r);
   };
-  auto resolve = [&](int i, TileSrc& t) {
+  auto resolve = [&](int i, TileSrc& t, int known) {
     t.src[0] = t.src[1] = -1;
     if (i >= gm.n_tiles) return;
     const int row0 = gm.r_begin + i * BK_TILE;
@@ -115,16 +129,16 @@ __device__ __forceinline__ void block_producer(const BlockArgs& a, const BlockGe
     if (row0 < gm.tail_pad) {
       if (lane * a.hp < valid) {
         const int p = gm.raw0 + row0 + lane * a.hp;
-        const int chunk = p / v.C;
-        t.src[0] = page_row(chunk, p - chunk * v.C);
+        const int chunk = (int)a.by_c.div((uint32_t)p);
+        t.src[0] = page_row(known != -1 ? known : v.page_table[sb + chunk], p - chunk * v.C);
       }
     } else if (a.mode == ATTN_RAW) {
       if (lane * a.hp < valid) {
         const int ll = row0 - gm.tail_pad + lane * a.hp;
-        const int ci = ll / v.C;
+        const int ci = (int)a.by_c.div((uint32_t)ll);
         int chunk = v.keep_idx[sb + ci];
         if (chunk < 0 || chunk >= a.n_chunks) { set_status(v.status, ERR_CAPACITY); chunk = 0; }
-        t.src[0] = page_row(chunk, ll - ci * v.C);
+        t.src[0] = page_row(v.page_table[sb + chunk], ll - ci * v.C);
       }
     } else {
       // kept summary rows sit compacted, one contiguous run per sequence: boxes of BK_SUM_BOX rows, lane j the j-th
@@ -164,14 +178,14 @@ __device__ __forceinline__ void block_producer(const BlockArgs& a, const BlockGe
     return true;
   };
   TileSrc t0, t1, t2;
-  resolve(0, t0);
-  resolve(1, t1);
-  resolve(2, t2);
+  resolve(0, t0, first.page[0]);
+  resolve(1, t1, first.page[1]);
+  resolve(2, t2, first.page[2]);
   for (int i = 0; i < gm.n_tiles; i += 3) {
     if (!issue(i, t0)) break;
-    resolve(i + 3, t0);
-    if (i + 1 < gm.n_tiles) { if (!issue(i + 1, t1)) break; resolve(i + 4, t1); }
-    if (i + 2 < gm.n_tiles) { if (!issue(i + 2, t2)) break; resolve(i + 5, t2); }
+    resolve(i + 3, t0, -1);
+    if (i + 1 < gm.n_tiles) { if (!issue(i + 1, t1)) break; resolve(i + 4, t1, -1); }
+    if (i + 2 < gm.n_tiles) { if (!issue(i + 2, t2)) break; resolve(i + 5, t2, -1); }
   }
 }
 

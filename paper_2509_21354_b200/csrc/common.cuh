@@ -105,6 +105,9 @@ __device__ __forceinline__ void bulk_g2s(void* dst_smem, const void* src_gmem, u
       : "memory");
 }
 
+// fetch of the line into L2, nothing returned
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // 16-byte asynchronous copy global -> shared (bypassing L1); `live` false writes 16 zero bytes instead
 __device__ __forceinline__ void cp_async16(void* dst_smem, const void* src_gmem, bool live) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst_smem)), "l"(src_gmem),
