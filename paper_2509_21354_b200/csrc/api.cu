@@ -182,6 +182,16 @@ int stale_chunks(const kvE_config& c, int n) { return n > c.W ? (n - c.W) / c.C 
 
 bool bad_layer(const kvE_store* st, int layer) { return !st || layer < 0 || layer >= st->cfg.n_layers; }
 
+// the address under which the device reads and writes a host buffer, or null (memory that is not pinned)
+void* device_address(const void* host) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
+}
+
 // every launch goes to the current device: it must be the one the handle's buffers live on
 bool wrong_device(const kvE_store* st) {
   int dev = -1;
@@ -704,13 +714,29 @@ static int decode_step_host(kvE_store* st, int layer, const void* k_new_host, co
   const size_t row_bytes = (size_t)st->S * 128 * 2;
   char* stage = static_cast<char*>(st->buf.workspace) + st->off_stage;
   char *dk = stage, *dv = stage + row_bytes, *dq = stage + 2 * row_bytes, *dout = stage + 3 * row_bytes;
-  cudaError_t e = cudaMemcpyAsync(dk, k_new_host, row_bytes, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(dv, v_new_host, row_bytes, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(dq, q_host, row_bytes, cudaMemcpyHostToDevice, s);
-  if (e != cudaSuccess) return cuda_fail(st, e);
-  int rc = kvE_append(st, layer, dk, dv, 1, nullptr, stream);
-  if (rc != KVE_OK) return rc;
   LayerState& ls = st->layers[layer];
+  if (ls.n_tokens + 1 > st->cfg.max_tokens) return KVE_ERR_CAPACITY;
+  // Pinned buffers: the append kernel fetches the three inputs across PCIe itself, and attention writes its result there.  Others:
+  // copies to and from the staging rows.
+  const void *pk = device_address(k_new_host), *pv = device_address(v_new_host), *pq = device_address(q_host);
+  void* pout = device_address(out_host);
+  const bool in_place = pk && pv && pq;
+  cudaError_t e = cudaSuccess;
+  int rc;
+  if (in_place) {
+    Prof prof(st, KVE_K_APPEND, s);
+    e = launch_append(view(st, layer), pk, pv, 1, ls.n_tokens, s, pq, dq);
+    if (e != cudaSuccess) return cuda_fail(st, e);
+    ls.n_tokens += 1;
+    ls.reserve_upper = 0;
+  } else {
+    e = cudaMemcpyAsync(dk, k_new_host, row_bytes, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dv, v_new_host, row_bytes, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dq, q_host, row_bytes, cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) return cuda_fail(st, e);
+    rc = kvE_append(st, layer, dk, dv, 1, nullptr, stream);
+    if (rc != KVE_OK) return rc;
+  }
   const int nc = stale_chunks(st->cfg, ls.n_tokens);
   if (from_scratch) {
     rc = kvE_refresh(st, layer, aw, lw, tau, stream);
@@ -733,9 +759,9 @@ static int decode_step_host(kvE_store* st, int layer, const void* k_new_host, co
     rc = kvE_compact(st, layer, tau, stream);
     if (rc != KVE_OK) return rc;
   }
-  rc = kvE_decode_attn(st, layer, dq, dout, nullptr, scale, stream);
+  rc = kvE_decode_attn(st, layer, dq, pout ? pout : dout, nullptr, scale, stream);
   if (rc != KVE_OK) return rc;
-  e = cudaMemcpyAsync(out_host, dout, row_bytes, cudaMemcpyDeviceToHost, s);
+  if (!pout) e = cudaMemcpyAsync(out_host, dout, row_bytes, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess && wait) e = cudaStreamSynchronize(s);
   return e == cudaSuccess ? KVE_OK : cuda_fail(st, e);
 }

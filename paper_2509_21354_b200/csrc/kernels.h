@@ -64,7 +64,9 @@ struct AttnPlan {
 constexpr int ATTN_TILE_ROWS = 64;
 constexpr int ATTN_PARTIAL_FLOATS = 132;       // acc[128], m, l, 2 pad: keeps every record 16-byte aligned
 
-cudaError_t launch_append(const LayerView& v, const void* k_new, const void* v_new, int n_new, int pos0, cudaStream_t st);
+// q_src, q_dst: S rows to copy along, or null
+cudaError_t launch_append(const LayerView& v, const void* k_new, const void* v_new, int n_new, int pos0, cudaStream_t st,
+                          const void* q_src = nullptr, void* q_dst = nullptr);
 // n_listed >= 0: also set the device copy of the keep list's coverage to it
 cudaError_t launch_set_len(const LayerView& v, int n, int n_listed, cudaStream_t st);
 cudaError_t launch_append_next(const LayerView& v, const void* k_new, const void* v_new, int n_new, int32_t* ticket,

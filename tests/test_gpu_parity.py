@@ -1279,3 +1279,42 @@ def test_decode_step_over_tiles_of_many_and_of_broken_chunks(C, pages):
     assert st.poll_status() == 0
     Kd, Vd = pages_to_plain(st, 0, n0 + steps)
     assert np.array_equal(Kd, K) and np.array_equal(Vd, V)
+
+
+@pytest.mark.parametrize("n_new", [1, 7, 33, 250])
+def test_append_of_odd_counts_over_chunk_boundaries(n_new):
+    """Every token of every append at its own position, byte for byte."""
+    b = _binding()
+    n = 4 * n_new + 13
+    wl = wlm.Workload("append", B=2, H=5, n=n, C=48, W=n, d_g=64, seed=n_new)
+    K, V = wlm.gen_kv(wl, n=n)
+    st = make_store(wl)
+    for a in range(0, n, n_new):
+        e = min(n, a + n_new)
+        st.append(0, b.bits_to_bf16(np.ascontiguousarray(K[:, a:e])), b.bits_to_bf16(np.ascontiguousarray(V[:, a:e])))
+    Kd, Vd = pages_to_plain(st, 0, n)
+    assert st.poll_status() == 0 and int(st.seq_len[0, 0]) == n
+    assert np.array_equal(Kd, K) and np.array_equal(Vd, V)
+
+
+def test_decode_step_host_from_pageable_buffers_and_chained_through_one_buffer():
+    """Pinned buffers are read and written in place, pageable ones through staging copies: the same results; and a step whose
+    query is the buffer that the step before writes its result to (asynchronous form) sees that result."""
+    b = _binding()
+    wl = wlm.CFG1.small(n=700, n_append=3, seed=8)
+    K, V = wlm.gen_kv(wl)
+    lw = b.LstmWeights(wlm.gen_lstm_weights(wl))
+    rows = [b.bits_to_bf16(x, "cpu").reshape(wl.S, 128) for x in (*wlm.gen_new_tokens(wl, 0, 0), *wlm.gen_new_tokens(wl, 0, 1))]
+    q = b.bits_to_bf16(wlm.gen_q(wl), "cpu")
+    results = []
+    for pinned in (False, True):
+        st = make_store(wl)
+        load_kv(st, 0, K, V)
+        hold = lambda t: t.clone().pin_memory() if pinned else t.clone()
+        k0, v0, k1, v1, buf, out = (hold(t) for t in (*rows, q, torch.zeros_like(q)))
+        st.decode_step_host(0, k0, v0, buf, buf, None, lw, 0.5, from_scratch=True, wait=not pinned)
+        st.decode_step_host(0, k1, v1, buf, out, None, lw, 0.5, from_scratch=False, wait=not pinned)
+        torch.cuda.synchronize()
+        assert st.poll_status() == 0
+        results.append((buf.clone(), out.clone()))
+    assert torch.equal(results[0][0], results[1][0]) and torch.equal(results[0][1], results[1][1])
