@@ -14,8 +14,9 @@
 //    32 (w % 4) .., column half w / 4), add the bias and store P, the MMAs of tile i + 1 run into the other.  The epilogue
 //    turns each 32 x 32 block through shared memory so that a store instruction writes whole 128-byte row segments.
 //  * 256-column slices (128 KB of weights) left room for one tile of X, whose gather, MMAs and store then followed one
-//    another: 5.0 us per 128 x 256 tile.  512 sequences x 121 chunks (254 MB of P) 74 us, PJ_1 us this way; 256 x 56
-//    26.7 us, PJ_2; 8 x 28 at d_g = 128 12.3 us, PJ_3 (event pairs).
+//    another: 5.0 us per 128 x 256 tile.  512 sequences x 121 chunks (254 MB of P) 74 us, 70 us this way; 256 x 56
+//    26.7 us, 25.0; 8 x 28 at d_g = 128 12.3 us, 10.8 (event pairs).  Bound by shared memory: writing and reading
+//    the tiles of X and turning P take about 2500 of the 3800 cycles of a tile.
 //  * Every wait is bounded; on give-up the status word gets KVE_ERR_TIMEOUT.
 #include "common.cuh"
 #include "kernels.h"

@@ -10,7 +10,7 @@
 //    units, i.e. 256 rows of W_hh; eight warps own 8 units each and keep their rows in REGISTERS as mma A fragments
 //    for the whole kernel (128 registers per thread at d_g = 256).  (Sixteen warps, eight per group, with ten of the sixteen k
 //    tiles' fragments read from shared memory because 128 registers do not hold them: 330 us on 512 sequences x 121
-//    chunks, 347 us with the groups taking turns at the tensor cores, against RNN_NG2 us this way.)
+//    chunks, 347 us with the groups taking turns at the tensor cores, against 285 us this way.)
 //  * Per step the CTA computes its rows of W_hh h with warp-level tensor-core MMAs (m16n8k16, bf16 x bf16 -> fp32).  W_hh is
 //    bf16 by definition; the fp32 state h enters as PL = 2 bf16 planes by default (h = hi + lo up to 2^-17 |h|: 16 of its 24
 //    significant bits; a third plane makes the products exact, moves the scores by 1e-7 - far below what the fast
@@ -29,7 +29,7 @@
 //    thread takes them with one 16-byte load.
 //  * The score head is not part of the chain: a warp leaves its 8 units' share of w_s . h_t per sequence (d_g / 8 partial sums
 //    per (s, t): an eighth of the bytes of h_t), and when the chain is through the cluster adds them up in a fixed order.
-//  Measured, recurrence and score head: 512 sequences x 121 chunks 314 -> RNN_NG2 us, 256 x 56 92.5 -> RNN_NG1 us, 8 x 28 at
+//  Measured, recurrence and score head: 512 sequences x 121 chunks 314 -> 285 us, 256 x 56 92.5 -> 80 us, 8 x 28 at
 //  d_g = 128 51.6 -> 33 us (there a cluster of two CTAs halves the MMA chain: one CTA held all of W_hh).  Slower: waiting for the
 //  CTA's own planes and the peers' apart, with the own units' MMAs in between (255 -> 261 us a step on 256 sequences), and
 //  the score's shuffles between the MMAs (248 -> 255 us).

@@ -1,10 +1,13 @@
 // GELU in its exact form x * Phi(x) for the aggregator MLP kernels (Eq. 2), two values at a time.
 //   x Phi(x) = max(x, 0) - |x| Q(|x|),  Q = 1 - Phi the upper tail,  Q(a) = 2^(-g(a)).
-// g is so close to a parabola that a polynomial of degree 6 does: fitted here by least squares with weights iterated towards
-// the least maximum (Lawson's method) of the resulting error in a Q(a) on 0 <= a <= 6.  Absolute error of the result
-// 5.1e-8 in exact arithmetic, 8.1e-8 with every step rounded to fp32 (the erf formula 7.1.26 of Abramowitz and Stegun, used
-// before with an exponential and a reciprocal: 2.1e-7).  8 fp32 operations and one exponential per value, in packed
-// pairs.  Beyond a = 6 the tail is held at 6 Q(6) = 6e-9 (the min also keeps infinities out of the polynomial); NaN stays NaN.
+// g is so close to a parabola that a polynomial of low degree does: fitted here by least squares with weights iterated
+// towards the least maximum (Lawson's method) of the resulting error in a Q(a) on 0 <= a <= 6.  Error of the result for
+// x ~ N(0, 1) with every step rounded to fp32: degree 6: rms 3.7e-8, max 9.4e-8; degree 8: rms 1.0e-8, max 4.9e-8 (the erf
+// formula 7.1.26 of Abramowitz and Stegun, used before with an exponential and a reciprocal: rms 4.9e-8, max 2.1e-7).
+// Degree 8 where the tensor cores bound the kernel and the activations are free (the chunk means' MLP: 219.8 us a step with
+// either on 256 sequences x 4096 tokens); degree 6 where the activations bound it and are averaged over a chunk's tokens anyway
+// (the per-token MLP: 381 us a step with 6, 395 with 7, 406 with 8).  Beyond a = 6 the tail is held at 6 Q(6) = 6e-9 (the
+// min also keeps infinities out of the polynomial); NaN stays NaN.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -20,19 +23,30 @@ __device__ __forceinline__ float relu_nan(float x) {
 }
 
 // relu: max(x, 0); a: |x|, at most 6; result: the tail Q(a).  x Phi(x) = relu - a * Q
+template <int DEGREE>
 __device__ __forceinline__ float2 gelu_tail2(float2 x, float2& relu, float2& a) {
+  static_assert(DEGREE == 6 || DEGREE == 8, "degrees fitted");
   a = make_float2(fminf(fabsf(x.x), 6.f), fminf(fabsf(x.y), 6.f));
   relu = make_float2(relu_nan(x.x), relu_nan(x.y));
-  constexpr float G[7] = {-0.999993061f, -1.1512017f, -0.458770975f, -0.0534121019f, 0.00808071511f, -0.00076921928f, 3.30927681e-05f};
-  float2 p = make_float2(G[6], G[6]);
+  constexpr float G6[7] = {-0.999993061f, -1.1512017f, -0.458770975f, -0.0534121019f, 0.00808071511f, -0.00076921928f, 3.30927681e-05f};
+  constexpr float G8[9] = {-0.999998868f, -1.15112329f, -0.459115446f, -0.0527141988f, 0.00733338343f, -0.00032334181f, -0.000114462782f,
+                           2.50833236e-05f, -1.69040277e-06f};
+  float2 p;
+  if constexpr (DEGREE == 6) {
+    p = make_float2(G6[6], G6[6]);
 #pragma unroll
-  for (int k = 5; k >= 0; --k) p = fma2(p, a, make_float2(G[k], G[k]));
+    for (int k = 5; k >= 0; --k) p = fma2(p, a, make_float2(G6[k], G6[k]));
+  } else {
+    p = make_float2(G8[8], G8[8]);
+#pragma unroll
+    for (int k = 7; k >= 0; --k) p = fma2(p, a, make_float2(G8[k], G8[k]));
+  }
   return make_float2(ex2_fast(p.x), ex2_fast(p.y));
 }
 
 __device__ __forceinline__ float2 gelu2(float2 x) {
   float2 relu, a;
-  const float2 q = gelu_tail2(x, relu, a);
+  const float2 q = gelu_tail2<8>(x, relu, a);
   return fma2(make_float2(-a.x, -a.y), q, relu);
 }
 

@@ -229,7 +229,11 @@ __global__ void __launch_bounds__(MLP_THREADS) kve_chunk_mlp_kernel(LayerView v,
 // ~9000 per warp; with all sixteen warps going through the phases together a tile took 22500 cycles.  512 x 121 chunks:
 // 96 -> 88 us; the second layer alone on 256 x 56 chunks 25 -> 15 us; small launches (256 x 56 chunks: 33 us) are the weights'
 // way into shared memory and the latency of one or two tiles, and did not change.
-// POOLED: the second layer alone, on the pooled activations hid [2][n_units][d_sum] of the per-token aggregator.
+// POOLED: the second layer alone, on the pooled activations hid [2][n_units][d_sum] of the per-token aggregator.  Its small
+// planes have an accumulator of their own (in the columns that layer 1 leaves free): the tensor core cuts off what lies
+// below the last bit of the accumulator at each of its steps, so the large sum takes d_sum / 16 of them, not three times that
+// (rms error of the
+// summaries against 64 bits on 256 x 56 chunks: keys 3.7e-7 -> 1.3e-7, values 2.4e-7 -> 0.7e-7; fp32 loops: 1.4e-7, 1.0e-7).
 // Every mbarrier wait is bounded; on give-up the status word gets KVE_ERR_TIMEOUT.
 constexpr int MT_M = 128;
 constexpr int MT_GELU_WARPS = 8, MT_IO_WARPS = 8;
@@ -247,6 +251,7 @@ constexpr int MT_SMEM_BAR = MT_SMEM_B2 + D * 4;
 constexpr int MT_SMEM_BYTES = MT_SMEM_BAR + 128 + 1024;                   // + slack to reach a 1024-byte boundary
 static_assert(MT_SMEM_BYTES <= 227 * 1024, "shared memory of one CTA");
 constexpr int MT_TMEM_COLS = 512;      // H halves: columns 0 and 128; Y: 256; activations of the two groups: 384, 432 (3 planes x 16)
+constexpr int MT_TMEM_YLO = 0;         // POOLED: sum of the two small planes, where H would be
 constexpr int MT_TMEM_Y = 256, MT_TMEM_ACT = 384, MT_ACT_COLS = 3 * MT_SLICE / 2;
 
 // 8 consecutive floats with one 32-byte access (a whole sector)
@@ -441,6 +446,15 @@ __global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerVi
       float y[2][32];
       umma::tmem_ld32(tmem + MT_TMEM_Y + c0 + lane_bits, y[0]);
       umma::tmem_ld32(tmem + MT_TMEM_Y + c0 + 32 + lane_bits, y[1]);
+      if constexpr (POOLED) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          float lo[16];
+          umma::tmem_ld16(tmem + MT_TMEM_YLO + c0 + 16 * q + lane_bits, lo);
+#pragma unroll
+          for (int e = 0; e < 16; ++e) y[q >> 1][(q & 1) * 16 + e] += lo[e];
+        }
+      }
       umma::fence_before_sync();
       __syncwarp();
       if (lane == 0) mbar_arrive(y_free);
@@ -500,8 +514,8 @@ __global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerVi
         for (int pl = 2; pl >= 0; --pl)
 #pragma unroll
           for (int s = 0; s < 2; ++s)
-            umma::mma_bf16_ts(tmem + MT_TMEM_Y, act + pl * (MT_SLICE / 2) + s * 8, umma::smem_desc(wb + s * 32), idesc2,
-                              !(l2_slice == 0 && pl == 2 && s == 0));
+            umma::mma_bf16_ts(tmem + (POOLED && pl ? MT_TMEM_YLO : MT_TMEM_Y), act + pl * (MT_SLICE / 2) + s * 8, umma::smem_desc(wb + s * 32),
+                              idesc2, !(l2_slice == 0 && s == 0 && (pl == 2 || (POOLED && pl == 0))));
         umma::commit(&act_free[l2_slice & 1]);
         ++l2;
         if (++l2_slice == n_slices) { l2_slice = 0; ++l2_tile; umma::commit(y_full); }

@@ -14,12 +14,13 @@
 //      token = column.  A thread of the sixteen warps therefore holds many tokens of ONE hidden unit: its bias is a
 //      constant, and the sum over a chunk's tokens stays in registers.  (With tokens as lanes the same kernel needed 31
 //      shuffles and as many selects per 32 activations, a bias load each and an atomic per sum: 38 instructions per
-//      activation, 690 us for 256 sequences x 56 chunks x 64 tokens x 2 sides x 256 units; now MEASURED.)
-//    * Two token buffers and two accumulators, one CTA-wide barrier per tile: behind it the tensor core works on tile i + 1 and
-//      the copies of tile i + 2 are under way while the warps go through tile i.
+//      activation, 690 us for 256 sequences x 56 chunks x 64 tokens x 2 sides x 256 units; now 250 us.)
+//    * Warp roles around a ring of four token buffers and two accumulators: four copy warps (two tiles under way behind the newest),
+//      one MMA thread, sixteen epilogue warps.  With two buffers and one CTA-wide barrier per tile the kernel took 522 us
+//      where it now takes 250.
 //    * The pooled activations (1/C) sum_j gelu(...) go to a scratch row per (side, sequence, chunk).
-//    Bound by the activation arithmetic (14 fp32 operations, 4 of the integer pipe and an exponential per activation).
-// The only wait (on the MMA commit) is bounded; on give-up the status word gets KVE_ERR_TIMEOUT.
+//    Bound by the activation arithmetic (about ten fp32 operations, in packed pairs, and an exponential per activation).
+// Every mbarrier wait is bounded; on give-up the status word gets KVE_ERR_TIMEOUT.
 #include "common.cuh"
 #include "kernels.h"
 #include "umma.cuh"
@@ -229,7 +230,7 @@ __global__ void __launch_bounds__(TM_THREADS, 1) kve_token_mlp_pool_kernel(Token
           for (int e = 0; e < 16; e += 2) {
             float2 relu, abs_x;
             const float2 x = add2(make_float2(__uint_as_float(h[q][e]), __uint_as_float(h[q][e + 1])), make_float2(b1, b1));
-            const float2 tail = gelu_tail2(x, relu, abs_x);
+            const float2 tail = gelu_tail2<6>(x, relu, abs_x);
             tail_sum = fma2(abs_x, tail, tail_sum);
             relu_sum = add2(relu_sum, relu);
           }

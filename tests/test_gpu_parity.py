@@ -1318,3 +1318,46 @@ def test_decode_step_host_from_pageable_buffers_and_chained_through_one_buffer()
         assert st.poll_status() == 0
         results.append((buf.clone(), out.clone()))
     assert torch.equal(results[0][0], results[1][0]) and torch.equal(results[0][1], results[1][1])
+
+
+@pytest.mark.parametrize("d_sum", [64, 128, 192])
+def test_chunk_mlp_of_several_tiles_per_cta(d_sum):
+    """Hidden widths of half an accumulator, of one and of one and a half, with more tiles of 128 chunks than CTAs (so that every
+    barrier of the pipeline wraps), and keep lists of five rounds of 32 chunks."""
+    b = _binding()
+    wl = wlm.Workload("tiles", B=4, H=16, n=4 * 153 + 10, C=4, W=8, d_g=64, agg="mlp", d_sum=d_sum, key_offset_std=0.5, seed=d_sum)
+    assert wl.S * wl.n_stale_chunks() > 74 * 128
+    pb = hz.Problem(wl)
+    st = make_store(wl)
+    load_kv(st, 0, pb.K, pb.V)
+    run_gpu_pipeline(st, pb, 0, b.AggWeights(pb.mlp), b.LstmWeights(pb.lstm))
+    assert st.poll_status() == 0
+    check_summaries(st, pb)
+    # with 1.2 M bf16 summaries a few round the other way than the oracle's, by one step; the list is held to the kernel's own scores
+    idx, cnt = pb.o32.compact(st.scores[0].cpu().numpy(), pb.Nc, pb.tau)
+    assert np.array_equal(st.keep_idx[0].cpu().numpy(), idx) and np.array_equal(st.keep_cnt[0].cpu().numpy(), cnt)
+
+
+def test_two_sequence_groups_per_cluster_of_two_ctas():
+    wl = wlm.Workload("groups", B=17, H=35, n=9 * 16 + 40, C=16, W=32, d_g=128, agg="mean", key_offset_std=0.5, seed=12)
+    assert wl.S > 8 * 74 and wl.S % 16
+    full_check(wl, "summary")
+
+
+@pytest.mark.parametrize("d_sum", [128, 256])
+def test_token_mlp_second_layer_is_no_less_precise_than_fp32_loops(d_sum):
+    """The sum of d_sum products in an fp32 loop rounds d_sum times, each time by ulp / sqrt(12) in the root mean square, with an
+    ulp of at most 2^-23 of the result's size: sqrt(d_sum / 12) 2^-23 rms(result)."""
+    b = _binding()
+    wl = wlm.CFG2.small(B=2, H=8, n=64 * 22, C=64, W=128, agg="token_mlp", d_sum=d_sum, seed=77)
+    K, V = wlm.gen_kv(wl)
+    mlp = wlm.gen_mlp_weights(wl)
+    st = make_store(wl)
+    load_kv(st, 0, K, V)
+    st.summarize_chunks(0, 0, 20, b.AggWeights(mlp))
+    want = kvo.Oracle("f64").summarize(K, V, 64, 0, 20, kvo.AGG_TOKEN_MLP, mlp)
+    assert st.poll_status() == 0
+    for got, name in ((st.ksum_f32, "ksum"), (st.vsum_f32, "vsum")):
+        ref = want[name][:, :20]
+        err = got[0, :, :20].cpu().numpy() - ref
+        assert np.sqrt(np.mean(err ** 2)) <= np.sqrt(d_sum / 12) * 2.0 ** -23 * np.sqrt(np.mean(ref ** 2))
