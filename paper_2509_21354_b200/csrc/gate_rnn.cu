@@ -10,7 +10,7 @@
 //    units, i.e. 256 rows of W_hh; eight warps own 8 units each and keep their rows in REGISTERS as mma A fragments
 //    for the whole kernel (128 registers per thread at d_g = 256).  (Sixteen warps, eight per group, with ten of the sixteen k
 //    tiles' fragments read from shared memory because 128 registers do not hold them: 330 us on 512 sequences x 121
-//    chunks, 347 us with the groups taking turns at the tensor cores, against 285 us this way.)
+//    chunks, 347 us with the groups taking turns at the tensor cores, against 285 us then.)
 //  * Per step the CTA computes its rows of W_hh h with warp-level tensor-core MMAs (m16n8k16, bf16 x bf16 -> fp32).  W_hh is
 //    bf16 by definition; the fp32 state h enters as PL = 2 bf16 planes by default (h = hi + lo up to 2^-17 |h|: 16 of its 24
 //    significant bits; a third plane makes the products exact, moves the scores by 1e-7 - far below what the fast
@@ -20,17 +20,18 @@
 //    same (hidden unit, sequence): the cell update is thread-local, c lives in registers.  f, i and g share one reciprocal
 //    and o and tanh(c) another (five exponentials and two reciprocals per element instead of five and five: the
 //    special-function unit is what the cell update waits for).
-//  * Exchange of h_t: a warp gathers the planes of its 8 hidden units in a small staging area of its own; bulk copies put them
-//    into the double-buffered h planes of every other CTA of the cluster and count their bytes on an mbarrier there (the own
-//    copy is a plain store followed by a local arrive), so a step costs one one-way transfer and no cluster-wide barrier.
-//    A CTA can only be sent step t+1 data after it has itself sent step t data, i.e. after all its warps have finished
+//  * Exchange of h_t: a warp writes the planes of its 8 hidden units into its own CTA's double-buffered h planes (two units per
+//    4-byte word, after one shuffle); from there bulk copies put the block into those of every other CTA of the cluster and count
+//    their bytes on an mbarrier there, so a step costs one one-way transfer and no cluster-wide barrier.  (With the planes
+//    gathered in a staging area in 2-byte stores and copied to the own buffer from there: 8.6 us more on 512 sequences x 121 chunks,
+//    1.5 us on 256 x 56, 0.8 us on 8 x 28 at d_g = 128.)  A CTA can only be sent step t+1 data after it has itself sent step t data, i.e. after all its warps have finished
 //    reading the buffer that is being overwritten.
 //  * P_{t+1} is fetched a round ahead: the projection kernel stores the four pre-activations of a hidden unit side by side, so a
 //    thread takes them with one 16-byte load.
 //  * The score head is not part of the chain: a warp leaves its 8 units' share of w_s . h_t per sequence (d_g / 8 partial sums
 //    per (s, t): an eighth of the bytes of h_t), and when the chain is through the cluster adds them up in a fixed order.
-//  Measured, recurrence and score head: 512 sequences x 121 chunks 314 -> 285 us, 256 x 56 92.5 -> 80 us, 8 x 28 at
-//  d_g = 128 51.6 -> 33 us (there a cluster of two CTAs halves the MMA chain: one CTA held all of W_hh).  Slower: waiting for the
+//  Measured, recurrence and score head: 512 sequences x 121 chunks 314 -> 276 us, 256 x 56 92.5 -> 79 us, 8 x 28 at
+//  d_g = 128 51.6 -> 32 us (there a cluster of two CTAs halves the MMA chain: one CTA held all of W_hh).  Slower: waiting for the
 //  CTA's own planes and the peers' apart, with the own units' MMAs in between (255 -> 261 us a step on 256 sequences), and
 //  the score's shuffles between the MMAs (248 -> 255 us).
 // Every mbarrier wait is bounded (one second); on give-up the status word gets KVE_ERR_TIMEOUT and
@@ -78,14 +79,13 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RNN_THREADS, 1) kve
   constexpr int KBLK = PL * NS * 8;                     // bf16 elements of one k-block (8 units): [plane][sequence][8]
   constexpr int HS_BUF = (DG / 8) * KBLK;               // bf16 elements per h buffer
   constexpr uint32_t H_BYTES = PL * NS * (DG - HU) * 2; // bytes of h planes a CTA receives from its peers per step and group
-  constexpr int OFF_STAGE = NG * 2 * HS_BUF * 2;
-  constexpr int OFF_BARS = OFF_STAGE + NG * RNN_WARPS * KBLK * 2;
+  constexpr int OFF_BARS = NG * 2 * HS_BUF * 2;
+  constexpr int BULK_PENDING = 2 * NG - 1;              // a group's copies of two steps ago: all but the newest 2 NG - 1 commits
   static_assert(HU == 8 * RNN_WARPS && KT % 2 == 0, "one pair of m16 tiles (8 units x 4 gates) per warp");
-  static_assert(OFF_STAGE % 16 == 0 && OFF_BARS % 16 == 0, "16-byte pieces");
+  static_assert(OFF_BARS % 16 == 0, "16-byte pieces");
 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint16_t* hs = reinterpret_cast<uint16_t*>(smem_raw);                          // [NG][2][DG / 8][PL][NS][8]
-  uint16_t* stage = reinterpret_cast<uint16_t*>(smem_raw + OFF_STAGE);           // [NG][warps][PL][NS][8]
   uint64_t* hbar = reinterpret_cast<uint64_t*>(smem_raw + OFF_BARS);             // [NG][2] h planes landed
 
   const int tid = threadIdx.x, lane = tid & 31;
@@ -201,7 +201,6 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RNN_THREADS, 1) kve
 #pragma unroll
     for (int gi = 0; gi < NG; ++gi) {
       uint16_t* hs_g = hs + gi * 2 * HS_BUF;
-      uint16_t* my_stage = stage + (gi * RNN_WARPS + warp) * KBLK;
       uint64_t* hbar_g = hbar + 2 * gi;
       // P of the next round, used there: requested before the wait (one group), while the MMAs drain (two, where nothing waits)
       float4 pv[2];
@@ -252,9 +251,11 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RNN_THREADS, 1) kve
         if (!__all_sync(0xffffffffu, alive)) break;
         load_p((gi + 1) % NG, step + (gi + 1) / NG, pv);
       }
-      // ---- cell update (thread-local), planes of h_t into the warp's staging area ---------------------
-      if (CL > 1) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-      __syncwarp();      // earlier copies have read the staging area
+      // ---- cell update (thread-local), planes of h_t into this CTA's buffer ---------------------
+      // the copies from there two steps ago have been read: those of the group's last step may still be under way
+      if (CL > 1) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(BULK_PENDING) : "memory");
+      __syncwarp();
+      uint32_t split[2][3];
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
         float pre[4];
@@ -268,30 +269,32 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RNN_THREADS, 1) kve
         }
         const float hv = lstm_cell(pre, c[gi][e]);
         hlast[gi][e] = hv;
-        if (send_h) {
-          uint32_t pl3[3];
-          split3(hv, pl3);
-          const int j = tig * 2 + e;
-#pragma unroll
-          for (int pl = 0; pl < PL; ++pl) my_stage[(pl * NS + j) * 8 + g] = (uint16_t)pl3[pl];
-        }
+        split3(hv, split[e]);
       }
       KVE_RNN_MARK(3);
       // ---- the warp's k-block (8 units: [plane][sequence][8], contiguous) to every CTA of the cluster ----
       if (send_h) {
         const uint32_t off = (uint32_t)(((gi * 2 + (buf ^ 1)) * HS_BUF + ((int)rank * RNN_WARPS + warp) * KBLK) * 2);
-        if (CL > 1) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // staging writes -> visible to the bulk copies
+        // lanes g and g ^ 1 hold neighbouring units: an even g takes both units of sequence 2 tig, an odd one those of 2 tig + 1, and
+        // a warp's store instruction is a whole plane of the block: 128 bytes in a row
+        const bool odd = (g & 1) != 0;
+        unsigned char* mine = reinterpret_cast<unsigned char*>(hs) + off + (tig * 2 + (g & 1)) * 16 + (g >> 1) * 4;
+        const uint32_t keep = odd ? split[1][0] | split[1][1] << 16 : split[0][0] | split[0][1] << 16;
+        const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? split[0][0] | split[0][1] << 16 : split[1][0] | split[1][1] << 16, 4);
+        *reinterpret_cast<uint32_t*>(mine) = __byte_perm(odd ? got : keep, odd ? keep : got, 0x5410);
+        *reinterpret_cast<uint32_t*>(mine + NS * 16) = __byte_perm(odd ? got : keep, odd ? keep : got, 0x7632);
+        if constexpr (PL == 3) {
+          const uint32_t keep2 = odd ? split[1][2] : split[0][2], got2 = __shfl_xor_sync(0xffffffffu, odd ? split[0][2] : split[1][2], 4);
+          *reinterpret_cast<uint32_t*>(mine + 2 * NS * 16) = (odd ? got2 : keep2) | (odd ? keep2 : got2) << 16;
+        }
+        if (CL > 1) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // visible to the bulk copies
         __syncwarp();
-        // own CTA: plain 16-byte stores (ordered by this warp's arrive below)
-        for (int idx = lane; idx < KBLK / 8; idx += 32)
-          *reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(hs) + off + idx * 16) = *reinterpret_cast<const uint4*>(my_stage + idx * 8);
         if (CL > 1) {
-          // peers: one bulk copy each, its bytes counted on the receiver's barrier
+          // peers: one bulk copy each out of the own buffer, its bytes counted on the receiver's barrier
           if (lane < CL && lane != (int)rank)
-            bulk_s2cluster(peer_hs + off, smem_u32(my_stage), KBLK * 2, peer_bar + (2 * gi + (buf ^ 1)) * 8);
+            bulk_s2cluster(peer_hs + off, smem_u32(hs) + off, KBLK * 2, peer_bar + (2 * gi + (buf ^ 1)) * 8);
           asm volatile("cp.async.bulk.commit_group;" ::: "memory");
         }
-        __syncwarp();
         if (lane == 0) mbar_arrive(&hbar_g[buf ^ 1]);     // release: this warp's own pieces are in place
       }
       KVE_RNN_MARK(4);
@@ -347,7 +350,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RNN_THREADS, 1) kve
 template <int DG, int CL, int NG, int PL>
 static cudaError_t launch_rnn_t(const RnnArgs& a, cudaStream_t st) {
   constexpr int KBLK_BYTES = PL * 8 * 8 * 2;
-  constexpr int smem = NG * 2 * (DG / 8) * KBLK_BYTES + NG * RNN_WARPS * KBLK_BYTES + NG * 2 * 8;
+  constexpr int smem = NG * 2 * (DG / 8) * KBLK_BYTES + NG * 2 * 8;
   static DeviceFlags opted;
   {
     cudaError_t e = smem_opt_in(opted, kve_gate_rnn_kernel<DG, CL, NG, PL>, smem);
