@@ -422,8 +422,9 @@ int kvE_set_gate_planes(kvE_store* st, int planes) {
   return KVE_OK;
 }
 
-int kvE_summarize_chunks(kvE_store* st, int layer, int chunk_begin, int chunk_end, const kvE_agg_weights* w,
-                         void* stream) {
+// beside: the launch may run beside the gate recurrence launched just before it
+static int summarize_chunks(kvE_store* st, int layer, int chunk_begin, int chunk_end, const kvE_agg_weights* w, bool beside,
+                            void* stream) {
   if (bad_layer(st, layer) || chunk_begin < 0 || chunk_end < chunk_begin) return KVE_ERR_ARG;
   if (wrong_device(st)) return KVE_ERR_STATE;
   LayerState& ls = st->layers[layer];
@@ -439,7 +440,8 @@ int kvE_summarize_chunks(kvE_store* st, int layer, int chunk_begin, int chunk_en
   const int list_cut = lower_listed(ls, chunk_begin);      // the compacted copies of these summaries are stale
   if (!token_mlp) {
     Prof prof(st, KVE_K_CHUNK_MEAN, s);
-    e = launch_chunk_mean(v, chunk_begin, chunk_end, !mlp, st->cfg.agg == KVE_AGG_MAX, s, -1, list_cut);
+    e = beside ? launch_chunk_mean_beside(v, chunk_begin, chunk_end, !mlp, st->cfg.agg == KVE_AGG_MAX, s)
+               : launch_chunk_mean(v, chunk_begin, chunk_end, !mlp, st->cfg.agg == KVE_AGG_MAX, s, -1, list_cut);
   } else {
     Prof prof(st, KVE_K_CHUNK_MLP, s);
     MlpWeights mw;
@@ -460,6 +462,11 @@ int kvE_summarize_chunks(kvE_store* st, int layer, int chunk_begin, int chunk_en
   if (e != cudaSuccess) return cuda_fail(st, e);
   if (chunk_begin <= ls.n_summarised && chunk_end > ls.n_summarised) ls.n_summarised = chunk_end;
   return KVE_OK;
+}
+
+int kvE_summarize_chunks(kvE_store* st, int layer, int chunk_begin, int chunk_end, const kvE_agg_weights* w,
+                         void* stream) {
+  return summarize_chunks(st, layer, chunk_begin, chunk_end, w, false, stream);
 }
 
 int kvE_gate(kvE_store* st, int layer, int chunk_begin, int chunk_end, const kvE_lstm_weights* w, void* stream) {
@@ -592,11 +599,39 @@ int kvE_adopt_device_state(kvE_store* st, int layer, void* stream) {
   return KVE_OK;
 }
 
+// How many of its nc chunks kvE_refresh summarises and gates before the rest (all: nc).  The recurrence is a chain of short
+// steps that leaves HBM idle, the chunk mean a stream that leaves everything else idle: of two ranges, the means of the second
+// are taken while the recurrence goes through the first (kve_chunk_mean_beside_kernel).  With M and R the microseconds of
+// the means and of the recurrence alone, x = M / (M + 0.7 R) of the chunks first lets both end at about the same time; M (1 - x)
+// is then hidden, and the second launches of MLP, projection and recurrence and the slower recurrence are paid.  Measured, one
+// range -> two (us a step): 512 sequences x 121 chunks of 128, MLP 1055 -> 1010; 128 x 121 of 128, MLP 370 -> 350; 256 x 240
+// of 32, MLP 604 -> 562; 512 x 56 of 64, mean 344 -> 333; 256 x 120 of 64, mean 364 -> 340, MLP 407 -> 393; below the lines:
+// 256 x 56 of 64 with 28 us to hide, mean 194 -> 189, MLP 218 -> 226; 32 x 250 of 64, mean, 33 us: 356 -> 364.
+constexpr double REFRESH_HIDE_US = 40, REFRESH_HIDE_MLP_US = 60;
+
+static int first_range(const kvE_store* st, int nc, const kvE_lstm_weights* lw) {
+  const kvE_config& c = st->cfg;
+  if (c.agg == KVE_AGG_TOKEN_MLP) return nc;      // its kernel takes whole SMs
+  if (st->profiling) return nc;                   // one launch of each kernel, alone
+  if (!lw || !lw->W_ih || !lw->W_hh || !lw->b_ih || !lw->b_hh || !lw->w_s) return nc;      // refused by kvE_gate
+  const double mean_us = (double)st->S * nc * c.C * 512 / 6.6e6;
+  const double rnn_us = nc * gate_rnn_us_per_chunk(st->S, c.d_g, st->gate_planes);
+  const double x = mean_us / (mean_us + 0.7 * rnn_us);
+  if (mean_us * (1 - x) < (c.agg == KVE_AGG_MLP ? REFRESH_HIDE_MLP_US : REFRESH_HIDE_US)) return nc;
+  const int first = (int)(nc * x + 0.5);
+  return first < 1 ? 1 : first;
+}
+
 int kvE_refresh(kvE_store* st, int layer, const kvE_agg_weights* aw, const kvE_lstm_weights* lw, float tau, void* stream) {
   if (bad_layer(st, layer)) return KVE_ERR_ARG;
   const int nc = stale_chunks(st->cfg, st->layers[layer].n_tokens);
-  int rc = kvE_summarize_chunks(st, layer, 0, nc, aw, stream);
-  if (rc == KVE_OK) rc = kvE_gate(st, layer, 0, nc, lw, stream);
+  const int first = nc > 0 ? first_range(st, nc, lw) : nc;
+  int rc = summarize_chunks(st, layer, 0, first, aw, false, stream);
+  if (rc == KVE_OK) rc = kvE_gate(st, layer, 0, first, lw, stream);
+  if (first < nc) {
+    if (rc == KVE_OK) rc = summarize_chunks(st, layer, first, nc, aw, true, stream);
+    if (rc == KVE_OK) rc = kvE_gate(st, layer, first, nc, lw, stream);
+  }
   if (rc == KVE_OK) rc = kvE_compact(st, layer, tau, stream);
   return rc;
 }

@@ -95,7 +95,6 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RNN_THREADS, 1) kve
   const int seq0 = (blockIdx.x / CL) * NS * NG;      // group gi owns sequences seq0 + 8 gi .. + 7
   const int ug = (int)rank * HU + warp * 8 + g;                // this thread's hidden unit
 
-  pdl_launch_dependents();
   KVE_RNN_ONCE(0);
   if (tid == 0) {
     for (int i = 0; i < 2 * NG; ++i) mbar_init(&hbar[i], RNN_WARPS + (CL > 1 ? 1 : 0));
@@ -134,6 +133,8 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RNN_THREADS, 1) kve
 
   KVE_RNN_ONCE(1);
   pdl_wait();      // W_hh is in place; the carried state and P come from earlier kernels
+  // only now, when all earlier work is complete: a launch may run beside this kernel without waiting for anything (kvE_refresh)
+  pdl_launch_dependents();
   KVE_RNN_ONCE(2);
   // ---- initial state: every CTA needs the full h of its sequences as planes in buffer 0 of each group -------------
   for (int i = tid; i < NG * NS * (DG / 2); i += RNN_THREADS) {
@@ -357,17 +358,40 @@ static cudaError_t launch_rnn_t(const RnnArgs& a, cudaStream_t st) {
     if (e != cudaSuccess) return e;
   }
   const int clusters = (a.S + 8 * NG - 1) / (8 * NG);
-  return launch_pdl(kve_gate_rnn_kernel<DG, CL, NG, PL>, dim3(clusters * CL), dim3(RNN_THREADS), smem, st, a);
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  // an SM keeps its division of shared memory and L1 as long as a CTA is there: all of it shared, for what may run beside this kernel
+  attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  attr[1].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(clusters * CL);
+  cfg.blockDim = dim3(RNN_THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kve_gate_rnn_kernel<DG, CL, NG, PL>, a);
 }
 
-// two groups of 8 sequences per cluster once one group per cluster would need more than one wave of clusters
+// CTAs of a cluster; two groups of 8 sequences per cluster once one group per cluster would need more than one wave of clusters
+static int cluster_ctas(int d_g) { return d_g / 64; }
+static bool two_groups(int S, int d_g) { return (S + 7) / 8 > sm_count() / cluster_ctas(d_g); }
+
+// Microseconds per chunk as measured (two planes of h, d_g = 256): 1.22 with one group of sequences per cluster, 2.28 with two
+double gate_rnn_us_per_chunk(int S, int d_g, int planes) {
+  const bool two = two_groups(S, d_g);
+  const int clusters = (S + (two ? 15 : 7)) / (two ? 16 : 8), wave = sm_count() / cluster_ctas(d_g);
+  return (two ? 2.28 : 1.22) * (planes == 3 ? 1.25 : 1.0) * ((clusters + wave - 1) / wave);
+}
+
 template <int PL>
 static cudaError_t launch_rnn_planes(const RnnArgs& a, int d_g, cudaStream_t st) {
-  const int groups = (a.S + 7) / 8;
+  const bool two = two_groups(a.S, d_g);
   switch (d_g) {
-    case 256: return groups > sm_count() / 4 ? launch_rnn_t<256, 4, 2, PL>(a, st) : launch_rnn_t<256, 4, 1, PL>(a, st);
-    case 128: return groups > sm_count() / 2 ? launch_rnn_t<128, 2, 2, PL>(a, st) : launch_rnn_t<128, 2, 1, PL>(a, st);
-    case 64:  return groups > sm_count() ? launch_rnn_t<64, 1, 2, PL>(a, st) : launch_rnn_t<64, 1, 1, PL>(a, st);
+    case 256: return two ? launch_rnn_t<256, 4, 2, PL>(a, st) : launch_rnn_t<256, 4, 1, PL>(a, st);
+    case 128: return two ? launch_rnn_t<128, 2, 2, PL>(a, st) : launch_rnn_t<128, 2, 1, PL>(a, st);
+    case 64:  return two ? launch_rnn_t<64, 1, 2, PL>(a, st) : launch_rnn_t<64, 1, 1, PL>(a, st);
     default:  return cudaErrorInvalidValue;
   }
 }

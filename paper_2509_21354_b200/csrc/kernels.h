@@ -76,6 +76,7 @@ cudaError_t launch_append_next(const LayerView& v, const void* k_new, const void
 // else the launch does nothing (a trigger that is replayed from a CUDA graph)
 // list_cut >= 0 (here, launch_chunk_token_mlp, launch_gate_proj): the keep list covers no more than that many chunks from now on
 cudaError_t launch_chunk_mean(const LayerView& v, int t0, int t1, bool final_output, bool pool_max, cudaStream_t st, int dev_window, int list_cut);
+cudaError_t launch_chunk_mean_beside(const LayerView& v, int t0, int t1, bool final_output, bool pool_max, cudaStream_t st);
 cudaError_t launch_chunk_mlp(const LayerView& v, int t0, int t1, const MlpWeights& w, int d_sum, cudaStream_t st, int dev_window);
 // the MLP's second layer on pooled activations hid [2][S * (t1 - t0)][d_sum]: Kbar = W2 hid + b2 (d_sum 128 or 256)
 cudaError_t launch_pooled_out(const LayerView& v, int t0, int t1, const MlpWeights& w, int d_sum, const float* hid, cudaStream_t st);
@@ -85,6 +86,7 @@ cudaError_t launch_chunk_token_mlp(const LayerView& v, int t0, int t1, const Mlp
 cudaError_t launch_gate_proj(const LayerView& v, int t0, int t1, const uint16_t* W_ih, const float* b_ih,
                              const float* b_hh, int d_g, float* P, int list_cut, cudaStream_t st);
 // planes: bf16 planes of the fp32 state h that enter the recurrent product (2, or 3 = exact products)
+double gate_rnn_us_per_chunk(int S, int d_g, int planes);
 cudaError_t launch_gate_rnn(const LayerView& v, int t0, int t1, const uint16_t* W_hh, const float* w_s, float b_s,
                             int d_g, const float* P, float* H, bool reset_state, int planes, cudaStream_t st);
 // one LSTM step on chunk t with the carried state, its score, and chunk t appended to the keep list for tau (which must

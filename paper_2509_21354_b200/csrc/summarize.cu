@@ -98,6 +98,126 @@ cudaError_t launch_chunk_mean(const LayerView& v, int t0, int t1, bool final_out
                   : cudaLaunchKernelEx(&cfg, kve_chunk_mean_kernel<false>, v, t0, n_range, by_range, final_output ? 1 : 0, dev_window, list_cut);
 }
 
+// ---- the same mean for a launch that runs beside the gate recurrence -----------------------------------------------
+// The recurrence leaves an SM a sixth of its registers and most of its shared memory, so the rows on their way wait there: a
+// warp's pages come in bulk copies of 16 rows, eight of them in flight, and are added up row by row as above (the same rounding).
+// A CTA takes several units in a row, so that the copies of the next one are under way while the last is added up.
+// 4.1 TB/s beside the recurrence of 512 sequences, which takes 22 % longer meanwhile (pages of 128 tokens; the kernel above, its
+// rows in registers: 3 TB/s).  Fewer rows in flight were slower for the whole step (eight pieces of 8 rows +1 %, four +9 %), asynchronous
+// 16-byte copies +0.6 %; 256 rows per CTA +1 %, 512 +2 %, and a CTA per page +4 % with pages of 32 tokens.
+constexpr int MB_ROWS = 16, MB_STAGES = 8;
+constexpr int MB_CTA_ROWS = 128;                      // rows of K (or V) that a CTA takes, about
+constexpr int MB_STAGE_BYTES = MB_ROWS * D * 2;
+constexpr int MB_SMEM_BAR = MEAN_WARPS * MB_STAGES * MB_STAGE_BYTES;
+constexpr int MB_SMEM_BYTES = MB_SMEM_BAR + MEAN_WARPS * MB_STAGES * 8;
+
+template <bool POOL_MAX>
+__global__ void __launch_bounds__(MEAN_WARPS * 32) kve_chunk_mean_beside_kernel(LayerView v, int t0, int n_range, FastDiv by_range, int n_units,
+                                                                               int units_per_cta, int final_output) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  pdl_launch_dependents();
+  if (blockIdx.x == gridDim.x - 1) {      // an extra CTA, the last to be placed: this launch is not over before the one it runs beside
+    pdl_wait();
+    return;
+  }
+  const int lane = threadIdx.x & 31, is_v = threadIdx.x >> 5;
+  const int unit0 = (int)blockIdx.x * units_per_cta, n_mine = min(units_per_cta, n_units - unit0);      // 1 .. 32
+  // lane u keeps the page and the summary row of unit u
+  long long page = -1, row_of = 0;
+  if (lane < n_mine) {
+    const int s = (int)by_range.div((uint32_t)(unit0 + lane)), t = t0 + (unit0 + lane - s * n_range);
+    row_of = (long long)s * v.max_chunks + t;
+    page = v.page_table[row_of];
+    if (page < 0 || page >= v.n_pages) {
+      set_status(v.status, ERR_CAPACITY);
+      page = -1;
+    }
+  }
+  unsigned char* ring = smem_raw + is_v * MB_STAGES * MB_STAGE_BYTES;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw + MB_SMEM_BAR) + is_v * MB_STAGES;
+  const uint16_t* pool = is_v ? v.v_pages : v.k_pages;
+  const int per_unit = (v.C + MB_ROWS - 1) / MB_ROWS;      // pieces of a page; one without a page has none
+  int f_unit = 0, f_piece = 0, n_fetched = 0;              // the next piece to fetch (the same in all lanes)
+  auto fetch = [&]() {
+    long long p = -1;
+    while (f_unit < n_mine && (p = __shfl_sync(0xffffffffu, page, f_unit)) < 0) ++f_unit;
+    if (f_unit >= n_mine) return;
+    if (lane == 0) {
+      const uint32_t bytes = (uint32_t)min(MB_ROWS, v.C - f_piece * MB_ROWS) * D * 2;
+      uint64_t* bar = &full[n_fetched % MB_STAGES];
+      mbar_arrive_expect_tx(bar, bytes);
+      bulk_g2s(ring + (n_fetched % MB_STAGES) * MB_STAGE_BYTES, pool + (p * v.C + f_piece * MB_ROWS) * D, bytes, bar);
+    }
+    ++n_fetched;
+    if (++f_piece == per_unit) { f_piece = 0; ++f_unit; }
+  };
+  if (lane == 0) {
+    for (int i = 0; i < MB_STAGES; ++i) mbar_init(&full[i], 1);
+    mbar_fence_init();
+  }
+  __syncwarp();
+  for (int i = 0; i < MB_STAGES; ++i) fetch();
+  bool ok = true;
+  int i = 0;                                               // the next piece to add up
+  for (int u = 0; u < n_mine && ok; ++u) {
+    if (__shfl_sync(0xffffffffu, page, u) < 0) continue;
+    float acc[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) acc[x] = POOL_MAX ? -INFINITY : 0.f;
+    auto take = [&](const uint2& w) {
+      const float f[4] = {bf16lo(w.x), bf16hi(w.x), bf16lo(w.y), bf16hi(w.y)};
+#pragma unroll
+      for (int x = 0; x < 4; ++x) acc[x] = POOL_MAX ? fmaxf(acc[x], f[x]) : acc[x] + f[x];
+    };
+    for (int p = 0; p < per_unit; ++p, ++i) {
+      ok = __all_sync(0xffffffffu, mbar_wait_bounded(&full[i % MB_STAGES], (uint32_t)((i / MB_STAGES) & 1)));
+      if (!ok) break;
+      const uint2* row = reinterpret_cast<const uint2*>(ring + (i % MB_STAGES) * MB_STAGE_BYTES) + lane;
+      const int rows = min(MB_ROWS, v.C - p * MB_ROWS);
+      if (rows == MB_ROWS) {
+#pragma unroll
+        for (int j = 0; j < MB_ROWS; ++j) take(row[j * (D / 4)]);
+      } else {
+        for (int j = 0; j < rows; ++j) take(row[j * (D / 4)]);
+      }
+      __syncwarp();
+      fetch();
+    }
+    if (!ok) break;
+    if (!POOL_MAX) {
+      const float fc = (float)v.C;
+#pragma unroll
+      for (int x = 0; x < 4; ++x) acc[x] = __fdiv_rn(acc[x], fc);
+    }
+    const long long o = __shfl_sync(0xffffffffu, row_of, u) * D + lane * 4;
+    *reinterpret_cast<float4*>((is_v ? v.vsum_f32 : v.ksum_f32) + o) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+    if (final_output)
+      *reinterpret_cast<uint2*>((is_v ? v.vsum_bf16 : v.ksum_bf16) + o) = make_uint2(pack_bf16x2(acc[0], acc[1]), pack_bf16x2(acc[2], acc[3]));
+  }
+  if (!ok) {      // a wait ran out: the other copies under way are still waited for
+    if (lane == 0) set_status(v.status, ERR_TIMEOUT);
+    for (++i; i < n_fetched; ++i) mbar_wait_bounded(&full[i % MB_STAGES], (uint32_t)((i / MB_STAGES) & 1));
+  }
+}
+
+cudaError_t launch_chunk_mean_beside(const LayerView& v, int t0, int t1, bool final_output, bool pool_max, cudaStream_t st) {
+  const int n_range = t1 - t0;
+  const long long n_units = (long long)v.S * n_range;
+  if (n_units <= 0 || n_units >= (1LL << 31) - 64) return cudaErrorInvalidValue;
+  static DeviceFlags opted, opted_max;
+  const cudaError_t e = pool_max ? smem_opt_in(opted_max, kve_chunk_mean_beside_kernel<true>, MB_SMEM_BYTES)
+                                 : smem_opt_in(opted, kve_chunk_mean_beside_kernel<false>, MB_SMEM_BYTES);
+  if (e != cudaSuccess) return e;
+  int per_cta = v.C < MB_CTA_ROWS ? MB_CTA_ROWS / v.C : 1;
+  if (per_cta > 32) per_cta = 32;
+  while (per_cta > 1 && n_units / per_cta < 4 * sm_count()) per_cta /= 2;
+  const dim3 grid((unsigned)((n_units + per_cta - 1) / per_cta) + 1), block(MEAN_WARPS * 32);
+  const FastDiv by_range = fast_div((uint32_t)n_range);
+  return pool_max ? launch_pdl(kve_chunk_mean_beside_kernel<true>, grid, block, MB_SMEM_BYTES, st, v, t0, n_range, by_range, (int)n_units, per_cta, 1)
+                  : launch_pdl(kve_chunk_mean_beside_kernel<false>, grid, block, MB_SMEM_BYTES, st, v, t0, n_range, by_range, (int)n_units, per_cta,
+                               final_output ? 1 : 0);
+}
+
 // ---- aggregator MLP (Eq. 2 read as mean -> d_sum -> d, exact-erf GELU), fp32 FMA ------------------
 // A CTA takes MLP_ROWS (sequence, chunk) units of one side (blockIdx.y: 0 = keys, 1 = values).
 // The unit's mean sits in ksum_f32 / vsum_f32 (written by chunk_mean); the MLP output overwrites it

@@ -1361,3 +1361,39 @@ def test_token_mlp_second_layer_is_no_less_precise_than_fp32_loops(d_sum):
         ref = want[name][:, :20]
         err = got[0, :, :20].cpu().numpy() - ref
         assert np.sqrt(np.mean(err ** 2)) <= np.sqrt(d_sum / 12) * 2.0 ** -23 * np.sqrt(np.mean(ref ** 2))
+
+
+@pytest.mark.parametrize("agg,d_g,B,C,n", [("mean", 128, 16, 64, 4300), ("max", 256, 16, 40, 4100), ("mlp", 256, 16, 136, 8300), ("mean", 64, 4, 7, 9000)])
+def test_refresh_with_means_beside_the_recurrence_equals_the_stepwise_calls(agg, d_g, B, C, n):
+    """Sizes at which kvE_refresh takes two ranges, the means of the second beside the recurrence over the first: pages of whole and of
+    broken pieces of 16 rows, one and several to a CTA, both group counts; bit for bit what the three calls give, again when
+    repeated, and a bad page id in the second range is reported and nothing of it written."""
+    b = _binding()
+    wl = wlm.Workload("beside", B=B, H=32, n=n, C=C, W=128, d_g=d_g, agg=agg, d_sum=256 if agg == "mlp" else 0, seed=C)
+    mlp = wlm.gen_mlp_weights(wl)
+    aw, lw = b.AggWeights(mlp) if mlp is not None else None, b.LstmWeights(wlm.gen_lstm_weights(wl))
+    st = make_store(wl)
+    st.k_pages.normal_(generator=torch.Generator(device="cuda").manual_seed(1))
+    st.v_pages.normal_(generator=torch.Generator(device="cuda").manual_seed(2))
+    st.set_len(0, n)
+    N = wl.n_stale_chunks()
+    state = lambda: [t.clone() for t in (st.ksum_f32, st.vsum_f32, st.ksum_bf16, st.vsum_bf16, st.scores, st.keep_idx, st.keep_cnt, st.lstm_h, st.lstm_c)]
+    st.summarize_chunks(0, 0, N, aw)
+    st.gate(0, 0, N, lw)
+    st.compact(0, 0.5)
+    want = state()
+    for _ in range(2):
+        for t in (st.ksum_f32, st.vsum_f32, st.ksum_bf16, st.vsum_bf16, st.scores, st.lstm_h, st.lstm_c):
+            t.zero_()
+        st.refresh(0, aw, lw, 0.5)
+        torch.cuda.synchronize()
+        assert st.poll_status() == 0
+        for got, ref in zip(state(), want):
+            assert torch.equal(got, ref)
+    if agg != "mlp":
+        st.ksum_f32[0, 3, N - 1] = 7.0
+        st.page_table[0, 3, N - 1] = -1
+        st.refresh(0, aw, lw, 0.5)
+        torch.cuda.synchronize()
+        assert st.poll_status() == -3
+        assert bool((st.ksum_f32[0, 3, N - 1] == 7.0).all()) and torch.equal(st.ksum_f32[0, 4:], want[0][0, 4:])
