@@ -43,10 +43,17 @@ METRIC = "gated_decode_attention_steps_per_sec"
 UNIT = "steps/s"
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 SCALE = 1.0 / math.sqrt(128.0)
-def kernels_per_step(wl, Nc):
-    """kernel launches of one from-scratch step: set_len, append, chunk mean [+ chunk MLP], gate projection,
-    recurrence with its score head, keep list with its gather, attention"""
-    return 7 + (1 if wl.agg == "mlp" else 0)
+def launches_per_step(step):
+    """the library's kernel launches in one step, counted by the profiler over four of them (outside every timed region):
+    length, append, chunk mean [+ MLP], projection and recurrence - twice where kvE_refresh takes two ranges -, keep list, attention"""
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+    torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        for _ in range(4):
+            step()
+        torch.cuda.synchronize()
+    return sum("kve::" in e.name for e in prof.events()) // 4
 
 
 def load_peaks():
@@ -803,6 +810,7 @@ def run_ours(args, rank, world, local_rank):
     assert st.poll_status() == 0
     loops = [max_over_ranks([t], world)[0] for t in loops] if world > 1 else loops
     ms_total = float(np.median(loops))
+    launches = launches_per_step(rig.step_full)
 
     # ---- steady-state decode step (between two gate triggers): append one token, gated attention ----
     for _ in range(3):
@@ -895,7 +903,7 @@ def run_ours(args, rank, world, local_rank):
         "e2e": {"value": world * args.steps / e2e_s, "unit": UNIT, "h2d_bytes_per_step": 3 * S * 256,
                 "d2h_bytes_per_step": S * 256,
                 "max_abs_diff_vs_device_path": e2e_diff, "max_abs_output": e2e_ref},
-        "gpu_launches": kernels_per_step(wl, rig.Nc) * args.steps * repeats,
+        "gpu_launches": launches * args.steps * repeats,
         "clocks": clk.summary(),
         "roofline": roofline,
         "roofline_largest_hbm_kernel": roofline_hbm,
