@@ -9,6 +9,7 @@ kvE_gate, kvE_compact, kvE_decode_attn, ...) and take the same arguments with to
 of device pointers; `Store` bundles the caller-owned buffers a handle needs.
 """
 import ctypes as C
+import importlib.util
 import os
 
 import numpy as np
@@ -58,6 +59,21 @@ class kvE_lstm_weights(C.Structure):
 
 
 _lib = None
+_bind = None
+
+
+def _load_bind(build_if_missing: bool):
+    """the extension module behind Store.decode_step (csrc/bind.cpp)"""
+    global _bind
+    if _bind is None:
+        path = _build.build_bind() if build_if_missing else _build.BIND
+        if not os.path.exists(path):
+            raise RuntimeError(f"{path} is missing: run `python -m paper_2509_21354_b200.build`")
+        spec = importlib.util.spec_from_file_location("_kve_bind", path)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        _bind = module
+    return _bind
 
 
 def load_library(build_if_missing: bool = True) -> C.CDLL:
@@ -70,6 +86,7 @@ def load_library(build_if_missing: bool = True) -> C.CDLL:
         path = _build.build()
     if not os.path.exists(path):
         raise RuntimeError(f"{path} is missing: run `python -m paper_2509_21354_b200.build`")
+    _load_bind(build_if_missing)
     lib = C.CDLL(path)
     lib.kvE_workspace_bytes.restype = C.c_size_t
     lib.kvE_workspace_bytes.argtypes = [C.POINTER(kvE_config)]
@@ -198,6 +215,8 @@ class Store:
         if not torch.cuda.is_available():
             raise RuntimeError("libkve needs a CUDA device; there is no CPU path")
         self.lib = load_library()
+        self._decode_step = _bind.decode_step
+        self._decode_step_fn = C.cast(self.lib.kvE_decode_step, C.c_void_p).value
         self.device = torch.device(device)
         self.Hq = H if Hq is None else Hq
         self.cfg = kvE_config(B=B, Hq=self.Hq, Hkv=H, d=128, C=C_, W=W, max_tokens=max_tokens, n_layers=n_layers,
@@ -309,11 +328,10 @@ class Store:
 
     def decode_step(self, layer, k_new, v_new, q, out=None, lse=None, scale=None, n_reserve=0, stream=None):
         """append one token per sequence (k_new, v_new: bf16 [S, 128]) at the device-held length and attend, one launch"""
-        shape = self.row_shape
         if out is None:
             out = torch.empty_like(q)
-        rc = self.lib.kvE_decode_step(self.handle, layer, _rows(k_new, shape), _rows(v_new, shape), _rows(q, shape), _p(out), _p(lse),
-                                      _DEFAULT_SCALE if scale is None else scale, n_reserve, _stream(self, stream))
+        rc = self._decode_step(self._decode_step_fn, self.handle and self.handle.value, self.S, self.device_index, layer, k_new, v_new, q, out,
+                               lse, _DEFAULT_SCALE if scale is None else scale, n_reserve, None if stream is None else stream.cuda_stream)
         if rc:
             _check("kvE_decode_step", rc, self.handle)
         return out

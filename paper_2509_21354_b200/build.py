@@ -10,14 +10,37 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libkve.so")
+BIND = os.path.join(HERE, "_kve_bind.so")      # the decode step's call from Python (csrc/bind.cpp)
 SOURCES = ["api.cu", "append.cu", "summarize.cu", "summarize_token.cu", "gate_proj.cu", "gate_rnn.cu", "gate_step.cu", "compact.cu", "attn.cu", "attn_block.cu", "attn_block_tc.cu", "selftest.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xptxas", "-v"]
 
 
 def _deps_mtime() -> float:
-    files = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(HERE, "..", "include", "kve.h")]
+    files = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if not f.endswith(".cpp")] + [os.path.join(HERE, "..", "include", "kve.h")]
     return max(os.path.getmtime(f) for f in files)
+
+
+def build_bind(force: bool = False) -> str:
+    """Compiles csrc/bind.cpp (an extension module against this interpreter and this torch; no device code)."""
+    src = os.path.join(CSRC, "bind.cpp")
+    if not force and os.path.exists(BIND) and os.path.getmtime(BIND) >= os.path.getmtime(src):
+        return BIND
+    import sysconfig
+    import torch
+    root = os.path.join(os.path.dirname(torch.__file__))
+    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+    include = [sysconfig.get_paths()["include"], os.path.join(root, "include"),
+               os.path.join(root, "include", "torch", "csrc", "api", "include"), os.path.join(cuda, "include")]
+    tmp = f"{BIND}.{os.getpid()}"
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+           *[f"-I{d}" for d in include], src, "-o", tmp, "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        sys.stderr.write(r.stderr)
+        raise RuntimeError("g++ failed on bind.cpp")
+    os.replace(tmp, BIND)
+    return BIND
 
 
 def build(force: bool = False, verbose: bool = False, defines=(), lib: str = LIB, obj_dir: str = OBJ) -> str:
@@ -53,3 +76,4 @@ def build(force: bool = False, verbose: bool = False, defines=(), lib: str = LIB
 
 if __name__ == "__main__":
     print(build(force="--force" in sys.argv, verbose="--verbose" in sys.argv))
+    print(build_bind(force="--force" in sys.argv))

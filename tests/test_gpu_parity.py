@@ -1397,3 +1397,33 @@ def test_refresh_with_means_beside_the_recurrence_equals_the_stepwise_calls(agg,
         torch.cuda.synchronize()
         assert st.poll_status() == -3
         assert bool((st.ksum_f32[0, 3, N - 1] == 7.0).all()) and torch.equal(st.ksum_f32[0, 4:], want[0][0, 4:])
+
+
+def test_decode_step_call_checks_its_tensors_and_takes_a_stream():
+    b = _binding()
+    wl = wlm.CFG1.small(n=300, n_append=2, seed=4)
+    K, V = wlm.gen_kv(wl)
+    k, v = (b.bits_to_bf16(x).reshape(wl.S, 128) for x in wlm.gen_new_tokens(wl))
+    q = b.bits_to_bf16(wlm.gen_q(wl))
+    outs = []
+    for use_stream in (False, True):
+        st = make_store(wl)
+        load_kv(st, 0, K, V)
+        for bad in (q.float(), q[:, :64], q[:-1], q.t().contiguous().t(), q.cpu(), q.reshape(-1)):
+            with pytest.raises(AssertionError):
+                st.decode_step(0, bad, v, q)
+            with pytest.raises(AssertionError):
+                st.decode_step(0, k, v, bad)
+        with pytest.raises(AssertionError):
+            st.decode_step(0, k, v, q, q.clone().cpu())
+        with pytest.raises(TypeError):
+            st.decode_step(0, k.data_ptr(), v, q)
+        with pytest.raises(b.KveError):
+            st.decode_step(1, k, v, q)                    # one layer only
+        lse = torch.zeros(wl.S, device="cuda")
+        torch.cuda.synchronize()
+        side = torch.cuda.Stream()
+        outs.append((st.decode_step(0, k, v, q, lse=lse, scale=0.1, n_reserve=1, stream=side if use_stream else None), lse))
+        torch.cuda.synchronize()
+        assert st.poll_status() == 0 and st.layer_state()["n_tokens"] == 301
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
