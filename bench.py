@@ -426,9 +426,7 @@ class Rig:
         st, wl = self.st, self.wl
         st.set_len(0, self.n0 - 1)
         st.append(0, self.k3, self.v3)
-        st.summarize_chunks(0, 0, self.Nc, self.aw)
-        st.gate(0, 0, self.Nc, self.lw)
-        st.compact(0, wl.tau)
+        st.refresh(0, self.aw, self.lw, wl.tau)
         st.decode_attn(0, self.q, self.out)
 
     def step_steady(self):

@@ -109,7 +109,7 @@ typedef struct {
 
 typedef struct kvE_store kvE_store;
 
-/* Bytes of workspace the handle needs: the gate projection buffer and the h_t rows of one kvE_gate call, the split-K partial records and tickets of
+/* Bytes of workspace the handle needs: the gate projection buffer and the score's partial sums of one kvE_gate call, the split-K partial records and tickets of
  * the attention kernels (those of kvE_decode_attn_block only when cfg.max_query_tokens > 0), staging rows of the
  * host-buffer step, scratch of kvE_reclaim_pages.  0 if the geometry is not supported. */
 size_t kvE_workspace_bytes(const kvE_config* cfg);
@@ -299,11 +299,11 @@ int kvE_decode_attn_block(kvE_store* st, int layer, const void* q, int n_query_t
 int kvE_decode_attn_static(kvE_store* st, int layer, const void* q, void* out, float* lse, float scale,
                            void* stream);
 
-/* One whole decode step of `layer` from HOST memory: copies k_new, v_new, q (bf16 [S][d] each,
- * ideally pinned) to the device, appends the token, brings summaries, gate and keep list up to
+/* One whole decode step of `layer` from HOST memory: takes k_new, v_new, q (bf16 [S][d] each; pinned buffers that the
+ * device can address are read in place by the kernels, others are copied) to the device, appends the token, brings summaries, gate and keep list up to
  * date for every chunk that has left the window (from scratch, through kvE_refresh, if `from_scratch` != 0), runs
- * kvE_decode_attn and copies out (bf16 [S][d]) back to host memory.  Staging uses the tail of the
- * workspace.  Waits for the stream before returning. */
+ * kvE_decode_attn and brings out (bf16 [S][d]) back to host memory (pinned: written by attention itself).  Staging uses
+ * the tail of the workspace.  Waits for the stream before returning. */
 int kvE_decode_step_host(kvE_store* st, int layer, const void* k_new_host, const void* v_new_host,
                          const void* q_host, void* out_host, const kvE_agg_weights* aw,
                          const kvE_lstm_weights* lw, float tau, float scale, int from_scratch,
@@ -328,7 +328,8 @@ int kvE_layer_state(const kvE_store* st, int layer, int* n_tokens, int* n_summar
 /* Per-kernel timing.  While enabled, every kernel launch of this handle is bracketed by a pair of CUDA
  * events on the launch stream (events are created on the first enable; no device memory).
  * kvE_profile_read synchronises the device and writes, per kernel id, the duration in microseconds
- * of that kernel's most recent launch, or -1 if it has not run since profiling was enabled. */
+ * of that kernel's most recent launch, or -1 if it has not run since profiling was enabled.  While enabled,
+ * kvE_refresh takes all chunks in one range, so that a duration is that of the kernel alone. */
 enum { KVE_K_APPEND = 0, KVE_K_CHUNK_MEAN, KVE_K_CHUNK_MLP, KVE_K_GATE_PROJ, KVE_K_GATE_RNN, KVE_K_COMPACT,
        KVE_K_ATTN, KVE_K_ATTN_DENSE, KVE_K_ATTN_BLOCK, KVE_K_COUNT };
 int kvE_profile(kvE_store* st, int enable);

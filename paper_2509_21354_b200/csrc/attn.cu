@@ -34,8 +34,8 @@
 //    ticket; the CTA that draws a sequence's last ticket merges its records by log-sum-exp.  Nobody
 //    spins on another CTA.
 //  * Fused append (kvE_decode_step): the step's new token need not be in its page yet.  Its row is streamed from the
-//    caller's buffer as the last row of the raw tail, the CTA that streams it also stores it in the page, and the last
-//    CTA to finish advances the stored length: one launch per decode step and layer instead of two.
+//    caller's buffer as the last row of the raw tail, the CTA that streams it also stores it in the page, and the stored
+//    length is advanced once every CTA has read the old one: one launch per decode step and layer instead of two.
 // Every mbarrier wait is bounded; on give-up the status word gets KVE_ERR_TIMEOUT.
 #include "common.cuh"
 #include "kernels.h"

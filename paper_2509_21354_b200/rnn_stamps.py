@@ -20,7 +20,7 @@ if ROOT not in sys.path:
 from paper_2509_21354_b200 import build as kb  # noqa: E402
 
 PHASES = ["wait for the peers' h (mbarrier)", "ldmatrix + MMA chain (W_hh h)", "prefetch of the next step's P",
-          "cell update + plane split", "send h (staging, fence, bulk copies, arrive)",
+          "cell update + plane split", "send h (planes, fence, bulk copies, arrive)",
           "round to round (P_{t+1} lands in place, expect_tx)"]
 SLOTS = [6, 0, 1, 2, 3, 4]
 
