@@ -1390,6 +1390,17 @@ def test_refresh_with_means_beside_the_recurrence_equals_the_stepwise_calls(agg,
         assert st.poll_status() == 0
         for got, ref in zip(state(), want):
             assert torch.equal(got, ref)
+    graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()      # the same from a replayed graph
+    with torch.cuda.stream(side), torch.cuda.graph(graph, stream=side):
+        st.refresh(0, aw, lw, 0.5)
+    for _ in range(2):
+        for t in (st.ksum_f32, st.vsum_f32, st.ksum_bf16, st.vsum_bf16, st.scores, st.lstm_h, st.lstm_c):
+            t.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert st.poll_status() == 0
+        for got, ref in zip(state(), want):
+            assert torch.equal(got, ref)
     if agg != "mlp":
         st.ksum_f32[0, 3, N - 1] = 7.0
         st.page_table[0, 3, N - 1] = -1
