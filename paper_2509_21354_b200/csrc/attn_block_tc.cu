@@ -45,12 +45,13 @@ constexpr int TC_OFF_Q = 0;
 constexpr int TC_OFF_P = TC_OFF_Q + TC_Q_BYTES;
 constexpr int TC_OFF_RING = TC_OFF_P + 2 * TC_PLANES * TC_P_BYTES;
 constexpr int TC_OFF_BAR = TC_OFF_RING + TC_STAGES * BK_STAGE_BYTES;
-constexpr int TC_N_BARS = 2 * TC_STAGES + 8;
+constexpr int TC_N_BARS = 2 * TC_STAGES + 10;
 constexpr int TC_OFF_MISC = TC_OFF_BAR + TC_N_BARS * 8;            // tensor-memory base, ticket flag
-constexpr int TC_SMEM_BYTES = TC_OFF_MISC + 16;                    // 224 KB: everything an SM has, so no alignment slack;
+constexpr int TC_OFF_MX = TC_OFF_MISC + 16;                        // [2 tile parities][2 groups][128 lanes] column maxima
+constexpr int TC_SMEM_BYTES = TC_OFF_MX + 4 * 128 * 4;             // 226.2 KB: everything an SM has, so no alignment slack;
                                                                    // the kernel checks that the base is 1024-byte aligned
-constexpr int TC_OFF_REFS = 2 * 128 * BK_REC * 4;                  // final merge: the lanes' references, behind their records
-static_assert(TC_OFF_REFS + 2 * 128 * 4 <= TC_OFF_BAR, "the areas of the final merge lie in the Q / P / ring region");
+constexpr int TC_OFF_L = 128 * BK_REC * 4;                         // [2 groups][128 lanes] partial row sums, behind the exchange
+                                                                   // area of the final merge (both valid once the ring is free)
 static_assert(TC_SMEM_BYTES <= 227 * 1024, "shared memory of one CTA");
 constexpr int TC_THREADS = 320;
 constexpr int TC_TMEM_COLS = 512;                  // O of the two groups: 2 x 128 columns, then S: two buffers of 64
@@ -80,8 +81,11 @@ kve_decode_attn_block_tc_kernel(const __grid_constant__ CUtensorMap tmK, const _
   uint64_t* s_free = s_full + 2;            // [2] S buffer read by the four warps of its softmax group
   uint64_t* p_full = s_free + 2;            // [2] P buffer written by the four warps of its softmax group
   uint64_t* pv_done = p_full + 2;           // [2] O += P V of the buffer's tile complete (MMA commit)
+  uint64_t* mx_full = pv_done + 2;          // [2] the group's four warps have posted their column maxima
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + TC_OFF_MISC);
   int* flag = reinterpret_cast<int*>(tmem_slot + 1);
+  float* mx_x = reinterpret_cast<float*>(smem + TC_OFF_MX);
+  float* l_x = reinterpret_cast<float*>(smem + TC_OFF_L);      // valid only after the tile loops
 
   pdl_launch_dependents();
   const LayerView& v = a.v;
@@ -109,6 +113,7 @@ kve_decode_attn_block_tc_kernel(const __grid_constant__ CUtensorMap tmK, const _
       mbar_init(&s_free[i], 4);       // one arrival per warp of the group (an arrival per thread would
       mbar_init(&p_full[i], 4);       // serialise 128 updates of one shared-memory word)
       mbar_init(&pv_done[i], 1);
+      mbar_init(&mx_full[i], 4);
     }
     mbar_fence_init();
   }
@@ -217,17 +222,16 @@ kve_decode_attn_block_tc_kernel(const __grid_constant__ CUtensorMap tmK, const _
     // Tensor-memory lane L carries query row L % RB, RB = 128 / REP: with few query rows the block is
     // replicated REP times down the 128 lanes (the tensor core computes all 128 rows of S anyway) and
     // replica L / RB works on its own CW = 64 / REP columns of every tile, so a tile's softmax is spread
-    // over all four warps of the group (one per scheduler) instead of sitting on one.  Replicas are independent queries
-    // over their own columns: own m_ref, own sum, own row of P (zero in the other replicas' columns, once and for all)
-    // and own row of O - the product computes all 128 rows in any case - and are merged at the end.  (With one row of P
-    // and O per query the replicas had to agree on the maximum, an exchange through shared memory and a barrier per
-    // tile: 22.0 us on 128 sequences x 1084 rows, 21.4 us now together with the earlier look-ups.)
+    // over all four warps of the group (one per scheduler) instead of sitting on one.  The replicas
+    // of a row exchange their column maxima through shared memory once per tile, keep identical
+    // m_ref, write their columns of P into the row of replica 0, and add up their sums at the end.
     constexpr int RB = 128 / REP, CW = 64 / REP;
     const int group = (warp - 2) >> 2;                  // 0: even tiles, 1: odd tiles
     const int quarter = warp & 3;                       // the lanes a warp may touch follow from its index
     const int L = quarter * 32 + lane;
     const int row = L % RB, rep = L / RB;
     const bool warp_active = (quarter * 32) % RB < a.R; // some lane of this warp carries a real query row
+    const bool owns_o = warp_active && rep == 0;        // rows of O live in the lanes of replica 0
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
     const uint32_t my_o = tmem_o + lane_addr + group * 128, my_s = tmem_s + lane_addr + group * 64 + rep * CW;
     const float sl2 = a.scale * 1.44269504088896340736f;   // logits in log2 units
@@ -275,12 +279,22 @@ kve_decode_attn_block_tc_kernel(const __grid_constant__ CUtensorMap tmK, const _
         mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
         if (plain) mx *= sl2;
       }
+      if (REP > 1) {
+        // the row's maximum over all replicas' columns (buffers alternate, one barrier phase per tile)
+        float* slot = mx_x + ((j & 1) * 2 + group) * 128;
+        slot[L] = mx;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&mx_full[group]);
+        if (!warp_wait(&mx_full[group], j & 1)) { alive = false; break; }
+#pragma unroll
+        for (int r2 = 0; r2 < REP; ++r2) mx = fmaxf(mx, slot[row + r2 * RB]);
+      }
       if (warp_active) {
         if (__any_sync(0xffffffffu, mx > m_ref + TC_RESCALE_STEP)) {      // m_ref = -inf on the group's first tile
           const float m_new = fmaxf(m_ref, mx);
           if (j > 0) {
             const float f = (m_ref == -INFINITY) ? 0.f : ex2_fast(m_ref - m_new);      // nothing accumulated yet: O row is 0
-            {
+            if (owns_o) {
               // O holds this group's earlier tiles once their last product is complete; rescale this warp's rows
               if (!warp_wait(&pv_done[b], (j + 1) & 1)) { alive = false; break; }
               umma::fence_after_sync();
@@ -311,7 +325,7 @@ kve_decode_attn_block_tc_kernel(const __grid_constant__ CUtensorMap tmK, const _
       }
       if (j > 0 && !warp_wait(&pv_done[b], (j + 1) & 1)) { alive = false; break; }   // P buffer b is free
       if (warp_active) {
-        unsigned char* prow = Ps + (b * TC_PLANES) * TC_P_BYTES + L * 128;
+        unsigned char* prow = Ps + (b * TC_PLANES) * TC_P_BYTES + row * 128;
         float l4[4] = {0.f, 0.f, 0.f, 0.f};
         // (a row that has not seen a single column yet has m_ref = -inf: its p are 0, not exp2(-inf + inf))
         const float neg_m = (m_ref == -INFINITY) ? 0.f : -m_ref, mul = plain ? sl2 : 1.f;      // the masked path has stored s * sl2 already
@@ -330,7 +344,7 @@ kve_decode_attn_block_tc_kernel(const __grid_constant__ CUtensorMap tmK, const _
           lo.y = pack_bf16x2(p[2] - bf16lo(hi.y), p[3] - bf16hi(hi.y));
           lo.z = pack_bf16x2(p[4] - bf16lo(hi.z), p[5] - bf16hi(hi.z));
           lo.w = pack_bf16x2(p[6] - bf16lo(hi.w), p[7] - bf16hi(hi.w));
-          const int off = ((rep * (CW / 8) + c) ^ (L & 7)) << 4;
+          const int off = ((rep * (CW / 8) + c) ^ (row & 7)) << 4;
           *reinterpret_cast<uint4*>(prow + off) = hi;
           if (TC_PLANES == 2) *reinterpret_cast<uint4*>(prow + TC_P_BYTES + off) = lo;
         }
@@ -342,56 +356,80 @@ kve_decode_attn_block_tc_kernel(const __grid_constant__ CUtensorMap tmK, const _
       last_tile = i;
     }
 
-    // ---- the lanes' results (m_ref, l, O), merged per query row: everybody learns the row's common reference, brings its own
-    // record to it on the way out of tensor memory, and the records are added up ----
+    // ---- the group's result (m_ref, l, O); the odd group hands its rows over through shared memory ----
     if (alive && last_tile >= 0) alive = warp_wait(&pv_done[group], (last_tile >> 1) & 1);
     umma::fence_after_sync();
     // every product of BOTH groups has completed after this barrier (or the CTA has given up): Q, P and the
-    // ring are free
-    float* xch = reinterpret_cast<float*>(smem);      // [2 groups][128 lanes][BK_REC]: O, and at 129 the sum
-    float* refs = reinterpret_cast<float*>(smem + TC_OFF_REFS);      // [2 groups][128 lanes]
-    const bool any = last_tile >= 0 && alive;
+    // ring are free.  Exchange areas: [128 rows][BK_REC] fp32 from the start of shared memory, the
+    // replicas' partial row sums behind it
+    float* xch = reinterpret_cast<float*>(smem);
+    static_assert(TC_OFF_L + 2 * 128 * 4 <= TC_OFF_BAR, "exchange areas lie in the Q / P / ring region");
     asm volatile("bar.sync 1, 256;" ::: "memory");
-    refs[group * 128 + L] = any ? m_ref : -INFINITY;
+    l_x[group * 128 + L] = l_run;
     asm volatile("bar.sync 1, 256;" ::: "memory");
-    auto common_ref = [&](int r) {
-      float m = -INFINITY;
+    float l_tot = 0.f;
 #pragma unroll
-      for (int k = 0; k < 2 * REP; ++k) m = fmaxf(m, refs[(k / REP) * 128 + (k % REP) * RB + r]);
-      return m;
-    };
-    if (warp_active) {
-      float* mine = xch + (group * 128 + L) * BK_REC;
-      const float f = (any && m_ref != -INFINITY) ? exp2f(m_ref - common_ref(row)) : 0.f;
+    for (int r2 = 0; r2 < REP; ++r2) l_tot += l_x[group * 128 + row + r2 * RB];
+    if (group == 1 && owns_o) {
+      float* mine = xch + row * BK_REC;
 #pragma unroll 1
       for (int c = 0; c < 4; ++c) {
         float o[32];
-        if (any) umma::tmem_ld32(my_o + c * 32, o);
+        if (last_tile >= 0 && alive) umma::tmem_ld32(my_o + c * 32, o);
+        else {
+#pragma unroll
+          for (int x = 0; x < 32; ++x) o[x] = 0.f;
+        }
 #pragma unroll
         for (int x = 0; x < 32; x += 4)
-          *reinterpret_cast<float4*>(mine + c * 32 + x) = f != 0.f ? make_float4(o[x] * f, o[x + 1] * f, o[x + 2] * f, o[x + 3] * f) : make_float4(0.f, 0.f, 0.f, 0.f);
+          *reinterpret_cast<float4*>(mine + c * 32 + x) = make_float4(o[x], o[x + 1], o[x + 2], o[x + 3]);
       }
-      mine[129] = l_run * f;
+      mine[128] = (last_tile >= 0 && alive) ? m_ref : -INFINITY;
+      mine[129] = l_tot;
     }
     asm volatile("bar.sync 1, 256;" ::: "memory");
-#pragma unroll 2
-    for (int it = (warp - 2) * 32 + lane; it < a.R * 32; it += 256) {
-      const int r = it >> 5, c4 = it & 31;
-      float lC = 0.f;
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (group == 0 && owns_o && alive) {
+      const float* other = xch + row * BK_REC;
+      const float m1 = other[128], l1 = other[129];
+      const float m0 = (last_tile >= 0) ? m_ref : -INFINITY;
+      const float mC = fmaxf(m0, m1);
+      const float f0 = (m0 == -INFINITY) ? 0.f : exp2f(m0 - mC), f1 = (m1 == -INFINITY) ? 0.f : exp2f(m1 - mC);
+      const float lC = l_tot * f0 + l1 * f1;
+      const bool direct = gm.n_splits == 1;
+      const float inv = (lC > 0.f) ? 1.f / lC : 0.f;
+      float* rec = a.partials + (((long long)s * a.max_splits + split) * a.rec_rows + row) * BK_REC;
+      const long long off = q_row_offset(a, s, min(row, a.R - 1));
+#pragma unroll 1
+      for (int c = 0; c < 4; ++c) {
+        float o[32];
+        if (last_tile >= 0) umma::tmem_ld32(my_o + c * 32, o);
 #pragma unroll
-      for (int k = 0; k < 2 * REP; ++k) {
-        const float* rec = xch + ((k / REP) * 128 + (k % REP) * RB + r) * BK_REC;
-        const float4 o = *reinterpret_cast<const float4*>(rec + c4 * 4);
-        lC += rec[129];
-        acc.x += o.x; acc.y += o.y; acc.z += o.z; acc.w += o.w;
+        for (int x = 0; x < 32; ++x) {
+          const float o0 = (last_tile >= 0) ? o[x] * f0 : 0.f;
+          o[x] = (f1 != 0.f) ? fmaf(other[c * 32 + x], f1, o0) : o0;
+        }
+        if (row < a.R) {
+          if (direct) {
+#pragma unroll
+            for (int x = 0; x < 32; x += 8) {
+              uint4 w;
+              w.x = pack_bf16x2(o[x] * inv, o[x + 1] * inv); w.y = pack_bf16x2(o[x + 2] * inv, o[x + 3] * inv);
+              w.z = pack_bf16x2(o[x + 4] * inv, o[x + 5] * inv); w.w = pack_bf16x2(o[x + 6] * inv, o[x + 7] * inv);
+              *reinterpret_cast<uint4*>(a.out + off + c * 32 + x) = w;
+            }
+          } else {
+#pragma unroll
+            for (int x = 0; x < 32; x += 4)
+              *reinterpret_cast<float4*>(rec + c * 32 + x) = make_float4(o[x], o[x + 1], o[x + 2], o[x + 3]);
+          }
+        }
       }
-      if (gm.n_splits == 1) {
-        write_block_out(a, s, r, c4, acc, common_ref(r), lC);
-      } else {
-        float* rec = a.partials + (((long long)s * a.max_splits + split) * a.rec_rows + r) * BK_REC;
-        *reinterpret_cast<float4*>(rec + c4 * 4) = acc;
-        if (c4 == 0) *reinterpret_cast<float2*>(rec + 128) = make_float2(common_ref(r), lC);
+      if (row < a.R) {
+        if (direct) {
+          if (a.lse) a.lse[off / D] = (lC > 0.f) ? (mC + log2f(lC)) * 0.69314718055994530942f : -INFINITY;
+        } else {
+          *reinterpret_cast<float2*>(rec + 128) = make_float2(mC, lC);
+        }
       }
     }
     umma::fence_before_sync();

@@ -299,3 +299,29 @@ def test_block_attention_random_geometries(seed):
         causal = False                      # the oracle's causal form wants the block's tokens inside the raw tail
     _check(b, pb, st, attend, G, T, causal=causal)
     _check(b, pb, st, attend, G, T, dense=True, step=1, causal=causal)
+
+
+@pytest.mark.parametrize("G,T", [(4, 1), (4, 7), (8, 8), (8, 16)])
+@pytest.mark.parametrize("dense", [False, True])
+def test_block_attention_keeps_infinite_values_and_nan_keys_where_they_belong(dense, G, T):
+    """One element of V is infinite: that output element of every query of its KV sequence is infinite (its weight is
+    positive, nothing else about the sum is) and no other one is touched.  Sixteen keys in a row of another sequence are NaN, a quarter of
+    a tile's columns: every output of that KV sequence is NaN."""
+    wl = wlm.CFG1.small(B=1, H=3, n=2443, W=300, seed=22)
+    b, pb, st = _prepared(wl, "summary", G, T)
+    q = b.bits_to_bf16(wlm.gen_q_block(wl, T, wl.H * G, 0, 0))
+    plain = st.decode_attn_block(0, q, dense=dense).float()
+    pages = st.page_table[0].long()
+    tok = wl.n - 40                                      # in the raw tail
+    st.v_pages[pages[0, tok // wl.C], tok % wl.C, 5] = float("inf")
+    st.k_pages[pages[2, wl.n // wl.C - 1], 16:32] = float("nan")
+    lse = torch.zeros((1, T, wl.H * G), dtype=torch.float32, device="cuda")
+    out = st.decode_attn_block(0, q, dense=dense, lse=lse).float().reshape(T, wl.H, G, 128)
+    plain = plain.reshape(T, wl.H, G, 128)
+    assert st.poll_status() == 0
+    assert torch.isposinf(out[:, 0, :, 5]).all()
+    others = torch.ones(128, dtype=torch.bool, device="cuda")
+    others[5] = False
+    assert torch.equal(out[:, 0][..., others], plain[:, 0][..., others]) and torch.equal(out[:, 1], plain[:, 1])
+    assert torch.isnan(out[:, 2]).all()
+    assert torch.isfinite(lse.reshape(T, wl.H, G)[:, :2]).all()
