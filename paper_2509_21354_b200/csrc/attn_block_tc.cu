@@ -50,7 +50,7 @@ constexpr int TC_OFF_MISC = TC_OFF_BAR + TC_N_BARS * 8;            // tensor-mem
 constexpr int TC_OFF_MX = TC_OFF_MISC + 16;                        // [2 tile parities][2 groups][128 lanes] column maxima
 constexpr int TC_SMEM_BYTES = TC_OFF_MX + 4 * 128 * 4;             // 226.2 KB: everything an SM has, so no alignment slack;
                                                                    // the kernel checks that the base is 1024-byte aligned
-constexpr int TC_OFF_L = 128 * BK_REC * 4;                         // [2 groups][128 lanes] partial row sums, behind the exchange
+constexpr int TC_OFF_L = 2 * 128 * BK_REC * 4;                     // [2 groups][128 lanes] partial row sums, behind the exchange
                                                                    // area of the final merge (both valid once the ring is free)
 static_assert(TC_SMEM_BYTES <= 227 * 1024, "shared memory of one CTA");
 constexpr int TC_THREADS = 320;
@@ -356,26 +356,33 @@ kve_decode_attn_block_tc_kernel(const __grid_constant__ CUtensorMap tmK, const _
       last_tile = i;
     }
 
-    // ---- the group's result (m_ref, l, O); the odd group hands its rows over through shared memory ----
+    // ---- the groups' results (m_ref, l, O) meet in shared memory ----
     if (alive && last_tile >= 0) alive = warp_wait(&pv_done[group], (last_tile >> 1) & 1);
     umma::fence_after_sync();
     // every product of BOTH groups has completed after this barrier (or the CTA has given up): Q, P and the
-    // ring are free.  Exchange areas: [128 rows][BK_REC] fp32 from the start of shared memory, the
+    // ring are free.  Exchange areas: [2 groups][128 rows][BK_REC] fp32 from the start of shared memory, the
     // replicas' partial row sums behind it
     float* xch = reinterpret_cast<float*>(smem);
     static_assert(TC_OFF_L + 2 * 128 * 4 <= TC_OFF_BAR, "exchange areas lie in the Q / P / ring region");
+    const bool any = last_tile >= 0 && alive;
+    // In general all columns go to shared memory and the eight warps merge a row at a time, which leaves in whole lines (a thread
+    // per row: 0.5 to 1 us more per launch with few rows, 2 to 4 us with 128 rows and many splits).  A block of more than 64 rows
+    // that a CTA finishes by itself: every lane holds a row, the groups hand each other half of the columns and merge the rest
+    // out of tensor memory (128 rows, 128 sequences x 1084 rows 17.4 us, 18.9 the other way).
+    const bool direct = gm.n_splits == 1, halves = REP == 1 && direct;
+    const int piece0 = halves ? 2 * (1 - group) : 0, piece1 = halves ? piece0 + 2 : 4;      // 32-column pieces a group puts into shared memory
     asm volatile("bar.sync 1, 256;" ::: "memory");
     l_x[group * 128 + L] = l_run;
     asm volatile("bar.sync 1, 256;" ::: "memory");
-    float l_tot = 0.f;
+    if (owns_o) {
+      float l_tot = 0.f;
 #pragma unroll
-    for (int r2 = 0; r2 < REP; ++r2) l_tot += l_x[group * 128 + row + r2 * RB];
-    if (group == 1 && owns_o) {
-      float* mine = xch + row * BK_REC;
+      for (int r2 = 0; r2 < REP; ++r2) l_tot += l_x[group * 128 + row + r2 * RB];
+      float* mine = xch + (group * 128 + row) * BK_REC;
 #pragma unroll 1
-      for (int c = 0; c < 4; ++c) {
+      for (int c = piece0; c < piece1; ++c) {
         float o[32];
-        if (last_tile >= 0 && alive) umma::tmem_ld32(my_o + c * 32, o);
+        if (any) umma::tmem_ld32(my_o + c * 32, o);
         else {
 #pragma unroll
           for (int x = 0; x < 32; ++x) o[x] = 0.f;
@@ -384,53 +391,63 @@ kve_decode_attn_block_tc_kernel(const __grid_constant__ CUtensorMap tmK, const _
         for (int x = 0; x < 32; x += 4)
           *reinterpret_cast<float4*>(mine + c * 32 + x) = make_float4(o[x], o[x + 1], o[x + 2], o[x + 3]);
       }
-      mine[128] = (last_tile >= 0 && alive) ? m_ref : -INFINITY;
+      mine[128] = any ? m_ref : -INFINITY;
       mine[129] = l_tot;
     }
     asm volatile("bar.sync 1, 256;" ::: "memory");
-    if (group == 0 && owns_o && alive) {
-      const float* other = xch + row * BK_REC;
-      const float m1 = other[128], l1 = other[129];
-      const float m0 = (last_tile >= 0) ? m_ref : -INFINITY;
-      const float mC = fmaxf(m0, m1);
-      const float f0 = (m0 == -INFINITY) ? 0.f : exp2f(m0 - mC), f1 = (m1 == -INFINITY) ? 0.f : exp2f(m1 - mC);
-      const float lC = l_tot * f0 + l1 * f1;
-      const bool direct = gm.n_splits == 1;
+    auto merged = [&](int r, float& mC, float& f0, float& f1, float& lC) {      // even tiles (0) and odd tiles (1) of row r
+      const float *r0 = xch + r * BK_REC, *r1 = r0 + 128 * BK_REC;
+      const float m0 = r0[128], m1 = r1[128];
+      mC = fmaxf(m0, m1);
+      f0 = (m0 == -INFINITY) ? 0.f : exp2f(m0 - mC);
+      f1 = (m1 == -INFINITY) ? 0.f : exp2f(m1 - mC);
+      lC = r0[129] * f0 + r1[129] * f1;
+    };
+    float mC, f0, f1, lC;
+    if (!halves) {
+#pragma unroll 4
+      for (int it = (warp - 2) * 32 + lane; it < a.R * 32; it += 256) {
+        const int r = it >> 5, c4 = it & 31;
+        merged(r, mC, f0, f1, lC);
+        const float *r0 = xch + r * BK_REC, *r1 = r0 + 128 * BK_REC;
+        const float4 o0 = *reinterpret_cast<const float4*>(r0 + c4 * 4), o1 = *reinterpret_cast<const float4*>(r1 + c4 * 4);
+        float4 acc = make_float4(o0.x * f0, o0.y * f0, o0.z * f0, o0.w * f0);
+        if (f1 != 0.f) acc = make_float4(fmaf(o1.x, f1, acc.x), fmaf(o1.y, f1, acc.y), fmaf(o1.z, f1, acc.z), fmaf(o1.w, f1, acc.w));
+        if (direct) {
+          write_block_out(a, s, r, c4, acc, mC, lC);
+        } else {
+          float* rec = a.partials + (((long long)s * a.max_splits + split) * a.rec_rows + r) * BK_REC;
+          *reinterpret_cast<float4*>(rec + c4 * 4) = acc;
+          if (c4 == 0) *reinterpret_cast<float2*>(rec + 128) = make_float2(mC, lC);
+        }
+      }
+    } else if (owns_o) {      // (the whole warp: rows beyond the last one only write nothing)
+      merged(row, mC, f0, f1, lC);
       const float inv = (lC > 0.f) ? 1.f / lC : 0.f;
-      float* rec = a.partials + (((long long)s * a.max_splits + split) * a.rec_rows + row) * BK_REC;
+      const float* other = xch + ((1 - group) * 128 + row) * BK_REC;
       const long long off = q_row_offset(a, s, min(row, a.R - 1));
+      const bool live = row < a.R;
 #pragma unroll 1
-      for (int c = 0; c < 4; ++c) {
+      for (int c = 2 * group; c < 2 * group + 2; ++c) {
         float o[32];
-        if (last_tile >= 0) umma::tmem_ld32(my_o + c * 32, o);
+        if (any) umma::tmem_ld32(my_o + c * 32, o);
 #pragma unroll
         for (int x = 0; x < 32; ++x) {
-          const float o0 = (last_tile >= 0) ? o[x] * f0 : 0.f;
-          o[x] = (f1 != 0.f) ? fmaf(other[c * 32 + x], f1, o0) : o0;
+          const float mine = any ? o[x] : 0.f, theirs = other[c * 32 + x];
+          const float even = (group == 0 ? mine : theirs) * f0;
+          o[x] = (f1 != 0.f) ? fmaf(group == 0 ? theirs : mine, f1, even) : even;
         }
-        if (row < a.R) {
-          if (direct) {
+        if (live) {
 #pragma unroll
-            for (int x = 0; x < 32; x += 8) {
-              uint4 w;
-              w.x = pack_bf16x2(o[x] * inv, o[x + 1] * inv); w.y = pack_bf16x2(o[x + 2] * inv, o[x + 3] * inv);
-              w.z = pack_bf16x2(o[x + 4] * inv, o[x + 5] * inv); w.w = pack_bf16x2(o[x + 6] * inv, o[x + 7] * inv);
-              *reinterpret_cast<uint4*>(a.out + off + c * 32 + x) = w;
-            }
-          } else {
-#pragma unroll
-            for (int x = 0; x < 32; x += 4)
-              *reinterpret_cast<float4*>(rec + c * 32 + x) = make_float4(o[x], o[x + 1], o[x + 2], o[x + 3]);
+          for (int x = 0; x < 32; x += 8) {
+            uint4 w;
+            w.x = pack_bf16x2(o[x] * inv, o[x + 1] * inv); w.y = pack_bf16x2(o[x + 2] * inv, o[x + 3] * inv);
+            w.z = pack_bf16x2(o[x + 4] * inv, o[x + 5] * inv); w.w = pack_bf16x2(o[x + 6] * inv, o[x + 7] * inv);
+            *reinterpret_cast<uint4*>(a.out + off + c * 32 + x) = w;
           }
         }
       }
-      if (row < a.R) {
-        if (direct) {
-          if (a.lse) a.lse[off / D] = (lC > 0.f) ? (mC + log2f(lC)) * 0.69314718055994530942f : -INFINITY;
-        } else {
-          *reinterpret_cast<float2*>(rec + 128) = make_float2(mC, lC);
-        }
-      }
+      if (group == 0 && live && a.lse) a.lse[off / D] = (lC > 0.f) ? (mC + log2f(lC)) * 0.69314718055994530942f : -INFINITY;
     }
     umma::fence_before_sync();
   }
