@@ -299,10 +299,10 @@ int kvE_decode_attn_block(kvE_store* st, int layer, const void* q, int n_query_t
 int kvE_decode_attn_static(kvE_store* st, int layer, const void* q, void* out, float* lse, float scale,
                            void* stream);
 
-/* One whole decode step of `layer` from HOST memory: takes k_new, v_new, q (bf16 [S][d] each; pinned buffers that the
- * device can address are read in place by the kernels, others are copied) to the device, appends the token, brings summaries, gate and keep list up to
+/* One whole decode step of `layer` from HOST memory: takes k_new, v_new, q (bf16 [S][d] each; pinned buffers that
+ * start on 16 bytes are read in place by the kernels, others, of any alignment, are copied) to the device, appends the token, brings summaries, gate and keep list up to
  * date for every chunk that has left the window (from scratch, through kvE_refresh, if `from_scratch` != 0), runs
- * kvE_decode_attn and brings out (bf16 [S][d]) back to host memory (pinned: written by attention itself).  Staging uses
+ * kvE_decode_attn and brings out (bf16 [S][d]) back to host memory (pinned and on 16 bytes: written by attention itself).  Staging uses
  * the tail of the workspace.  Waits for the stream before returning. */
 int kvE_decode_step_host(kvE_store* st, int layer, const void* k_new_host, const void* v_new_host,
                          const void* q_host, void* out_host, const kvE_agg_weights* aw,

@@ -182,14 +182,21 @@ int stale_chunks(const kvE_config& c, int n) { return n > c.W ? (n - c.W) / c.C 
 
 bool bad_layer(const kvE_store* st, int layer) { return !st || layer < 0 || layer >= st->cfg.n_layers; }
 
-// the address under which the device reads and writes a host buffer, or null (memory that is not pinned)
-void* device_address(const void* host) {
-  cudaPointerAttributes at;
-  if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
-    cudaGetLastError();
-    return nullptr;
-  }
-  return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
+// The address under which kernels read and write a host buffer, or null where they cannot take it as it is: memory that is not
+// pinned from its first byte to its last, or that does not start on 16 bytes (their accesses are that wide; a copy does not mind)
+void* device_address(const void* host, size_t bytes) {
+  auto look_up = [](const void* p) -> char* {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    return at.type == cudaMemoryTypeHost ? static_cast<char*>(at.devicePointer) : nullptr;
+  };
+  if (reinterpret_cast<uintptr_t>(host) % 16 != 0) return nullptr;
+  char* first = look_up(host);
+  if (!first || reinterpret_cast<uintptr_t>(first) % 16 != 0) return nullptr;
+  return look_up(static_cast<const char*>(host) + bytes - 1) == first + (bytes - 1) ? first : nullptr;
 }
 
 // every launch goes to the current device: it must be the one the handle's buffers live on
@@ -751,10 +758,10 @@ static int decode_step_host(kvE_store* st, int layer, const void* k_new_host, co
   char *dk = stage, *dv = stage + row_bytes, *dq = stage + 2 * row_bytes, *dout = stage + 3 * row_bytes;
   LayerState& ls = st->layers[layer];
   if (ls.n_tokens + 1 > st->cfg.max_tokens) return KVE_ERR_CAPACITY;
-  // Pinned buffers: the append kernel fetches the three inputs across PCIe itself, and attention writes its result there.  Others:
-  // copies to and from the staging rows.
-  const void *pk = device_address(k_new_host), *pv = device_address(v_new_host), *pq = device_address(q_host);
-  void* pout = device_address(out_host);
+  // Pinned buffers on 16 bytes: the append kernel fetches the three inputs across PCIe itself, and attention writes its result
+  // there.  Others: copies to and from the staging rows.
+  const void *pk = device_address(k_new_host, row_bytes), *pv = device_address(v_new_host, row_bytes), *pq = device_address(q_host, row_bytes);
+  void* pout = device_address(out_host, row_bytes);
   const bool in_place = pk && pv && pq;
   cudaError_t e = cudaSuccess;
   int rc;

@@ -1438,3 +1438,33 @@ def test_decode_step_call_checks_its_tensors_and_takes_a_stream():
         torch.cuda.synchronize()
         assert st.poll_status() == 0 and st.layer_state()["n_tokens"] == 301
     assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+
+
+@pytest.mark.parametrize("wait", [True, False])
+@pytest.mark.parametrize("odd", [(0,), (1,), (2,), (3,), (0, 1, 2, 3)])
+def test_decode_step_host_takes_pinned_buffers_of_any_alignment(odd, wait):
+    """A pinned view that starts on an odd element (or on 8 bytes) is copied, not read 16 bytes at a time by the kernels: same
+    result as from aligned buffers, whichever of k, v, q and out it is."""
+    b = _binding()
+    wl = wlm.CFG1.small(n=700, seed=11)
+    K, V = wlm.gen_kv(wl)
+    q = wlm.gen_q(wl)
+    lw = b.LstmWeights(wlm.gen_lstm_weights(wl))
+    results = []
+    for shift in (0, 1, 4):                    # elements: aligned, 2 bytes, 8 bytes
+        st = make_store(wl)
+        load_kv(st, 0, K[:, :-1], V[:, :-1])
+        bufs = []
+        for i, bits in enumerate((K[:, -1], V[:, -1], q, np.zeros_like(q))):
+            at = shift if i in odd else 0
+            slab = torch.zeros(wl.S * 128 + 8, dtype=torch.bfloat16).pin_memory()
+            view = slab[at:at + wl.S * 128].view(wl.S, 128)
+            view.copy_(b.bits_to_bf16(np.ascontiguousarray(bits), "cpu"))
+            assert view.is_pinned() and view.data_ptr() % 16 == 2 * at
+            bufs.append((view, slab))
+        st.decode_step_host(0, *(v for v, _ in bufs), None, lw, 0.5, from_scratch=True, wait=wait)
+        torch.cuda.synchronize()
+        assert st.poll_status() == 0
+        results.append(bufs[3][0].clone())
+    assert results[0].float().abs().max() > 0
+    assert torch.equal(results[0], results[1]) and torch.equal(results[0], results[2])
