@@ -69,7 +69,8 @@ typedef struct {
 
 /* max_chunks = ceil(max_tokens / C) is the chunk stride of every per-chunk array below. */
 
-/* Caller-owned DEVICE buffers. */
+/* Caller-owned DEVICE buffers.  Pages and summaries start on 16 bytes (kvE_create refuses others with KVE_ERR_ARG), and so does
+ * lstm_h where kvE_gate_next or kvE_refresh_next are used. */
 typedef struct {
   void* k_pages;        /* bf16 [n_pages][C][d]: one page = one chunk of one (layer, b, h) */
   void* v_pages;        /* bf16 [n_pages][C][d] */

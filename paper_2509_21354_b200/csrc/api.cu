@@ -308,6 +308,9 @@ int kvE_create(const kvE_config* cfg, const kvE_buffers* buf, kvE_store** out) {
       !buf->vsum_f32 || !buf->ksum_bf16 || !buf->vsum_bf16 || !buf->scores || !buf->keep_idx || !buf->keep_cnt ||
       !buf->lstm_h || !buf->lstm_c || !buf->workspace || !buf->status_word || buf->n_pages <= 0)
     return KVE_ERR_ARG;
+  // what the kernels access 16 bytes at a time
+  for (const void* p : {buf->k_pages, buf->v_pages, (void*)buf->ksum_f32, (void*)buf->vsum_f32, buf->ksum_bf16, buf->vsum_bf16})
+    if (reinterpret_cast<uintptr_t>(p) % 16 != 0) return KVE_ERR_ARG;
   const Carve k = carve(*cfg);
   if (buf->workspace_bytes < k.total) return KVE_ERR_CAPACITY;
   if (reinterpret_cast<uintptr_t>(buf->workspace) % ALIGN != 0) return KVE_ERR_ARG;

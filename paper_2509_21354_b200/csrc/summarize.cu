@@ -374,17 +374,28 @@ constexpr int MT_TMEM_COLS = 512;      // H halves: columns 0 and 128; Y: 256; a
 constexpr int MT_TMEM_YLO = 0;         // POOLED: sum of the two small planes, where H would be
 constexpr int MT_TMEM_Y = 256, MT_TMEM_ACT = 384, MT_ACT_COLS = 3 * MT_SLICE / 2;
 
-// 8 consecutive floats with one 32-byte access (a whole sector)
-__device__ __forceinline__ void load8(const float* p, float (&x)[8]) {
-  asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]), "=f"(x[4]), "=f"(x[5]), "=f"(x[6]), "=f"(x[7])
-               : "l"(p)
-               : "memory");
+// 8 consecutive floats: one 32-byte access (a whole sector) where the array starts on such a boundary, two of 16 bytes otherwise
+__device__ __forceinline__ void load8(const float* p, float (&x)[8], bool wide) {
+  if (wide) {
+    asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]), "=f"(x[4]), "=f"(x[5]), "=f"(x[6]), "=f"(x[7])
+                 : "l"(p)
+                 : "memory");
+  } else {
+    const float4 lo = *reinterpret_cast<const float4*>(p), hi = *reinterpret_cast<const float4*>(p + 4);
+    x[0] = lo.x; x[1] = lo.y; x[2] = lo.z; x[3] = lo.w;
+    x[4] = hi.x; x[5] = hi.y; x[6] = hi.z; x[7] = hi.w;
+  }
 }
-__device__ __forceinline__ void store8(float* p, const float (&x)[8]) {
-  asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]), "f"(x[4]),
-               "f"(x[5]), "f"(x[6]), "f"(x[7])
-               : "memory");
+__device__ __forceinline__ void store8(float* p, const float (&x)[8], bool wide) {
+  if (wide) {
+    asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]), "f"(x[4]),
+                 "f"(x[5]), "f"(x[6]), "f"(x[7])
+                 : "memory");
+  } else {
+    *reinterpret_cast<float4*>(p) = make_float4(x[0], x[1], x[2], x[3]);
+    *reinterpret_cast<float4*>(p + 4) = make_float4(x[4], x[5], x[6], x[7]);
+  }
 }
 // splits 8 consecutive fp32 values and stores the three 16-byte pieces at dst + pl * plane_stride
 __device__ __forceinline__ void store_split8(const float (&x)[8], unsigned char* dst, int plane_stride) {
@@ -500,8 +511,8 @@ __global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerVi
 #pragma unroll
             for (int e = 0; e < 16; ++e) h[e] = 0.f;
             if (unit < n_units) {
-              load8(src, reinterpret_cast<float(&)[8]>(h[0]));
-              load8(src + 8, reinterpret_cast<float(&)[8]>(h[8]));
+              load8(src, reinterpret_cast<float(&)[8]>(h[0]), true);      // (workspace)
+              load8(src + 8, reinterpret_cast<float(&)[8]>(h[8]), true);
             }
           } else {
             umma::tmem_ld16(tmem + hb * 128 + (j & 3) * MT_SLICE + q * 16 + lane_bits, h);
@@ -537,6 +548,7 @@ __global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerVi
   } else if (warp < MT_MMA_WARP) {
     // ================= means in, summaries out =================
     const int c0 = ((warp - MT_GELU_WARPS) >> 2) * 64;      // this thread's 64 columns of its row: K-block c0 / 64
+    const bool wide = (reinterpret_cast<uintptr_t>(sum_f32) & 31) == 0;      // the caller's buffer: 16 bytes are enough
     // a thread keeps its 32-byte column and walks down 8 rows, so that a warp's load covers whole rows
     const int io = tid - MT_GELU_WARPS * 32, pc = io & 15;
     for (int k = POOLED ? 0 : -1; k < my_tiles && ok; ++k) {      // round k: the means of tile k + 1 in, then the summaries of tile k out
@@ -548,7 +560,7 @@ __global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerVi
           const int unit = unit0 + 16 * i;
 #pragma unroll
           for (int e = 0; e < 8; ++e) x[i][e] = 0.f;
-          if (unit < n_units) load8(sum_f32 + summary_row(unit) * D + pc * 8, x[i]);
+          if (unit < n_units) load8(sum_f32 + summary_row(unit) * D + pc * 8, x[i], wide);
         }
         if (k >= 0) ok = __all_sync(0xffffffffu, mbar_wait_bounded(a_free, (uint32_t)(k & 1)));
         if (!ok) break;
@@ -586,7 +598,7 @@ __global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerVi
           float z[8];
 #pragma unroll
           for (int e = 0; e < 8; ++e) z[e] = y[q >> 2][(q & 3) * 8 + e] + b2s[c0 + q * 8 + e];
-          store8(sum_f32 + o + q * 8, z);
+          store8(sum_f32 + o + q * 8, z, wide);
           *reinterpret_cast<uint4*>(sum_b16 + o + q * 8) =
               make_uint4(pack_bf16x2(z[0], z[1]), pack_bf16x2(z[2], z[3]), pack_bf16x2(z[4], z[5]), pack_bf16x2(z[6], z[7]));
         }

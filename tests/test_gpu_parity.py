@@ -1468,3 +1468,34 @@ def test_decode_step_host_takes_pinned_buffers_of_any_alignment(odd, wait):
         results.append(bufs[3][0].clone())
     assert results[0].float().abs().max() > 0
     assert torch.equal(results[0], results[1]) and torch.equal(results[0], results[2])
+
+
+@pytest.mark.parametrize("agg,d_sum", [("mlp", 256), ("mlp", 64), ("token_mlp", 128)])
+def test_summary_buffers_on_16_byte_boundaries(agg, d_sum):
+    """Summaries that start on 16 but not on 32 bytes, as an arena hands them out: the same values, bit for bit."""
+    import ctypes as C
+    b = _binding()
+    wl = wlm.CFG1.small(B=1, H=5, n=1100, C=32, agg=agg, d_sum=d_sum, seed=12)
+    K, V = wlm.gen_kv(wl)
+    aw, lw = b.AggWeights(wlm.gen_mlp_weights(wl)), b.LstmWeights(wlm.gen_lstm_weights(wl))
+    got = []
+    for shift in (0, 4):                       # floats
+        st = make_store(wl)
+        if shift:
+            for name in ("ksum_f32", "vsum_f32"):
+                old = getattr(st, name)
+                flat = torch.zeros(old.numel() + 8, device="cuda")[shift:shift + old.numel()]
+                setattr(st, name, flat.view(old.shape))
+                setattr(st.buf, name, flat.data_ptr())
+                assert flat.data_ptr() % 32 == 16
+            st.lib.kvE_destroy(st.handle)
+            st.handle = C.c_void_p()
+            assert st.lib.kvE_create(C.byref(st.cfg), C.byref(st.buf), C.byref(st.handle)) == 0
+        load_kv(st, 0, K, V)
+        st.refresh(0, aw, lw, 0.5)
+        torch.cuda.synchronize()
+        assert st.poll_status() == 0
+        got.append([t.clone() for t in (st.ksum_f32, st.vsum_f32, st.ksum_bf16, st.vsum_bf16, st.scores)])
+    assert got[0][0].abs().max() > 0
+    for x, y in zip(*got):
+        assert torch.equal(x, y)

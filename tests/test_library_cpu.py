@@ -90,3 +90,16 @@ def test_generators_are_seeded_and_bf16_exact():
     k2, _ = wlm.gen_chunk(wl, 0, 1, 2, 2)
     assert k.shape == (64, 128) and not np.array_equal(k, k2)
     assert [c.n_stale_chunks() for c in (wlm.CFG1, wlm.CFG2, wlm.CFG3, wlm.CFG4)] == [28, 56, 61, 121]
+
+
+def test_create_refuses_buffers_that_do_not_start_on_16_bytes():
+    """before anything touches a device: the addresses below are not memory"""
+    lib = binding.load_library()
+    cfg = binding.kvE_config(B=1, Hq=1, Hkv=1, d=128, C=64, W=64, max_tokens=256, n_layers=1, agg=1, d_sum=256, d_g=64, attend=0)
+    fields = [f for f, _ in binding.kvE_buffers._fields_ if f not in ("n_pages", "workspace_bytes")]
+    for name in ("k_pages", "v_pages", "ksum_f32", "vsum_f32", "ksum_bf16", "vsum_bf16"):
+        for off in (2, 4, 8):
+            buf = binding.kvE_buffers(n_pages=4, workspace_bytes=lib.kvE_workspace_bytes(C.byref(cfg)),
+                                      **{f: 0x10000 * (i + 1) + (off if f == name else 0) for i, f in enumerate(fields)})
+            out = C.c_void_p()
+            assert lib.kvE_create(C.byref(cfg), C.byref(buf), C.byref(out)) == -1, (name, off)
