@@ -25,6 +25,16 @@ bool address(PyObject* o, int64_t rows, void** p) {
   return true;
 }
 
+// int(o): a float or any other number is taken too
+long whole_number(PyObject* o) {
+  if (PyLong_Check(o)) return PyLong_AsLong(o);
+  PyObject* n = PyNumber_Long(o);
+  if (!n) return -1;
+  const long x = PyLong_AsLong(n);
+  Py_DECREF(n);
+  return x;
+}
+
 // decode_step(function address, handle, S, device, layer, k_new, v_new, q, out, lse or None, scale, n_reserve, stream or None) -> status
 PyObject* decode_step(PyObject*, PyObject* const* a, Py_ssize_t n) {
   if (n != 13) {
@@ -36,7 +46,7 @@ PyObject* decode_step(PyObject*, PyObject* const* a, Py_ssize_t n) {
     void* handle = a[1] == Py_None ? nullptr : PyLong_AsVoidPtr(a[1]);
     const long rows = PyLong_AsLong(a[2]), device = PyLong_AsLong(a[3]), layer = PyLong_AsLong(a[4]);
     const double scale = PyFloat_AsDouble(a[10]);
-    const long n_reserve = PyLong_AsLong(a[11]);
+    const long n_reserve = whole_number(a[11]);
     void* stream = a[12] == Py_None ? nullptr : PyLong_AsVoidPtr(a[12]);
     if (PyErr_Occurred()) return nullptr;
     if (layer != (int)layer || n_reserve != (int)n_reserve) {

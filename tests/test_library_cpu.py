@@ -103,3 +103,16 @@ def test_create_refuses_buffers_that_do_not_start_on_16_bytes():
                                       **{f: 0x10000 * (i + 1) + (off if f == name else 0) for i, f in enumerate(fields)})
             out = C.c_void_p()
             assert lib.kvE_create(C.byref(cfg), C.byref(buf), C.byref(out)) == -1, (name, off)
+
+
+def test_decode_step_takes_any_number_as_the_reserve():
+    """n_reserve is int(n_reserve), as in append_next: the call gets as far as refusing tensors that are not on a device"""
+    import pytest
+    import torch
+    binding.load_library()
+    t = torch.zeros(2, 128, dtype=torch.bfloat16)
+    for reserve in (3, 3.0, np.float32(3), np.int64(3), torch.tensor(3)):
+        with pytest.raises(AssertionError):
+            binding._bind.decode_step(0, None, 2, 0, 0, t, t, t, t, None, 0.1, reserve, 0)
+    with pytest.raises(TypeError):
+        binding._bind.decode_step(0, None, 2, 0, 0, t, t, t, t, None, 0.1, None, 0)
