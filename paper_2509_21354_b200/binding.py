@@ -11,6 +11,7 @@ of device pointers; `Store` bundles the caller-owned buffers a handle needs.
 import ctypes as C
 import importlib.util
 import os
+import warnings
 
 import numpy as np
 import torch
@@ -63,16 +64,18 @@ _bind = None
 
 
 def _load_bind(build_if_missing: bool):
-    """the extension module behind Store.decode_step (csrc/bind.cpp)"""
+    """The extension module behind Store.decode_step (csrc/bind.cpp).  Where it cannot be built or loaded (no compiler, no
+    headers) that one call goes through ctypes like all others, 2 us slower."""
     global _bind
     if _bind is None:
-        path = _build.build_bind() if build_if_missing else _build.BIND
-        if not os.path.exists(path):
-            raise RuntimeError(f"{path} is missing: run `python -m paper_2509_21354_b200.build`")
-        spec = importlib.util.spec_from_file_location("_kve_bind", path)
-        module = importlib.util.module_from_spec(spec)
-        spec.loader.exec_module(module)
-        _bind = module
+        try:
+            path = _build.build_bind() if build_if_missing else _build.bind_path()
+            spec = importlib.util.spec_from_file_location("_kve_bind", path)
+            module = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(module)
+            _bind = module
+        except Exception as e:
+            warnings.warn(f"the decode step's extension module is not available ({e}); calling through ctypes")
     return _bind
 
 
@@ -215,7 +218,7 @@ class Store:
         if not torch.cuda.is_available():
             raise RuntimeError("libkve needs a CUDA device; there is no CPU path")
         self.lib = load_library()
-        self._decode_step = _bind.decode_step
+        self._decode_step = _bind.decode_step if _bind is not None else None
         self._decode_step_fn = C.cast(self.lib.kvE_decode_step, C.c_void_p).value
         self.device = torch.device(device)
         self.Hq = H if Hq is None else Hq
@@ -330,6 +333,12 @@ class Store:
         """append one token per sequence (k_new, v_new: bf16 [S, 128]) at the device-held length and attend, one launch"""
         if out is None:
             out = torch.empty_like(q)
+        if self._decode_step is None:
+            rc = self.lib.kvE_decode_step(self.handle, layer, _rows(k_new, self.row_shape), _rows(v_new, self.row_shape), _rows(q, self.row_shape),
+                                          _p(out), _p(lse), _DEFAULT_SCALE if scale is None else scale, int(n_reserve), _stream(self, stream))
+            if rc:
+                _check("kvE_decode_step", rc, self.handle)
+            return out
         rc = self._decode_step(self._decode_step_fn, self.handle and self.handle.value, self.S, self.device_index, layer, k_new, v_new, q, out,
                                lse, _DEFAULT_SCALE if scale is None else scale, n_reserve, None if stream is None else stream.cuda_stream)
         if rc:

@@ -10,7 +10,6 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libkve.so")
-BIND = os.path.join(HERE, "_kve_bind.so")      # the decode step's call from Python (csrc/bind.cpp)
 SOURCES = ["api.cu", "append.cu", "summarize.cu", "summarize_token.cu", "gate_proj.cu", "gate_rnn.cu", "gate_step.cu", "compact.cu", "attn.cu", "attn_block.cu", "attn_block_tc.cu", "selftest.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xptxas", "-v"]
@@ -21,9 +20,19 @@ def _deps_mtime() -> float:
     return max(os.path.getmtime(f) for f in files)
 
 
+def bind_path() -> str:
+    """Where the decode step's extension module (csrc/bind.cpp) lies for this interpreter and this torch: it is compiled against
+    the headers of both, and one that was built for others must not be loaded."""
+    import hashlib
+    import sysconfig
+    import torch
+    key = f"{sysconfig.get_config_var('SOABI')} {torch.__version__} {torch.version.cuda} {int(torch.compiled_with_cxx11_abi())}"
+    return os.path.join(HERE, f"_kve_bind.{hashlib.sha256(key.encode()).hexdigest()[:12]}.so")
+
+
 def build_bind(force: bool = False) -> str:
     """Compiles csrc/bind.cpp (an extension module against this interpreter and this torch; no device code)."""
-    src = os.path.join(CSRC, "bind.cpp")
+    src, BIND = os.path.join(CSRC, "bind.cpp"), bind_path()
     if not force and os.path.exists(BIND) and os.path.getmtime(BIND) >= os.path.getmtime(src):
         return BIND
     import sysconfig

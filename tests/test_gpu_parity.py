@@ -1499,3 +1499,27 @@ def test_summary_buffers_on_16_byte_boundaries(agg, d_sum):
     assert got[0][0].abs().max() > 0
     for x, y in zip(*got):
         assert torch.equal(x, y)
+
+
+def test_decode_step_through_ctypes_equals_the_extension_module():
+    b = _binding()
+    wl = wlm.CFG1.small(n=500, seed=13)
+    K, V = wlm.gen_kv(wl)
+    q, k1, v1 = (b.bits_to_bf16(np.ascontiguousarray(x)) for x in (wlm.gen_q(wl), *(x[:, 0] for x in wlm.gen_new_tokens(wl))))
+    got = []
+    for ctypes_call in (False, True):
+        st = make_store(wl.small(n_append=2))
+        assert st._decode_step is not None
+        if ctypes_call:
+            st._decode_step = None
+        load_kv(st, 0, K, V)
+        lse = torch.zeros(wl.S, device="cuda")
+        outs = [st.decode_step(0, k1, v1, q, lse=lse, n_reserve=1.0).clone() for _ in range(2)]
+        with pytest.raises(AssertionError):
+            st.decode_step(0, k1.float(), v1, q)
+        with pytest.raises(b.KveError) as e:              # the cache is full
+            st.decode_step(0, k1, v1, q)
+        assert e.value.rc == -3 and st.poll_status() == 0
+        got.append((outs[0], outs[1], lse))
+    for x, y in zip(*got):
+        assert torch.equal(x, y)

@@ -116,3 +116,21 @@ def test_decode_step_takes_any_number_as_the_reserve():
             binding._bind.decode_step(0, None, 2, 0, 0, t, t, t, t, None, 0.1, reserve, 0)
     with pytest.raises(TypeError):
         binding._bind.decode_step(0, None, 2, 0, 0, t, t, t, t, None, 0.1, None, 0)
+
+
+def test_extension_module_is_kept_apart_by_torch_version_and_is_not_required(monkeypatch):
+    import pytest
+    import torch
+    from paper_2509_21354_b200 import build
+    here = build.bind_path()
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    assert build.bind_path() != here
+
+    def no_compiler(*a, **kw):
+        raise RuntimeError("no compiler")
+    monkeypatch.setattr(build, "build_bind", no_compiler)
+    monkeypatch.setattr(binding, "_bind", None)
+    monkeypatch.setattr(binding, "_lib", None)
+    with pytest.warns(UserWarning, match="ctypes"):
+        lib = binding.load_library()
+    assert binding._bind is None and lib.kvE_poll_status(None, None) == -1
