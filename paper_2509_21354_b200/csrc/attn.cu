@@ -506,17 +506,24 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
         // the dims in another order than even ones, so that a quarter warp's two rows (256 bytes apart) lie in different banks:
         // of the eight columns, all of which hold q, those of the row's own parity are its logit.
         const uint4* kt = reinterpret_cast<const uint4*>(Ks + stage * AT_STAGE_ELEMS + (gwarp * AT_SUB) * D) + g8 * 16 + tig;
-        float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
+        // Every MMA starts from zero and the sums of 16 products are added up here: the tensor core cuts off what lies below the
+        // last bit of its accumulator, an ordinary addition rounds.  (Two chains of four MMAs: a logit
+        // of N(0, 1) rows off by 7.3e-8 rms and biased towards zero by 2.9e-8, 6.1e-8 and no bias so; 8 layers of 128 sequences x 330
+        // rows 7.04 and 7.17 us a layer.)
+        float d0[4], d1[4];      // rows g8, g8 + 8
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
+          float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
           const uint4 ra = kt[4 * (j ^ odd)], rb = kt[4 * (j ^ odd) + 8 * 16];
           const uint32_t A0[4] = {ra.x, rb.x, ra.y, rb.y}, A1[4] = {ra.z, rb.z, ra.w, rb.w};
           mma_bf16_16816(c0, A0, qf[j].x, qf[j].y);
           mma_bf16_16816(c1, A1, qf[j].z, qf[j].w);
+          d0[j] = odd ? c0[1] + c1[1] : c0[0] + c1[0];
+          d1[j] = odd ? c0[3] + c1[3] : c0[2] + c1[2];
         }
         // ---- online softmax ----
-        const float s0 = (g8 < nvalid) ? (odd ? c0[1] + c1[1] : c0[0] + c1[0]) * sl2 : -INFINITY;
-        const float s1 = (g8 + 8 < nvalid) ? (odd ? c0[3] + c1[3] : c0[2] + c1[2]) * sl2 : -INFINITY;
+        const float s0 = (g8 < nvalid) ? ((d0[0] + d0[1]) + (d0[2] + d0[3])) * sl2 : -INFINITY;
+        const float s1 = (g8 + 8 < nvalid) ? ((d1[0] + d1[1]) + (d1[2] + d1[3])) * sl2 : -INFINITY;
         float mx = fmaxf(s0, s1);
 #pragma unroll
         for (int o = 4; o <= 16; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
