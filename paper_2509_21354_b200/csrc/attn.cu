@@ -528,8 +528,10 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
 #pragma unroll
         for (int o = 4; o <= 16; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         const float m_new = fmaxf(m, mx);
-        const float p0 = ex2_fast(s0 - m_new), p1 = ex2_fast(s1 - m_new);
-        const float alpha = ex2_fast(m - m_new);
+        // (logits of -inf only, so far: their weights are 0, not exp2(-inf + inf))
+        const float m_sub = m_new == -INFINITY ? 0.f : m_new;
+        const float p0 = ex2_fast(s0 - m_sub), p1 = ex2_fast(s1 - m_sub);
+        const float alpha = ex2_fast(m - m_sub);
         l = fmaf(l, alpha, p0 + p1);
         m = m_new;
 #pragma unroll

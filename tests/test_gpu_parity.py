@@ -1549,3 +1549,22 @@ def test_logits_are_not_biased():
     err = np.concatenate(err)
     assert np.sqrt((err ** 2).mean()) < 1e-7
     assert abs(err.mean()) < 1e-8, err.mean()
+
+
+@pytest.mark.parametrize("lo,hi", [(64, 128), (0, 16), (80, 96), (112, 144), (0, 300)])
+def test_attention_over_keys_whose_logits_are_minus_infinity(lo, hi):
+    """Keys of the type's lowest value give logits of -inf in fp32: weight 0, wherever they lie among the warps that share the rows"""
+    b = _binding()
+    wl = wlm.CFG1.small(B=1, H=4, n=333, W=333, seed=14)
+    K, V = wlm.gen_kv(wl)
+    K[:, lo:hi] = 0xFF7F                                 # the lowest bf16
+    st = make_store(wl)
+    load_kv(st, 0, K, V)
+    q = wlm.gen_q(wl) & 0x7FFF                           # positive
+    lse = torch.zeros(wl.S, device="cuda")
+    out = st.decode_attn_dense(0, b.bits_to_bf16(q), lse=lse)
+    assert st.poll_status() == 0
+    rows = [i for i in range(wl.n) if not lo <= i < hi]
+    want, _, want_lse = kvo.Oracle("f64").attn_dense(q, np.ascontiguousarray(K[:, rows]), np.ascontiguousarray(V[:, rows]), hz.SCALE)
+    hz.check_output(b.bf16_to_bits(out), want, "lowest keys")
+    assert np.abs(lse.cpu().numpy() - want_lse).max() <= 1e-3
