@@ -53,7 +53,12 @@ def launches_per_step(step):
         for _ in range(4):
             step()
         torch.cuda.synchronize()
-    return sum("kve::" in e.name for e in prof.events()) // 4
+    return whole_launches(sum("kve::" in e.name for e in prof.events()), 4)
+
+
+def whole_launches(events, steps):
+    """launches per step, or None where the profiler saw none or lost some: then the count is not known"""
+    return events // steps if events > 0 and events % steps == 0 else None
 
 
 def load_peaks():
@@ -901,7 +906,8 @@ def run_ours(args, rank, world, local_rank):
         "e2e": {"value": world * args.steps / e2e_s, "unit": UNIT, "h2d_bytes_per_step": 3 * S * 256,
                 "d2h_bytes_per_step": S * 256,
                 "max_abs_diff_vs_device_path": e2e_diff, "max_abs_output": e2e_ref},
-        "gpu_launches": launches * args.steps * repeats,
+        "gpu_launches": launches * args.steps * repeats if launches else None,
+        **({} if launches else {"gpu_launches_unknown": "the profiler recorded no kernels, or not the same number in each step"}),
         "clocks": clk.summary(),
         "roofline": roofline,
         "roofline_largest_hbm_kernel": roofline_hbm,

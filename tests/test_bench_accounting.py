@@ -28,3 +28,8 @@ def test_algorithmic_flops_of_cfg2():
     assert fl["chunk_mlp"] == 2 * units * 2 * (128 * 256 + 256 * 128) == 3_758_096_384
     assert fl["gate_rnn"] == units * (2 * 256 * 1024 + 512)
     assert "chunk_mlp" not in bench.algorithmic_flops(wlm.CFG1, 28)                        # mean aggregator: no MLP
+
+
+def test_launch_count_is_not_reported_when_events_are_missing():
+    assert bench.whole_launches(28, 4) == 7
+    assert bench.whole_launches(0, 4) is None and bench.whole_launches(27, 4) is None
