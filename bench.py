@@ -657,8 +657,9 @@ def trigger_leg(wl, attend, seed, steady_ms, n_triggers=24):
 def token_mlp_leg(wl, peaks, peak_kind, flush, seed):
     """Eq. 2 taken literally (KVE_AGG_TOKEN_MLP): the aggregator MLP on EVERY stale token, outputs mean-pooled, on the
     workload's geometry.  The first layer is a tcgen05 contraction [tokens, 128] x [128, d_sum]; the kernel is bound by
-    the activation arithmetic of its epilogue (erf GELU: about 21 FP32-pipe instructions and 2 special-function ops per
-    activation, plus the pooling shuffles), so its roofline is the FP32 issue rate: SMs x 128 lanes x clock / 21."""
+    the activation arithmetic of its epilogue.  Per pair of activations: bias, polynomial of degree 6 and the two sums in packed
+    instructions (9), |x| capped and max(x, 0) one by one (4), two exponentials.  The exponentials are the tighter bound (16 a
+    cycle and SM, against 128 / 6.5 = 19.7 activations that fit the issue slots): the roofline is SMs x 16 x clock."""
     import torch
     d_sum = 256
     g = wl.small(agg="token_mlp", d_sum=d_sum)
@@ -678,7 +679,7 @@ def token_mlp_leg(wl, peaks, peak_kind, flush, seed):
     acts = 2 * tokens * d_sum
     kv_bytes = tokens * 512
     sm_mhz = peaks.get("sm_max_mhz", 1965.0)
-    alu_peak = 148 * 128 * sm_mhz * 1e6 / 21.0          # activations per second if the FP32 pipe did nothing else
+    alu_peak = 148 * 16 * sm_mhz * 1e6          # activations per second: one exponential each, 16 a cycle and SM
     tensor_peak = peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"])
     res = {"what": f"kvE_summarize_chunks with the per-token MLP aggregator (d_sum {d_sum}) over all {rig.Nc} stale chunks of "
                    f"{g.S} sequences ({tokens} tokens per side), both kernels, L2 flushed",
@@ -687,7 +688,7 @@ def token_mlp_leg(wl, peaks, peak_kind, flush, seed):
            "activations": acts, "Gact/s": acts / us / 1e3,
            "roofline": {"bound": "alu", "achieved": acts / us / 1e3, "peak": alu_peak / 1e9, "unit": "Gact/s",
                         "frac": acts / us / 1e3 / (alu_peak / 1e9),
-                        "peak_kind": "derived: 148 SMs x 128 FP32 lanes x max SM clock / 21 instructions per activation"},
+                        "peak_kind": "derived: 148 SMs x 16 exponentials a cycle x max SM clock, one exponential per activation"},
            "peak_kind": f"of {peak_kind}"}
     st.close()
     return res
