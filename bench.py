@@ -885,6 +885,7 @@ def run_ours(args, rank, world, local_rank):
         roofline = {"kernel": dominant, "bound": "hbm", "achieved": kern[dominant]["GB/s"], "peak": hbm, "unit": "GB/s",
                     "frac": kern[dominant]["GB/s"] / hbm, "traffic": traffic, "peak_kind": f"of {peak_kind}",
                     "algorithmic_bytes": kern[dominant]["bytes"], "us_per_launch": kern[dominant]["us"]}
+    roofline["schedule"] = "kernels timed one by one, all chunks in one range; the step itself may take them in two"
     hbm_kernel = max((k for k in ("chunk_mean", "attn") if k in in_step), key=lambda k: in_step[k]["us"])
     roofline_hbm = {"kernel": hbm_kernel, "bound": "hbm", "achieved": kern[hbm_kernel]["GB/s"], "peak": hbm, "unit": "GB/s",
                     "frac": kern[hbm_kernel]["GB/s"] / hbm, "algorithmic_bytes": kern[hbm_kernel]["bytes"],
@@ -1056,6 +1057,17 @@ def run_reference(args, rank):
             "gpu_launches": 0, "wall_s": wall}
 
 
+# What the result line holds; everything else a run measured (kernels, other configurations, sweep, ...) goes to standard error
+# as a line of its own, so that the result stays a few kilobytes.
+RESULT_KEYS = ("impl", "unavailable", "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+               "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "gpu_launches_unknown", "clocks", "roofline", "roofline_largest_hbm_kernel",
+               "gated_attention", "steady_state", "cpu_baseline", "wall_s")
+
+
+def split_result(res):
+    return {k: res[k] for k in RESULT_KEYS if k in res}, {k: v for k, v in res.items() if k not in RESULT_KEYS}
+
+
 ALL_LEGS = "per_config,sweep,trigger,token_mlp,query_block,tick_graph,cpu"
 
 
@@ -1101,7 +1113,10 @@ def main():
             dist.barrier()
             dist.destroy_process_group()
     if res is not None:
-        print(json.dumps(res))
+        line, detail = split_result(res)
+        if detail:
+            print(json.dumps(detail), file=sys.stderr, flush=True)
+        print(json.dumps(line))
 
 
 if __name__ == "__main__":

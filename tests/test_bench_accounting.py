@@ -33,3 +33,11 @@ def test_algorithmic_flops_of_cfg2():
 def test_launch_count_is_not_reported_when_events_are_missing():
     assert bench.whole_launches(28, 4) == 7
     assert bench.whole_launches(0, 4) is None and bench.whole_launches(27, 4) is None
+
+
+def test_result_line_is_short_and_nothing_is_lost():
+    res = {k: {"x": [1.0] * 8} for k in bench.RESULT_KEYS}
+    res.update(per_config={"cfg1": [0.0] * 5000}, sweep=[1] * 5000, kernels={})
+    line, detail = bench.split_result(res)
+    assert set(line) | set(detail) == set(res) and not set(line) & set(detail)
+    assert set(detail) == {"per_config", "sweep", "kernels"}
