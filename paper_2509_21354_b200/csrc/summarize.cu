@@ -77,11 +77,123 @@ __global__ void __launch_bounds__(MEAN_WARPS * 32) kve_chunk_mean_kernel(LayerVi
     *reinterpret_cast<uint2*>((is_v ? v.vsum_bf16 : v.ksum_bf16) + o) = make_uint2(pack_bf16x2(acc[0], acc[1]), pack_bf16x2(acc[2], acc[3]));
 }
 
+// ---- the same mean over short chunks ---------------------------------------------------------------------------------
+// With few rows per page a CTA per unit spends its time starting up (and the summaries, 1536 bytes a unit, become the larger
+// part of the traffic).  Here a warp takes a unit, K in its lower and V in its upper lanes, 16 bytes each, SHORT_ROWS rows in flight, or
+// (MULTI) as many units of up to four rows as make up that number; eight warps to a CTA.
+//   us, a CTA per unit -> this: 128 sequences x 4160 tokens in chunks of 1, 4, 8, 16, 24 tokens 962 -> 165, 270 -> 74, 144 -> 57, 74 -> 45,
+//   55 -> 42; 60 x 2000 in chunks of 1, 4, 8 204 -> 39, 52 -> 15, 29 -> 11.  From 9 tokens on a launch that leaves SMs without work is
+//   better off with all rows of a page in flight: 8 x 2048 in chunks of 24 6.1 us this way, 4.0 the other; 60 x 2000 14.8 and 12.8.
+constexpr int SHORT_WARPS = 8, SHORT_ROWS = 8;
+
+template <bool POOL_MAX, bool MULTI>
+__global__ void __launch_bounds__(SHORT_WARPS * 32, 4) kve_chunk_mean_short_kernel(LayerView v, int t0, int n_range, FastDiv by_range, int n_units,
+                                                                                  int final_output, int dev_window, int list_cut) {
+  pdl_launch_dependents();
+  pdl_wait();
+  if (list_cut >= 0 && blockIdx.x == 0 && threadIdx.x == 0) *v.n_listed = list_cut;
+  if (dev_window >= 0) {      // one chunk per sequence, found on the device
+    const NextChunk nx = next_chunk(v.n_listed, v.seq_len, v.C, dev_window, v.max_chunks);
+    if (!nx.due) return;
+    t0 = nx.t;
+  }
+  const int lane = threadIdx.x & 31, is_v = lane >> 4, l16 = lane & 15;
+  const int per_warp = MULTI ? SHORT_ROWS / v.C : 1;
+  const long long unit0 = ((long long)blockIdx.x * SHORT_WARPS + (threadIdx.x >> 5)) * per_warp;
+  const int n_mine = (int)min((long long)per_warp, n_units - unit0);
+  if (n_mine <= 0) return;
+  // lane u keeps the page and the summary row of unit u
+  int page = -1;
+  long long row_of = 0;
+  if (lane < n_mine) {
+    const int unit = (int)unit0 + lane, s = (int)by_range.div((uint32_t)unit);
+    row_of = (long long)s * v.max_chunks + t0 + (unit - s * n_range);
+    page = v.page_table[row_of];
+    if (page < 0 || page >= v.n_pages) {
+      set_status(v.status, ERR_CAPACITY);
+      page = -1;
+    }
+  }
+  const uint4* pool = reinterpret_cast<const uint4*>(is_v ? v.v_pages : v.k_pages) + l16;
+  float acc[8];
+  auto clear = [&]() {
+#pragma unroll
+    for (int x = 0; x < 8; ++x) acc[x] = POOL_MAX ? -INFINITY : 0.f;
+  };
+  auto take = [&](const uint4& w) {      // the next row
+    const float f[8] = {bf16lo(w.x), bf16hi(w.x), bf16lo(w.y), bf16hi(w.y), bf16lo(w.z), bf16hi(w.z), bf16lo(w.w), bf16hi(w.w)};
+#pragma unroll
+    for (int x = 0; x < 8; ++x) acc[x] = POOL_MAX ? fmaxf(acc[x], f[x]) : acc[x] + f[x];
+  };
+  auto finish = [&](int u) {
+    const long long o = __shfl_sync(0xffffffffu, row_of, u) * D + l16 * 8;
+    if (__shfl_sync(0xffffffffu, page, u) < 0) return;
+    const float fc = (float)v.C;
+#pragma unroll
+    for (int x = 0; x < 8; ++x)
+      if (!POOL_MAX) acc[x] = __fdiv_rn(acc[x], fc);
+    float4* out = reinterpret_cast<float4*>((is_v ? v.vsum_f32 : v.ksum_f32) + o);
+    out[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+    out[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+    if (final_output)
+      *reinterpret_cast<uint4*>((is_v ? v.vsum_bf16 : v.ksum_bf16) + o) =
+          make_uint4(pack_bf16x2(acc[0], acc[1]), pack_bf16x2(acc[2], acc[3]), pack_bf16x2(acc[4], acc[5]), pack_bf16x2(acc[6], acc[7]));
+  };
+  uint4 w[SHORT_ROWS];
+  clear();
+  if constexpr (MULTI) {
+    int u = 0, row = 0;
+#pragma unroll
+    for (int x = 0; x < SHORT_ROWS; ++x) {
+      const int p = __shfl_sync(0xffffffffu, page, u);
+      if (p >= 0) w[x] = __ldcs(pool + ((long long)p * v.C + row) * 16);      // (lanes without a unit hold -1)
+      if (++row == v.C) { row = 0; ++u; }
+    }
+    u = row = 0;
+#pragma unroll
+    for (int x = 0; x < SHORT_ROWS; ++x) {
+      if (u >= n_mine) break;
+      take(w[x]);
+      if (++row == v.C) {
+        finish(u);
+        clear();
+        row = 0;
+        ++u;
+      }
+    }
+  } else {
+    const int p = __shfl_sync(0xffffffffu, page, 0);
+    if (p < 0) return;
+    const uint4* src = pool + (long long)p * v.C * 16;
+    for (int j = 0; j < v.C; j += SHORT_ROWS) {
+#pragma unroll
+      for (int x = 0; x < SHORT_ROWS; ++x)
+        if (j + x < v.C) w[x] = __ldcs(src + (j + x) * 16);
+#pragma unroll
+      for (int x = 0; x < SHORT_ROWS; ++x)
+        if (j + x < v.C) take(w[x]);
+    }
+    finish(0);
+  }
+}
+
+static cudaError_t launch_chunk_mean_short(const LayerView& v, int t0, int n_range, long long n_units, bool final_output, bool pool_max,
+                                           cudaStream_t st, int dev_window, int list_cut) {
+  const bool multi = 2 * v.C <= SHORT_ROWS && n_units * v.C / SHORT_ROWS > 16LL * sm_count();      // (16 warps for every SM first)
+  const long long per_cta = (long long)SHORT_WARPS * (multi ? SHORT_ROWS / v.C : 1);
+  const dim3 grid((unsigned)((n_units + per_cta - 1) / per_cta)), block(SHORT_WARPS * 32);
+  const FastDiv by_range = fast_div((uint32_t)n_range);
+  auto* kernel = pool_max ? (multi ? kve_chunk_mean_short_kernel<true, true> : kve_chunk_mean_short_kernel<true, false>)
+                          : (multi ? kve_chunk_mean_short_kernel<false, true> : kve_chunk_mean_short_kernel<false, false>);
+  return launch_pdl(kernel, grid, block, 0, st, v, t0, n_range, by_range, (int)n_units, pool_max || final_output ? 1 : 0, dev_window, list_cut);
+}
+
 cudaError_t launch_chunk_mean(const LayerView& v, int t0, int t1, bool final_output, bool pool_max, cudaStream_t st, int dev_window, int list_cut) {
   const int n_range = dev_window >= 0 ? 1 : t1 - t0;
   const long long n_units = (long long)v.S * n_range;
   if (n_units <= 0) return cudaSuccess;
   if (n_units >= (1LL << 31)) return cudaErrorInvalidValue;
+  if (v.C <= SHORT_ROWS || (v.C < 32 && n_units > 64LL * sm_count())) return launch_chunk_mean_short(v, t0, n_range, n_units, final_output, pool_max, st, dev_window, list_cut);
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;

@@ -1568,3 +1568,35 @@ def test_attention_over_keys_whose_logits_are_minus_infinity(lo, hi):
     want, _, want_lse = kvo.Oracle("f64").attn_dense(q, np.ascontiguousarray(K[:, rows]), np.ascontiguousarray(V[:, rows]), hz.SCALE)
     hz.check_output(b.bf16_to_bits(out), want, "lowest keys")
     assert np.abs(lse.cpu().numpy() - want_lse).max() <= 1e-3
+
+
+@pytest.mark.parametrize("agg", ["mean", "max"])
+@pytest.mark.parametrize("C,B,H,n", [(1, 1, 3, 77), (2, 1, 5, 1001), (7, 3, 3, 500), (8, 4, 32, 300), (16, 2, 9, 640), (24, 1, 1, 3000), (31, 1, 7, 400)])
+def test_summaries_of_short_chunks(C, B, H, n, agg):
+    """Chunks below 32 tokens, several to a warp: the fp32 sum in temporal order and an IEEE division, bit for bit; a unit without
+    a page is flagged and left alone, its neighbours are not."""
+    b = _binding()
+    wl = wlm.CFG1.small(B=B, H=H, n=n, C=C, W=5, agg=("identity" if C == 1 and agg == "mean" else agg), seed=16)
+    K, V = wlm.gen_kv(wl)
+    nc = wl.n_stale_chunks()
+    st = make_store(wl)
+    load_kv(st, 0, K, V)
+    st.summarize_chunks(0, 0, nc)
+    assert st.poll_status() == 0
+    for bits, f32, b16 in ((K, st.ksum_f32, st.ksum_bf16), (V, st.vsum_f32, st.vsum_bf16)):
+        x = wlm.bf16_bits_to_f32(bits[:, :nc * C]).reshape(wl.S, nc, C, 128)
+        want = x[:, :, 0].copy()
+        for r in range(1, C):
+            want = np.maximum(want, x[:, :, r]) if agg == "max" else want + x[:, :, r]
+        if agg != "max":
+            want = want / np.float32(C)
+        assert np.array_equal(f32[0, :, :nc].cpu().numpy(), want)
+        assert np.array_equal(b.bf16_to_bits(b16[0, :, :nc]), wlm.f32_to_bf16_bits(want))
+    s, t = wl.S // 2, nc // 2
+    st.page_table[0, s, t] = -1
+    before = st.ksum_f32.clone()
+    st.ksum_f32.zero_()
+    st.summarize_chunks(0, 0, nc)
+    assert st.poll_status() == -3
+    before[0, s, t] = 0
+    assert torch.equal(st.ksum_f32, before)
