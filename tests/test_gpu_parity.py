@@ -1600,3 +1600,21 @@ def test_summaries_of_short_chunks(C, B, H, n, agg):
     assert st.poll_status() == -3
     before[0, s, t] = 0
     assert torch.equal(st.ksum_f32, before)
+
+
+@pytest.mark.parametrize("d_sum", [64, 128, 256])
+def test_mlp_summaries_are_no_further_off_than_fp32_loops(d_sum):
+    """The aggregator MLP sums in pieces that the tensor core cuts off and ordinary additions round: against 64 bits its rms error stays
+    within that of the oracle's fp32 build, plain loops over the same inputs."""
+    b = _binding()
+    wl = wlm.CFG2.small(B=1, H=12, n=2200, d_sum=d_sum, seed=19)
+    pb = hz.Problem(wl)
+    st = make_store(wl)
+    load_kv(st, 0, pb.K, pb.V)
+    st.summarize_chunks(0, 0, pb.Nc, b.AggWeights(pb.mlp))
+    assert st.poll_status() == 0
+    for name in ("ksum", "vsum"):
+        want = pb.sm64[name][:, :pb.Nc].astype(np.float64)
+        rms = lambda x: np.sqrt(((x[:, :pb.Nc].astype(np.float64) - want) ** 2).mean())
+        got = getattr(st, name + "_f32")[0].cpu().numpy()
+        assert rms(got) <= rms(pb.sm32[name]), (name, rms(got), rms(pb.sm32[name]))
