@@ -1618,3 +1618,32 @@ def test_mlp_summaries_are_no_further_off_than_fp32_loops(d_sum):
         rms = lambda x: np.sqrt(((x[:, :pb.Nc].astype(np.float64) - want) ** 2).mean())
         got = getattr(st, name + "_f32")[0].cpu().numpy()
         assert rms(got) <= rms(pb.sm32[name]), (name, rms(got), rms(pb.sm32[name]))
+
+
+@pytest.mark.parametrize("B,H,C,n", [(1, 3, 1, 700), (1, 2, 2, 3000), (2, 40, 1, 400)])
+@pytest.mark.parametrize("keep", [0.0, 0.4, 1.0])
+def test_long_keep_lists(B, H, C, n, keep):
+    """Lists of more than 256 chunks, with few sequences and with many: ids, counts and the rows that attention reads"""
+    b = _binding()
+    wl = wlm.CFG1.small(B=B, H=H, n=n, C=C, W=20, agg="identity" if C == 1 else "mean", seed=17)
+    K, V = wlm.gen_kv(wl)
+    nc = wl.n_stale_chunks()
+    st = make_store(wl)
+    load_kv(st, 0, K, V)
+    st.summarize_chunks(0, 0, nc)
+    st.gate(0, 0, nc, b.LstmWeights(wlm.gen_lstm_weights(wl)))
+    scores = np.random.default_rng(17).random((wl.S, nc), dtype=np.float32) * 0.998 + 0.001
+    st.scores[0, :, :nc] = torch.from_numpy(scores).cuda()
+    st.compact(0, 1.0 - keep)
+    kept = scores >= np.float32(1.0 - keep)
+    assert st.poll_status() == 0 and np.array_equal(st.keep_cnt[0].cpu().numpy(), kept.sum(1))
+    idx = st.keep_idx[0].cpu().numpy()
+    for s in range(wl.S):
+        m = int(kept[s].sum())
+        assert np.array_equal(idx[s, :m], np.nonzero(kept[s])[0]) and (idx[s, m:] == -1).all()
+    q = wlm.gen_q(wl)
+    out = st.decode_attn(0, b.bits_to_bf16(q))
+    o = kvo.Oracle("f64")
+    cnt = kept.sum(1).astype(np.int32)
+    want, _, _, _ = o.attn(q, K, V, C, nc, idx, cnt, b.bf16_to_bits(st.ksum_bf16[0]), b.bf16_to_bits(st.vsum_bf16[0]), hz.ATT["summary"], hz.SCALE)
+    hz.check_output(b.bf16_to_bits(out), want, "long list")
