@@ -230,13 +230,15 @@ AttnCut attention_cut(const kvE_store* st, AttnMode mode, const LayerState& ls) 
   if (tiles < 1) tiles = 1;
   const long long G = st->attn_grid_max, S = st->S;
   const long long k_max = tiles < MAX_SPLITS ? tiles : MAX_SPLITS;
+  // a tile of short chunks is up to 2 * 64 / C copies, which is what bounds it below 16 tokens
+  const double copies_us = st->cfg.C < 16 ? 4.0 / st->cfg.C - 4.0 / 16 : 0.0;
   const double hbm_us = (double)S * (double)(tail + lead) * 512.0 / 6.4e6;
   auto cost_of = [&](long long k) {
     const unsigned parts = (unsigned)(S * k), grid = parts < (unsigned)G ? parts : (unsigned)G;
     const unsigned rounds = (parts + grid - 1) / grid;                 // parts of the busiest CTA
     const double busiest = rounds == 1 ? (double)(((unsigned)tiles + (unsigned)k - 1) / (unsigned)k) : (double)rounds * (double)tiles / (double)k;
     const double ends = k == 1 ? 0.0 : 1.7 + 0.05 * (double)k + (rounds > 1 ? 1.8 : 0.0);
-    const double us = busiest * (2 * grid <= (unsigned)G ? 0.9 : 1.25) + ends;
+    const double us = busiest * ((2 * grid <= (unsigned)G ? 0.9 : 1.25) + copies_us) + ends;
     const double stream = hbm_us + 0.35 * (busiest - (double)(S * tiles) / (double)grid);
     return us > stream ? us : stream;
   };

@@ -67,7 +67,8 @@ constexpr int AT_SUB = AT_TILE / AT_GWARPS;   // 16 rows per warp per tile: the 
 constexpr int AT_PRODUCER = AT_CWARPS;        // warp ids
 constexpr int AT_THREADS = (AT_CWARPS + 2) * 32;
 constexpr int AT_STAGE_ELEMS = AT_TILE * D;   // bf16 elements of one K (or V) tile
-constexpr int AT_LANE_SEGS = 3;               // chunks a tile may touch for one lane to issue its copies: chunks of 32 tokens and more
+constexpr int AT_LANE_SEGS = 3;               // chunks a tile may touch for one lane to issue its copies
+constexpr int AT_SHORT_CHUNK = AT_TILE / (AT_LANE_SEGS - 1);      // that holds for all tiles with chunks of 32 tokens and more
 constexpr int AT_PREFETCH_TILES = 2;          // most tiles a CTA pulls into L2 before its predecessor has finished
 static_assert(AT_SUB == 16, "the logits of a warp's rows are one m16n8k16 tile");
 
@@ -220,6 +221,8 @@ __device__ __forceinline__ void prefetch_first_tiles(const AttnArgs& a, uint32_t
   }
 }
 
+// SHORT: chunks below 32 tokens, of which a tile may touch more than AT_LANE_SEGS
+template <bool SHORT>
 __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   uint16_t* Ks = reinterpret_cast<uint16_t*>(smem + AT_OFF_K);
@@ -352,10 +355,18 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
     if (a.k_new != nullptr && !g.appending && blockIdx.x == 0 && lane == 0) set_status(v.status, ERR_CAPACITY);   // cache full
 
     // The copies of tile i of the batch: lane i waits for the stage, publishes the tile's description and issues one K and one V
-    // copy per chunk the tile touches, all from its own registers; the lanes take turns.  Chunks so short that a tile
-    // has more than AT_LANE_SEGS of them: the whole warp, 32 chunks at a time.  False on a timed-out wait.
+    // copy per chunk the tile touches, all from its own registers; the lanes take turns.  Chunks so short that a tile may
+    // have more than AT_LANE_SEGS of them: the whole warp, 32 chunks at a time, their pages `pg` looked up a tile ahead, and chunks
+    // that follow one another in the pool (pages dealt out in order) in one copy.  (One copy per chunk, looked up when its
+    // turn came: 60 sequences x 2000 rows in chunks of one token 48.8 us, 17.5 so with the pages in order, 43.3 scattered; 128 x 4160 in
+    // chunks of 4 and 16 tokens 71 -> 66 and 51 -> 48.)  False on a timed-out wait.
+    auto look_up = [&](const TilePlan& p, int i, int (&pg)[2]) {
+      const int n_seg = __shfl_sync(0xffffffffu, p.n_seg, i), c0 = __shfl_sync(0xffffffffu, p.c0, i), list = __shfl_sync(0xffffffffu, p.list, i);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) pg[h] = n_seg > AT_LANE_SEGS && lane + 32 * h < n_seg ? page_of(p.s, list, c0 + lane + 32 * h) : -1;
+    };
     int it = 0;
-    auto issue = [&](const TilePlan& p, int i) -> bool {
+    auto issue = [&](const TilePlan& p, int i, const int (&pg)[2]) -> bool {
       const int stage = it % AT_STAGES, round = it / AT_STAGES;
       ++it;
       uint16_t *kd = Ks + stage * AT_STAGE_ELEMS, *vd = Vs + stage * AT_STAGE_ELEMS;
@@ -396,19 +407,29 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
         }
       }
       ok = __shfl_sync(0xffffffffu, (int)ok, i) != 0;
-      if (v.C < AT_TILE / (AT_LANE_SEGS - 1)) {
+      if constexpr (SHORT) {
         const int n_seg = __shfl_sync(0xffffffffu, p.n_seg, i);
         if (ok && n_seg > AT_LANE_SEGS) {
           const int row0 = __shfl_sync(0xffffffffu, p.row0, i), c0 = __shfl_sync(0xffffffffu, p.c0, i);
-          const int rows = __shfl_sync(0xffffffffu, p.rows, i) - (with_new ? 1 : 0), list = __shfl_sync(0xffffffffu, p.list, i);
-          for (int x = lane; x < n_seg; x += 32) {
-            const TileSegment sg = tile_segment(row0, rows, v.C, c0 + x);
-            if (sg.len <= 0) continue;
-            int page = page_of(p.s, list, sg.pos);
-            if (page < 0 || page >= v.n_pages) { set_status(v.status, ERR_CAPACITY); page = 0; }
-            const long long off = ((long long)page * v.C + sg.r) * D;
-            bulk_g2s(kd + sg.dst * D, v.k_pages + off, (uint32_t)sg.len * ROW_BYTES, &full[stage]);
-            bulk_g2s(vd + sg.dst * D, v.v_pages + off, (uint32_t)sg.len * ROW_BYTES, &full[stage]);
+          const int rows = __shfl_sync(0xffffffffu, p.rows, i) - (with_new ? 1 : 0);
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            if (32 * h >= n_seg) break;
+            TileSegment sg = tile_segment(row0, rows, v.C, c0 + lane + 32 * h);
+            if (lane + 32 * h >= n_seg) sg.len = 0;
+            int page = pg[h];
+            if (sg.len > 0 && (page < 0 || page >= v.n_pages)) { set_status(v.status, ERR_CAPACITY); page = 0; }
+            const long long row = (long long)page * v.C + sg.r;      // of the pool
+            const long long end = row + sg.len, end_before = __shfl_up_sync(0xffffffffu, end, 1);
+            const bool head = sg.len > 0 && (lane == 0 || row != end_before);
+            const unsigned heads = __ballot_sync(0xffffffffu, head), live = __ballot_sync(0xffffffffu, sg.len > 0);      // live: the first lanes
+            const unsigned above = lane == 31 ? 0u : heads & ~((2u << lane) - 1u);
+            const int last = (above ? __ffs(above) - 1 : __popc(live)) - 1;      // last chunk of the run that starts here
+            const int run = __shfl_sync(0xffffffffu, sg.dst + sg.len, last & 31) - sg.dst;
+            if (head) {
+              bulk_g2s(kd + sg.dst * D, v.k_pages + row * D, (uint32_t)run * ROW_BYTES, &full[stage]);
+              bulk_g2s(vd + sg.dst * D, v.v_pages + row * D, (uint32_t)run * ROW_BYTES, &full[stage]);
+            }
           }
           __syncwarp();
         }
@@ -416,10 +437,17 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
       return ok;
     };
     bool ok = true;
+    int pg[2] = {-1, -1}, pg_next[2] = {-1, -1};
+    if (SHORT && cur.n > 0) look_up(cur, 0, pg);
     while (ok && cur.n > 0) {
       for (int i = 0; ok && i < cur.n; ++i) {
         if (i == cur.n - 1) make_plan(nxt, nullptr);      // its look-ups run while this batch's last copies are issued
-        ok = issue(cur, i);
+        if constexpr (SHORT) {
+          if (i < cur.n - 1) look_up(cur, i + 1, pg_next);
+          else if (nxt.n > 0) look_up(nxt, 0, pg_next);
+        }
+        ok = issue(cur, i, pg);
+        if constexpr (SHORT) { pg[0] = pg_next[0]; pg[1] = pg_next[1]; }
         KVE_STAMP(it == 1 && lane == 0, 2);
       }
       if (cur.i_new >= 0) {
@@ -510,7 +538,7 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
         // last bit of its accumulator, an ordinary addition rounds.  (Two chains of four MMAs: a logit
         // of N(0, 1) rows off by 7.3e-8 rms and biased towards zero by 2.9e-8, 6.1e-8 and no bias so; 8 layers of 128 sequences x 330
         // rows 7.04 and 7.17 us a layer.)
-        float d0[4], d1[4];      // rows g8, g8 + 8
+        float2 d0[4], d1[4];      // rows g8, g8 + 8: both parities
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
@@ -518,12 +546,13 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
           const uint32_t A0[4] = {ra.x, rb.x, ra.y, rb.y}, A1[4] = {ra.z, rb.z, ra.w, rb.w};
           mma_bf16_16816(c0, A0, qf[j].x, qf[j].y);
           mma_bf16_16816(c1, A1, qf[j].z, qf[j].w);
-          d0[j] = odd ? c0[1] + c1[1] : c0[0] + c1[0];
-          d1[j] = odd ? c0[3] + c1[3] : c0[2] + c1[2];
+          d0[j] = add2(make_float2(c0[0], c0[1]), make_float2(c1[0], c1[1]));
+          d1[j] = add2(make_float2(c0[2], c0[3]), make_float2(c1[2], c1[3]));
         }
+        const float2 l0 = add2(add2(d0[0], d0[1]), add2(d0[2], d0[3])), l1 = add2(add2(d1[0], d1[1]), add2(d1[2], d1[3]));
         // ---- online softmax ----
-        const float s0 = (g8 < nvalid) ? ((d0[0] + d0[1]) + (d0[2] + d0[3])) * sl2 : -INFINITY;
-        const float s1 = (g8 + 8 < nvalid) ? ((d1[0] + d1[1]) + (d1[2] + d1[3])) * sl2 : -INFINITY;
+        const float s0 = (g8 < nvalid) ? (odd ? l0.y : l0.x) * sl2 : -INFINITY;
+        const float s1 = (g8 + 8 < nvalid) ? (odd ? l1.y : l1.x) * sl2 : -INFINITY;
         float mx = fmaxf(s0, s1);
 #pragma unroll
         for (int o = 4; o <= 16; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -664,9 +693,11 @@ cudaError_t launch_attn(const LayerView& v, AttnMode mode, int n_chunks, int par
                         float* lse, float scale, const void* kkept, const void* vkept, float* partials, int32_t* counters,
                         const void* k_new, const void* v_new, int32_t* ticket, cudaStream_t st) {
   if (v.S <= 0) return cudaSuccess;
-  static DeviceFlags opted;
+  const bool is_short = v.C < AT_SHORT_CHUNK;
+  static DeviceFlags opted, opted_short;
   {
-    cudaError_t e = smem_opt_in(opted, kve_decode_attn_kernel, AT_SMEM_BYTES);
+    const cudaError_t e = is_short ? smem_opt_in(opted_short, kve_decode_attn_kernel<true>, AT_SMEM_BYTES)
+                                   : smem_opt_in(opted, kve_decode_attn_kernel<false>, AT_SMEM_BYTES);
     if (e != cudaSuccess) return e;
   }
   AttnArgs a;
@@ -676,7 +707,7 @@ cudaError_t launch_attn(const LayerView& v, AttnMode mode, int n_chunks, int par
   a.kkept = static_cast<const uint16_t*>(kkept); a.vkept = static_cast<const uint16_t*>(vkept);
   a.partials = partials; a.counters = counters;
   a.k_new = static_cast<const uint16_t*>(k_new); a.v_new = static_cast<const uint16_t*>(v_new); a.ticket = ticket;
-  return launch_pdl(kve_decode_attn_kernel, dim3((unsigned)(grid < 1 ? 1 : grid)), dim3(AT_THREADS), AT_SMEM_BYTES, st, a);
+  return launch_pdl(is_short ? kve_decode_attn_kernel<true> : kve_decode_attn_kernel<false>, dim3((unsigned)(grid < 1 ? 1 : grid)), dim3(AT_THREADS), AT_SMEM_BYTES, st, a);
 }
 
 }  // namespace kve

@@ -1647,3 +1647,40 @@ def test_long_keep_lists(B, H, C, n, keep):
     cnt = kept.sum(1).astype(np.int32)
     want, _, _, _ = o.attn(q, K, V, C, nc, idx, cnt, b.bf16_to_bits(st.ksum_bf16[0]), b.bf16_to_bits(st.vsum_bf16[0]), hz.ATT["summary"], hz.SCALE)
     hz.check_output(b.bf16_to_bits(out), want, "long list")
+
+
+@pytest.mark.parametrize("C,n", [(1, 333), (2, 130), (4, 1000), (7, 500), (20, 700)])
+@pytest.mark.parametrize("page_perm", ["random", None, "pairs"])
+def test_attention_over_short_chunks_in_any_page_order(page_perm, C, n):
+    """Chunks below 32 tokens, many to a tile: pages scattered, in order (one copy for a run of them) and in runs of two; a page that
+    names nothing inside a run is flagged, and the rest is as before"""
+    b = _binding()
+    wl = wlm.CFG1.small(B=1, H=3, n=n, C=C, W=n // 3, agg="identity" if C == 1 else "mean", n_append=1, seed=18)
+    perm = page_perm
+    if page_perm == "pairs":
+        ids = np.arange(wl.S * wl.max_chunks + 2, dtype=np.int32)[:wl.S * wl.max_chunks // 2 * 2].reshape(-1, 2)
+        ids = ids[np.random.default_rng(1).permutation(len(ids))].reshape(-1)
+        perm = np.concatenate([ids, np.arange(len(ids), wl.S * wl.max_chunks, dtype=np.int32)]).reshape(1, wl.S, wl.max_chunks)
+    K, V = wlm.gen_kv(wl)
+    nc = wl.n_stale_chunks()
+    lw = b.LstmWeights(wlm.gen_lstm_weights(wl))
+    q = wlm.gen_q(wl)
+    k1, v1 = wlm.gen_new_tokens(wl)
+    o = kvo.Oracle("f64")
+    K1, V1 = (np.ascontiguousarray(np.concatenate(x, axis=1)) for x in ((K, k1), (V, v1)))
+    for attend in ("summary", "raw"):
+        st = make_store(wl, attend=attend, page_perm=perm)
+        load_kv(st, 0, K, V)
+        st.refresh(0, None, lw, 0.5)
+        out = st.decode_step(0, *(b.bits_to_bf16(np.ascontiguousarray(x)) for x in (k1[:, 0], v1[:, 0], q)))
+        idx, cnt = st.keep_idx[0].cpu().numpy(), st.keep_cnt[0].cpu().numpy()
+        want, _, _, _ = o.attn(q, K1, V1, C, nc, idx, cnt, b.bf16_to_bits(st.ksum_bf16[0]), b.bf16_to_bits(st.vsum_bf16[0]), hz.ATT[attend], hz.SCALE)
+        hz.check_output(b.bf16_to_bits(out), want, attend)
+        dense = st.decode_attn_dense(0, b.bits_to_bf16(q))
+        want, _, _ = o.attn_dense(q, K1, V1, hz.SCALE)
+        hz.check_output(b.bf16_to_bits(dense), want, "dense")
+        assert st.poll_status() == 0
+    st.page_table[0, 1, wl.max_chunks // 2] = -1
+    again = st.decode_attn_dense(0, b.bits_to_bf16(q))
+    assert st.poll_status() == -3
+    assert torch.equal(again[0], dense[0]) and torch.equal(again[2], dense[2])
