@@ -19,8 +19,8 @@
 //    size, shuffles, 64-bit addresses) and held everything back: 8 layers of 128 sequences x 330 rows 9.75 us a
 //    layer, 8.75 us so.  (With the page of every ROW looked up, 512 sequences x 1100 rows took 56.7 us, 5.0 TB/s;
 //    49.8 us now.)
-//  * While the predecessor on the stream still runs, the producer goes through its first tiles once on what the tables hold (a
-//    guess, repeated with the real values after the wait) and the consumers pull the guessed rows of two tiles into L2:
+//  * While the predecessor on the stream still runs, a warp goes through the CTA's first tiles on what the tables hold (a
+//    guess, which tells the producer after its wait where to look) and others pull the guessed rows of two tiles into L2:
 //    12.7 -> 11.4 us a layer in that setting.
 //  * Warps 0-7 (consumers) are two groups of four that take tiles in turn, 16 rows per warp.  (One group: 8.75 us a layer, two:
 //    8.2 us - a tile is ~1400 cycles of dependent steps, and two of them now run at a time.)  The logits q.k are eight
@@ -65,11 +65,13 @@ constexpr int AT_GWARPS = 4;                  // warps of a group
 constexpr int AT_CWARPS = AT_CGROUPS * AT_GWARPS;
 constexpr int AT_SUB = AT_TILE / AT_GWARPS;   // 16 rows per warp per tile: the rows of one m16n8k16 MMA
 constexpr int AT_PRODUCER = AT_CWARPS;        // warp ids
+constexpr int AT_GUESSER = 4;                 // consumer that guesses the first plan: the producer's scheduler, and no tile to prefetch
 constexpr int AT_THREADS = (AT_CWARPS + 2) * 32;
 constexpr int AT_STAGE_ELEMS = AT_TILE * D;   // bf16 elements of one K (or V) tile
 constexpr int AT_LANE_SEGS = 3;               // chunks a tile may touch for one lane to issue its copies
 constexpr int AT_SHORT_CHUNK = AT_TILE / (AT_LANE_SEGS - 1);      // that holds for all tiles with chunks of 32 tokens and more
 constexpr int AT_PREFETCH_TILES = 2;          // most tiles a CTA pulls into L2 before its predecessor has finished
+static_assert(AT_GUESSER % 4 == AT_PRODUCER % 4 && AT_GUESSER >= AT_PREFETCH_TILES && AT_GUESSER < AT_CWARPS, "the guessing warp");
 static_assert(AT_SUB == 16, "the logits of a warp's rows are one m16n8k16 tile");
 
 // shared-memory carve-up (bytes)
@@ -80,8 +82,9 @@ constexpr int AT_OFF_COMB = AT_OFF_Q + AT_STAGES * ROW_BYTES;                   
 constexpr int AT_OFF_INFO = AT_OFF_COMB + 2 * AT_CWARPS * ATTN_PARTIAL_FLOATS * 4;  // [stages] int4
 constexpr int AT_OFF_FINFO = AT_OFF_INFO + AT_STAGES * 16;                          // [2] int4
 constexpr int AT_OFF_BAR = AT_OFF_FINFO + 2 * 16;                                   // full[3], empty[3], ffull[2], fempty[2]
-constexpr int AT_SMEM_BYTES = AT_OFF_BAR + (2 * AT_STAGES + 4) * 8;
-static_assert(AT_OFF_COMB % 16 == 0 && AT_OFF_INFO % 16 == 0 && AT_OFF_BAR % 8 == 0, "alignment of the carve-up");
+constexpr int AT_OFF_GUESS = AT_OFF_BAR + (2 * AT_STAGES + 4) * 8;                  // [32] int4: the guessed first plan; a flag
+constexpr int AT_SMEM_BYTES = AT_OFF_GUESS + 32 * 16 + 16;
+static_assert(AT_OFF_COMB % 16 == 0 && AT_OFF_INFO % 16 == 0 && AT_OFF_BAR % 8 == 0 && AT_OFF_GUESS % 16 == 0, "alignment of the carve-up");
 
 int attn_smem_bytes() { return AT_SMEM_BYTES; }
 
@@ -235,6 +238,8 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
   uint64_t* empty = full + AT_STAGES;
   uint64_t* ffull = empty + AT_STAGES;
   uint64_t* fempty = ffull + 2;
+  int4* guess = reinterpret_cast<int4*>(smem + AT_OFF_GUESS);
+  volatile int* guessed = reinterpret_cast<volatile int*>(guess + 32);
 
   pdl_launch_dependents();
   const LayerView& v = a.v;
@@ -244,11 +249,9 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
   const uint32_t c = blockIdx.x, uk = (uint32_t)a.k;
   const uint32_t n_items = (uint32_t)v.S * uk, n_pieces = min(gridDim.x, n_items);
   const uint32_t i0 = piece_begin(c, n_items, n_pieces), i1 = piece_begin(c + 1, n_items, n_pieces);
-  if (i0 < i1) {
-    if (warp == AT_PRODUCER) prefetch_sequence_metadata(a, (int)(i0 / uk), lane);
-    else if (warp < AT_CWARPS) prefetch_first_tiles(a, i0, i1, warp, lane);
-  }
+  if (i0 < i1 && warp == AT_PRODUCER) prefetch_sequence_metadata(a, (int)(i0 / uk), lane);
   if (threadIdx.x == 0) {
+    *guessed = 0;
     for (int i = 0; i < AT_STAGES; ++i) {
       mbar_init(&full[i], 1);
       mbar_init(&empty[i], AT_CWARPS);
@@ -260,8 +263,8 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
     mbar_fence_init();
   }
   __syncthreads();
-  if (warp == AT_PRODUCER) {
-    // ================= producer warp =================
+  if (warp == AT_PRODUCER || warp == AT_GUESSER) {
+    // ================= producer warp (and, up to the first plan, a consumer that has nothing to do yet) =================
     // walks the CTA's parts in order, sequence by sequence; within a sequence the tiles [j, j_hi) that its parts in this CTA
     // cover (part p of a sequence with T tiles: tiles [p T / k, (p + 1) T / k))
     const int s_first = (int)(i0 / uk), s_last = i0 < i1 ? (int)((i1 - 1u) / uk) : s_first;
@@ -325,167 +328,180 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
       }
     };
 
-    // The first tiles are worked out twice: once from what the tables hold while the predecessor still runs - only a guess at
-    // where to look, and a way to have the code at hand - and again from the real values, when the look-ups of the
-    // length, the coverage, the keep count and the guessed page ids go out together.
+    // The first tiles are worked out twice: by a consumer warp from what the tables hold while the predecessor still runs - only
+    // a guess at where to look, and a way to have the code at hand - and by the producer from the real values, when the look-ups
+    // of the length, the coverage, the keep count and the guessed page ids go out together.  Without a predecessor there is no
+    // guess yet when the producer comes by, and it does not wait for one.  (The producer guessing first, in
+    // front of its own wait, and the rows' prefetch in front of the barrier below: 8 sequences behind a kernel of another library 8.4 us,
+    // 6.6 so; 128 x 330 rows 8.4 and 6.6; in chains of decode steps 0.1 us for it.)
     TilePlan cur, nxt;
     nxt.n = 0;
-#pragma unroll 1
-    for (int pass = 0; pass < 2; ++pass) {
-      if (pass == 1) {
-        pdl_wait();      // lengths, keep lists, summaries and the new token come from earlier kernels
-        KVE_STAMP(lane == 0, 1);
-      }
-      const int len_stored = load_hint(v.seq_len);
-      // chunks the keep list covers: the device's own count, so that a launch replayed from a CUDA graph follows the
-      // gate triggers that happened since it was captured (the launch argument is only the host's view at capture time)
-      const int listed = (a.mode == ATTN_DENSE) ? 0 : load_hint(v.n_listed);
-      const int keep_cnt = (a.mode == ATTN_DENSE || i0 >= i1) ? 0 : load_hint(v.keep_cnt + s_first);
-      if (pass == 1 && cur.n > 0) {
-        nxt = cur;
-#pragma unroll
-        for (int x = 0; x < AT_LANE_SEGS; ++x) nxt.page[x] = (nxt.list == 0 && x < nxt.n_seg) ? page_of(s_first, 0, nxt.c0 + x) : -1;
-      }
-      g = make_geometry(a, len_stored, listed);
-      s = s_first;
-      done = i0 >= i1;
-      if (!done) enter_sequence(keep_cnt);
-      make_plan(cur, pass == 1 && nxt.n > 0 ? &nxt : nullptr);
+    const bool real = warp == AT_PRODUCER;
+    if (real) {
+      pdl_wait();      // lengths, keep lists, summaries and the new token come from earlier kernels
+      KVE_STAMP(lane == 0, 1);
     }
-    if (a.k_new != nullptr && !g.appending && blockIdx.x == 0 && lane == 0) set_status(v.status, ERR_CAPACITY);   // cache full
+    const int len_stored = load_hint(v.seq_len);
+    // chunks the keep list covers: the device's own count, so that a launch replayed from a CUDA graph follows the
+    // gate triggers that happened since it was captured (the launch argument is only the host's view at capture time)
+    const int listed = (a.mode == ATTN_DENSE) ? 0 : load_hint(v.n_listed);
+    const int keep_cnt = (a.mode == ATTN_DENSE || done) ? 0 : load_hint(v.keep_cnt + s_first);
+    if (real && !done && __shfl_sync(0xffffffffu, *guessed, 0) != 0) {
+      __threadfence_block();
+      const int4 gs = guess[lane];
+      nxt.n = 1;
+      nxt.list = gs.x; nxt.c0 = gs.y; nxt.n_seg = gs.z;
+#pragma unroll
+      for (int x = 0; x < AT_LANE_SEGS; ++x) nxt.page[x] = (nxt.list == 0 && x < nxt.n_seg) ? page_of(s_first, 0, nxt.c0 + x) : -1;
+    }
+    g = make_geometry(a, len_stored, listed);
+    if (!done) enter_sequence(keep_cnt);
+    make_plan(cur, nxt.n > 0 ? &nxt : nullptr);
+    if (!real) {
+      if (cur.n > 0) {
+        guess[lane] = make_int4(cur.list, cur.c0, cur.n_seg, 0);
+        __threadfence_block();
+        __syncwarp();
+        if (lane == 0) *guessed = 1;
+      }
+    } else {
+      if (a.k_new != nullptr && !g.appending && blockIdx.x == 0 && lane == 0) set_status(v.status, ERR_CAPACITY);   // cache full
 
-    // The copies of tile i of the batch: lane i waits for the stage, publishes the tile's description and issues one K and one V
-    // copy per chunk the tile touches, all from its own registers; the lanes take turns.  Chunks so short that a tile may
-    // have more than AT_LANE_SEGS of them: the whole warp, 32 chunks at a time, their pages `pg` looked up a tile ahead, and chunks
-    // that follow one another in the pool (pages dealt out in order) in one copy.  (One copy per chunk, looked up when its
-    // turn came: 60 sequences x 2000 rows in chunks of one token 48.8 us, 17.5 so with the pages in order, 43.3 scattered; 128 x 4160 in
-    // chunks of 4 and 16 tokens 71 -> 66 and 51 -> 48.)  False on a timed-out wait.
-    auto look_up = [&](const TilePlan& p, int i, int (&pg)[2]) {
-      const int n_seg = __shfl_sync(0xffffffffu, p.n_seg, i), c0 = __shfl_sync(0xffffffffu, p.c0, i), list = __shfl_sync(0xffffffffu, p.list, i);
+      // The copies of tile i of the batch: lane i waits for the stage, publishes the tile's description and issues one K and one V
+      // copy per chunk the tile touches, all from its own registers; the lanes take turns.  Chunks so short that a tile may
+      // have more than AT_LANE_SEGS of them: the whole warp, 32 chunks at a time, their pages `pg` looked up a tile ahead, and chunks
+      // that follow one another in the pool (pages dealt out in order) in one copy.  (One copy per chunk, looked up when its
+      // turn came: 60 sequences x 2000 rows in chunks of one token 48.8 us, 17.5 so with the pages in order, 43.3 scattered; 128 x 4160 in
+      // chunks of 4 and 16 tokens 71 -> 66 and 51 -> 48.)  False on a timed-out wait.
+      auto look_up = [&](const TilePlan& p, int i, int (&pg)[2]) {
+        const int n_seg = __shfl_sync(0xffffffffu, p.n_seg, i), c0 = __shfl_sync(0xffffffffu, p.c0, i), list = __shfl_sync(0xffffffffu, p.list, i);
 #pragma unroll
-      for (int h = 0; h < 2; ++h) pg[h] = n_seg > AT_LANE_SEGS && lane + 32 * h < n_seg ? page_of(p.s, list, c0 + lane + 32 * h) : -1;
-    };
-    int it = 0;
-    auto issue = [&](const TilePlan& p, int i, const int (&pg)[2]) -> bool {
-      const int stage = it % AT_STAGES, round = it / AT_STAGES;
-      ++it;
-      uint16_t *kd = Ks + stage * AT_STAGE_ELEMS, *vd = Vs + stage * AT_STAGE_ELEMS;
-      const bool with_new = i == p.i_new;
-      bool ok = true;
-      if (lane == i) {
-        ok = round == 0 || mbar_wait_bounded(&empty[stage], (round - 1) & 1);
-        if (ok) {
-          info[stage] = make_int4(p.s, p.rows, p.flags, p.list);
-          const bool with_q = (p.flags & TF_NEW) != 0;
-          mbar_arrive_expect_tx(&full[stage], (uint32_t)p.rows * 2u * ROW_BYTES + (with_q ? (uint32_t)ROW_BYTES : 0u));      // release: whoever sees the phase sees the description
-          if (p.n_seg > 0 && p.n_seg <= AT_LANE_SEGS) {
-            int r = p.row0 - p.c0 * v.C, dst = 0, rest = p.rows - (with_new ? 1 : 0);
+        for (int h = 0; h < 2; ++h) pg[h] = n_seg > AT_LANE_SEGS && lane + 32 * h < n_seg ? page_of(p.s, list, c0 + lane + 32 * h) : -1;
+      };
+      int it = 0;
+      auto issue = [&](const TilePlan& p, int i, const int (&pg)[2]) -> bool {
+        const int stage = it % AT_STAGES, round = it / AT_STAGES;
+        ++it;
+        uint16_t *kd = Ks + stage * AT_STAGE_ELEMS, *vd = Vs + stage * AT_STAGE_ELEMS;
+        const bool with_new = i == p.i_new;
+        bool ok = true;
+        if (lane == i) {
+          ok = round == 0 || mbar_wait_bounded(&empty[stage], (round - 1) & 1);
+          if (ok) {
+            info[stage] = make_int4(p.s, p.rows, p.flags, p.list);
+            const bool with_q = (p.flags & TF_NEW) != 0;
+            mbar_arrive_expect_tx(&full[stage], (uint32_t)p.rows * 2u * ROW_BYTES + (with_q ? (uint32_t)ROW_BYTES : 0u));      // release: whoever sees the phase sees the description
+            if (p.n_seg > 0 && p.n_seg <= AT_LANE_SEGS) {
+              int r = p.row0 - p.c0 * v.C, dst = 0, rest = p.rows - (with_new ? 1 : 0);
 #pragma unroll
-            for (int x = 0; x < AT_LANE_SEGS; ++x) {
-              const int len = min(v.C - r, rest);
-              if (len > 0) {
-                int page = p.page[x];
-                if (page < 0 || page >= v.n_pages) { set_status(v.status, ERR_CAPACITY); page = 0; }
-                const long long off = ((long long)page * v.C + r) * D;
-                bulk_g2s(kd + dst * D, v.k_pages + off, (uint32_t)len * ROW_BYTES, &full[stage]);
-                bulk_g2s(vd + dst * D, v.v_pages + off, (uint32_t)len * ROW_BYTES, &full[stage]);
+              for (int x = 0; x < AT_LANE_SEGS; ++x) {
+                const int len = min(v.C - r, rest);
+                if (len > 0) {
+                  int page = p.page[x];
+                  if (page < 0 || page >= v.n_pages) { set_status(v.status, ERR_CAPACITY); page = 0; }
+                  const long long off = ((long long)page * v.C + r) * D;
+                  bulk_g2s(kd + dst * D, v.k_pages + off, (uint32_t)len * ROW_BYTES, &full[stage]);
+                  bulk_g2s(vd + dst * D, v.v_pages + off, (uint32_t)len * ROW_BYTES, &full[stage]);
+                }
+                dst += len; rest -= len; r = 0;
               }
-              dst += len; rest -= len; r = 0;
+            } else if (p.n_seg == 0 && p.rows > 0) {      // kept summary rows: one contiguous run per sequence
+              const long long off = ((long long)p.s * v.max_chunks + p.row0) * D;
+              bulk_g2s(kd, a.kkept + off, (uint32_t)p.rows * ROW_BYTES, &full[stage]);
+              bulk_g2s(vd, a.vkept + off, (uint32_t)p.rows * ROW_BYTES, &full[stage]);
             }
-          } else if (p.n_seg == 0 && p.rows > 0) {      // kept summary rows: one contiguous run per sequence
-            const long long off = ((long long)p.s * v.max_chunks + p.row0) * D;
-            bulk_g2s(kd, a.kkept + off, (uint32_t)p.rows * ROW_BYTES, &full[stage]);
-            bulk_g2s(vd, a.vkept + off, (uint32_t)p.rows * ROW_BYTES, &full[stage]);
+            if (with_new) {
+              bulk_g2s(kd + (p.rows - 1) * D, a.k_new + (long long)p.s * D, ROW_BYTES, &full[stage]);
+              bulk_g2s(vd + (p.rows - 1) * D, a.v_new + (long long)p.s * D, ROW_BYTES, &full[stage]);
+            }
+            if (with_q) bulk_g2s(Qs + stage * D, a.q + (long long)p.s * D, ROW_BYTES, &full[stage]);
+          } else {
+            set_status(v.status, ERR_TIMEOUT);
           }
-          if (with_new) {
-            bulk_g2s(kd + (p.rows - 1) * D, a.k_new + (long long)p.s * D, ROW_BYTES, &full[stage]);
-            bulk_g2s(vd + (p.rows - 1) * D, a.v_new + (long long)p.s * D, ROW_BYTES, &full[stage]);
+        }
+        ok = __shfl_sync(0xffffffffu, (int)ok, i) != 0;
+        if constexpr (SHORT) {
+          const int n_seg = __shfl_sync(0xffffffffu, p.n_seg, i);
+          if (ok && n_seg > AT_LANE_SEGS) {
+            const int row0 = __shfl_sync(0xffffffffu, p.row0, i), c0 = __shfl_sync(0xffffffffu, p.c0, i);
+            const int rows = __shfl_sync(0xffffffffu, p.rows, i) - (with_new ? 1 : 0);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              if (32 * h >= n_seg) break;
+              TileSegment sg = tile_segment(row0, rows, v.C, c0 + lane + 32 * h);
+              if (lane + 32 * h >= n_seg) sg.len = 0;
+              int page = pg[h];
+              if (sg.len > 0 && (page < 0 || page >= v.n_pages)) { set_status(v.status, ERR_CAPACITY); page = 0; }
+              const long long row = (long long)page * v.C + sg.r;      // of the pool
+              const long long end = row + sg.len, end_before = __shfl_up_sync(0xffffffffu, end, 1);
+              const bool head = sg.len > 0 && (lane == 0 || row != end_before);
+              const unsigned heads = __ballot_sync(0xffffffffu, head), live = __ballot_sync(0xffffffffu, sg.len > 0);      // live: the first lanes
+              const unsigned above = lane == 31 ? 0u : heads & ~((2u << lane) - 1u);
+              const int last = (above ? __ffs(above) - 1 : __popc(live)) - 1;      // last chunk of the run that starts here
+              const int run = __shfl_sync(0xffffffffu, sg.dst + sg.len, last & 31) - sg.dst;
+              if (head) {
+                bulk_g2s(kd + sg.dst * D, v.k_pages + row * D, (uint32_t)run * ROW_BYTES, &full[stage]);
+                bulk_g2s(vd + sg.dst * D, v.v_pages + row * D, (uint32_t)run * ROW_BYTES, &full[stage]);
+              }
+            }
+            __syncwarp();
           }
-          if (with_q) bulk_g2s(Qs + stage * D, a.q + (long long)p.s * D, ROW_BYTES, &full[stage]);
+        }
+        return ok;
+      };
+      bool ok = true;
+      int pg[2] = {-1, -1}, pg_next[2] = {-1, -1};
+      if (SHORT && cur.n > 0) look_up(cur, 0, pg);
+      while (ok && cur.n > 0) {
+        for (int i = 0; ok && i < cur.n; ++i) {
+          if (i == cur.n - 1) make_plan(nxt, nullptr);      // its look-ups run while this batch's last copies are issued
+          if constexpr (SHORT) {
+            if (i < cur.n - 1) look_up(cur, i + 1, pg_next);
+            else if (nxt.n > 0) look_up(nxt, 0, pg_next);
+          }
+          ok = issue(cur, i, pg);
+          if constexpr (SHORT) { pg[0] = pg_next[0]; pg[1] = pg_next[1]; }
+          KVE_STAMP(it == 1 && lane == 0, 2);
+        }
+        if (cur.i_new >= 0) {
+          if (cur.new_page >= 0 && cur.new_page < v.n_pages)
+            *(reinterpret_cast<uint4*>((lane >> 4 ? v.v_pages : v.k_pages) + ((long long)cur.new_page * v.C + (g.n - 1 - (int)a.by_c.div((uint32_t)(g.n - 1)) * v.C)) * D) + (lane & 15)) = cur.new_row;
+          else if (lane == 0) set_status(v.status, ERR_CAPACITY);
+        }
+        cur = nxt;
+      }
+      // a description without a tile takes a stage of its own (no copies): that is how the consumers learn that they are done
+      if (ok && lane == 0) {
+        const int stage = it % AT_STAGES, round = it / AT_STAGES;
+        if (round == 0 || mbar_wait_bounded(&empty[stage], (round - 1) & 1)) {
+          info[stage] = make_int4(-1, 0, TF_END, 0);
+          mbar_arrive(&full[stage]);
         } else {
           set_status(v.status, ERR_TIMEOUT);
         }
       }
-      ok = __shfl_sync(0xffffffffu, (int)ok, i) != 0;
-      if constexpr (SHORT) {
-        const int n_seg = __shfl_sync(0xffffffffu, p.n_seg, i);
-        if (ok && n_seg > AT_LANE_SEGS) {
-          const int row0 = __shfl_sync(0xffffffffu, p.row0, i), c0 = __shfl_sync(0xffffffffu, p.c0, i);
-          const int rows = __shfl_sync(0xffffffffu, p.rows, i) - (with_new ? 1 : 0);
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            if (32 * h >= n_seg) break;
-            TileSegment sg = tile_segment(row0, rows, v.C, c0 + lane + 32 * h);
-            if (lane + 32 * h >= n_seg) sg.len = 0;
-            int page = pg[h];
-            if (sg.len > 0 && (page < 0 || page >= v.n_pages)) { set_status(v.status, ERR_CAPACITY); page = 0; }
-            const long long row = (long long)page * v.C + sg.r;      // of the pool
-            const long long end = row + sg.len, end_before = __shfl_up_sync(0xffffffffu, end, 1);
-            const bool head = sg.len > 0 && (lane == 0 || row != end_before);
-            const unsigned heads = __ballot_sync(0xffffffffu, head), live = __ballot_sync(0xffffffffu, sg.len > 0);      // live: the first lanes
-            const unsigned above = lane == 31 ? 0u : heads & ~((2u << lane) - 1u);
-            const int last = (above ? __ffs(above) - 1 : __popc(live)) - 1;      // last chunk of the run that starts here
-            const int run = __shfl_sync(0xffffffffu, sg.dst + sg.len, last & 31) - sg.dst;
-            if (head) {
-              bulk_g2s(kd + sg.dst * D, v.k_pages + row * D, (uint32_t)run * ROW_BYTES, &full[stage]);
-              bulk_g2s(vd + sg.dst * D, v.v_pages + row * D, (uint32_t)run * ROW_BYTES, &full[stage]);
-            }
-          }
-          __syncwarp();
+      // Fused append: the length advances as soon as every CTA has read the old one, which is what the tickets count (nothing else
+      // in the launch reads it; later launches wait for this one to complete).
+      if (g.appending) {
+        __syncwarp();
+        int last = 0;
+        if (lane == 0) {
+          int arrived;
+          asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(arrived) : "l"(a.ticket) : "memory");
+          last = arrived == (int)gridDim.x - 1;
+        }
+        last = __shfl_sync(0xffffffffu, last, 0);
+        if (last) {
+          for (int b = lane; b < v.B; b += 32) v.seq_len[b] = g.n;
+          if (lane == 0) *a.ticket = 0;      // clean for the next launch
         }
       }
-      return ok;
-    };
-    bool ok = true;
-    int pg[2] = {-1, -1}, pg_next[2] = {-1, -1};
-    if (SHORT && cur.n > 0) look_up(cur, 0, pg);
-    while (ok && cur.n > 0) {
-      for (int i = 0; ok && i < cur.n; ++i) {
-        if (i == cur.n - 1) make_plan(nxt, nullptr);      // its look-ups run while this batch's last copies are issued
-        if constexpr (SHORT) {
-          if (i < cur.n - 1) look_up(cur, i + 1, pg_next);
-          else if (nxt.n > 0) look_up(nxt, 0, pg_next);
-        }
-        ok = issue(cur, i, pg);
-        if constexpr (SHORT) { pg[0] = pg_next[0]; pg[1] = pg_next[1]; }
-        KVE_STAMP(it == 1 && lane == 0, 2);
-      }
-      if (cur.i_new >= 0) {
-        if (cur.new_page >= 0 && cur.new_page < v.n_pages)
-          *(reinterpret_cast<uint4*>((lane >> 4 ? v.v_pages : v.k_pages) + ((long long)cur.new_page * v.C + (g.n - 1 - (int)a.by_c.div((uint32_t)(g.n - 1)) * v.C)) * D) + (lane & 15)) = cur.new_row;
-        else if (lane == 0) set_status(v.status, ERR_CAPACITY);
-      }
-      cur = nxt;
+      KVE_STAMP(lane == 0, 6);
     }
-    // a description without a tile takes a stage of its own (no copies): that is how the consumers learn that they are done
-    if (ok && lane == 0) {
-      const int stage = it % AT_STAGES, round = it / AT_STAGES;
-      if (round == 0 || mbar_wait_bounded(&empty[stage], (round - 1) & 1)) {
-        info[stage] = make_int4(-1, 0, TF_END, 0);
-        mbar_arrive(&full[stage]);
-      } else {
-        set_status(v.status, ERR_TIMEOUT);
-      }
-    }
-    // Fused append: the length advances as soon as every CTA has read the old one, which is what the tickets count (nothing else
-    // in the launch reads it; later launches wait for this one to complete).
-    if (g.appending) {
-      __syncwarp();
-      int last = 0;
-      if (lane == 0) {
-        int arrived;
-        asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(arrived) : "l"(a.ticket) : "memory");
-        last = arrived == (int)gridDim.x - 1;
-      }
-      last = __shfl_sync(0xffffffffu, last, 0);
-      if (last) {
-        for (int b = lane; b < v.B; b += 32) v.seq_len[b] = g.n;
-        if (lane == 0) *a.ticket = 0;      // clean for the next launch
-      }
-    }
-    KVE_STAMP(lane == 0, 6);
-  } else if (warp < AT_CWARPS) {
+  }
+  if (warp < AT_CWARPS) {
     // ================= consumer warps =================
+    if (i0 < i1) prefetch_first_tiles(a, i0, i1, warp, lane);
     pdl_wait();
     const float sl2 = a.scale * 1.44269504088896340736f;   // logits kept in log2 units
     const int gwarp = warp % AT_GWARPS;
@@ -606,7 +622,7 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
         ++n_flush;
       }
     }
-  } else {
+  } else if (warp > AT_PRODUCER) {
     // ================= merger warp =================
     pdl_wait();
     for (int f = 0;; ++f) {
