@@ -136,8 +136,9 @@ def load_library(build_if_missing: bool = True) -> C.CDLL:
 
 
 # Marshalling is on the path of every decode step (a token of a small cache takes the GPU 7 us), so it passes plain integers and
-# floats (argtypes converts them), asks torch for the raw stream handle and compares shapes as tuples: set_len and 7 decode
-# steps issued call by call 172 us with ctypes objects, stream objects and numpy scalars, 119 us so.
+# floats (argtypes converts them), asks torch for the raw stream handle and compares shapes as tuples: with ctypes objects, stream
+# objects and numpy scalars set_len and 7 decode steps issued call by call took 1.4 times as long (172 and 119 us on one machine;
+# host times differ by a fifth between machines).
 _BF16 = torch.bfloat16
 _DEFAULT_SCALE = 1.0 / 128.0 ** 0.5
 

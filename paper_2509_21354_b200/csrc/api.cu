@@ -109,8 +109,9 @@ Carve carve(const kvE_config& c) {
   size_t p_floats = S * max_chunks * 4 * (size_t)c.d_g;
   if (c.agg == KVE_AGG_TOKEN_MLP && 2 * S * max_chunks * (size_t)c.d_sum > p_floats) p_floats = 2 * S * max_chunks * (size_t)c.d_sum;
   k.off_P = o;        o = align_up(o + p_floats * sizeof(float));
-  // h_t of every gated (sequence, chunk) of one kvE_gate call, [S max_chunks][d_g]: what the score head reads
-  k.off_H = o;        o = align_up(o + S * max_chunks * (size_t)c.d_g * sizeof(float));
+  // partial sums of w_s . h_t of every gated (sequence, chunk) of one kvE_gate call, [S max_chunks][d_g / 8], one per warp of the
+  // recurrence: what its score head adds up
+  k.off_H = o;        o = align_up(o + S * max_chunks * (size_t)(c.d_g / 8) * sizeof(float));
   // attention partial records: the one of (sequence s, CTA c) at s + c, at most ATTN_GRID_LIMIT CTAs
   k.off_partials = o; o = align_up(o + (S + ATTN_GRID_LIMIT) * ATTN_PARTIAL_FLOATS * sizeof(float));
   k.off_counters = o; o = align_up(o + S * sizeof(int32_t));
@@ -618,7 +619,10 @@ int kvE_adopt_device_state(kvE_store* st, int layer, void* stream) {
 // is then hidden, and the second launches of MLP, projection and recurrence and the slower recurrence are paid.  Measured, one
 // range -> two (us a step): 512 sequences x 121 chunks of 128, MLP 1055 -> 1010; 128 x 121 of 128, MLP 370 -> 350; 256 x 240
 // of 32, MLP 604 -> 562; 512 x 56 of 64, mean 344 -> 333; 256 x 120 of 64, mean 364 -> 340, MLP 407 -> 393; below the lines:
-// 256 x 56 of 64 with 28 us to hide, mean 194 -> 189, MLP 218 -> 226; 32 x 250 of 64, mean, 33 us: 356 -> 364.
+// 256 x 56 of 64 with 28 us to hide, mean 194 -> 189, MLP 218 -> 226; 32 x 250 of 64, mean, 33 us: 356 -> 364.  (The figures of the
+// recurrence are those of d_g = 256; at 64 and 128 it is faster, which makes x too small rather than too large.  The rule over 240 settings
+// - d_g 64, 128, 256; 8 to 1024 sequences of 4160 to 16512 tokens in chunks of 32 to 512; mean and MLP - and 28 with three planes: never more than
+// 2 % behind one range, up to 23 % ahead of it, 128 x 127 of 128 at d_g = 64.)
 constexpr double REFRESH_HIDE_US = 40, REFRESH_HIDE_MLP_US = 60;
 
 static int first_range(const kvE_store* st, int nc, const kvE_lstm_weights* lw) {

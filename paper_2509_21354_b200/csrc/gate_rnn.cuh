@@ -1,6 +1,6 @@
-// Pieces shared by the LSTM recurrence kernels: launch arguments, cluster addressing, stores and bulk
-// copies into a peer CTA's shared memory that count bytes on the peer's mbarrier, bounded cluster
-// waits, the fast activations and the exact 3-way bf16 split of an fp32 value.
+// Pieces shared by the LSTM recurrence kernels: launch arguments, cluster addressing, bulk copies into a peer CTA's shared
+// memory that count bytes on the peer's mbarrier, bounded cluster waits, the fast activations and the exact 3-way bf16 split
+// of an fp32 value.
 #pragma once
 #include "common.cuh"
 #include "kernels.h"
@@ -32,18 +32,6 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t smem_addr, uint32_t ran
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(rank));
   return r;
-}
-// stores into the shared memory of a CTA of the cluster (address from mapa) that count their bytes
-// on an mbarrier of the same CTA when they land
-__device__ __forceinline__ void st_async_u32(uint32_t addr, uint32_t val, uint32_t bar) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.u32 [%0], %1, [%2];" ::"r"(addr), "r"(val),
-               "r"(bar)
-               : "memory");
-}
-__device__ __forceinline__ void st_async_v4(uint32_t addr, const uint4& v, uint32_t bar) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.u32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr),
-               "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar)
-               : "memory");
 }
 // bulk copy from this CTA's shared memory into a peer's (addresses from mapa), bytes counted on the peer's barrier
 __device__ __forceinline__ void bulk_s2cluster(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
