@@ -1686,3 +1686,23 @@ def test_attention_over_short_chunks_in_any_page_order(page_perm, C, n):
     again = st.decode_attn_dense(0, b.bits_to_bf16(q))
     assert st.poll_status() == -3
     assert torch.equal(again[0], dense[0]) and torch.equal(again[2], dense[2])
+
+
+@pytest.mark.parametrize("C", [2, 8, 20])
+def test_device_positioned_trigger_with_short_chunks(C):
+    """kvE_refresh_next finds its chunk on the device with chunks below 32 tokens too: the summary is the one of the call by position"""
+    b = _binding()
+    wl = wlm.CFG1.small(B=2, H=3, n=300, C=C, W=40, n_append=C, seed=20)
+    K, V = wlm.gen_kv(wl, n=wl.n + C)
+    lw = b.LstmWeights(wlm.gen_lstm_weights(wl))
+    nc = wl.n_stale_chunks()
+    st = make_store(wl)
+    load_kv(st, 0, K[:, :wl.n], V[:, :wl.n])
+    st.refresh(0, None, lw, 0.5)
+    st.append(0, b.bits_to_bf16(np.ascontiguousarray(K[:, wl.n:])), b.bits_to_bf16(np.ascontiguousarray(V[:, wl.n:])))
+    st.refresh_next(0, None, lw, 0.5)
+    assert st.poll_status() == 0 and st.layer_state()["n_gated"] == nc + 1
+    got = [st.ksum_f32[0, :, :nc + 1].clone(), st.vsum_f32[0, :, :nc + 1].clone()]
+    st.summarize_chunks(0, 0, nc + 1)
+    assert torch.equal(got[0], st.ksum_f32[0, :, :nc + 1]) and torch.equal(got[1], st.vsum_f32[0, :, :nc + 1])
+    assert got[0][:, nc].abs().max() > 0
