@@ -592,11 +592,6 @@ __global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerVi
   }
   const int my_tiles = n_tiles > (int)blockIdx.x ? (n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
   const int n_halves = (d_sum + 127) / 128, n_slices = d_sum / MT_SLICE;
-  // The second layer's sum is taken in two parts, each overwriting Y and added up by the output warps (POOLED has its accumulator
-  // for the small planes instead): the tensor core cuts off what lies
-  // below the last bit of the sum at each of its steps.  Key summaries of 64 x 61 chunks, rms against 64 bits: 2.7e-7 in one part, 1.5e-7 in
-  // two (d_sum 64: 8.8e-8 and 5.8e-8); 512 x 121 chunks 86 -> 92 us.
-  const int y_parts = POOLED ? 1 : 2, part_slices = n_slices / y_parts;      // (n_slices is even)
   auto summary_row = [&](int unit) -> long long {
     const int s = (int)by_range.div((uint32_t)unit);
     return (long long)s * v.max_chunks + t0 + (unit - s * n_range);
@@ -689,27 +684,12 @@ __global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerVi
         if (lane == 0) mbar_arrive(a_full);
       }
       if (k < 0) continue;
-      float y[2][32];
-      ok = __all_sync(0xffffffffu, mbar_wait_bounded(y_full, (uint32_t)((k * y_parts) & 1)));
+      ok = __all_sync(0xffffffffu, mbar_wait_bounded(y_full, (uint32_t)(k & 1)));
       if (!ok) break;
       umma::fence_after_sync();
+      float y[2][32];
       umma::tmem_ld32(tmem + MT_TMEM_Y + c0 + lane_bits, y[0]);
       umma::tmem_ld32(tmem + MT_TMEM_Y + c0 + 32 + lane_bits, y[1]);
-      if (y_parts == 2) {
-        umma::fence_before_sync();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(y_free);
-        ok = __all_sync(0xffffffffu, mbar_wait_bounded(y_full, (uint32_t)((k * y_parts + 1) & 1)));
-        if (!ok) break;
-        umma::fence_after_sync();
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          float more[16];
-          umma::tmem_ld16(tmem + MT_TMEM_Y + c0 + 16 * q + lane_bits, more);
-#pragma unroll
-          for (int e = 0; e < 16; ++e) y[q >> 1][(q & 1) * 16 + e] += more[e];
-        }
-      }
       if constexpr (POOLED) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -742,7 +722,7 @@ __global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerVi
     const uint32_t a_base = smem_u32(As), w1_base = smem_u32(W1s), w2_base = smem_u32(W2s);
     constexpr uint32_t idesc2 = umma::instr_desc_bf16(MT_M, D);
     const int n_l1 = POOLED ? 0 : my_tiles * n_halves, n_l2 = my_tiles * n_slices;
-    int l1 = 0, l2 = 0, l1_tile = 0, l1_half = 0, l2_tile = 0, l2_slice = 0, part_slice = 0, n_parts = 0;      // n_parts: parts of Y begun before
+    int l1 = 0, l2 = 0, l1_tile = 0, l1_half = 0, l2_tile = 0, l2_slice = 0;
     uint32_t idle = 0;
     while (l2 < n_l2) {
       bool progress = false;
@@ -768,9 +748,9 @@ __global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerVi
         if (++l1_half == n_halves) { l1_half = 0; ++l1_tile; umma::commit(a_free); }
         progress = true;
       }
-      // layer 2: 32 hidden units; the first slice of a part overwrites Y, once that has been read
+      // layer 2: 32 hidden units; the first slice of a tile overwrites Y, once that has been read
       if (mbar_test_wait(&act_full[l2_slice & 1], (uint32_t)(((l2_tile * n_slices + l2_slice) >> 1) & 1)) &&
-          (part_slice > 0 || n_parts == 0 || mbar_test_wait(y_free, (uint32_t)((n_parts - 1) & 1)))) {
+          (l2_slice > 0 || l2_tile == 0 || mbar_test_wait(y_free, (uint32_t)((l2_tile - 1) & 1)))) {
         umma::fence_after_sync();
         const uint32_t act = tmem + MT_TMEM_ACT + (l2_slice & 1) * MT_ACT_COLS;
         const uint32_t wb = w2_base + (l2_slice >> 1) * MT_PLANE_KB_BYTES + (l2_slice & 1) * 64;
@@ -779,11 +759,10 @@ __global__ void __launch_bounds__(MT_THREADS, 1) kve_chunk_mlp_tc_kernel(LayerVi
 #pragma unroll
           for (int s = 0; s < 2; ++s)
             umma::mma_bf16_ts(tmem + (POOLED && pl ? MT_TMEM_YLO : MT_TMEM_Y), act + pl * (MT_SLICE / 2) + s * 8, umma::smem_desc(wb + s * 32),
-                              idesc2, !(part_slice == 0 && s == 0 && (pl == 2 || (POOLED && pl == 0))));
+                              idesc2, !(l2_slice == 0 && s == 0 && (pl == 2 || (POOLED && pl == 0))));
         umma::commit(&act_free[l2_slice & 1]);
         ++l2;
-        if (++part_slice == part_slices) { part_slice = 0; ++n_parts; umma::commit(y_full); }
-        if (++l2_slice == n_slices) { l2_slice = 0; ++l2_tile; }
+        if (++l2_slice == n_slices) { l2_slice = 0; ++l2_tile; umma::commit(y_full); }
         progress = true;
       }
       if (progress) idle = 0;
