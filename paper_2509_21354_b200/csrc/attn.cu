@@ -82,7 +82,7 @@ constexpr int AT_OFF_COMB = AT_OFF_Q + AT_STAGES * ROW_BYTES;                   
 constexpr int AT_OFF_INFO = AT_OFF_COMB + 2 * AT_CWARPS * ATTN_PARTIAL_FLOATS * 4;  // [stages] int4
 constexpr int AT_OFF_FINFO = AT_OFF_INFO + AT_STAGES * 16;                          // [2] int4
 constexpr int AT_OFF_BAR = AT_OFF_FINFO + 2 * 16;                                   // full[3], empty[3], ffull[2], fempty[2]
-constexpr int AT_OFF_GUESS = AT_OFF_BAR + (2 * AT_STAGES + 4) * 8;                  // [32] int4: the guessed first plan; a flag
+constexpr int AT_OFF_GUESS = AT_OFF_BAR + (2 * AT_STAGES + 4) * 8;                  // [32] int4: the guessed first plan; its barrier
 constexpr int AT_SMEM_BYTES = AT_OFF_GUESS + 32 * 16 + 16;
 static_assert(AT_OFF_COMB % 16 == 0 && AT_OFF_INFO % 16 == 0 && AT_OFF_BAR % 8 == 0 && AT_OFF_GUESS % 16 == 0, "alignment of the carve-up");
 
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
   uint64_t* ffull = empty + AT_STAGES;
   uint64_t* fempty = ffull + 2;
   int4* guess = reinterpret_cast<int4*>(smem + AT_OFF_GUESS);
-  volatile int* guessed = reinterpret_cast<volatile int*>(guess + 32);
+  uint64_t* guessed = reinterpret_cast<uint64_t*>(guess + 32);
 
   pdl_launch_dependents();
   const LayerView& v = a.v;
@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
   const uint32_t i0 = piece_begin(c, n_items, n_pieces), i1 = piece_begin(c + 1, n_items, n_pieces);
   if (i0 < i1 && warp == AT_PRODUCER) prefetch_sequence_metadata(a, (int)(i0 / uk), lane);
   if (threadIdx.x == 0) {
-    *guessed = 0;
+    mbar_init(guessed, 1);
     for (int i = 0; i < AT_STAGES; ++i) {
       mbar_init(&full[i], 1);
       mbar_init(&empty[i], AT_CWARPS);
@@ -346,8 +346,7 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
     // gate triggers that happened since it was captured (the launch argument is only the host's view at capture time)
     const int listed = (a.mode == ATTN_DENSE) ? 0 : load_hint(v.n_listed);
     const int keep_cnt = (a.mode == ATTN_DENSE || done) ? 0 : load_hint(v.keep_cnt + s_first);
-    if (real && !done && __shfl_sync(0xffffffffu, *guessed, 0) != 0) {
-      __threadfence_block();
+    if (real && !done && __all_sync(0xffffffffu, mbar_test_wait(guessed, 0))) {
       const int4 gs = guess[lane];
       nxt.n = 1;
       nxt.list = gs.x; nxt.c0 = gs.y; nxt.n_seg = gs.z;
@@ -360,9 +359,8 @@ __global__ void __launch_bounds__(AT_THREADS, 2) kve_decode_attn_kernel(AttnArgs
     if (!real) {
       if (cur.n > 0) {
         guess[lane] = make_int4(cur.list, cur.c0, cur.n_seg, 0);
-        __threadfence_block();
         __syncwarp();
-        if (lane == 0) *guessed = 1;
+        if (lane == 0) mbar_arrive(guessed);      // release
       }
     } else {
       if (a.k_new != nullptr && !g.appending && blockIdx.x == 0 && lane == 0) set_status(v.status, ERR_CAPACITY);   // cache full
