@@ -12,57 +12,69 @@ constexpr int COMPACT_WARPS = 4;
 // rows ("compacted chunk tokens", Sec. 3.3: attention then fetches them with one bulk copy per 64 rows), lanes 0-15 the
 // K row, lanes 16-31 the V row, 16 bytes each, GATHER_ROWS loads in flight.  (As two kernels, one warp per sequence and then
 // one per 8 kept rows, a second launch and a round trip of the list through memory: 2.2 us more in a chain of small launches.)
-// A long list of one of few sequences is more than four warps should copy: there (gather == 0) this kernel writes the ids only
-// and the rows follow in a launch of their own.  (8 sequences x 1792 chunks: 26.5 us in one launch, 11.1 so; 60 x 1744:
-// 29.6 and 16.7; 128 x 3904, where every SM has a CTA: 109.5, 100.4 in one launch.  Loads of the scores a group of rounds ahead in all three.)
+// A long list is more than four warps should copy: there (GATHER false) this kernel writes the ids only, every warp those of its
+// round in a group whose scores were requested a group ahead, and the rows follow in a launch of their own.
+// (us, in one launch -> in two: 8 sequences x 448 chunks 9.1 -> 6.0, 8 x 1792 26.6 -> 8.6, 60 x 436 9.2 -> 7.4, 128 x 1952 57 -> 33,
+// 512 x 2000 97.5 -> 95.9; in one: 128 x 976 21.5, 512 x 1000 51.)
 constexpr int GATHER_ROWS = 8;
-constexpr int COMPACT_LONG = 256;      // chunks from which that pays, below half a CTA of four warps per SM
+constexpr int COMPACT_LONG = 256, COMPACT_VERY_LONG = 1024;      // chunks from which that pays: below half a CTA per SM, and always
 
-__global__ void __launch_bounds__(COMPACT_WARPS * 32) kve_compact_kernel(LayerView v, int n_chunks, float tau, int gather,
-                                                                        uint4* __restrict__ kkept, uint4* __restrict__ vkept) {
+template <bool GATHER>
+__global__ void __launch_bounds__(COMPACT_WARPS * 32) kve_compact_kernel(LayerView v, int n_chunks, float tau, uint4* __restrict__ kkept,
+                                                                        uint4* __restrict__ vkept) {
   pdl_launch_dependents();
   pdl_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int s = blockIdx.x;
   const long long sb = (long long)s * v.max_chunks;
-  const int is_v = lane >> 4, l16 = lane & 15;
-  const uint4* src = reinterpret_cast<const uint4*>(is_v ? v.vsum_bf16 : v.ksum_bf16) + l16;
-  uint4* dst = (is_v ? vkept : kkept) + l16;
   int base = 0;
-  float sc[COMPACT_WARPS], next[COMPACT_WARPS];      // scores of COMPACT_WARPS rounds, one for each warp to write, and of the rounds after them
-  auto load = [&](int t0, float (&x)[COMPACT_WARPS]) {
+  if constexpr (GATHER) {
+    const int is_v = lane >> 4, l16 = lane & 15;
+    const uint4* src = reinterpret_cast<const uint4*>(is_v ? v.vsum_bf16 : v.ksum_bf16) + l16;
+    uint4* dst = (is_v ? vkept : kkept) + l16;
+    for (int t0 = 0, round = 0; t0 < n_chunks; t0 += 32, ++round) {
+      const int t = t0 + lane;
+      const bool keep = (t < n_chunks) && (v.scores[sb + t] >= tau);
+      unsigned mask = __ballot_sync(0xffffffffu, keep);
+      const int kept = __popc(mask);
+      if (round % COMPACT_WARPS == warp) {
+        if (keep) v.keep_idx[sb + base + __popc(mask & ((1u << lane) - 1u))] = t;
+        for (int i = 0; i < kept; i += GATHER_ROWS) {
+          uint4 w[GATHER_ROWS];
+          unsigned m = mask;
 #pragma unroll
-    for (int r = 0; r < COMPACT_WARPS; ++r) x[r] = t0 + r * 32 + lane < n_chunks ? v.scores[sb + t0 + r * 32 + lane] : 0.f;
-  };
-  load(0, sc);
-  for (int t0 = 0; t0 < n_chunks; t0 += COMPACT_WARPS * 32) {
-    if (t0 + COMPACT_WARPS * 32 < n_chunks) load(t0 + COMPACT_WARPS * 32, next);
-    unsigned mask = 0;      // of this warp's round
-    int first = base, all = 0;
+          for (int r = 0; r < GATHER_ROWS; ++r) {
+            if (i + r < kept) w[r] = __ldg(src + (sb + t0 + __ffs(m) - 1) * 16);
+            m &= m - 1;
+          }
+          mask = m;
 #pragma unroll
-    for (int r = 0; r < COMPACT_WARPS; ++r) {
-      if (t0 + r * 32 >= n_chunks) break;
-      const unsigned m = __ballot_sync(0xffffffffu, t0 + r * 32 + lane < n_chunks && sc[r] >= tau);
-      if (r < warp) first += __popc(m);
-      if (r == warp) mask = m;
-      all += __popc(m);
-      sc[r] = next[r];
-    }
-    base += all;
-    const int mine0 = t0 + warp * 32, kept = __popc(mask);
-    if (mask >> lane & 1u) v.keep_idx[sb + first + __popc(mask & ((1u << lane) - 1u))] = mine0 + lane;
-    for (int i = 0; gather && i < kept; i += GATHER_ROWS) {
-      uint4 w[GATHER_ROWS];
-      unsigned m = mask;
-#pragma unroll
-      for (int r = 0; r < GATHER_ROWS; ++r) {
-        if (i + r < kept) w[r] = __ldg(src + (sb + mine0 + __ffs(m) - 1) * 16);
-        m &= m - 1;
+          for (int r = 0; r < GATHER_ROWS; ++r)
+            if (i + r < kept) dst[(sb + base + i + r) * 16] = w[r];
+        }
       }
-      mask = m;
+      base += kept;
+    }
+  } else {
+    float sc[COMPACT_WARPS], next[COMPACT_WARPS];
+    auto load = [&](int t0, float (&x)[COMPACT_WARPS]) {
 #pragma unroll
-      for (int r = 0; r < GATHER_ROWS; ++r)
-        if (i + r < kept) dst[(sb + first + i + r) * 16] = w[r];
+      for (int r = 0; r < COMPACT_WARPS; ++r) x[r] = t0 + r * 32 + lane < n_chunks ? v.scores[sb + t0 + r * 32 + lane] : 0.f;
+    };
+    load(0, sc);
+    for (int t0 = 0; t0 < n_chunks; t0 += COMPACT_WARPS * 32) {
+      load(t0 + COMPACT_WARPS * 32, next);
+      unsigned mask = 0;      // of this warp's round
+      int first = base;
+#pragma unroll
+      for (int r = 0; r < COMPACT_WARPS; ++r) {
+        const unsigned m = __ballot_sync(0xffffffffu, t0 + r * 32 + lane < n_chunks && sc[r] >= tau);
+        if (r < warp) first += __popc(m);
+        if (r == warp) mask = m;
+        base += __popc(m);
+        sc[r] = next[r];
+      }
+      if (mask >> lane & 1u) v.keep_idx[sb + first + __popc(mask & ((1u << lane) - 1u))] = t0 + warp * 32 + lane;
     }
   }
   for (int t = base + (int)threadIdx.x; t < v.max_chunks; t += COMPACT_WARPS * 32) v.keep_idx[sb + t] = -1;
@@ -112,9 +124,9 @@ static cudaError_t launch_keep_gather(const LayerView& v, int n_chunks, void* kk
 }
 
 cudaError_t launch_compact(const LayerView& v, int n_chunks, float tau, void* kkept, void* vkept, cudaStream_t st) {
-  const bool apart = n_chunks > COMPACT_LONG && 2 * v.S < sm_count();
-  const cudaError_t e = launch_pdl(kve_compact_kernel, dim3((unsigned)v.S), dim3(COMPACT_WARPS * 32), 0, st, v, n_chunks, tau, apart ? 0 : 1,
-                                   static_cast<uint4*>(kkept), static_cast<uint4*>(vkept));
+  const bool apart = n_chunks > COMPACT_VERY_LONG || (n_chunks > COMPACT_LONG && 2 * v.S < sm_count());
+  const cudaError_t e = launch_pdl(apart ? kve_compact_kernel<false> : kve_compact_kernel<true>, dim3((unsigned)v.S), dim3(COMPACT_WARPS * 32), 0, st,
+                                   v, n_chunks, tau, static_cast<uint4*>(kkept), static_cast<uint4*>(vkept));
   return e == cudaSuccess && apart ? launch_keep_gather(v, n_chunks, kkept, vkept, st) : e;
 }
 

@@ -1602,7 +1602,7 @@ def test_summaries_of_short_chunks(C, B, H, n, agg):
     assert torch.equal(st.ksum_f32, before)
 
 
-@pytest.mark.parametrize("B,H,C,n", [(1, 3, 1, 700), (1, 2, 2, 3000), (2, 40, 1, 400)])
+@pytest.mark.parametrize("B,H,C,n", [(1, 3, 1, 700), (1, 2, 2, 3000), (2, 40, 1, 400), (2, 40, 1, 1100)])
 @pytest.mark.parametrize("keep", [0.0, 0.4, 1.0])
 def test_long_keep_lists(B, H, C, n, keep):
     """Lists of more than 256 chunks, with few sequences and with many: ids, counts and the rows that attention reads"""
