@@ -110,7 +110,7 @@ typedef struct {
 
 typedef struct kvE_store kvE_store;
 
-/* Bytes of workspace the handle needs: the gate projection buffer and the score's partial sums of one kvE_gate call, the split-K partial records and tickets of
+/* Bytes of workspace the handle needs: the score's partial sums of one kvE_gate call, pooled activations of KVE_AGG_TOKEN_MLP, the split-K partial records and tickets of
  * the attention kernels (those of kvE_decode_attn_block only when cfg.max_query_tokens > 0), staging rows of the
  * host-buffer step, scratch of kvE_reclaim_pages.  0 if the geometry is not supported. */
 size_t kvE_workspace_bytes(const kvE_config* cfg);
@@ -330,7 +330,8 @@ int kvE_layer_state(const kvE_store* st, int layer, int* n_tokens, int* n_summar
  * events on the launch stream (events are created on the first enable; no device memory).
  * kvE_profile_read synchronises the device and writes, per kernel id, the duration in microseconds
  * of that kernel's most recent launch, or -1 if it has not run since profiling was enabled.  While enabled,
- * kvE_refresh takes all chunks in one range, so that a duration is that of the kernel alone. */
+ * kvE_refresh takes all chunks in one range, so that a duration is that of the kernel alone.  KVE_K_GATE_RNN is the
+ * whole gate, the input projection included (KVE_K_GATE_PROJ: no kernel of its own, always -1). */
 enum { KVE_K_APPEND = 0, KVE_K_CHUNK_MEAN, KVE_K_CHUNK_MLP, KVE_K_GATE_PROJ, KVE_K_GATE_RNN, KVE_K_COMPACT,
        KVE_K_ATTN, KVE_K_ATTN_DENSE, KVE_K_ATTN_BLOCK, KVE_K_COUNT };
 int kvE_profile(kvE_store* st, int enable);

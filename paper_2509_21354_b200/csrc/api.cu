@@ -28,11 +28,12 @@ struct kvE_store {
   int device = -1;       // the device that was current at kvE_create: owner of every buffer; calls check it
   int S, max_chunks;
   // workspace carve-up (byte offsets)
-  size_t off_P, off_H, off_partials, off_counters, off_stage, off_reclaim, off_ticket, off_block, off_kept_k, off_kept_v, off_listed, ws_needed;
+  size_t off_pooled, off_H, off_partials, off_counters, off_stage, off_reclaim, off_ticket, off_block, off_kept_k, off_kept_v, off_listed, ws_needed;
   int attn_grid_max;     // most CTAs an attention launch uses (two per SM of the handle's device): sizes the partial records
   // block-of-queries attention: tensor maps over the page pools and the summary store (encoded at
   // create when cfg.max_query_tokens > 0), rows per page box, split cap the workspace was sized for
   alignas(64) unsigned char block_maps[4 * ATTN_BLOCK_MAP_BYTES];
+  alignas(64) unsigned char gate_maps[2 * GATE_MAP_BYTES];
   bool block_ready = false;
   int block_hp = 0, block_split_cap = 1;
   std::vector<LayerState> layers;
@@ -87,7 +88,7 @@ int check_config(const kvE_config* c) {
 }
 
 struct Carve {
-  size_t off_P, off_H, off_partials, off_counters, off_stage, off_reclaim, off_ticket, off_block, off_kept_k, off_kept_v, off_listed, total;
+  size_t off_pooled, off_H, off_partials, off_counters, off_stage, off_reclaim, off_ticket, off_block, off_kept_k, off_kept_v, off_listed, total;
 };
 // most CTAs of one attention launch: two resident per SM (148 SMs assumed where no device can be asked)
 int attn_grid_cap() {
@@ -104,11 +105,11 @@ Carve carve(const kvE_config& c) {
   const size_t max_chunks = ((size_t)c.max_tokens + c.C - 1) / c.C;
   Carve k;
   size_t o = 0;
-  // gate projection P [S max_chunks][4 d_g]; the per-token MLP aggregator, which runs before the gate, borrows it
-  // for its pooled activations [2][S max_chunks][d_sum]
-  size_t p_floats = S * max_chunks * 4 * (size_t)c.d_g;
-  if (c.agg == KVE_AGG_TOKEN_MLP && 2 * S * max_chunks * (size_t)c.d_sum > p_floats) p_floats = 2 * S * max_chunks * (size_t)c.d_sum;
-  k.off_P = o;        o = align_up(o + p_floats * sizeof(float));
+  // pooled activations of the per-token MLP aggregator, [2][S max_chunks][d_sum]; never less than [S max_chunks][4 d_g], the
+  // pre-activations that the gate once kept here: the workspace stays as large as callers know it
+  size_t pooled = S * max_chunks * 4 * (size_t)c.d_g;
+  if (c.agg == KVE_AGG_TOKEN_MLP && 2 * S * max_chunks * (size_t)c.d_sum > pooled) pooled = 2 * S * max_chunks * (size_t)c.d_sum;
+  k.off_pooled = o;   o = align_up(o + pooled * sizeof(float));
   // partial sums of w_s . h_t of every gated (sequence, chunk) of one kvE_gate call, [S max_chunks][d_g / 8], one per warp of the
   // recurrence: what its score head adds up
   k.off_H = o;        o = align_up(o + S * max_chunks * (size_t)(c.d_g / 8) * sizeof(float));
@@ -327,11 +328,15 @@ int kvE_create(const kvE_config* cfg, const kvE_buffers* buf, kvE_store** out) {
   }
   st->S = cfg->B * cfg->Hkv;
   st->max_chunks = (cfg->max_tokens + cfg->C - 1) / cfg->C;
-  st->off_P = k.off_P; st->off_H = k.off_H; st->off_partials = k.off_partials; st->off_counters = k.off_counters;
+  st->off_pooled = k.off_pooled; st->off_H = k.off_H; st->off_partials = k.off_partials; st->off_counters = k.off_counters;
   st->off_stage = k.off_stage; st->off_reclaim = k.off_reclaim; st->off_ticket = k.off_ticket; st->off_block = k.off_block;
   st->off_kept_k = k.off_kept_k; st->off_kept_v = k.off_kept_v; st->off_listed = k.off_listed; st->ws_needed = k.total;
   st->attn_grid_max = attn_grid_cap();
   if ((size_t)st->attn_grid_max > ATTN_GRID_LIMIT) st->attn_grid_max = (int)ATTN_GRID_LIMIT;
+  if (encode_gate_maps(st->gate_maps, buf->ksum_bf16, buf->vsum_bf16, (long long)cfg->n_layers * st->S, st->max_chunks, st->S, cfg->d_g) != cudaSuccess) {
+    delete st;
+    return KVE_ERR_CUDA;
+  }
   if (cfg->max_query_tokens > 0) {
     st->block_hp = attn_block_hp(cfg->C);
     st->block_split_cap = block_split_cap(st->S);
@@ -462,7 +467,7 @@ static int summarize_chunks(kvE_store* st, int layer, int chunk_begin, int chunk
     mw.W1V = static_cast<const uint16_t*>(w->W1V); mw.W2V = static_cast<const uint16_t*>(w->W2V);
     mw.b1K = w->b1K; mw.b2K = w->b2K; mw.b1V = w->b1V; mw.b2V = w->b2V;
     e = launch_chunk_token_mlp(v, chunk_begin, chunk_end, mw, st->cfg.d_sum,
-                               reinterpret_cast<float*>(static_cast<char*>(st->buf.workspace) + st->off_P), list_cut, s);
+                               reinterpret_cast<float*>(static_cast<char*>(st->buf.workspace) + st->off_pooled), list_cut, s);
   }
   if (e == cudaSuccess && mlp) {
     Prof prof(st, KVE_K_CHUNK_MLP, s);
@@ -495,18 +500,12 @@ int kvE_gate(kvE_store* st, int layer, int chunk_begin, int chunk_end, const kvE
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const LayerView v = view(st, layer);
-  float* P = reinterpret_cast<float*>(static_cast<char*>(st->buf.workspace) + st->off_P);
   cudaError_t e;
   {
-    Prof prof(st, KVE_K_GATE_PROJ, s);
-    e = launch_gate_proj(v, chunk_begin, chunk_end, static_cast<const uint16_t*>(w->W_ih), w->b_ih, w->b_hh,
-                         st->cfg.d_g, P, lower_listed(ls, chunk_begin), s);      // scores change under the keep list
-  }
-  if (e == cudaSuccess) {
     Prof prof(st, KVE_K_GATE_RNN, s);
-    e = launch_gate_rnn(v, chunk_begin, chunk_end, static_cast<const uint16_t*>(w->W_hh), w->w_s, w->b_s, st->cfg.d_g,
-                        P, reinterpret_cast<float*>(static_cast<char*>(st->buf.workspace) + st->off_H), chunk_begin == 0,
-                        st->gate_planes, s);
+    e = launch_gate_rnn(v, st->gate_maps, layer * st->S, chunk_begin, chunk_end, static_cast<const uint16_t*>(w->W_ih), static_cast<const uint16_t*>(w->W_hh), w->b_ih, w->b_hh,
+                        w->w_s, w->b_s, st->cfg.d_g, reinterpret_cast<float*>(static_cast<char*>(st->buf.workspace) + st->off_H), chunk_begin == 0,
+                        st->gate_planes, lower_listed(ls, chunk_begin), s);      // scores change under the keep list
   }
   if (e != cudaSuccess) return cuda_fail(st, e);
   ls.n_gated = chunk_end;

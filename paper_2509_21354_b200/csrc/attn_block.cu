@@ -1,6 +1,7 @@
 // Host side of the block-of-queries attention (kvE_decode_attn_block): tensor maps over the page pools
 // and the summary store, and the launch.  The kernel is in attn_block_tc.cu.
 #include "attn_block.cuh"
+#include "tensor_map.h"
 
 namespace kve {
 
@@ -15,27 +16,11 @@ int attn_block_hp(int C) {
 
 // [rows][128] bf16, boxes of 64 columns x box_rows rows, 128-byte swizzle
 static cudaError_t encode_rows_map(CUtensorMap* tm, const void* base, unsigned long long rows, unsigned box_rows) {
-  typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                               const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                               CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-  static EncodeFn encode = nullptr;
-  if (!encode) {
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres);
-    if (e != cudaSuccess) return e;
-    if (qres != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
-    encode = reinterpret_cast<EncodeFn>(fn);
-  }
   if (rows == 0 || rows >= (1ULL << 31)) return cudaErrorInvalidValue;
   const cuuint64_t dims[2] = {(cuuint64_t)D, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)ROW_BYTES};
   const cuuint32_t box[2] = {64u, box_rows};
-  const cuuint32_t estr[2] = {1u, 1u};
-  const CUresult r = encode(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+  return encode_bf16_map(tm, base, 2, dims, strides, box);
 }
 
 static_assert(sizeof(CUtensorMap) == ATTN_BLOCK_MAP_BYTES, "tensor map size");

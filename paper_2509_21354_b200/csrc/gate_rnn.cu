@@ -1,7 +1,6 @@
-// LSTM recurrence + score head of the gate (Eq. 3): for every sequence, chunks oldest first,
-//   pre_t = P_t + W_hh h_{t-1};  i,f,o = sigmoid, g = tanh;  c_t = f c_{t-1} + i g;  h_t = o tanh(c_t)
+// The gate (Eq. 3): input projection, LSTM recurrence and score head, for every sequence, chunks oldest first:
+//   pre_t = W_ih [Kbar_t ; Vbar_t] + b_ih + b_hh + W_hh h_{t-1};  i,f,o = sigmoid, g = tanh;  c_t = f c_{t-1} + i g;  h_t = o tanh(c_t)
 //   s_t   = sigmoid(w_s . h_t + b_s)
-// P_t (= W_ih x_t + b_ih + b_hh) comes from the projection GEMM.
 //
 // The chain over t is strictly sequential, so the kernel is built for latency per step:
 //  * A thread-block cluster of CL CTAs owns NG groups of 8 sequences for all steps (NG = 2 when one
@@ -15,35 +14,67 @@
 //    bf16 by definition; the fp32 state h enters as PL = 2 bf16 planes by default (h = hi + lo up to 2^-17 |h|: 16 of its 24
 //    significant bits; a third plane makes the products exact, moves the scores by 1e-7 - far below what the fast
 //    exponentials of the cell update contribute, 5e-5 - and costs a third more MMAs).  Each plane has its own
-//    accumulators (as many independent MMA chains), added smallest plane first at the end.
+//    accumulators (as many independent MMA chains), added smallest plane first at the end.  128 MMAs per scheduler and round take
+//    ~1000 cycles of ~2400, whether one warp or two issue them, and in as many chains as one likes: that is their rate.
 //  * MMA rows are ordered so that one thread ends up holding the i, f, g, o pre-activations of the
 //    same (hidden unit, sequence): the cell update is thread-local, c lives in registers.  f, i and g share one reciprocal
 //    and o and tanh(c) another (five exponentials and two reciprocals per element instead of five and five: the
 //    special-function unit is what the cell update waits for).
+//  * Input projection: a warp of a third warpgroup multiplies W_ih x_t a batch of GX_ROUNDS rounds (step, group) ahead on tcgen05.  The
+//    CTA's 256 rows of W_ih are the left operand and stay in TENSOR memory (half of it); a batch's summary rows, 64 columns
+//    of the product, come as four tiled copies (8 or 16 sequences x 8 or 4 consecutive chunks of 64 elements each); the two sets of
+//    accumulators fill the other half.  Rows of W_ih are placed so that tcgen05.ld in its 16-lane shape hands a thread its own four
+//    pre-activations of two sequences in the layout of the MMA fragments: two instructions a round.  As a kernel of its own
+//    (a GEMM over all chunks, P = 254 MB on 512 sequences x 121 chunks written and read again) it took 70 us there, 25 us on 256 x 56, 11 us on
+//    8 x 28 at d_g = 128; here it adds what its MMAs (32 a batch, ~68 cycles each whatever the columns) take away from the recurrence's:
+//    ~45 cycles each, 6 us on 256 x 56.  Issued by the recurrence's own warps it cost another 2 to 4 us and, with the branches
+//    around it, 10 % of a round.
 //  * Exchange of h_t: a warp writes the planes of its 8 hidden units into its own CTA's double-buffered h planes (two units per
-//    4-byte word, after one shuffle); from there bulk copies put the block into those of every other CTA of the cluster and count
-//    their bytes on an mbarrier there, so a step costs one one-way transfer and no cluster-wide barrier.  (With the planes
-//    gathered in a staging area in 2-byte stores and copied to the own buffer from there: 8.6 us more on 512 sequences x 121 chunks,
-//    1.5 us on 256 x 56, 0.8 us on 8 x 28 at d_g = 128.)  A CTA can only be sent step t+1 data after it has itself sent step t data, i.e. after all its warps have finished
-//    reading the buffer that is being overwritten.
-//  * P_{t+1} is fetched a round ahead: the projection kernel stores the four pre-activations of a hidden unit side by side, so a
-//    thread takes them with one 16-byte load.
-//  * The score head is not part of the chain: a warp leaves its 8 units' share of w_s . h_t per sequence (d_g / 8 partial sums
-//    per (s, t): an eighth of the bytes of h_t), and when the chain is through the cluster adds them up in a fixed order.
-//  Measured, recurrence and score head: 512 sequences x 121 chunks 314 -> 276 us, 256 x 56 92.5 -> 79 us, 8 x 28 at
-//  d_g = 128 51.6 -> 32 us (there a cluster of two CTAs halves the MMA chain: one CTA held all of W_hh).  Slower: waiting for the
-//  CTA's own planes and the peers' apart, with the own units' MMAs in between (255 -> 261 us a step on 256 sequences), and
-//  the score's shuffles between the MMAs (248 -> 255 us).
+//    4-byte word, after one shuffle), and sends them from there to every other CTA of the cluster in 16-byte asynchronous stores that
+//    count their bytes on an mbarrier there, so a step costs one one-way transfer and no cluster-wide barrier.  (By bulk copies, with the proxy
+//    fence that they need: 82 us on 256 sequences x 56 chunks, 80 so; 512 x 121 293 and 279 us.)  A CTA can only be sent step t+1 data after it has
+//    itself sent step t data, i.e. after all its warps have finished reading the buffer that is being overwritten.
+//  * The score head is not part of the chain: a warp leaves the products of w_s and h_t in shared memory, another warp of the third
+//    warpgroup adds up its 8 units (d_g / 8 partial sums per (s, t) go to memory: an eighth of the bytes of h_t) and announces the bytes of
+//    the next exchange, and when the chain is through the cluster adds the partial sums up in a fixed order.  (Both by the recurrence's
+//    warps: 77 us on 60 sequences x 80 chunks at d_g = 128, 73.6 so.)
+//  Measured, the whole gate: 512 sequences x 121 chunks 318 -> 277 us, 256 x 56 87.7 -> 78.6 us, 128 x 61 86 -> 83 us, 8 x 28 at d_g = 128
+//  32 -> 27.7 us, 60 x 5 at d_g = 128 12.7 -> 8.9 us (before: projection and recurrence as two kernels, back to back).
+//  Slower, with the kernels of that time: waiting for the CTA's own planes and the peers' apart, with the own units' MMAs in between (255 -> 261 us a step
+//  on 256 sequences), the two warps of a scheduler taking turns at the tensor cores (512 x 121 279 -> 317 us), and the sums of the even and the
+//  odd k tiles in accumulators of their own (286 -> 308 us).
 // Every mbarrier wait is bounded (one second); on give-up the status word gets KVE_ERR_TIMEOUT and
 // the CTA stops sending, which lets its peers run into their own limits and leave as well.
 #include "gate_rnn.cuh"
+#include "tensor_map.h"
+#include "umma.cuh"
 
 namespace kve {
 
+// the input projection: rounds (step, group) of a batch, 8 columns of the product each; shared and tensor memory
+constexpr int GX_ROUNDS = 8;
+constexpr int GX_N = GX_ROUNDS * 8;                          // columns of a batch: (step, group, sequence)
+constexpr int GX_KB = 2 * D / umma::KBLOCK_ELEMS;            // K-blocks of 64: keys' summary, values' summary
+constexpr int GX_KB_BYTES = GX_N * umma::KBLOCK_ROW_BYTES;   // 8 KB
+constexpr int GX_BYTES = GX_KB * GX_KB_BYTES;                // 32 KB
+constexpr int GX_TMEM_W = 0;                                 // two tiles of 128 rows of W_ih, 128 columns (256 bf16) each
+constexpr int GX_TMEM_ACC = 2 * D;                           // [batch & 1][tile][GX_N]
+constexpr int GX_TMEM_COLS = 512;
+static_assert(GX_TMEM_ACC + 4 * GX_N == GX_TMEM_COLS, "tensor memory");
+// two warpgroups of the recurrence and a third with the projector and the score warp (a warpgroup, because registers move
+// between whole warpgroups: with 9 warps of equal shares the recurrence would have 168 registers)
+constexpr int GATE_THREADS = RNN_THREADS + 128;
+// registers per thread of the recurrence and of the third warpgroup, which share out those of the launch
+template <int DG, int PL>
+constexpr int RNN_REGS = DG == 256 ? (PL == 3 ? 232 : 208) : (DG == 128 ? 184 : 136);
+constexpr int PROJ_REGS = 40;
+template <int DG, int PL>
+constexpr int GATE_REGS = (2 * RNN_REGS<DG, PL> + PROJ_REGS) / 3;
+
 // Optional cycle budget of one recurrence step (build with -DKVE_RNN_STAMPS, see rnn_stamps.py): warp 0 of CTA 0 adds
 // up, over all steps and groups, the clock64 cycles between five points of a step - 0: waiting for the peers' h,
-// 1: fragment loads + MMA chain, 2: prefetch of the next step's P, 3: cell update and plane split, 4: sending h,
-// 6: from the end of one round to the start of the next (the loaded P moves into place, barrier bookkeeping) - and
+// 1: fragment loads + MMA chain, 2: start of a round (pre-activations asked for), 3: cell update, 4: splitting and sending h,
+// 6: the rest of a round - and
 // slot 5 counts the (step, group) rounds.  The marks are contiguous: the slots add up to the whole step loop.  Compiled out of the product library.
 #ifdef KVE_RNN_STAMPS
 __device__ unsigned long long g_rnn_cycles[8];
@@ -71,25 +102,44 @@ __device__ unsigned long long g_rnn_once[8];
 #define KVE_RNN_ONCE(slot) do { } while (0)
 #endif
 
+// bytes in front of the summary rows: h buffers, products of the score, barriers
+template <int DG, int NG, int PL>
+constexpr int RNN_SMEM_X = NG * 2 * (DG / 8) * PL * 8 * 8 * 2 + NG * 2 * RNN_WARPS * 64 * 4 + (2 * NG + 5) * 8 + 8;
+
 template <int DG, int CL, int NG, int PL>
-__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RNN_THREADS, 1) kve_gate_rnn_kernel(RnnArgs a) {
+__global__ void __cluster_dims__(CL, 1, 1) __maxnreg__((GATE_REGS<DG, PL>))
+    kve_gate_rnn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, RnnArgs a) {
   constexpr int HU = DG / CL;            // hidden units owned by this CTA
   constexpr int KT = DG / 16;            // k tiles
   constexpr int NS = 8;                  // sequences per group: the n of the m16n8k16 MMA
   constexpr int KBLK = PL * NS * 8;                     // bf16 elements of one k-block (8 units): [plane][sequence][8]
   constexpr int HS_BUF = (DG / 8) * KBLK;               // bf16 elements per h buffer
   constexpr uint32_t H_BYTES = PL * NS * (DG - HU) * 2; // bytes of h planes a CTA receives from its peers per step and group
-  constexpr int OFF_BARS = NG * 2 * HS_BUF * 2;
-  constexpr int BULK_PENDING = 2 * NG - 1;              // a group's copies of two steps ago: all but the newest 2 NG - 1 commits
+  constexpr int OFF_PROD = NG * 2 * HS_BUF * 2;
+  constexpr int PROD_BUF = RNN_WARPS * 8 * NS;          // floats: w_s h of a round, [warp][sequence & 1][sequence / 2][8 units]
+  constexpr int OFF_BARS = OFF_PROD + NG * 2 * PROD_BUF * 4;
+  constexpr int T = GX_ROUNDS / NG;                     // steps of a batch of the input projection
+  constexpr bool P_LATE = DG < 256;                     // pre-activations fetched behind the MMAs, not in front: 77 us, 79 (60 sequences x 80 chunks, d_g = 128)
+  constexpr int SENDS = ((CL - 1) * PL * NS + 31) / 32;         // 16-byte messages to the peers per lane, step and group
   static_assert(HU == 8 * RNN_WARPS && KT % 2 == 0, "one pair of m16 tiles (8 units x 4 gates) per warp");
+  // what the warpgroups ask for is exactly what the launch has, or the last one to ask would wait for good
+  static_assert(3 * GATE_REGS<DG, PL> == 2 * RNN_REGS<DG, PL> + PROJ_REGS && GATE_REGS<DG, PL> % 8 == 0 && RNN_REGS<DG, PL> % 8 == 0, "register split");
   static_assert(OFF_BARS % 16 == 0, "16-byte pieces");
 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   uint16_t* hs = reinterpret_cast<uint16_t*>(smem_raw);                          // [NG][2][DG / 8][PL][NS][8]
+  float* prod = reinterpret_cast<float*>(smem_raw + OFF_PROD);                   // [NG][2][PROD_BUF]
   uint64_t* hbar = reinterpret_cast<uint64_t*>(smem_raw + OFF_BARS);             // [NG][2] h planes landed
+  uint64_t* x_full = hbar + 2 * NG;                                              // rows of a batch landed
+  uint64_t* x_done = x_full + 1;                                                 // [2] pre-activations of a batch computed
+  uint64_t* x_read = x_done + 2;                                                 // [2] ... and read by all warps
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(x_read + 2);
+  volatile uint32_t* rounds_done = tmem_slot + 1;                                // MMA chains that warp 0 has behind it
+  // [GX_KB] K-blocks of summary rows, on a 1024-byte boundary
+  unsigned char* xs = smem_raw + ((smem_u32(smem_raw) + RNN_SMEM_X<DG, NG, PL> + 1023u) & ~1023u) - smem_u32(smem_raw);
 
   const int tid = threadIdx.x, lane = tid & 31;
-  const int warp = tid >> 5;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);      // (the same in all lanes, for the compiler to see)
   const int g = lane >> 2, tig = lane & 3;
   const uint32_t rank = cluster_rank();
   const int seq0 = (blockIdx.x / CL) * NS * NG;      // group gi owns sequences seq0 + 8 gi .. + 7
@@ -97,9 +147,131 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RNN_THREADS, 1) kve
 
   KVE_RNN_ONCE(0);
   if (tid == 0) {
-    for (int i = 0; i < 2 * NG; ++i) mbar_init(&hbar[i], RNN_WARPS + (CL > 1 ? 1 : 0));
+    for (int i = 0; i < 2 * NG; ++i) mbar_init(&hbar[i], RNN_WARPS + 1);
+    *rounds_done = 0;
+    mbar_init(x_full, 1);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&x_done[i], 1);
+      mbar_init(&x_read[i], RNN_WARPS);
+    }
     mbar_fence_init();
   }
+  if (warp == 0) umma::tmem_alloc(tmem_slot, GX_TMEM_COLS);
+  umma::fence_before_sync();
+  __syncthreads();
+  umma::fence_after_sync();
+  const uint32_t tmem = *tmem_slot;
+
+  const int n_batches = (a.n_range + T - 1) / T;
+  // a warp's worth of partial sums from the products of a round: lane = (warp, sequence / 2), for both halves of the sequences
+  auto put_scores = [&](int gi, int step) {
+    const float* src = prod + (gi * 2 + (step & 1)) * PROD_BUF;
+    const int w = lane & 7, pair = lane >> 3;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const float4 x = *reinterpret_cast<const float4*>(src + ((w * 2 + e) * 4 + pair) * 8), y = *reinterpret_cast<const float4*>(src + ((w * 2 + e) * 4 + pair) * 8 + 4);
+      const int s = seq0 + gi * NS + pair * 2 + e;
+      if (s < a.S) a.H[(long long)(s * a.n_range + step) * (DG / 8) + rank * RNN_WARPS + w] = ((x.x + x.y) + (x.z + x.w)) + ((y.x + y.y) + (y.z + y.w));
+    }
+  };
+  if (warp >= RNN_WARPS) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(PROJ_REGS));
+    // ================= projector warp =================
+    // Pre-activations W_ih x_t a batch of GX_ROUNDS rounds ahead of the recurrence.
+    pdl_wait();      // the summaries come from earlier kernels
+    __syncthreads();      // W_ih is in tensor memory, and xs, its staging area, is free
+    umma::fence_after_sync();
+    cluster_arrive();      // the recurrence's first meeting, which this warp has nothing to wait for
+    bool ok = true;
+    int n_fetched = 0, n_begun = 0;
+    if (warp == RNN_WARPS && lane == 0) {
+      asm volatile("fence.proxy.async.global;" ::: "memory");
+      for (int b = 0; b < n_batches && ok; ++b) {
+        const int buf = b & 1;
+        // the rows of all steps and sequences of the batch: a copy per K-block, zeros beyond the store (what it brings beyond the range
+        // or from another layer goes into columns that nobody reads)
+        mbar_arrive_expect_tx(x_full, GX_BYTES);
+#pragma unroll
+        for (int kb = 0; kb < GX_KB; ++kb)
+          tma_load_3d(smem_u32(xs) + kb * GX_KB_BYTES, kb < GX_KB / 2 ? &map_k : &map_v, (kb & 1) * umma::KBLOCK_ELEMS, a.seq_base + seq0, a.t0 + b * T, x_full);
+        n_fetched = b + 1;
+        ok = mbar_wait_bounded(x_full, (uint32_t)(b & 1)) && (b < 2 || mbar_wait_bounded(&x_read[buf], (uint32_t)(((b >> 1) - 1) & 1)));
+        if (!ok) break;
+        umma::fence_after_sync();
+        n_begun = b + 1;
+        // (A loop over the tiles: what runs once has to be fetched first, and a launch of 5 chunks took 4 us longer with the issue of 32 MMAs spelled out.)
+#pragma unroll 1
+        for (int tile = 0; tile < 2; ++tile) {
+          // The tensor cores work on one of the two products at a time.  With two groups the tiles go out one by one, when warp 0 has the
+          // MMAs of a round behind it (for the pace only: the wait gives up soon).  512 sequences x 121 chunks 285 us in one go, 277 so; with one
+          // group nothing is gained by it.
+          if (NG > 1 && b > 0)
+            for (int poll = 0; poll < 4096 && *rounds_done < (uint32_t)((b - 1) * GX_ROUNDS + tile * 3 + 2); ++poll) __nanosleep(20);
+          const uint32_t acc = tmem + GX_TMEM_ACC + (uint32_t)((buf * 2 + tile) * GX_N);
+#pragma unroll
+          for (int k = 0; k < 4 * GX_KB; ++k)
+            umma::mma_bf16_ts(acc, tmem + GX_TMEM_W + (uint32_t)(tile * D + k * 8), umma::smem_desc(smem_u32(xs) + (k >> 2) * GX_KB_BYTES + (k & 3) * 32),
+                              umma::instr_desc_bf16(128, GX_N), k != 0);
+        }
+        umma::commit(&x_done[buf]);
+        ok = mbar_wait_bounded(&x_done[buf], (uint32_t)((b >> 1) & 1));      // the rows may be overwritten
+      }
+      if (!ok) {      // nothing is under way any more when the CTA leaves
+        set_status(a.status, ERR_TIMEOUT);
+        mbar_wait_bounded(x_full, (uint32_t)((n_fetched - 1) & 1));
+        if (n_begun > 0) mbar_wait_bounded(&x_done[(n_begun - 1) & 1], (uint32_t)(((n_begun - 1) >> 1) & 1));
+      }
+    }
+    if (warp == RNN_WARPS + 1) {
+      // ================= score warp =================
+      // Announces the bytes of every exchange, and adds up what the warps leave of w_s . h_t when it is through (eight units in pairs;
+      // the warps' sums go to memory).  Its arrival for the next exchange says that it has read what that one will overwrite.
+      for (int step = 0; step + 1 < a.n_range && ok; ++step) {
+        const int buf = (step + 1) & 1;
+        if (lane < NG) {
+          if (CL > 1) mbar_arrive_expect_tx(&hbar[2 * lane + buf], H_BYTES);
+          else mbar_arrive(&hbar[2 * lane + buf]);
+        }
+        for (int gi = 0; gi < NG && ok; ++gi) {
+          ok = __all_sync(0xffffffffu, mbar_wait_cluster_bounded(&hbar[2 * gi + buf], (uint32_t)((step >> 1) & 1)));
+          if (ok) put_scores(gi, step);
+        }
+      }
+      if (!ok && lane == 0) set_status(a.status, ERR_TIMEOUT);
+    }
+    __syncwarp();
+    cluster_wait();
+    cluster_sync_all();
+    return;
+  }
+
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(RNN_REGS<DG, PL>));
+  // ---- W_ih rows of this CTA into tensor memory, the left operand of the input projection ------------------------
+  // Tile w / 4, lanes 32 (w % 4) .. are the rows of warp w in the order of its MMA fragments: lane l = row (l & 7) of gate l >> 3.
+  // A K-block (32 rows x 128 bytes) at a time through the warp's share of the X area.
+  const uint32_t tmem_mine = tmem + ((uint32_t)(warp & 3) << 21);      // this warp's quarter of the lanes
+  unsigned char* w_stage = xs + warp * (32 * umma::KBLOCK_ROW_BYTES);
+  auto fetch_w_ih = [&](int kb) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int r = i * 4 + (lane >> 3), p = lane & 7;
+      cp_async16(w_stage + umma::piece_offset(r, p),
+                 a.W_ih + ((long long)(r >> 3) * DG + (int)rank * HU + warp * 8 + (r & 7)) * (2 * D) + kb * umma::KBLOCK_ELEMS + p * 8, true);
+    }
+  };
+  auto store_w_ih = [&](int kb) {
+    cp_async_wait_all();
+    __syncwarp();
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      uint32_t r[16];
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+        *reinterpret_cast<uint4*>(&r[4 * p]) = *reinterpret_cast<const uint4*>(w_stage + umma::piece_offset(lane, half * 4 + p));
+      umma::tmem_st16_nowait(tmem_mine + GX_TMEM_W + (uint32_t)((warp >> 2) * D + kb * 32 + half * 16), r);
+    }
+    __syncwarp();      // read by all lanes: the next K-block may come
+  };
 
   // ---- W_hh rows of this CTA as A fragments ---------------------------------------------------------------------
   // Register j of the fragment of k tile kt holds the two bf16 at k = 16 kt + 8 (j >> 1) + 2 tig of row (j & 1): word
@@ -128,14 +300,27 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RNN_THREADS, 1) kve
   };
   uint32_t A[KT / 2][2][2][4];
 #pragma unroll
-  for (int kp = 0; kp < KT / 2; ++kp) load_pair(kp, A[kp]);
+  for (int kb = 0; kb < GX_KB; ++kb) {
+    fetch_w_ih(kb);
+#pragma unroll
+    for (int kp = kb * KT / 2 / GX_KB; kp < (kb + 1) * KT / 2 / GX_KB; ++kp) load_pair(kp, A[kp]);
+    store_w_ih(kb);
+  }
   const float w_score = __ldg(a.w_s + ug);
+  float bias[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) bias[q] = __ldg(a.b_ih + q * DG + ug) + __ldg(a.b_hh + q * DG + ug);
+  umma::tmem_st_wait();
 
   KVE_RNN_ONCE(1);
   pdl_wait();      // W_hh is in place; the carried state and P come from earlier kernels
   // only now, when all earlier work is complete: a launch may run beside this kernel without waiting for anything (kvE_refresh)
   pdl_launch_dependents();
+  if (a.list_cut >= 0 && blockIdx.x == 0 && tid == 0) *a.n_listed = a.list_cut;
   KVE_RNN_ONCE(2);
+  umma::fence_smem_to_async();
+  umma::fence_before_sync();
+  __syncthreads();      // W_ih is in tensor memory: the projector may start
   // ---- initial state: every CTA needs the full h of its sequences as planes in buffer 0 of each group -------------
   for (int i = tid; i < NG * NS * (DG / 2); i += RNN_THREADS) {
     const int js = i / (DG / 2), k2 = i % (DG / 2);      // js: sequence of the cluster, 0 .. 8 NG - 1
@@ -163,26 +348,11 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RNN_THREADS, 1) kve
       c[gi][e] = carried ? a.lstm_c[(long long)s * DG + ug] : 0.f;
       hlast[gi][e] = carried ? a.lstm_h[(long long)s * DG + ug] : 0.f;
     }
-  // the four pre-activations of a unit lie side by side in P: one 16-byte load
-  const float4* p_unit = reinterpret_cast<const float4*>(a.P) + ug;
-  auto load_p = [&](int gi, int step, float4 (&pv)[2]) {
+  // message m of a warp goes to peer (rank + 1 + m / rows of a block): row m % rows of that CTA's buffers, as an address in the cluster window
+  uint32_t peer_hs[SENDS > 0 ? SENDS : 1];
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int s = seq0 + gi * NS + tig * 2 + e;
-      const bool there = s < a.S && step < a.n_range;
-      const float4* p = p_unit + (long long)(s * a.n_range + step) * DG;
-      pv[e] = there ? __ldcs(p) : make_float4(0.f, 0.f, 0.f, 0.f);
-      // the 8 lanes of a group cover one 128-byte line of the row after it: one of them asks L2 for it
-      if (s < a.S && step + 1 < a.n_range && g == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + DG));
-    }
-  };
-  float4 pin[2];
-  load_p(0, 0, pin);
-  float* part_out = a.H + rank * RNN_WARPS + warp;
-
-  // lane r < CL feeds peer r: that CTA's h buffers and barriers, as addresses in the cluster window
-  const uint32_t peer_hs = map_to_rank(smem_u32(hs), lane < CL ? lane : 0);
-  const uint32_t peer_bar = map_to_rank(smem_u32(&hbar[0]), lane < CL ? lane : 0);
+  for (int x = 0; x < SENDS; ++x)
+    peer_hs[x] = map_to_rank(smem_u32(hs), (rank + 1 + (lane + 32 * x) / (PL * NS)) % CL) + (lane + 32 * x) % (PL * NS) * 16;
 
   // barriers initialised and buffer 0 filled in every CTA before anyone sends
   KVE_RNN_ONCE(3);
@@ -191,131 +361,138 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RNN_THREADS, 1) kve
 
   bool alive = true;
   KVE_RNN_MARK_BEGIN();
-  for (int step = 0; step < a.n_range && alive; ++step) {
-    const int buf = step & 1;
-    const bool send_h = step + 1 < a.n_range;
-    // this step's sends of the cluster land in buffer buf^1 of each group: announce the bytes
-    if (CL > 1 && send_h && tid == 0) {
-#pragma unroll
-      for (int gi = 0; gi < NG; ++gi) mbar_arrive_expect_tx(&hbar[2 * gi + (buf ^ 1)], H_BYTES);
+  for (int batch = 0; batch < n_batches && alive; ++batch) {
+    // ---- the pre-activations of the next T steps' inputs
+    alive = __all_sync(0xffffffffu, mbar_wait_bounded(&x_done[batch & 1], (uint32_t)((batch >> 1) & 1)));
+    if (!alive) {
+      if (lane == 0) set_status(a.status, ERR_TIMEOUT);
+      break;
     }
+    umma::fence_after_sync();
+    uint32_t acc_x = tmem_mine + GX_TMEM_ACC + (uint32_t)(((batch & 1) * 2 + (warp >> 2)) * GX_N);
+    const int step_end = min(batch * T + T, a.n_range);
+    for (int step = batch * T; step < step_end; ++step) {
+      const int buf = step & 1;
+      const bool send_h = step + 1 < a.n_range;
 #pragma unroll
-    for (int gi = 0; gi < NG; ++gi) {
-      uint16_t* hs_g = hs + gi * 2 * HS_BUF;
-      uint64_t* hbar_g = hbar + 2 * gi;
-      // P of the next round, used there: requested before the wait (one group), while the MMAs drain (two, where nothing waits)
-      float4 pv[2];
-      if (NG == 1) load_p(0, step + 1, pv);
-      KVE_RNN_MARK(2);
-      // ---- h_{t-1} from every CTA of the cluster (each buffer completes once per two steps) -----------------------------
-      if (step > 0) {
-        if (!mbar_wait_cluster_bounded(&hbar_g[buf], ((step - 1) >> 1) & 1)) {
-          if (lane == 0) set_status(a.status, ERR_TIMEOUT);
-          alive = false;
+      for (int gi = 0; gi < NG; ++gi) {
+        uint16_t* hs_g = hs + gi * 2 * HS_BUF;
+        uint64_t* hbar_g = hbar + 2 * gi;
+        // pre-activations of the round's inputs, in the layout of the MMA accumulators
+        uint32_t pin[2][4];
+        auto ask_pin = [&]() {
+          umma::tmem_ld_frag_nowait(acc_x, pin[0]);
+          umma::tmem_ld_frag_nowait(acc_x + (16u << 16), pin[1]);
+          acc_x += 8;
+        };
+        if (!P_LATE) ask_pin();
+        KVE_RNN_MARK(2);
+        // ---- h_{t-1} from every CTA of the cluster (each buffer completes once per two steps) -----------------------------
+        if (step > 0) {
+          // (one poll usually waits long enough: it is the only thing in the way then)
+          const uint32_t parity = ((step - 1) >> 1) & 1;
+          if (!__all_sync(0xffffffffu, mbar_try_wait_cluster(&hbar_g[buf], parity))) {
+            alive = __all_sync(0xffffffffu, mbar_wait_cluster_bounded(&hbar_g[buf], parity));
+            if (!alive) {
+              if (lane == 0) set_status(a.status, ERR_TIMEOUT);
+              break;
+            }
+          }
         }
-        alive = __all_sync(0xffffffffu, alive);
-        if (!alive) break;
-      }
-      KVE_RNN_MARK(0);
+        KVE_RNN_MARK(0);
 
-      // ---- W_hh h_{t-1} on the tensor cores: one accumulator set per plane ---------------------------------------------
-      float acc[PL][2][4];
+        // ---- W_hh h_{t-1} on the tensor cores: one accumulator set per plane ---------------------------------------------
+        float acc[PL][2][4];
 #pragma unroll
-      for (int pl = 0; pl < PL; ++pl)
+        for (int pl = 0; pl < PL; ++pl)
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
+          for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-          for (int e = 0; e < 4; ++e) acc[pl][mt][e] = 0.f;
-      // B fragments: one ldmatrix.x4 brings the 8 sequences x 32 k-values of a plane (two k tiles);
-      // lane l addresses row (l & 7) of the 8 x 8 block (l >> 3).
-      const uint32_t hb_lane = smem_u32(hs_g + buf * HS_BUF + (lane >> 3) * KBLK + (lane & 7) * 8);
-      uint32_t bf[2][PL][4];
-      auto load_b = [&](int kp) {
+            for (int e = 0; e < 4; ++e) acc[pl][mt][e] = 0.f;
+        // B fragments: one ldmatrix.x4 brings the 8 sequences x 32 k-values of a plane (two k tiles);
+        // lane l addresses row (l & 7) of the 8 x 8 block (l >> 3).
+        const uint32_t hb_lane = smem_u32(hs_g + buf * HS_BUF + (lane >> 3) * KBLK + (lane & 7) * 8);
+        uint32_t bf[2][PL][4];
+        auto load_b = [&](int kp) {
 #pragma unroll
-        for (int pl = 0; pl < PL; ++pl) ldmatrix_x4(bf[kp & 1][pl], hb_lane + (uint32_t)((kp * 4 * KBLK + pl * NS * 8) * 2));
-      };
-      load_b(0);
+          for (int pl = 0; pl < PL; ++pl) ldmatrix_x4(bf[kp & 1][pl], hb_lane + (uint32_t)((kp * 4 * KBLK + pl * NS * 8) * 2));
+        };
+        load_b(0);
 #pragma unroll
-      for (int kp = 0; kp < KT / 2; ++kp) {
-        if (kp + 1 < KT / 2) load_b(kp + 1);      // a pair of k tiles ahead
+        for (int kp = 0; kp < KT / 2; ++kp) {
+          if (kp + 1 < KT / 2) load_b(kp + 1);      // a pair of k tiles ahead
 #pragma unroll
-        for (int half = 0; half < 2; ++half)
+          for (int half = 0; half < 2; ++half)
 #pragma unroll
-          for (int pl = 0; pl < PL; ++pl)
+            for (int pl = 0; pl < PL; ++pl)
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt) mma_bf16_16816(acc[pl][mt], A[kp][mt][half], bf[kp & 1][pl][2 * half], bf[kp & 1][pl][2 * half + 1]);
-      }
-      KVE_RNN_MARK(1);
+              for (int mt = 0; mt < 2; ++mt) mma_bf16_16816(acc[pl][mt], A[kp][mt][half], bf[kp & 1][pl][2 * half], bf[kp & 1][pl][2 * half + 1]);
+        }
+        if (NG > 1 && tid == 0) *rounds_done = (uint32_t)(step * NG + gi + 1);
+        KVE_RNN_MARK(1);
 
-      if (NG > 1) {
-        // (the vote is a scheduling fence: without it the compiler spreads the loads' address arithmetic over the MMA chain)
+        // (the vote is a scheduling fence: without it the compiler draws what follows into the MMA chain, 10 % of a step)
         if (!__all_sync(0xffffffffu, alive)) break;
-        load_p((gi + 1) % NG, step + (gi + 1) / NG, pv);
-      }
-      // ---- cell update (thread-local), planes of h_t into this CTA's buffer ---------------------
-      // the copies from there two steps ago have been read: those of the group's last step may still be under way
-      if (CL > 1) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(BULK_PENDING) : "memory");
-      __syncwarp();
-      uint32_t split[2][3];
+        if (P_LATE) ask_pin();
+        umma::tmem_ld_wait_frags(pin[0], pin[1]);
+        // ---- cell update (thread-local), planes of h_t into this CTA's buffer ---------------------
+        float hv[2];
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        float pre[4];
+        for (int e = 0; e < 2; ++e) {
+          float pre[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {   // q: 0 = i, 1 = f (tile 0, rows g / g+8), 2 = g, 3 = o (tile 1)
-          const int mt = q >> 1, ai = (q & 1) * 2 + e;
-          float sum = acc[PL - 1][mt][ai];      // smallest plane first
+          for (int q = 0; q < 4; ++q) {   // q: 0 = i, 1 = f (tile 0, rows g / g+8), 2 = g, 3 = o (tile 1)
+            const int mt = q >> 1, ai = (q & 1) * 2 + e;
+            float sum = acc[PL - 1][mt][ai];      // smallest plane first
 #pragma unroll
-          for (int pl = PL - 2; pl >= 0; --pl) sum += acc[pl][mt][ai];
-          pre[q] = sum + (q == 0 ? pin[e].x : (q == 1 ? pin[e].y : (q == 2 ? pin[e].z : pin[e].w)));
+            for (int pl = PL - 2; pl >= 0; --pl) sum += acc[pl][mt][ai];
+            pre[q] = sum + (__uint_as_float(pin[mt][ai]) + bias[q]);
+          }
+          hlast[gi][e] = hv[e] = lstm_cell(pre, c[gi][e]);
         }
-        const float hv = lstm_cell(pre, c[gi][e]);
-        hlast[gi][e] = hv;
-        split3(hv, split[e]);
-      }
-      KVE_RNN_MARK(3);
-      // ---- the warp's k-block (8 units: [plane][sequence][8], contiguous) to every CTA of the cluster ----
-      if (send_h) {
-        const uint32_t off = (uint32_t)(((gi * 2 + (buf ^ 1)) * HS_BUF + ((int)rank * RNN_WARPS + warp) * KBLK) * 2);
-        // lanes g and g ^ 1 hold neighbouring units: an even g takes both units of sequence 2 tig, an odd one those of 2 tig + 1, and
-        // a warp's store instruction is a whole plane of the block: 128 bytes in a row
-        const bool odd = (g & 1) != 0;
-        unsigned char* mine = reinterpret_cast<unsigned char*>(hs) + off + (tig * 2 + (g & 1)) * 16 + (g >> 1) * 4;
-        const uint32_t keep = odd ? split[1][0] | split[1][1] << 16 : split[0][0] | split[0][1] << 16;
-        const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? split[0][0] | split[0][1] << 16 : split[1][0] | split[1][1] << 16, 4);
-        *reinterpret_cast<uint32_t*>(mine) = __byte_perm(odd ? got : keep, odd ? keep : got, 0x5410);
-        *reinterpret_cast<uint32_t*>(mine + NS * 16) = __byte_perm(odd ? got : keep, odd ? keep : got, 0x7632);
-        if constexpr (PL == 3) {
-          const uint32_t keep2 = odd ? split[1][2] : split[0][2], got2 = __shfl_xor_sync(0xffffffffu, odd ? split[0][2] : split[1][2], 4);
-          *reinterpret_cast<uint32_t*>(mine + 2 * NS * 16) = (odd ? got2 : keep2) | (odd ? keep2 : got2) << 16;
+        KVE_RNN_MARK(3);
+        // products of the score: nothing of the chain waits for their sum
+        {
+          float* mine = prod + (gi * 2 + buf) * PROD_BUF + (warp * 2 * 4 + tig) * 8 + g;
+          mine[0] = w_score * hv[0];
+          mine[4 * 8] = w_score * hv[1];
         }
-        if (CL > 1) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // visible to the bulk copies
-        __syncwarp();
-        if (CL > 1) {
-          // peers: one bulk copy each out of the own buffer, its bytes counted on the receiver's barrier
-          if (lane < CL && lane != (int)rank)
-            bulk_s2cluster(peer_hs + off, smem_u32(hs) + off, KBLK * 2, peer_bar + (2 * gi + (buf ^ 1)) * 8);
-          asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+        // ---- the warp's k-block (8 units: [plane][sequence][8], contiguous) to every CTA of the cluster ----
+        if (send_h) {
+          const uint32_t off = (uint32_t)(((gi * 2 + (buf ^ 1)) * HS_BUF + ((int)rank * RNN_WARPS + warp) * KBLK) * 2);
+          // lanes g and g ^ 1 hold neighbouring units: an even g takes both units of sequence 2 tig, an odd one those of 2 tig + 1, and
+          // a warp's store instruction is a whole plane of the block: 128 bytes in a row
+          const bool odd = (g & 1) != 0;
+          unsigned char* mine = reinterpret_cast<unsigned char*>(hs) + off + (tig * 2 + (g & 1)) * 16 + (g >> 1) * 4;
+          uint32_t pl[3];      // planes of both sequences, the even one below
+          split3_pair(hv[0], hv[1], pl);
+          const uint32_t h0 = __byte_perm(pl[0], pl[1], 0x5410), h1 = __byte_perm(pl[0], pl[1], 0x7632);      // two planes of a sequence
+          const uint32_t keep = odd ? h1 : h0, got = __shfl_xor_sync(0xffffffffu, odd ? h0 : h1, 4);
+          *reinterpret_cast<uint32_t*>(mine) = __byte_perm(odd ? got : keep, odd ? keep : got, 0x5410);
+          *reinterpret_cast<uint32_t*>(mine + NS * 16) = __byte_perm(odd ? got : keep, odd ? keep : got, 0x7632);
+          if constexpr (PL == 3) {
+            const uint32_t got2 = __shfl_xor_sync(0xffffffffu, pl[2], 4);
+            *reinterpret_cast<uint32_t*>(mine + 2 * NS * 16) = __byte_perm(odd ? got2 : pl[2], odd ? pl[2] : got2, odd ? 0x7632 : 0x5410);
+          }
+          __syncwarp();
+          // peers: 16-byte rows out of the own block, each counted in bytes on the receiver's barrier; lane l sends message l, l + 32 ..
+#pragma unroll
+          for (int x = 0; x < SENDS; ++x) {
+            const uint4 row = *reinterpret_cast<const uint4*>(reinterpret_cast<const unsigned char*>(hs) + off + (lane + 32 * x) % (PL * NS) * 16);
+            if (x * 32 + lane < (CL - 1) * PL * NS)
+              st_async_cluster(peer_hs[x] + off, row, peer_hs[x] - (lane + 32 * x) % (PL * NS) * 16 + OFF_BARS + (2 * gi + (buf ^ 1)) * 8);
+          }
+          if (lane == 0) mbar_arrive(&hbar_g[buf ^ 1]);     // release: this warp's own pieces are in place
         }
-        if (lane == 0) mbar_arrive(&hbar_g[buf ^ 1]);     // release: this warp's own pieces are in place
-      }
-      KVE_RNN_MARK(4);
-      // ---- this warp's share of the score, behind the sends: lane group g = 0 ends up with sequence 2 tig, g = 1 with 2 tig + 1 ----
-      {
-        const bool odd = (g & 1) != 0;
-        const float d0 = w_score * hlast[gi][0], d1 = w_score * hlast[gi][1];
-        float d = (odd ? d1 : d0) + __shfl_xor_sync(0xffffffffu, odd ? d0 : d1, 4);
-        d += __shfl_xor_sync(0xffffffffu, d, 8);
-        d += __shfl_xor_sync(0xffffffffu, d, 16);
-        const int s = seq0 + gi * NS + tig * 2 + (g & 1);
-        if (g < 2 && s < a.S) part_out[(long long)(s * a.n_range + step) * (DG / 8)] = d;
-      }
+        KVE_RNN_MARK(4);
 #ifdef KVE_RNN_STAMPS
-      if (blockIdx.x == 0 && tid == 0) atomicAdd(&g_rnn_cycles[5], 1ull);
+        if (blockIdx.x == 0 && tid == 0) atomicAdd(&g_rnn_cycles[5], 1ull);
 #endif
-      pin[0] = pv[0];
-      pin[1] = pv[1];
-      KVE_RNN_MARK(6);
+        KVE_RNN_MARK(6);
+      }
+      if (!alive) break;
     }
+    if (lane == 0) mbar_arrive(&x_read[batch & 1]);
   }
 
   KVE_RNN_ONCE(5);
@@ -330,9 +507,13 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RNN_THREADS, 1) kve
         a.lstm_h[(long long)s * DG + ug] = hlast[gi][e];
       }
     }
+  // (the last step's products, which no exchange follows)
+  asm volatile("bar.sync 1, %0;" ::"n"(RNN_THREADS) : "memory");
+  if (warp < NG && alive) put_scores(warp, a.n_range - 1);
   // nobody leaves while a peer may still be sending into its shared memory; the partial sums of all CTAs are in place behind it
   cluster_sync_all();
   KVE_RNN_ONCE(6);
+  if (warp == 0) umma::tmem_dealloc(tmem, GX_TMEM_COLS);
   // ---- score head: s_t = sigmoid(w_s . h_t + b_s); a row's d_g / 8 partial sums lie side by side and are added in order -----------
   const int n_seq = min(NS * NG, a.S - seq0);
   for (int i = (int)rank * RNN_THREADS + tid; i < n_seq * a.n_range; i += CL * RNN_THREADS) {
@@ -349,9 +530,8 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(RNN_THREADS, 1) kve
 }
 
 template <int DG, int CL, int NG, int PL>
-static cudaError_t launch_rnn_t(const RnnArgs& a, cudaStream_t st) {
-  constexpr int KBLK_BYTES = PL * 8 * 8 * 2;
-  constexpr int smem = NG * 2 * (DG / 8) * KBLK_BYTES + NG * 2 * 8;
+static cudaError_t launch_rnn_t(const RnnArgs& a, const CUtensorMap* maps, cudaStream_t st) {
+  constexpr int smem = RNN_SMEM_X<DG, NG, PL> + GX_BYTES + 1024;      // + slack to reach a 1024-byte boundary
   static DeviceFlags opted;
   {
     cudaError_t e = smem_opt_in(opted, kve_gate_rnn_kernel<DG, CL, NG, PL>, smem);
@@ -366,12 +546,12 @@ static cudaError_t launch_rnn_t(const RnnArgs& a, cudaStream_t st) {
   attr[1].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(clusters * CL);
-  cfg.blockDim = dim3(RNN_THREADS);
+  cfg.blockDim = dim3(GATE_THREADS);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, kve_gate_rnn_kernel<DG, CL, NG, PL>, a);
+  return cudaLaunchKernelEx(&cfg, kve_gate_rnn_kernel<DG, CL, NG, PL>, maps[0], maps[1], a);
 }
 
 // CTAs of a cluster; two groups of 8 sequences per cluster once one group per cluster would need more than one wave of clusters
@@ -386,24 +566,42 @@ double gate_rnn_us_per_chunk(int S, int d_g, int planes) {
 }
 
 template <int PL>
-static cudaError_t launch_rnn_planes(const RnnArgs& a, int d_g, cudaStream_t st) {
+static cudaError_t launch_rnn_planes(const RnnArgs& a, const CUtensorMap* maps, int d_g, cudaStream_t st) {
   const bool two = two_groups(a.S, d_g);
   switch (d_g) {
-    case 256: return two ? launch_rnn_t<256, 4, 2, PL>(a, st) : launch_rnn_t<256, 4, 1, PL>(a, st);
-    case 128: return two ? launch_rnn_t<128, 2, 2, PL>(a, st) : launch_rnn_t<128, 2, 1, PL>(a, st);
-    case 64:  return two ? launch_rnn_t<64, 1, 2, PL>(a, st) : launch_rnn_t<64, 1, 1, PL>(a, st);
+    case 256: return two ? launch_rnn_t<256, 4, 2, PL>(a, maps, st) : launch_rnn_t<256, 4, 1, PL>(a, maps, st);
+    case 128: return two ? launch_rnn_t<128, 2, 2, PL>(a, maps, st) : launch_rnn_t<128, 2, 1, PL>(a, maps, st);
+    case 64:  return two ? launch_rnn_t<64, 1, 2, PL>(a, maps, st) : launch_rnn_t<64, 1, 1, PL>(a, maps, st);
     default:  return cudaErrorInvalidValue;
   }
 }
 
-cudaError_t launch_gate_rnn(const LayerView& v, int t0, int t1, const uint16_t* W_hh, const float* w_s, float b_s,
-                            int d_g, const float* P, float* H, bool reset_state, int planes, cudaStream_t st) {
+cudaError_t encode_gate_maps(void* maps, const void* ksum, const void* vsum, long long n_seq, int max_chunks, int S, int d_g) {
+  static_assert(sizeof(CUtensorMap) == GATE_MAP_BYTES, "tensor map size");
+  const int ng = two_groups(S, d_g) ? 2 : 1;
+  for (int i = 0; i < 2; ++i) {
+    // element, sequence, chunk: a box holds the sequences of a cluster at GX_ROUNDS / ng consecutive chunks
+    const cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)n_seq, (cuuint64_t)max_chunks};
+    const cuuint64_t strides[2] = {(cuuint64_t)max_chunks * ROW_BYTES, (cuuint64_t)ROW_BYTES};
+    const cuuint32_t box[3] = {(cuuint32_t)umma::KBLOCK_ELEMS, (cuuint32_t)(8 * ng), (cuuint32_t)(GX_ROUNDS / ng)};
+    const cudaError_t e = encode_bf16_map(static_cast<CUtensorMap*>(maps) + i, i ? vsum : ksum, 3, dims, strides, box);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t launch_gate_rnn(const LayerView& v, const void* maps, int seq_base, int t0, int t1, const uint16_t* W_ih, const uint16_t* W_hh, const float* b_ih, const float* b_hh,
+                            const float* w_s, float b_s, int d_g, float* H, bool reset_state, int planes, int list_cut, cudaStream_t st) {
   if (t1 <= t0 || v.S <= 0) return cudaSuccess;
+  if ((long long)v.S * (t1 - t0) >= (1LL << 31) - 128) return cudaErrorInvalidValue;
+  const CUtensorMap* tm = static_cast<const CUtensorMap*>(maps);
   RnnArgs a;
-  a.P = P; a.H = H; a.W_hh = W_hh; a.w_s = w_s; a.b_s = b_s;
+  a.seq_base = seq_base; a.W_ih = W_ih; a.b_ih = b_ih; a.b_hh = b_hh;
+  a.n_listed = v.n_listed; a.list_cut = list_cut;
+  a.H = H; a.W_hh = W_hh; a.w_s = w_s; a.b_s = b_s;
   a.scores = v.scores; a.lstm_h = v.lstm_h; a.lstm_c = v.lstm_c; a.status = v.status;
   a.S = v.S; a.max_chunks = v.max_chunks; a.t0 = t0; a.n_range = t1 - t0; a.reset = reset_state ? 1 : 0;
-  return planes == 3 ? launch_rnn_planes<3>(a, d_g, st) : launch_rnn_planes<2>(a, d_g, st);
+  return planes == 3 ? launch_rnn_planes<3>(a, tm, d_g, st) : launch_rnn_planes<2>(a, tm, d_g, st);
 }
 
 }  // namespace kve

@@ -1,7 +1,8 @@
-// Pieces shared by the LSTM recurrence kernels: launch arguments, cluster addressing, bulk copies into a peer CTA's shared
+// Pieces shared by the LSTM recurrence kernels: launch arguments, cluster addressing, asynchronous stores into a peer CTA's shared
 // memory that count bytes on the peer's mbarrier, bounded cluster waits, the fast activations and the exact 3-way bf16 split
 // of an fp32 value.
 #pragma once
+#include <cuda.h>
 #include "common.cuh"
 #include "kernels.h"
 
@@ -11,7 +12,10 @@ constexpr int RNN_WARPS = 8;
 constexpr int RNN_THREADS = RNN_WARPS * 32;
 
 struct RnnArgs {
-  const float* P;          // [S * n_range][4 d_g], column 4 u + gate: the pre-activations W_ih x + b of unit u
+  int seq_base;            // the layer's first sequence in the tensor maps over the bf16 summaries (the inputs x_t = [Kbar_t ; Vbar_t])
+  const uint16_t* W_ih;    // bf16 [4 d_g][256]
+  const float* b_ih;       // [4 d_g]
+  const float* b_hh;
   float* H;                // [S * n_range][d_g / 8]: partial sums of w_s . h_t
   const uint16_t* W_hh;    // bf16 [4 d_g][d_g]
   const float* w_s;        // [d_g]
@@ -20,6 +24,8 @@ struct RnnArgs {
   float* lstm_h;           // [S][d_g]
   float* lstm_c;
   int32_t* status;
+  int32_t* n_listed;       // set to list_cut if that is not negative
+  int list_cut;
   int S, max_chunks, t0, n_range, reset;
 };
 
@@ -33,11 +39,18 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t smem_addr, uint32_t ran
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(rank));
   return r;
 }
-// bulk copy from this CTA's shared memory into a peer's (addresses from mapa), bytes counted on the peer's barrier
-__device__ __forceinline__ void bulk_s2cluster(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-               "r"(src), "r"(bytes), "r"(bar)
+// 16 bytes into a peer's shared memory (addresses from mapa), counted on the peer's barrier
+__device__ __forceinline__ void st_async_cluster(uint32_t dst, const uint4& v, uint32_t bar) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(dst), "r"(v.x), "r"(v.y), "r"(v.z),
+               "r"(v.w), "r"(bar)
                : "memory");
+}
+// box of a tensor map (dimensions x, y, z) into this CTA's shared memory, bytes counted on `bar`.  No multicast.
+__device__ __forceinline__ void tma_load_3d(uint32_t dst_smem, const CUtensorMap* tm, int x, int y, int z, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(dst_smem),
+      "l"(tm), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z)
+      : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
@@ -64,6 +77,8 @@ __device__ __forceinline__ bool mbar_wait_cluster_bounded(uint64_t* bar, uint32_
   } while (t_now - t_start < deadline_ns);
   return false;
 }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }

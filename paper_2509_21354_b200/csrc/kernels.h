@@ -74,7 +74,7 @@ cudaError_t launch_append_next(const LayerView& v, const void* k_new, const void
 // dev_window < 0: chunks [t0, t1).  dev_window >= 0 (the window size W): ONE chunk per sequence whose index the kernel
 // finds on the device - the chunk behind the keep list's coverage, if the stored length says it has left the window,
 // else the launch does nothing (a trigger that is replayed from a CUDA graph)
-// list_cut >= 0 (here, launch_chunk_token_mlp, launch_gate_proj): the keep list covers no more than that many chunks from now on
+// list_cut >= 0 (here, launch_chunk_token_mlp, launch_gate_rnn): the keep list covers no more than that many chunks from now on
 cudaError_t launch_chunk_mean(const LayerView& v, int t0, int t1, bool final_output, bool pool_max, cudaStream_t st, int dev_window, int list_cut);
 cudaError_t launch_chunk_mean_beside(const LayerView& v, int t0, int t1, bool final_output, bool pool_max, cudaStream_t st);
 cudaError_t launch_chunk_mlp(const LayerView& v, int t0, int t1, const MlpWeights& w, int d_sum, cudaStream_t st, int dev_window);
@@ -83,12 +83,13 @@ cudaError_t launch_pooled_out(const LayerView& v, int t0, int t1, const MlpWeigh
 // per-token MLP aggregator: hid = scratch of 2 * S * (t1 - t0) * d_sum floats
 bool token_mlp_supported(int C, int d_sum);
 cudaError_t launch_chunk_token_mlp(const LayerView& v, int t0, int t1, const MlpWeights& w, int d_sum, float* hid, int list_cut, cudaStream_t st);
-cudaError_t launch_gate_proj(const LayerView& v, int t0, int t1, const uint16_t* W_ih, const float* b_ih,
-                             const float* b_hh, int d_g, float* P, int list_cut, cudaStream_t st);
 // planes: bf16 planes of the fp32 state h that enter the recurrent product (2, or 3 = exact products)
 double gate_rnn_us_per_chunk(int S, int d_g, int planes);
-cudaError_t launch_gate_rnn(const LayerView& v, int t0, int t1, const uint16_t* W_hh, const float* w_s, float b_s,
-                            int d_g, const float* P, float* H, bool reset_state, int planes, cudaStream_t st);
+// maps: two tensor maps over the bf16 summaries of all layers; seq_base: this layer's first sequence in them
+constexpr int GATE_MAP_BYTES = 128;
+cudaError_t encode_gate_maps(void* maps, const void* ksum, const void* vsum, long long n_seq, int max_chunks, int S, int d_g);
+cudaError_t launch_gate_rnn(const LayerView& v, const void* maps, int seq_base, int t0, int t1, const uint16_t* W_ih, const uint16_t* W_hh, const float* b_ih, const float* b_hh,
+                            const float* w_s, float b_s, int d_g, float* H, bool reset_state, int planes, int list_cut, cudaStream_t st);
 // one LSTM step on chunk t with the carried state, its score, and chunk t appended to the keep list for tau (which must
 // cover chunks [0, t)), its summary rows appended to kkept / vkept, the device's coverage count set to t + 1.
 // dev_window >= 0: t is found on the device as above (the argument t is ignored), nothing happens if no chunk is due

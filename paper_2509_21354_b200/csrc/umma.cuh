@@ -134,6 +134,17 @@ __device__ __forceinline__ void tmem_ld_wait16(uint32_t (&r)[16]) {
                  "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])::"memory");
 }
 
+// 16 lanes x 8 fp32 columns as the accumulator fragment of an m16n8 warp MMA (thread t: lanes t / 4 and t / 4 + 8, columns 2 (t % 4),
+// + 1), without waiting for the data; the address names the first of the 16 lanes
+__device__ __forceinline__ void tmem_ld_frag_nowait(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
+}
+// waits for the loads issued so far; a, b: what two of them bring (the values may not be touched before)
+__device__ __forceinline__ void tmem_ld_wait_frags(uint32_t (&a)[4], uint32_t (&b)[4]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3])::"memory");
+}
+
 // stores 32 consecutive fp32 columns of this thread's lane and waits until they are in tensor memory
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const float (&v)[32]) {
   asm volatile(

@@ -19,9 +19,8 @@ if ROOT not in sys.path:
 
 from paper_2509_21354_b200 import build as kb  # noqa: E402
 
-PHASES = ["wait for the peers' h (mbarrier)", "ldmatrix + MMA chain (W_hh h)", "prefetch of the next step's P",
-          "cell update + plane split", "send h (planes, fence, bulk copies, arrive)",
-          "round to round (P_{t+1} lands in place, expect_tx)"]
+PHASES = ["wait for the peers' h (mbarrier)", "ldmatrix + MMA chain (W_hh h)", "start of a round (pre-activations asked for)",
+          "cell update", "split and send h (planes, asynchronous stores)", "rest of a round"]
 SLOTS = [6, 0, 1, 2, 3, 4]
 
 
@@ -62,11 +61,11 @@ def main(cfgs):
                 tot += cyc
                 print(f"  {nm:52s} {cyc:8.0f} cycles  {cyc / mhz:6.3f} us   (per step and group)")
             o = (once.astype(np.int64) - int(once[0])) / 1e3
-            print(f"  CTA 0, us after its entry: W_hh fragments loaded {o[1]:.2f}, predecessor waited for {o[2]:.2f}, initial state and "
-                  f"first P {o[3]:.2f}, cluster barrier {o[4]:.2f}, step loop done {o[5]:.2f}, state out + cluster barrier {o[6]:.2f}")
+            print(f"  CTA 0, us after its entry: weights loaded {o[1]:.2f}, predecessor waited for {o[2]:.2f}, initial state "
+                  f"{o[3]:.2f}, cluster barrier {o[4]:.2f}, step loop done {o[5]:.2f}, state out + cluster barrier {o[6]:.2f}")
             loop_us = tot * rounds / mhz
             print(f"  {'sum':52s} {tot:8.0f} cycles  {tot / mhz:6.3f} us   x {groups} group(s) = {tot * groups / mhz:.3f} us per step; "
-                  f"step loop {loop_us:.1f} us of the {us_kernel:.1f} us (rest: W_hh fragments into registers, first P, "
+                  f"step loop {loop_us:.1f} us of the {us_kernel:.1f} us (rest: weights, first batch of the projection, "
                   "cluster syncs, score head)")
         rig.st.close()
 

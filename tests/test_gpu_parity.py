@@ -175,6 +175,35 @@ def test_two_sequence_groups_per_cluster(d_g, B, H):
     assert torch.equal(st.scores[0, :, :pb.Nc], want[:, :pb.Nc])
 
 
+@pytest.mark.parametrize("d_g,S", [(64, 3), (128, 17), (256, 9), (256, 299)])
+@pytest.mark.parametrize("planes", [2, 3])
+def test_input_projection_over_batches_of_chunks(d_g, S, planes):
+    # The projection runs in batches of 8 chunks (one group of sequences per cluster) or 4 (two, S = 299): ranges that end before,
+    # at and behind the edge of a batch, from scratch and behind a carried state, sequences that fill no group.  The input of a
+    # chunk behind the range, and of the layer's neighbour, must not show: those rows hold NaN.
+    b = _binding()
+    Nc = 19
+    wl = wlm.Workload("batches", B=1, H=S, n=(Nc + 6) * 16 + 40, C=16, W=32, d_g=d_g, agg="mean", key_offset_std=0.5, seed=d_g + S)
+    pb = hz.Problem(wl)
+    st = make_store(wl, n_layers=2)
+    load_kv(st, 0, pb.K, pb.V)
+    st.set_gate_planes(planes)
+    lw = b.LstmWeights(pb.lstm)
+    st.summarize_chunks(0, 0, pb.Nc, None)
+    torch.cuda.synchronize()
+    keep = st.ksum_bf16.clone(), st.vsum_bf16.clone()
+    for cuts in ((0, 1), (0, 4), (0, 5), (0, 7), (0, 8), (0, 9), (0, 16), (0, 17), (0, 3, 11, 19), (0, 8, 12, 16, 17)):
+        for buf, whole in zip((st.ksum_bf16, st.vsum_bf16), keep):
+            buf.fill_(float("nan"))
+            buf[0, :, :cuts[-1]] = whole[0, :, :cuts[-1]]
+        for t0, t1 in zip(cuts, cuts[1:]):
+            st.gate(0, t0, t1, lw)
+        torch.cuda.synchronize()
+        assert st.poll_status() == 0
+        got = st.scores[0, :, :cuts[-1]].cpu().numpy()
+        assert np.abs(got - pb.sc64[:, :cuts[-1]]).max() <= 2e-4, cuts      # the bound that scores are held to everywhere here
+
+
 def test_chunk_of_one_identity_keep_all_is_dense():
     # C = 1 with identity aggregation and tau = 0: the summary path reproduces dense attention
     b = _binding()
