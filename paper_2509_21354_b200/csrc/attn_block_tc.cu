@@ -1,5 +1,5 @@
-// Attention of a block of queries over the retained set (Sec. 3.3, softmax of Eq. 1) on the 5th-generation
-// tensor cores: the T query tokens decoded together times the G = Hq / Hkv query heads sharing a KV
+// Attention of a block of more than 32 query rows over the retained set (Sec. 3.3, softmax of Eq. 1; up to 32: attn_block_warp.cu) on
+// the 5th-generation tensor cores: the T query tokens decoded together times the G = Hq / Hkv query heads sharing a KV
 // head form R = T * G <= 128 query rows per KV sequence; out[r] = softmax(q[r] K'^T * scale) V'.
 //
 // Every retained K/V row is fetched once per KV sequence (HBM-bound), both products run as
@@ -22,9 +22,9 @@
 //               when a row's maximum has grown by more than 8 (log2 units) does the warp rescale its
 //               rows of O in tensor memory, so p stays below 2^8 and the usual per-tile rescale of O
 //               disappears.
-//  * with R <= 32 (<= 64) query rows the block is laid out four times (twice) down the 128 rows of the
-//    A operand, and each copy's warp takes a quarter (half) of a tile's 64 columns: the softmax of
-//    a tile then runs on all four warps of a group, one per scheduler, instead of on one.
+//  * with R <= 64 query rows the block is laid out twice down the 128 rows of the
+//    A operand, and each copy's warps take half of a tile's 64 columns: the softmax of
+//    a tile then runs on all four warps of a group, one per scheduler, instead of on two.
 //  * Q sits in shared memory as the K-major A operand for the whole CTA.
 //  * tile rows beyond the valid ones (ragged tail, partial tiles of kept rows) hold stale bytes:
 //    their logits are masked and their V rows are zeroed before P V (0 * NaN would poison O).
@@ -129,7 +129,7 @@ kve_decode_attn_block_tc_kernel(const __grid_constant__ CUtensorMap tmK, const _
 
   pdl_wait();      // lengths, keep lists, summaries and the queries come from earlier kernels
 
-  FirstPages first;
+  int first = -1;
   if (warp == 0) first = first_pages(a, s, split, lane);
   const BlockGeom gm = block_geometry(a, s, split);
   // the sequence has outgrown what this launch was sized for (a replayed launch): rows would be dropped
@@ -245,12 +245,8 @@ kve_decode_attn_block_tc_kernel(const __grid_constant__ CUtensorMap tmK, const _
       umma::fence_after_sync();
       float sv[CW];
       if (warp_active) {
-        if (CW == 16) {
-          umma::tmem_ld16(my_s, reinterpret_cast<float(&)[16]>(sv));
-        } else {
 #pragma unroll
-          for (int c = 0; c < CW / 32; ++c) umma::tmem_ld32(my_s + c * 32, reinterpret_cast<float(&)[32]>(sv[c * 32 % CW]));
-        }
+        for (int c = 0; c < CW / 32; ++c) umma::tmem_ld32(my_s + c * 32, reinterpret_cast<float(&)[32]>(sv[c * 32 % CW]));
       }
       umma::fence_before_sync();
       __syncwarp();
@@ -452,7 +448,7 @@ kve_decode_attn_block_tc_kernel(const __grid_constant__ CUtensorMap tmK, const _
     umma::fence_before_sync();
   }
 
-  if (gm.n_splits > 1) block_merge_splits(a, s, gm.n_splits, a.R, flag, TC_THREADS);
+  if (gm.n_splits > 1) block_merge_splits(a, s, gm.n_splits, flag, warp, lane, TC_THREADS / 32, [] { __syncthreads(); });
   umma::fence_before_sync();
   __syncthreads();
   if (warp == 1) umma::tmem_dealloc(tmem_base, TC_TMEM_COLS);
@@ -469,7 +465,6 @@ static cudaError_t launch_tc(const CUtensorMap* tm, const BlockArgs& a, dim3 gri
 }
 
 cudaError_t launch_attn_block_tc(const CUtensorMap* tm, const BlockArgs& a, dim3 grid, cudaStream_t st) {
-  if (a.R <= 32) return launch_tc<4>(tm, a, grid, st);
   if (a.R <= 64) return launch_tc<2>(tm, a, grid, st);
   return launch_tc<1>(tm, a, grid, st);
 }

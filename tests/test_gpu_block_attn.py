@@ -209,6 +209,17 @@ def test_action_token_loop_replays_from_a_cuda_graph():
     assert int(st.seq_len[0, 0]) == wl.n + steps * T
 
 
+@pytest.mark.parametrize("G,T", [(1, 15), (1, 16), (1, 17), (4, 8)])
+@pytest.mark.parametrize("n", [257, 272, 273, 320, 1500])
+def test_small_query_blocks_at_tile_edges_and_over_many_page_boxes(G, T, n):
+    # one and two 16-row tiles of queries, full and not; last tiles of 1, 16, 17 and 64 rows (a consumer warp owns 16 keys); 160
+    # sequences leave a CTA all tiles of one: pages of 8 rows are looked up in batches of 32, of which n = 1500 needs six
+    wl = wlm.CFG1.small(B=20, H=8, n=n, C=8, W=64, seed=50 + T)
+    b, pb, st = _prepared(wl, "raw", G, T)
+    _check(b, pb, st, "raw", G, T, causal=True)
+    _check(b, pb, st, "raw", G, T, dense=True, step=1)
+
+
 # causal blocks: the block's tokens are the newest rows of the cache and token t sees the cache up to itself
 @pytest.mark.parametrize("G,T,n", [(4, 7, 2443), (1, 33, 2200), (2, 40, 1989), (4, 32, 2048 + 31)])
 def test_causal_block_attention_matches_oracle(G, T, n):
