@@ -17,7 +17,8 @@
 //    accumulators (as many independent MMA chains), added smallest plane first at the end.  128 MMAs per scheduler and round take
 //    ~1000 cycles of ~2400, whether one warp or two issue them, and in as many chains as one likes: that is their rate.
 //  * MMA rows are ordered so that one thread ends up holding the i, f, g, o pre-activations of the
-//    same (hidden unit, sequence): the cell update is thread-local, c lives in registers.  f, i and g share one reciprocal
+//    same (hidden unit, sequence): the cell update is thread-local, c lives in registers.  The cells of two sequences are updated side by side
+//    in packed operations (256 x 56 75.1 -> 74.3 us).  f, i and g share one reciprocal
 //    and o and tanh(c) another (five exponentials and two reciprocals per element instead of five and five: the
 //    special-function unit is what the cell update waits for).
 //  * Input projection: a warp of a third warpgroup multiplies W_ih x_t a batch of GX_ROUNDS rounds (step, group) ahead on tcgen05.  The
@@ -26,8 +27,9 @@
 //    accumulators fill the other half.  Rows of W_ih are placed so that tcgen05.ld in its 16-lane shape hands a thread its own four
 //    pre-activations of two sequences in the layout of the MMA fragments: two instructions a round.  As a kernel of its own
 //    (a GEMM over all chunks, P = 254 MB on 512 sequences x 121 chunks written and read again) it took 70 us there, 25 us on 256 x 56, 11 us on
-//    8 x 28 at d_g = 128; here it adds what its MMAs (32 a batch, ~68 cycles each whatever the columns) take away from the recurrence's:
-//    ~45 cycles each, 6 us on 256 x 56.  Issued by the recurrence's own warps it cost another 2 to 4 us and, with the branches
+//    8 x 28 at d_g = 128; here it adds what the issue of its MMAs (32 a batch, ~68 cycles each whatever the columns) takes away from the
+//    recurrence's warps: 3 us on 256 x 56 (77.5 us without them, 3 more if one warp issues all).  A chain of 300 chunks of 8 sequences pays more for that than the
+//    GEMM cost it (348 -> 358 us), all others gain.  Issued by the recurrence's own warps it cost another 2 to 4 us and, with the branches
 //    around it, 10 % of a round.
 //  * Exchange of h_t: a warp writes the planes of its 8 hidden units into its own CTA's double-buffered h planes (two units per
 //    4-byte word, after one shuffle), and sends them from there to every other CTA of the cluster in 16-byte asynchronous stores that
@@ -38,8 +40,8 @@
 //    warpgroup adds up its 8 units (d_g / 8 partial sums per (s, t) go to memory: an eighth of the bytes of h_t) and announces the bytes of
 //    the next exchange, and when the chain is through the cluster adds the partial sums up in a fixed order.  (Both by the recurrence's
 //    warps: 77 us on 60 sequences x 80 chunks at d_g = 128, 73.6 so.)
-//  Measured, the whole gate: 512 sequences x 121 chunks 318 -> 277 us, 256 x 56 87.7 -> 78.6 us, 128 x 61 86 -> 83 us, 8 x 28 at d_g = 128
-//  32 -> 27.7 us, 60 x 5 at d_g = 128 12.7 -> 8.9 us (before: projection and recurrence as two kernels, back to back).
+//  Measured, the whole gate: 512 sequences x 121 chunks 318 -> 277 us, 256 x 56 87.6 -> 74.3 us, 32 x 250 298 -> 299.5 us, 8 x 28 at d_g = 128
+//  30.7 -> 27.0 us, 60 x 80 75.7 -> 69.1 us, 60 x 5 12.9 -> 8.9 us (before: projection and recurrence as two kernels, back to back).
 //  Slower, with the kernels of that time: waiting for the CTA's own planes and the peers' apart, with the own units' MMAs in between (255 -> 261 us a step
 //  on 256 sequences), the two warps of a scheduler taking turns at the tensor cores (512 x 121 279 -> 317 us), and the sums of the even and the
 //  odd k tiles in accumulators of their own (286 -> 308 us).
@@ -61,7 +63,7 @@ constexpr int GX_TMEM_W = 0;                                 // two tiles of 128
 constexpr int GX_TMEM_ACC = 2 * D;                           // [batch & 1][tile][GX_N]
 constexpr int GX_TMEM_COLS = 512;
 static_assert(GX_TMEM_ACC + 4 * GX_N == GX_TMEM_COLS, "tensor memory");
-// two warpgroups of the recurrence and a third with the projector and the score warp (a warpgroup, because registers move
+// two warpgroups of the recurrence and a third with the projectors and the score warp (a warpgroup, because registers move
 // between whole warpgroups: with 9 warps of equal shares the recurrence would have 168 registers)
 constexpr int GATE_THREADS = RNN_THREADS + 128;
 // registers per thread of the recurrence and of the third warpgroup, which share out those of the launch
@@ -120,6 +122,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __maxnreg__((GATE_REGS<DG, PL>))
   constexpr int OFF_BARS = OFF_PROD + NG * 2 * PROD_BUF * 4;
   constexpr int T = GX_ROUNDS / NG;                     // steps of a batch of the input projection
   constexpr bool P_LATE = DG < 256;                     // pre-activations fetched behind the MMAs, not in front: 77 us, 79 (60 sequences x 80 chunks, d_g = 128)
+  constexpr bool PACE_BY_SENDS = DG == 256 && NG == 1;  // where in a round the projector's MMAs go out
   constexpr int SENDS = ((CL - 1) * PL * NS + 31) / 32;         // 16-byte messages to the peers per lane, step and group
   static_assert(HU == 8 * RNN_WARPS && KT % 2 == 0, "one pair of m16 tiles (8 units x 4 gates) per warp");
   // what the warpgroups ask for is exactly what the launch has, or the last one to ask would wait for good
@@ -134,7 +137,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __maxnreg__((GATE_REGS<DG, PL>))
   uint64_t* x_done = x_full + 1;                                                 // [2] pre-activations of a batch computed
   uint64_t* x_read = x_done + 2;                                                 // [2] ... and read by all warps
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(x_read + 2);
-  volatile uint32_t* rounds_done = tmem_slot + 1;                                // MMA chains that warp 0 has behind it
+  volatile int* rounds_done = reinterpret_cast<volatile int*>(tmem_slot + 1);    // rounds of which warp 0 has its MMAs (or its sends) behind it
   // [GX_KB] K-blocks of summary rows, on a 1024-byte boundary
   unsigned char* xs = smem_raw + ((smem_u32(smem_raw) + RNN_SMEM_X<DG, NG, PL> + 1023u) & ~1023u) - smem_u32(smem_raw);
 
@@ -151,7 +154,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __maxnreg__((GATE_REGS<DG, PL>))
     *rounds_done = 0;
     mbar_init(x_full, 1);
     for (int i = 0; i < 2; ++i) {
-      mbar_init(&x_done[i], 1);
+      mbar_init(&x_done[i], 2);
       mbar_init(&x_read[i], RNN_WARPS);
     }
     mbar_fence_init();
@@ -176,42 +179,47 @@ __global__ void __cluster_dims__(CL, 1, 1) __maxnreg__((GATE_REGS<DG, PL>))
   };
   if (warp >= RNN_WARPS) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(PROJ_REGS));
-    // ================= projector warp =================
-    // Pre-activations W_ih x_t a batch of GX_ROUNDS rounds ahead of the recurrence.
+    // ================= projector warps =================
+    // Pre-activations W_ih x_t a batch of GX_ROUNDS rounds ahead of the recurrence.  Each of the two issues the MMAs of one tile: every
+    // issue holds up the other warps of its scheduler for some 45 cycles, wherever in the round it falls, and this way two schedulers
+    // share them (256 sequences x 56 chunks 78.5 -> 76.9 us, 32 x 250 320 -> 312).
     pdl_wait();      // the summaries come from earlier kernels
     __syncthreads();      // W_ih is in tensor memory, and xs, its staging area, is free
     umma::fence_after_sync();
     cluster_arrive();      // the recurrence's first meeting, which this warp has nothing to wait for
     bool ok = true;
     int n_fetched = 0, n_begun = 0;
-    if (warp == RNN_WARPS && lane == 0) {
+    if ((warp == RNN_WARPS || warp == RNN_WARPS + 2) && lane == 0) {
+      const int tile = warp == RNN_WARPS ? 0 : 1;
       asm volatile("fence.proxy.async.global;" ::: "memory");
       for (int b = 0; b < n_batches && ok; ++b) {
         const int buf = b & 1;
         // the rows of all steps and sequences of the batch: a copy per K-block, zeros beyond the store (what it brings beyond the range
         // or from another layer goes into columns that nobody reads)
-        mbar_arrive_expect_tx(x_full, GX_BYTES);
+        if (tile == 0) {
+          mbar_arrive_expect_tx(x_full, GX_BYTES);
 #pragma unroll
-        for (int kb = 0; kb < GX_KB; ++kb)
-          tma_load_3d(smem_u32(xs) + kb * GX_KB_BYTES, kb < GX_KB / 2 ? &map_k : &map_v, (kb & 1) * umma::KBLOCK_ELEMS, a.seq_base + seq0, a.t0 + b * T, x_full);
+          for (int kb = 0; kb < GX_KB; ++kb)
+            tma_load_3d(smem_u32(xs) + kb * GX_KB_BYTES, kb < GX_KB / 2 ? &map_k : &map_v, (kb & 1) * umma::KBLOCK_ELEMS, a.seq_base + seq0, a.t0 + b * T, x_full);
+        }
         n_fetched = b + 1;
         ok = mbar_wait_bounded(x_full, (uint32_t)(b & 1)) && (b < 2 || mbar_wait_bounded(&x_read[buf], (uint32_t)(((b >> 1) - 1) & 1)));
         if (!ok) break;
         umma::fence_after_sync();
         n_begun = b + 1;
-        // (A loop over the tiles: what runs once has to be fetched first, and a launch of 5 chunks took 4 us longer with the issue of 32 MMAs spelled out.)
+        const uint32_t acc = tmem + GX_TMEM_ACC + (uint32_t)((buf * 2 + tile) * GX_N);
+        // A K-block at a time, when warp 0 reports the right moment of a round (for the pace only: the wait gives up soon): behind its
+        // sends at d_g = 256, where the recurrence then waits for its peers (32 x 250 312 -> 303 us), behind its MMAs below (8 x 400 at
+        // d_g = 128 333 -> 321.5).  With two groups there is always somebody at work: a tile at a time (512 x 121 285 -> 277 us).
 #pragma unroll 1
-        for (int tile = 0; tile < 2; ++tile) {
-          // The tensor cores work on one of the two products at a time.  With two groups the tiles go out one by one, when warp 0 has the
-          // MMAs of a round behind it (for the pace only: the wait gives up soon).  512 sequences x 121 chunks 285 us in one go, 277 so; with one
-          // group nothing is gained by it.
-          if (NG > 1 && b > 0)
-            for (int poll = 0; poll < 4096 && *rounds_done < (uint32_t)((b - 1) * GX_ROUNDS + tile * 3 + 2); ++poll) __nanosleep(20);
-          const uint32_t acc = tmem + GX_TMEM_ACC + (uint32_t)((buf * 2 + tile) * GX_N);
+        for (int kb = 0; kb < GX_KB; ++kb) {
+          const int due = NG == 1 ? (b - 1) * GX_ROUNDS + 1 + 2 * kb : (b - 1) * GX_ROUNDS + 2 + 3 * tile;
+          if (b > 0 && (NG == 1 || kb == 0))
+            for (int poll = 0; poll < 2048 && *rounds_done < due; ++poll) __nanosleep(30);
 #pragma unroll
-          for (int k = 0; k < 4 * GX_KB; ++k)
-            umma::mma_bf16_ts(acc, tmem + GX_TMEM_W + (uint32_t)(tile * D + k * 8), umma::smem_desc(smem_u32(xs) + (k >> 2) * GX_KB_BYTES + (k & 3) * 32),
-                              umma::instr_desc_bf16(128, GX_N), k != 0);
+          for (int k = 0; k < 4; ++k)
+            umma::mma_bf16_ts(acc, tmem + GX_TMEM_W + (uint32_t)(tile * D + kb * 32 + k * 8), umma::smem_desc(smem_u32(xs) + kb * GX_KB_BYTES + k * 32),
+                              umma::instr_desc_bf16(128, GX_N), (kb | k) != 0);
         }
         umma::commit(&x_done[buf]);
         ok = mbar_wait_bounded(&x_done[buf], (uint32_t)((b >> 1) & 1));      // the rows may be overwritten
@@ -338,16 +346,16 @@ __global__ void __cluster_dims__(CL, 1, 1) __maxnreg__((GATE_REGS<DG, PL>))
       *reinterpret_cast<uint32_t*>(hs + js / NS * 2 * HS_BUF + (k2 >> 2) * KBLK + (pl * NS + j) * 8 + (k2 & 3) * 2) = p0[pl] | (p1[pl] << 16);
   }
   // state of the sequences 2 tig, 2 tig + 1 of every group
-  float c[NG][2], hlast[NG][2];
+  float2 c[NG], hlast[NG];
 #pragma unroll
-  for (int gi = 0; gi < NG; ++gi)
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int s = seq0 + gi * NS + tig * 2 + e;
-      const bool carried = !a.reset && s < a.S;
-      c[gi][e] = carried ? a.lstm_c[(long long)s * DG + ug] : 0.f;
-      hlast[gi][e] = carried ? a.lstm_h[(long long)s * DG + ug] : 0.f;
-    }
+  for (int gi = 0; gi < NG; ++gi) {
+    const int s = seq0 + gi * NS + tig * 2;
+    const bool even = !a.reset && s < a.S, odd = !a.reset && s + 1 < a.S;
+    const long long at = (long long)s * DG + ug;
+    c[gi] = make_float2(even ? a.lstm_c[at] : 0.f, odd ? a.lstm_c[at + DG] : 0.f);
+    hlast[gi] = make_float2(even ? a.lstm_h[at] : 0.f, odd ? a.lstm_h[at + DG] : 0.f);
+  }
+
   // message m of a warp goes to peer (rank + 1 + m / rows of a block): row m % rows of that CTA's buffers, as an address in the cluster window
   uint32_t peer_hs[SENDS > 0 ? SENDS : 1];
 #pragma unroll
@@ -428,7 +436,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __maxnreg__((GATE_REGS<DG, PL>))
 #pragma unroll
               for (int mt = 0; mt < 2; ++mt) mma_bf16_16816(acc[pl][mt], A[kp][mt][half], bf[kp & 1][pl][2 * half], bf[kp & 1][pl][2 * half + 1]);
         }
-        if (NG > 1 && tid == 0) *rounds_done = (uint32_t)(step * NG + gi + 1);
+        if (!PACE_BY_SENDS && tid == 0) *rounds_done = step * NG + gi + 1;
         KVE_RNN_MARK(1);
 
         // (the vote is a scheduling fence: without it the compiler draws what follows into the MMA chain, 10 % of a step)
@@ -436,26 +444,23 @@ __global__ void __cluster_dims__(CL, 1, 1) __maxnreg__((GATE_REGS<DG, PL>))
         if (P_LATE) ask_pin();
         umma::tmem_ld_wait_frags(pin[0], pin[1]);
         // ---- cell update (thread-local), planes of h_t into this CTA's buffer ---------------------
-        float hv[2];
+        float2 pre[4];       // both sequences: 0 = i, 1 = f (tile 0, rows g / g+8), 2 = g, 3 = o (tile 1)
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          float pre[4];
+        for (int q = 0; q < 4; ++q) {
+          const int mt = q >> 1, ai = (q & 1) * 2;
+          float2 sum = make_float2(acc[PL - 1][mt][ai], acc[PL - 1][mt][ai + 1]);      // smallest plane first
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {   // q: 0 = i, 1 = f (tile 0, rows g / g+8), 2 = g, 3 = o (tile 1)
-            const int mt = q >> 1, ai = (q & 1) * 2 + e;
-            float sum = acc[PL - 1][mt][ai];      // smallest plane first
-#pragma unroll
-            for (int pl = PL - 2; pl >= 0; --pl) sum += acc[pl][mt][ai];
-            pre[q] = sum + (__uint_as_float(pin[mt][ai]) + bias[q]);
-          }
-          hlast[gi][e] = hv[e] = lstm_cell(pre, c[gi][e]);
+          for (int pl = PL - 2; pl >= 0; --pl) sum = add2(sum, make_float2(acc[pl][mt][ai], acc[pl][mt][ai + 1]));
+          pre[q] = add2(sum, add2(make_float2(__uint_as_float(pin[mt][ai]), __uint_as_float(pin[mt][ai + 1])), make_float2(bias[q], bias[q])));
         }
+        const float2 hv = lstm_cell_pair(pre, c[gi]);
+        hlast[gi] = hv;
         KVE_RNN_MARK(3);
         // products of the score: nothing of the chain waits for their sum
         {
           float* mine = prod + (gi * 2 + buf) * PROD_BUF + (warp * 2 * 4 + tig) * 8 + g;
-          mine[0] = w_score * hv[0];
-          mine[4 * 8] = w_score * hv[1];
+          mine[0] = w_score * hv.x;
+          mine[4 * 8] = w_score * hv.y;
         }
         // ---- the warp's k-block (8 units: [plane][sequence][8], contiguous) to every CTA of the cluster ----
         if (send_h) {
@@ -465,7 +470,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __maxnreg__((GATE_REGS<DG, PL>))
           const bool odd = (g & 1) != 0;
           unsigned char* mine = reinterpret_cast<unsigned char*>(hs) + off + (tig * 2 + (g & 1)) * 16 + (g >> 1) * 4;
           uint32_t pl[3];      // planes of both sequences, the even one below
-          split3_pair(hv[0], hv[1], pl);
+          split3_pair(hv.x, hv.y, pl);
           const uint32_t h0 = __byte_perm(pl[0], pl[1], 0x5410), h1 = __byte_perm(pl[0], pl[1], 0x7632);      // two planes of a sequence
           const uint32_t keep = odd ? h1 : h0, got = __shfl_xor_sync(0xffffffffu, odd ? h0 : h1, 4);
           *reinterpret_cast<uint32_t*>(mine) = __byte_perm(odd ? got : keep, odd ? keep : got, 0x5410);
@@ -484,6 +489,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __maxnreg__((GATE_REGS<DG, PL>))
           }
           if (lane == 0) mbar_arrive(&hbar_g[buf ^ 1]);     // release: this warp's own pieces are in place
         }
+        if (PACE_BY_SENDS && tid == 0) *rounds_done = step + 1;
         KVE_RNN_MARK(4);
 #ifdef KVE_RNN_STAMPS
         if (blockIdx.x == 0 && tid == 0) atomicAdd(&g_rnn_cycles[5], 1ull);
@@ -503,8 +509,8 @@ __global__ void __cluster_dims__(CL, 1, 1) __maxnreg__((GATE_REGS<DG, PL>))
     for (int e = 0; e < 2; ++e) {
       const int s = seq0 + gi * NS + tig * 2 + e;
       if (s < a.S && alive) {
-        a.lstm_c[(long long)s * DG + ug] = c[gi][e];
-        a.lstm_h[(long long)s * DG + ug] = hlast[gi][e];
+        a.lstm_c[(long long)s * DG + ug] = e ? c[gi].y : c[gi].x;
+        a.lstm_h[(long long)s * DG + ug] = e ? hlast[gi].y : hlast[gi].x;
       }
     }
   // (the last step's products, which no exchange follows)

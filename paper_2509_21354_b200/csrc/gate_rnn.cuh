@@ -85,22 +85,29 @@ __device__ __forceinline__ void cluster_sync_all() {
 
 __device__ __forceinline__ float fast_sigmoid(float x) { return __fdividef(1.f, 1.f + __expf(-x)); }
 __device__ __forceinline__ float fast_tanh(float x) { return 2.f * fast_sigmoid(2.f * x) - 1.f; }
-// One LSTM cell: pre-activations in the order i, f, g, o; updates c, returns h.  With E(x) = 2^(-x log2 e):
+// Two LSTM cells at once, in packed operations where there are any: pre-activations in the order i, f, g, o; updates c, returns h.
+// With E(x) = 2^(-x log2 e):
 //   c = f c + i g = [c (1 + E_i)(1 + E_2g) + (1 - E_2g)(1 + E_f)] / [(1 + E_f)(1 + E_i)(1 + E_2g)],  h = (1 - E_2c) / [(1 + E_o)(1 + E_2c)]
-// five exponentials and two reciprocals.  The exponents stop at 40 (a sigmoid of 1e-12), which keeps the products finite.
-__device__ __forceinline__ float exp2_neg_capped(float x, float scale) {      // 2^(-x scale), at most 2^40; NaN stays NaN
-  float y;
-  asm("min.NaN.f32 %0, %1, 0f42200000;" : "=f"(y) : "f"(-x * scale));
-  return ex2_fast(y);
-}
-__device__ __forceinline__ float lstm_cell(const float (&pre)[4], float& c) {
+// five exponentials and two reciprocals per cell.  The exponents stop at 40 (a sigmoid of 1e-12), which keeps the products finite.
+__device__ __forceinline__ float2 lstm_cell_pair(const float2 (&pre)[4], float2& c) {
   constexpr float L2E = 1.44269504088896340736f;
-  const float ei = 1.f + exp2_neg_capped(pre[0], L2E), ef = 1.f + exp2_neg_capped(pre[1], L2E);
-  const float g2 = exp2_neg_capped(pre[2], 2.f * L2E), eo = 1.f + exp2_neg_capped(pre[3], L2E);
-  const float eg = 1.f + g2, ig = ei * eg;
-  c = __fdividef(fmaf(c, ig, (1.f - g2) * ef), ef * ig);
-  const float c2 = exp2_neg_capped(c, 2.f * L2E);
-  return __fdividef(1.f - c2, eo * (1.f + c2));
+  const float2 one = make_float2(1.f, 1.f);
+  auto e = [](float2 x, float scale) {      // 2^(-x scale), at most 2^40; NaN stays NaN
+    const float2 y = mul2(x, make_float2(-scale, -scale));
+    float2 z;
+    asm("min.NaN.f32 %0, %1, 0f42200000;" : "=f"(z.x) : "f"(y.x));
+    asm("min.NaN.f32 %0, %1, 0f42200000;" : "=f"(z.y) : "f"(y.y));
+    return make_float2(ex2_fast(z.x), ex2_fast(z.y));
+  };
+  auto minus = [&](float2 x) { return add2(one, make_float2(-x.x, -x.y)); };
+  const float2 ei = add2(one, e(pre[0], L2E)), ef = add2(one, e(pre[1], L2E));
+  const float2 g2 = e(pre[2], 2.f * L2E), eo = add2(one, e(pre[3], L2E));
+  const float2 ig = mul2(ei, add2(one, g2));
+  const float2 num = fma2(c, ig, mul2(minus(g2), ef)), den = mul2(ef, ig);
+  c = make_float2(__fdividef(num.x, den.x), __fdividef(num.y, den.y));
+  const float2 c2 = e(c, 2.f * L2E);
+  const float2 top = minus(c2), low = mul2(eo, add2(one, c2));
+  return make_float2(__fdividef(top.x, low.x), __fdividef(top.y, low.y));
 }
 // four 8 x 8 b16 blocks of shared memory as mma fragments (lane l gives the address of row l & 7 of block l >> 3)
 __device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], uint32_t addr) {
