@@ -22,13 +22,16 @@ __device__ __forceinline__ float relu_nan(float x) {
   return y;
 }
 
+// coefficients of -g at degree 6, lowest first
+#define KVE_GELU_TAIL6 {-0.999993061f, -1.1512017f, -0.458770975f, -0.0534121019f, 0.00808071511f, -0.00076921928f, 3.30927681e-05f}
+
 // relu: max(x, 0); a: |x|, at most 6; result: the tail Q(a).  x Phi(x) = relu - a * Q
 template <int DEGREE>
 __device__ __forceinline__ float2 gelu_tail2(float2 x, float2& relu, float2& a) {
   static_assert(DEGREE == 6 || DEGREE == 8, "degrees fitted");
   a = make_float2(fminf(fabsf(x.x), 6.f), fminf(fabsf(x.y), 6.f));
   relu = make_float2(relu_nan(x.x), relu_nan(x.y));
-  constexpr float G6[7] = {-0.999993061f, -1.1512017f, -0.458770975f, -0.0534121019f, 0.00808071511f, -0.00076921928f, 3.30927681e-05f};
+  constexpr float G6[7] = KVE_GELU_TAIL6;
   constexpr float G8[9] = {-0.999998868f, -1.15112329f, -0.459115446f, -0.0527141988f, 0.00733338343f, -0.00032334181f, -0.000114462782f,
                            2.50833236e-05f, -1.69040277e-06f};
   float2 p;

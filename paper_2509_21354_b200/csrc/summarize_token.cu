@@ -14,12 +14,19 @@
 //      token = column.  A thread of the sixteen warps therefore holds many tokens of ONE hidden unit: its bias is a
 //      constant, and the sum over a chunk's tokens stays in registers.  (With tokens as lanes the same kernel needed 31
 //      shuffles and as many selects per 32 activations, a bias load each and an atomic per sum: 38 instructions per
-//      activation, 690 us for 256 sequences x 56 chunks x 64 tokens x 2 sides x 256 units; now 250 us.)
-//    * Warp roles around a ring of four token buffers and two accumulators: four copy warps (two tiles under way behind the newest),
-//      one MMA thread, sixteen epilogue warps.  With two buffers and one CTA-wide barrier per tile the kernel took 522 us
-//      where it now takes 250.
+//      activation, 690 us for 256 sequences x 56 chunks x 64 tokens x 2 sides x 256 units; 250 us so.)
+//    * Warp roles around a ring of four token buffers and two accumulators (four with 128 hidden units): four copy warps (two tiles under
+//      way behind the newest), one MMA thread, sixteen epilogue warps.  With two buffers and one CTA-wide barrier per tile the kernel took 522 us
+//      where it now takes 223.
+//    * Each accumulator has epilogue warps of its own, and a thread goes through all 128 tokens of its hidden unit: one hand-over, one first load
+//      from tensor memory per 128 activations, no sums that meet in shared memory.  (All sixteen warps on every tile, 64 or 32 tokens a
+//      thread: 256 sequences x 56 chunks x 64 tokens x 256 units 254 us with the second layer, 238 so; 128 units 160 and 145 us; 64 x 30 x 128
+//      tokens 82 and 75 us.)  Items (chunks or groups of chunks) go through the accumulators in turn, so that the slices of a long chunk
+//      stay with the same threads.
+//    * The exponentials of eight tokens are taken beside the polynomial of the next eight.
 //    * The pooled activations (1/C) sum_j gelu(...) go to a scratch row per (side, sequence, chunk).
-//    Bound by the activation arithmetic (about ten fp32 operations, in packed pairs, and an exponential per activation).
+//    Bound by the activation arithmetic: 20 issue slots per pair of activations (18.6 cycles of the fp32 pipe, 16 of the exponentials'), 65 %
+//    of the schedulers' slots used.
 // Every mbarrier wait is bounded; on give-up the status word gets KVE_ERR_TIMEOUT.
 #include "common.cuh"
 #include "kernels.h"
@@ -40,10 +47,10 @@ constexpr int TM_SMEM_W1 = 0;                               // 2 K-blocks of [d_
 constexpr int TM_XBUFS = 4;                                  // token buffers
 constexpr int TM_LAG = 2;                                    // tiles whose copies are under way behind the newest
 constexpr int TM_SMEM_X = TM_SMEM_W1 + 2 * TM_MAX_DSUM * umma::KBLOCK_ROW_BYTES;   // 4 buffers x 2 K-blocks: 128 KB
-constexpr int TM_SMEM_POOL = TM_SMEM_X + TM_XBUFS * 2 * TM_KB_BYTES;          // [2 tile parities][4 groups of 32 tokens][d_sum] sums
-constexpr int TM_SMEM_BAR = TM_SMEM_POOL + 2 * 4 * TM_MAX_DSUM * 4;
-constexpr int TM_SMEM_BYTES = TM_SMEM_BAR + 128 + 1024;      // + slack to reach a 1024-byte boundary
-constexpr int TM_TMEM_COLS = 512;                           // two accumulators of up to two slabs x 128 columns
+constexpr int TM_TMEM_COLS = 512;                           // accumulators: one slab x 128 columns (four) or two (two)
+constexpr int TM_MAX_ACC = TM_TMEM_COLS / TM_N;
+constexpr int TM_SMEM_BAR = TM_SMEM_X + TM_XBUFS * 2 * TM_KB_BYTES;
+constexpr int TM_SMEM_BYTES = TM_SMEM_BAR + (2 * TM_XBUFS + 2 * TM_MAX_ACC) * 8 + 16 + 1024;      // + slack to reach a 1024-byte boundary
 static_assert(TM_SMEM_BYTES > 116 * 1024, "one CTA per SM: each allocates all of tensor memory");
 
 struct TokenMlpArgs {
@@ -58,21 +65,37 @@ struct TokenMlpArgs {
   float* hid;                // [2][n_units][d_sum] pooled activations (side, unit = s * n_range + (t - t0))
 };
 
+// The order in which a CTA goes through its tiles: as many items side by side as there are accumulators, slice by slice.
+template <int ACCS>
+struct TileWalk {
+  int my_items, tiles_per_item;      // items of this CTA: blockIdx.x + k gridDim.x
+  int k0 = 0, slice = 0, acc = 0;    // this tile: slice `slice` of item k0 + acc, in accumulator `acc`
+  __device__ __forceinline__ bool done() const { return k0 >= my_items; }
+  __device__ __forceinline__ int item() const { return (int)blockIdx.x + (k0 + acc) * (int)gridDim.x; }
+  __device__ __forceinline__ int turn() const { return k0 / ACCS * tiles_per_item + slice; }      // of the accumulator: 0, 1, ..
+  __device__ __forceinline__ void next() {
+    if (++acc < ACCS && k0 + acc < my_items) return;
+    acc = 0;
+    if (++slice < tiles_per_item) return;
+    slice = 0;
+    k0 += ACCS;
+  }
+};
+
 template <int DSUM>
 __global__ void __launch_bounds__(TM_THREADS, 1) kve_token_mlp_pool_kernel(TokenMlpArgs a) {
   constexpr int SLABS = DSUM / TM_SLAB;
-  constexpr int COLS = TM_N * SLABS / 4;       // tokens an epilogue thread goes through per tile: 64 or 32
-  constexpr int GROUPS = COLS / 32;
+  constexpr int ACCS = TM_TMEM_COLS / (TM_N * SLABS);          // accumulators, each with its own epilogue warps
+  constexpr int ACC_WARPS = TM_EPI_WARPS / ACCS;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   unsigned char* W1s = smem + TM_SMEM_W1;
   unsigned char* Xs = smem + TM_SMEM_X;
-  float* pool = reinterpret_cast<float*>(smem + TM_SMEM_POOL);
   uint64_t* x_full = reinterpret_cast<uint64_t*>(smem + TM_SMEM_BAR);      // [4] token buffer filled by the copy warps
   uint64_t* x_free = x_full + TM_XBUFS;                                     // [4] token buffer read (MMA commit)
-  uint64_t* acc_full = x_free + TM_XBUFS;                                   // [2] accumulator written (MMA commit)
-  uint64_t* acc_free = acc_full + 2;                                        // [2] accumulator read by the epilogue warps
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_free + 2);
+  uint64_t* acc_full = x_free + TM_XBUFS;                                   // [ACCS] accumulator written (MMA commit)
+  uint64_t* acc_free = acc_full + TM_MAX_ACC;                               // [ACCS] accumulator read by its epilogue warps
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_free + TM_MAX_ACC);
 
   pdl_launch_dependents();
   const LayerView& v = a.v;
@@ -92,9 +115,9 @@ __global__ void __launch_bounds__(TM_THREADS, 1) kve_token_mlp_pool_kernel(Token
       mbar_init(&x_full[i], TM_COPY_WARPS * 32);
       mbar_init(&x_free[i], 1);
     }
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < ACCS; ++i) {
       mbar_init(&acc_full[i], 1);
-      mbar_init(&acc_free[i], TM_EPI_WARPS);
+      mbar_init(&acc_free[i], ACC_WARPS);
     }
     mbar_fence_init();
   }
@@ -110,6 +133,7 @@ __global__ void __launch_bounds__(TM_THREADS, 1) kve_token_mlp_pool_kernel(Token
   // A CTA walks whole items (a chunk longer than a tile keeps all its 128-token slices on one CTA, in a row)
   const int my_items = a.n_items > (int)blockIdx.x ? (a.n_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
   const int n_tiles = my_items * a.tiles_per_item;      // of this CTA
+  TileWalk<ACCS> walk{my_items, a.tiles_per_item};
   const int chunk_shift = v.C >= TM_N ? 7 : (v.C == 64 ? 6 : 5);      // row r of a tile: chunk r >> chunk_shift
 
   if (warp >= TM_EPI_WARPS && warp < TM_MMA_WARP) {
@@ -117,14 +141,13 @@ __global__ void __launch_bounds__(TM_THREADS, 1) kve_token_mlp_pool_kernel(Token
     const int ct = tid - TM_EPI_WARPS * 32, p16 = ct & 15, r0 = ct >> 4;      // the 16-byte piece p16 of the rows r0 + 8 i
     const uint16_t* pages = (side ? v.v_pages : v.k_pages) + p16 * 8;
     unsigned char* dst0 = Xs + (p16 >> 3) * TM_KB_BYTES;
-    int item = blockIdx.x, slice = 0;
     int page[4];                                       // of the (up to four) chunks of the tile to come, looked up a tile ahead
     auto look_up = [&]() {
 #pragma unroll
       for (int x = 0; x < 4; ++x) {
-        const int u = item * a.units_per_item + x;
+        const int u = walk.item() * a.units_per_item + x;
         page[x] = -1;
-        if (x < a.units_per_item && item < a.n_items && u < a.n_units) {
+        if (x < a.units_per_item && !walk.done() && u < a.n_units) {
           const int s = (int)a.by_range.div((uint32_t)u);
           page[x] = v.page_table[(long long)s * v.max_chunks + a.t0 + (u - s * a.n_range)];
         }
@@ -140,10 +163,10 @@ __global__ void __launch_bounds__(TM_THREADS, 1) kve_token_mlp_pool_kernel(Token
 #pragma unroll
         for (int x = 0; x < 4; ++x) {
           const bool live = page[x] >= 0 && page[x] < v.n_pages;
-          if (!live && x < a.units_per_item && item * a.units_per_item + x < a.n_units) set_status(v.status, ERR_CAPACITY);
-          src[x] = live ? ((long long)page[x] * v.C + slice * TM_N) * D : -1;
+          if (!live && x < a.units_per_item && walk.item() * a.units_per_item + x < a.n_units) set_status(v.status, ERR_CAPACITY);
+          src[x] = live ? ((long long)page[x] * v.C + walk.slice * TM_N) * D : -1;
         }
-        if (++slice == a.tiles_per_item) { slice = 0; item += gridDim.x; }
+        walk.next();
         look_up();
 #pragma unroll
         for (int i = 0; i < TM_N / 8; ++i) {
@@ -166,10 +189,10 @@ __global__ void __launch_bounds__(TM_THREADS, 1) kve_token_mlp_pool_kernel(Token
     if (lane == 0) {
       constexpr uint32_t idesc = umma::instr_desc_bf16(TM_SLAB, TM_N);
       const uint32_t x_base = smem_u32(Xs), w1_base = smem_u32(W1s);
-      for (int tile = 0; tile < n_tiles; ++tile) {
-        const int buf = tile & 1, xb = tile % TM_XBUFS;
+      for (int tile = 0; tile < n_tiles; ++tile, walk.next()) {
+        const int buf = walk.acc, turn = walk.turn(), xb = tile % TM_XBUFS;
         if (!mbar_wait_bounded(&x_full[xb], (uint32_t)((tile / TM_XBUFS) & 1)) ||
-            (tile >= 2 && !mbar_wait_bounded(&acc_free[buf], (uint32_t)(((tile >> 1) - 1) & 1)))) {
+            (turn > 0 && !mbar_wait_bounded(&acc_free[buf], (uint32_t)((turn - 1) & 1)))) {
           set_status(v.status, ERR_TIMEOUT);
           break;
         }
@@ -189,82 +212,89 @@ __global__ void __launch_bounds__(TM_THREADS, 1) kve_token_mlp_pool_kernel(Token
     }
   } else {
     // ================= epilogue warps =================
-    // this thread's hidden unit and tokens: tensor-memory lane 32 (warp & 3) + lane of slab `slab`, columns [col0, col0 + COLS)
-    const int lg = warp & 3, quarter = warp >> 2;
-    const int slab = SLABS == 2 ? quarter >> 1 : 0, col0 = (SLABS == 2 ? quarter & 1 : quarter) * COLS;
+    // accumulator warp / ACC_WARPS, this thread's hidden unit: tensor-memory lane 32 (warp & 3) + lane of slab `slab`; all 128 tokens of
+    // a tile
+    const int buf = warp / ACC_WARPS, lg = warp & 3, slab = SLABS == 2 ? (warp >> 2) & 1 : 0;
     const int unit = slab * TM_SLAB + lg * 32 + lane;
     const float b1 = (side ? a.w.b1V : a.w.b1K)[unit];
-    const uint32_t tmem_t = tmem_d + (uint32_t)(slab * TM_N + col0) + ((uint32_t)(lg * 32) << 16);
+    const uint32_t cols = tmem_d + (uint32_t)((buf * SLABS + slab) * TM_N) + ((uint32_t)(lg * 32) << 16);
     const float inv_c = 1.f / (float)v.C;
-    float* hid = a.hid + (long long)side * a.n_units * DSUM;
-    // chunks no longer than this thread's tokens are summed by it alone; longer ones meet in shared memory
-    const int chunk_groups = (1 << chunk_shift) / 32;
-    float sum[GROUPS];                                  // per 32 tokens (of all slices of a long chunk)
-#pragma unroll
-    for (int g = 0; g < GROUPS; ++g) sum[g] = 0.f;
-    int item = blockIdx.x, slice = 0, item_parity = 0;
-    bool alive = true;      // a warp whose wait ran out goes on without waiting: the others meet it at the barrier below
-    for (int tile = 0; tile < n_tiles; ++tile) {
-      const int buf = tile & 1;
-      if (alive && !__all_sync(0xffffffffu, mbar_wait_bounded(&acc_full[buf], (uint32_t)((tile >> 1) & 1)))) {
-        alive = false;
-        if (lane == 0) set_status(v.status, ERR_TIMEOUT);
-      }
-      umma::fence_after_sync();
-      const uint32_t cols = tmem_t + (uint32_t)(buf * SLABS * TM_N);
-      uint32_t h[2][16];                                // 16 columns in work, 16 on their way
-      umma::tmem_ld16_nowait(cols, h[0]);
-#pragma unroll
-      for (int g = 0; g < GROUPS; ++g) {
-        float2 relu_sum = make_float2(0.f, 0.f), tail_sum = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          umma::tmem_ld_wait16(h[q]);
-          if (2 * g + q + 1 < 2 * GROUPS) umma::tmem_ld16_nowait(cols + (uint32_t)((2 * g + q + 1) * 16), h[(q + 1) & 1]);
-          else {
-            umma::fence_before_sync();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&acc_free[buf]);
-          }
-#pragma unroll
-          for (int e = 0; e < 16; e += 2) {
-            float2 relu, abs_x;
-            const float2 x = add2(make_float2(__uint_as_float(h[q][e]), __uint_as_float(h[q][e + 1])), make_float2(b1, b1));
-            const float2 tail = gelu_tail2<6>(x, relu, abs_x);
-            tail_sum = fma2(abs_x, tail, tail_sum);
-            relu_sum = add2(relu_sum, relu);
-          }
+    float* hid = a.hid + (long long)side * a.n_units * DSUM + unit;
+    constexpr float G6[7] = KVE_GELU_TAIL6;
+    int turn = 0;
+    for (int k = buf; k < my_items; k += ACCS) {
+      float sum[4] = {0.f, 0.f, 0.f, 0.f};              // per 32 tokens (of all slices of a long chunk)
+      bool alive = true;
+      for (int slice = 0; slice < a.tiles_per_item && alive; ++slice, ++turn) {
+        alive = __all_sync(0xffffffffu, mbar_wait_bounded(&acc_full[buf], (uint32_t)(turn & 1)));
+        if (!alive) {
+          if (lane == 0) set_status(v.status, ERR_TIMEOUT);
+          break;
         }
-        sum[g] += (relu_sum.x + relu_sum.y) - (tail_sum.x + tail_sum.y);
+        umma::fence_after_sync();
+        uint32_t h[2][16];                              // 16 columns in work, 16 on their way
+        umma::tmem_ld16_nowait(cols, h[0]);
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          // 32 tokens, eight at a time; the exponentials of the block before go out between the polynomial steps of this one
+          float2 relu_sum = make_float2(0.f, 0.f), tail_sum = make_float2(0.f, 0.f), abs_before[4], p_before[4];
+#pragma unroll
+          for (int blk = 0; blk <= 4; ++blk) {
+            float2 abs_x[4], p[4];
+            if (blk < 4) {
+              const int q = blk >> 1;
+              if (blk % 2 == 0) {
+                umma::tmem_ld_wait16(h[q]);
+                if (blk == 0 || g < 3) umma::tmem_ld16_nowait(cols + (uint32_t)(g * 32 + (q + 1) * 16), h[q ^ 1]);
+                else {
+                  umma::fence_before_sync();
+                  __syncwarp();
+                  if (lane == 0) mbar_arrive(&acc_free[buf]);
+                }
+              }
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const int e = (blk & 1) * 8 + 2 * i;
+                const float2 x = add2(make_float2(__uint_as_float(h[q][e]), __uint_as_float(h[q][e + 1])), make_float2(b1, b1));
+                abs_x[i] = make_float2(fminf(fabsf(x.x), 6.f), fminf(fabsf(x.y), 6.f));
+                relu_sum = add2(relu_sum, make_float2(relu_nan(x.x), relu_nan(x.y)));
+                p[i] = make_float2(G6[6], G6[6]);
+              }
+            }
+            float2 tail[4];
+#pragma unroll
+            for (int y = 0; y < 8; ++y) {      // an exponential of the block before, three steps of this one
+              if (blk > 0) {
+                if (y & 1) tail[y >> 1].y = ex2_fast(p_before[y >> 1].y);
+                else tail[y >> 1].x = ex2_fast(p_before[y >> 1].x);
+              }
+              if (blk < 4)
+#pragma unroll
+                for (int z = 3 * y; z < 3 * y + 3; ++z) p[z & 3] = fma2(p[z & 3], abs_x[z & 3], make_float2(G6[5 - z / 4], G6[5 - z / 4]));
+            }
+            if (blk > 0)
+#pragma unroll
+              for (int i = 0; i < 4; ++i) tail_sum = fma2(abs_before[i], tail[i], tail_sum);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { abs_before[i] = abs_x[i]; p_before[i] = p[i]; }
+          }
+          const float got = (relu_sum.x + relu_sum.y) - (tail_sum.x + tail_sum.y);
+          sum[g] += got;
+        }
       }
-      if (++slice < a.tiles_per_item) continue;
+      if (!alive) break;
       // the chunk(s) of this item are complete
-      if (chunk_groups <= GROUPS) {
-        const int first = item * a.units_per_item + col0 / 32 / chunk_groups;
-        if (GROUPS == 2 && chunk_groups == 2) {
-          if (first < a.n_units) hid[(long long)first * DSUM + unit] = (sum[0] + sum[GROUPS - 1]) * inv_c;
-        } else {
-#pragma unroll
-          for (int g = 0; g < GROUPS; ++g)
-            if (first + g < a.n_units) hid[(long long)(first + g) * DSUM + unit] = sum[g] * inv_c;
-        }
+      const int first = ((int)blockIdx.x + k * (int)gridDim.x) * a.units_per_item;
+      if (a.units_per_item == 1) {
+        hid[(long long)first * DSUM] = (((sum[0] + sum[1]) + sum[2]) + sum[3]) * inv_c;
+      } else if (a.units_per_item == 2) {
+        if (first < a.n_units) hid[(long long)first * DSUM] = (sum[0] + sum[1]) * inv_c;
+        if (first + 1 < a.n_units) hid[(long long)(first + 1) * DSUM] = (sum[2] + sum[3]) * inv_c;
       } else {
-        float* pl = pool + (item_parity & 1) * 4 * TM_MAX_DSUM;
 #pragma unroll
-        for (int g = 0; g < GROUPS; ++g) pl[(col0 / 32 + g) * TM_MAX_DSUM + unit] = sum[g];
-        asm volatile("bar.sync 1, %0;" ::"n"(TM_EPI_WARPS * 32) : "memory");      // the other parity keeps the next item apart
-        for (int i = tid; i < a.units_per_item * DSUM; i += TM_EPI_WARPS * 32) {
-          const int u_in = i / DSUM, col = i - u_in * DSUM, u = item * a.units_per_item + u_in;
-          float s = 0.f;
-          for (int g = 0; g < chunk_groups; ++g) s += pl[(u_in * chunk_groups + g) * TM_MAX_DSUM + col];
-          if (u < a.n_units) hid[(long long)u * DSUM + col] = s * inv_c;
-        }
-        ++item_parity;
+        for (int x = 0; x < 4; ++x)
+          if (first + x < a.n_units) hid[(long long)(first + x) * DSUM] = sum[x] * inv_c;
       }
-#pragma unroll
-      for (int g = 0; g < GROUPS; ++g) sum[g] = 0.f;
-      slice = 0;
-      item += gridDim.x;
     }
   }
   umma::fence_before_sync();

@@ -1070,6 +1070,30 @@ def test_token_mlp_aggregator_full_pipeline(C, d_sum):
     assert pb.Nc == 7
 
 
+@pytest.mark.parametrize("C,S", [(32, 97), (64, 97), (128, 53), (256, 53), (384, 41)])
+@pytest.mark.parametrize("d_sum", [128, 256])
+def test_token_mlp_with_several_items_per_cta(C, S, d_sum):
+    # three to six items (chunks, or groups of them) per CTA, not a multiple of its accumulators; chunks of one, two and three
+    # 128-token slices.  Reference: the MLP on every token and the mean in 64 bits; bound as for all MLP summaries.
+    b = _binding()
+    Nc = 9
+    wl = wlm.Workload("items", B=1, H=S, n=C * Nc + 32, C=C, W=32, d_g=64, agg="token_mlp", d_sum=d_sum, key_offset_std=0.5, seed=C + d_sum)
+    st = make_store(wl)
+    gen = torch.Generator(device="cuda").manual_seed(C)
+    k, v = (torch.randn(S, wl.n, 128, generator=gen, device="cuda").to(torch.bfloat16) for _ in range(2))
+    st.append(0, k, v)
+    mlp = wlm.gen_mlp_weights(wl)
+    st.summarize_chunks(0, 0, Nc, b.AggWeights(mlp))
+    torch.cuda.synchronize()
+    assert st.poll_status() == 0
+    for x, side, got in ((k, "K", st.ksum_f32), (v, "V", st.vsum_f32)):
+        W1, b1, W2, b2 = (torch.as_tensor(np.asarray(mlp[name + side]), device="cuda").double() for name in ("W1", "b1", "W2", "b2"))
+        for s0 in range(0, S, 8):
+            t = x[s0:s0 + 8, :Nc * C].double() @ W1.T + b1
+            want = torch.nn.functional.gelu(t).reshape(t.shape[0], Nc, C, d_sum).mean(2) @ W2.T + b2
+            assert (got[0, s0:s0 + 8, :Nc].double() - want).abs().max() <= 2e-5 * max(1.0, float(want.abs().max()))
+
+
 def test_token_mlp_aggregator_incremental_ranges_and_unsupported_geometry():
     b = _binding()
     wl = wlm.CFG2.small(B=1, H=5, n=64 * 11, C=64, W=128, agg="token_mlp", d_sum=256, seed=71)
