@@ -211,7 +211,7 @@ cudaError_t launch_chunk_mean(const LayerView& v, int t0, int t1, bool final_out
 }
 
 // ---- the same mean for a launch that runs beside the gate recurrence -----------------------------------------------
-// The recurrence leaves an SM a sixth of its registers and most of its shared memory, so the rows on their way wait there: a
+// The recurrence leaves an SM a tenth of its registers and two thirds of its shared memory (two CTAs of this kernel), so the rows on their way wait there: a
 // warp's pages come in bulk copies of 16 rows, eight of them in flight, and are added up row by row as above (the same rounding).
 // A CTA takes several units in a row, so that the copies of the next one are under way while the last is added up.
 // 4.1 TB/s beside the recurrence of 512 sequences, which takes 22 % longer meanwhile (pages of 128 tokens; the kernel above, its
