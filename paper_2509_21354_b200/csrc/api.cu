@@ -615,10 +615,11 @@ int kvE_adopt_device_state(kvE_store* st, int layer, void* stream) {
 // steps that leaves HBM idle, the chunk mean a stream that leaves everything else idle: of two ranges, the means of the second
 // are taken while the recurrence goes through the first (kve_chunk_mean_beside_kernel).  With M and R the microseconds of
 // the means and of the recurrence alone, x = M / (M + 0.7 R) of the chunks first lets both end at about the same time; M (1 - x)
-// is then hidden, and the second launches of MLP, projection and recurrence and the slower recurrence are paid.  Measured, one
-// range -> two (us a step): 512 sequences x 121 chunks of 128, MLP 1055 -> 1010; 128 x 121 of 128, MLP 370 -> 350; 256 x 240
-// of 32, MLP 604 -> 562; 512 x 56 of 64, mean 344 -> 333; 256 x 120 of 64, mean 364 -> 340, MLP 407 -> 393; below the lines:
-// 256 x 56 of 64 with 28 us to hide, mean 194 -> 189, MLP 218 -> 226; 32 x 250 of 64, mean, 33 us: 356 -> 364.  (The figures of the
+// is then hidden, and the second launches of MLP and gate and the slower recurrence are paid.  Measured, one
+// range -> two (us a step): 512 sequences x 121 chunks of 128, MLP 1008 -> 937; 128 x 121 of 128, MLP 353 -> 328; 256 x 240
+// of 32, MLP 570 -> 539; 512 x 56 of 64, mean 320 -> 300; 256 x 120 of 64, mean 340 -> 311, MLP 382 -> 366; 128 x 127 of 128 at d_g = 128, mean
+// 279 -> 244; below the lines, with the projection still a kernel of its own: 256 x 56 of 64 with 28 us to hide, mean 194 -> 189, MLP 218 -> 226; 32 x 250 of
+// 64, mean, 33 us: 356 -> 364.  (The figures of the
 // recurrence are those of d_g = 256; at 64 and 128 it is faster, which makes x too small rather than too large.  The rule over 240 settings
 // - d_g 64, 128, 256; 8 to 1024 sequences of 4160 to 16512 tokens in chunks of 32 to 512; mean and MLP - and 28 with three planes: never more than
 // 2 % behind one range, up to 23 % ahead of it, 128 x 127 of 128 at d_g = 64.)
