@@ -179,7 +179,7 @@ def algorithmic_bytes(wl, Nc, keep_mean, R, attend="summary"):
     by = {}
     by["chunk_mean"] = S * Nc * (2 * wl.C * 256 + 2 * 128 * 4)            # every stale K and V row once; fp32 means out
     by["chunk_mlp"] = S * Nc * 2 * (128 * 4 + 128 * 4 + 128 * 2)          # means in, fp32 + bf16 summaries out
-    by["gate_proj"] = S * Nc * (2 * 256 + 4 * d_g * 4)                    # bf16 summaries in, fp32 P out
+    by["gate_proj"] = S * Nc * (2 * 256 + 4 * d_g * 4)                    # as a kernel of its own: bf16 summaries in, fp32 P out
     by["gate_rnn"] = S * Nc * (4 * d_g * 4 + 4)                           # P in, scores out
     by["compact"] = S * (Nc * 4 + Nc * 4 + 4)
     rows_per_kept = wl.C if attend == "raw" else 1                          # a kept chunk: its C raw rows, or its one summary row
