@@ -498,6 +498,8 @@ __global__ void __cluster_dims__(CL, 1, 1) __maxnreg__((GATE_REGS<DG, PL>))
       }
       if (!alive) break;
     }
+    umma::fence_before_sync();      // this warp's loads out of the accumulators come before what the projector writes there next
+    __syncwarp();
     if (lane == 0) mbar_arrive(&x_read[batch & 1]);
   }
 

@@ -204,6 +204,33 @@ def test_input_projection_over_batches_of_chunks(d_g, S, planes):
         assert np.abs(got - pb.sc64[:, :cuts[-1]]).max() <= 2e-4, cuts      # the bound that scores are held to everywhere here
 
 
+@pytest.mark.parametrize("per_call", [8])
+@pytest.mark.parametrize("d_g,S,planes", [(64, 5, 2), (64, 1200, 2), (128, 16, 2), (128, 600, 3), (256, 9, 3), (256, 304, 2)])
+def test_long_gate_range_equals_short_ranges(d_g, S, planes, per_call):
+    # Buffers inside the gate kernel come round again in a long range and not in a short one: the two sets of the projection's accumulators
+    # after 16 chunks (8 with two groups of sequences per cluster).  The carried state is fp32 and splits the same way, so every bit is the same.
+    b = _binding()
+    Nc = 42
+    wl = wlm.Workload("rounds", B=1, H=S, n=Nc * 8 + 40, C=8, W=32, d_g=d_g, agg="mean", key_offset_std=0.5, seed=d_g + S)
+    st = make_store(wl)
+    gen = torch.Generator(device="cuda").manual_seed(S)
+    st.append(0, *(torch.randn(S, wl.n, 128, generator=gen, device="cuda").to(torch.bfloat16) for _ in range(2)))
+    st.set_gate_planes(planes)
+    lw = b.LstmWeights(wlm.gen_lstm_weights(wl))
+    st.summarize_chunks(0, 0, Nc, None)
+    got = []
+    for step in (per_call, Nc):
+        for rep in range(1 if step != Nc else 5):
+            for t in range(0, Nc, step):
+                st.gate(0, t, min(t + step, Nc), lw)
+            torch.cuda.synchronize()
+            assert st.poll_status() == 0
+            got.append([x.clone() for x in (st.scores[0, :, :Nc], st.lstm_h, st.lstm_c)])
+    assert all(torch.isfinite(x).all() and x.abs().max() > 0 for x in got[0])
+    for other in got[1:]:
+        assert all(torch.equal(x, y) for x, y in zip(got[0], other))
+
+
 def test_chunk_of_one_identity_keep_all_is_dense():
     # C = 1 with identity aggregation and tau = 0: the summary path reproduces dense attention
     b = _binding()
