@@ -244,6 +244,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __maxnreg__((GATE_REGS<DG, PL>))
           ok = __all_sync(0xffffffffu, mbar_wait_cluster_bounded(&hbar[2 * gi + buf], (uint32_t)((step >> 1) & 1)));
           if (ok) put_scores(gi, step);
         }
+        __syncwarp();      // all lanes have read: an arrival orders only what its own lane has done
       }
       if (!ok && lane == 0) set_status(a.status, ERR_TIMEOUT);
     }

@@ -204,11 +204,12 @@ def test_input_projection_over_batches_of_chunks(d_g, S, planes):
         assert np.abs(got - pb.sc64[:, :cuts[-1]]).max() <= 2e-4, cuts      # the bound that scores are held to everywhere here
 
 
-@pytest.mark.parametrize("per_call", [8])
+@pytest.mark.parametrize("per_call", [8, 2])
 @pytest.mark.parametrize("d_g,S,planes", [(64, 5, 2), (64, 1200, 2), (128, 16, 2), (128, 600, 3), (256, 9, 3), (256, 304, 2)])
 def test_long_gate_range_equals_short_ranges(d_g, S, planes, per_call):
     # Buffers inside the gate kernel come round again in a long range and not in a short one: the two sets of the projection's accumulators
-    # after 16 chunks (8 with two groups of sequences per cluster).  The carried state is fp32 and splits the same way, so every bit is the same.
+    # after 16 chunks (8 with two groups of sequences per cluster), the products of the score after 2.  The carried state is fp32 and splits
+    # the same way, so every bit is the same.
     b = _binding()
     Nc = 42
     wl = wlm.Workload("rounds", B=1, H=S, n=Nc * 8 + 40, C=8, W=32, d_g=d_g, agg="mean", key_offset_std=0.5, seed=d_g + S)
