@@ -343,7 +343,8 @@ const char* kvE_last_cuda_error(const kvE_store* st);
 /* ---- self-test (not part of the paper's path) ----------------------------------------------------------------------
  * Makes a bounded device-side wait run out on purpose, without a fault: a small kernel waits on a barrier that nothing
  * ever completes, with a limit of a few thousand polls (which == 0: the wait the copy pipelines and tensor-core
- * commits use) or two milliseconds (which == 1: the wait between the CTAs of a cluster in the gate recurrence).  The
+ * commits use) or two milliseconds (which == 1: the wait between the CTAs of a cluster in the gate recurrence), or gives up
+ * a ring of copies of which some are under way and waits for those before it leaves (which == 2).  The
  * kernel returns by itself, the status word reads KVE_ERR_TIMEOUT at the next kvE_poll_status, and the handle stays
  * usable.  A way to check, on the installed driver and GPU, that the failure path every kernel relies on works. */
 int kvE_selftest_timeout(kvE_store* st, int which, void* stream);

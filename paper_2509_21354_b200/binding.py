@@ -375,7 +375,8 @@ class Store:
         return kvE_poll_status(self)
 
     def selftest_timeout(self, which: int, stream=None):
-        """launches the kernel whose bounded wait runs out (which: 0 = CTA-scope wait, 1 = cluster-scope wait)"""
+        """launches the kernel whose bounded wait runs out (which: 0 = CTA-scope wait, 1 = cluster-scope wait, 2 = a ring of copies
+        given up with copies under way)"""
         _check("kvE_selftest_timeout", self.lib.kvE_selftest_timeout(self.handle, int(which), _stream(self, stream)), self.handle)
 
     def layer_state(self, layer=0) -> dict:

@@ -881,9 +881,10 @@ int kvE_profile_read(kvE_store* st, float* us) {
 const char* kvE_last_cuda_error(const kvE_store* st) { return st ? st->cuda_error.c_str() : ""; }
 
 int kvE_selftest_timeout(kvE_store* st, int which, void* stream) {
-  if (!st || (which != 0 && which != 1)) return KVE_ERR_ARG;
+  if (!st || which < 0 || which > 2) return KVE_ERR_ARG;
   if (wrong_device(st)) return KVE_ERR_STATE;
-  cudaError_t e = launch_selftest_timeout(which, st->buf.status_word, static_cast<cudaStream_t>(stream));
+  static_assert(SELFTEST_RING_BYTES <= ATTN_GRID_LIMIT * ATTN_PARTIAL_FLOATS * sizeof(float), "what the ring reads: partial records");
+  cudaError_t e = launch_selftest_timeout(which, static_cast<char*>(st->buf.workspace) + st->off_partials, st->buf.status_word, static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? KVE_OK : cuda_fail(st, e);
 }
 

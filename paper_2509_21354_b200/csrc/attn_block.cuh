@@ -99,7 +99,7 @@ __device__ __forceinline__ int first_pages(const BlockArgs& a, int s, int split,
 }
 
 // Producer warp: fetches the CTA's tiles with 2-D tensor copies into the ring `ring` (STAGES stages), arming full[stage] with the
-// byte count and waiting (bounded) on empty[stage] before a stage is reused.  Page ids are looked up 32 granules at a time, a
+// byte count and waiting (bounded) on empty[stage] before a stage is reused; comes back when the copies have landed.  Page ids are looked up 32 granules at a time, a
 // batch ahead, and looked at only when a copy needs them: a look-up is a trip to L2, and one per tile in the producer's way made 128
 // sequences x 1084 rows 18.5 us, 18.1 so (64 x 4099 35.2 and 34.6).  What a lane fetches for a tile: up to two boxes (K and V each, both 64-column halves):
 //   page tiles:    lane j < granules: hp rows of a page to tile row j * hp
@@ -125,7 +125,8 @@ __device__ __forceinline__ void block_producer(const BlockArgs& a, const BlockGe
   };
   int pages = look_up(gm.r_begin + lane * a.hp, true, first);
   int pages_next = look_up(gm.r_begin + (32 + lane) * a.hp, false, -1);
-  for (int i = 0; i < gm.n_tiles; ++i) {
+  int i = 0;
+  for (; i < gm.n_tiles; ++i) {
     const int stage = i % STAGES, round = i / STAGES;
     const int granule = i * per_tile;
     if (i > 0 && granule % 32 == 0) {
@@ -164,6 +165,7 @@ __device__ __forceinline__ void block_producer(const BlockArgs& a, const BlockGe
       tma_load_2d(vdst + BK_KBLOCK_BYTES, mv, 64, src, &full[stage]);
     }
   }
+  ring_drain<STAGES>(full, i);      // whoever waits for these tiles may have given up
 }
 
 // normalises one query row's columns 4 c4 .. +3 and writes them (bf16) and, from c4 == 0, the row's lse

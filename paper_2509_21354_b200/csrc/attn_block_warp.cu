@@ -55,6 +55,7 @@ kve_decode_attn_block_warp_kernel(const __grid_constant__ CUtensorMap tmK, const
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + BW_OFF_BAR);
   uint64_t* empty = full + BW_STAGES;
   int* flag = reinterpret_cast<int*>(empty + BW_STAGES);
+  volatile int* gave_up = flag + 1;      // a consumer's wait ran out
 
   pdl_launch_dependents();
   const LayerView& v = a.v;
@@ -76,6 +77,7 @@ kve_decode_attn_block_warp_kernel(const __grid_constant__ CUtensorMap tmK, const
       mbar_init(&empty[i], BW_GWARPS);
     }
     mbar_fence_init();
+    *gave_up = 0;
   }
   __syncthreads();
 
@@ -138,7 +140,10 @@ kve_decode_attn_block_warp_kernel(const __grid_constant__ CUtensorMap tmK, const
   for (int i = group; i < gm.n_tiles; i += 2) {
     const int stage = i % BW_STAGES;
     if (!__all_sync(0xffffffffu, mbar_wait_bounded(&full[stage], (uint32_t)((i / BW_STAGES) & 1)))) {
-      if (lane == 0) set_status(v.status, ERR_TIMEOUT);
+      if (lane == 0) {
+        set_status(v.status, ERR_TIMEOUT);
+        *gave_up = 1;
+      }
       break;
     }
     const int row0 = gm.r_begin + i * BK_TILE;
@@ -246,10 +251,11 @@ kve_decode_attn_block_warp_kernel(const __grid_constant__ CUtensorMap tmK, const
 
   // ---- the eight states (m_ref, l, O) meet in shared memory: [warp][row][BW_XP] from the start of the ring ----
   float* xch = reinterpret_cast<float*>(smem);
-  consumers_sync();      // every tile has been read
+  consumers_sync();      // every tile has been read, or somebody has given up: copies may be under way then, and the ring is left alone
+  const bool complete = *gave_up == 0;
   float* mine = xch + warp * 32 * BW_XP;
 #pragma unroll
-  for (int mt = 0; mt < MT; ++mt)
+  for (int mt = 0; mt < MT && complete; ++mt)
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
       float l = l_run[mt][e];
@@ -264,15 +270,15 @@ kve_decode_attn_block_warp_kernel(const __grid_constant__ CUtensorMap tmK, const
   const bool direct = gm.n_splits == 1;
   for (int r = warp; r < a.R; r += BW_CWARPS) {
     float2 ml[BW_CWARPS];
-    float mC = -INFINITY, lC = 0.f;
+    float mC = -INFINITY, lC = 0.f;      // (what a CTA that gave up has to say of its rows)
 #pragma unroll
-    for (int w = 0; w < BW_CWARPS; ++w) {
+    for (int w = 0; w < BW_CWARPS && complete; ++w) {
       ml[w] = *reinterpret_cast<const float2*>(xch + (w * 32 + r) * BW_XP + 128);
       mC = fmaxf(mC, ml[w].x);
     }
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int w = 0; w < BW_CWARPS; ++w) {
+    for (int w = 0; w < BW_CWARPS && complete; ++w) {
       const float f = (ml[w].x == -INFINITY) ? 0.f : exp2f(ml[w].x - mC);
       lC = fmaf(ml[w].y, f, lC);
       const float4 o = *reinterpret_cast<const float4*>(xch + (w * 32 + r) * BW_XP + lane * 4);

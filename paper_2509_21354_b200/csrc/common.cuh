@@ -95,6 +95,14 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
   return false;
 }
 
+// Waits for the copies of a ring of STAGES stages that may still be under way when those of the tiles 0 .. n_issued - 1 have been issued (tile i
+// into stage i % STAGES): shared memory is written to until they land, so a CTA that gives up a wait must not leave, nor use
+// the ring for something else, before.  Bounded by itself: a copy that never lands must not hold the CTA either.
+template <int STAGES>
+__device__ __forceinline__ void ring_drain(uint64_t* full, int n_issued) {
+  for (int i = n_issued > STAGES ? n_issued - STAGES : 0; i < n_issued; ++i) mbar_wait_bounded(&full[i % STAGES], (uint32_t)((i / STAGES) & 1), 1u << 16);
+}
+
 // 1-D bulk copy global -> this CTA's shared memory through the TMA engine, completion counted in
 // bytes on `bar`.  dst, src 16-byte aligned; bytes a multiple of 16.  No multicast.
 __device__ __forceinline__ void bulk_g2s(void* dst_smem, const void* src_gmem, uint32_t bytes, uint64_t* bar) {

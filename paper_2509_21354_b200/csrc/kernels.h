@@ -110,7 +110,8 @@ cudaError_t launch_attn(const LayerView& v, AttnMode mode, int n_chunks, int par
                         float* lse, float scale, const void* kkept, const void* vkept, float* partials, int32_t* counters,
                         const void* k_new, const void* v_new, int32_t* ticket, cudaStream_t st);
 int attn_smem_bytes();
-cudaError_t launch_selftest_timeout(int which, int32_t* status, cudaStream_t st);
+constexpr int SELFTEST_RING_BYTES = 16384;      // read from src (which 2)
+cudaError_t launch_selftest_timeout(int which, const void* src, int32_t* status, cudaStream_t st);
 
 // block-of-queries attention (grouped query heads x query tokens), tensor-map fed
 constexpr int ATTN_BLOCK_MAX_ROWS = 128;       // query rows (tokens x heads per KV head) per KV sequence

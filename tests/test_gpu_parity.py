@@ -574,6 +574,21 @@ def test_a_bounded_wait_that_runs_out_reports_timeout_and_leaves_the_handle_usab
     check_gate_and_keep(st, pb)
 
 
+def test_a_ring_that_is_given_up_is_drained_before_the_kernel_leaves():
+    """As above for a ring of copies: -6 says that the wait ran out and that the copies still under way had landed when the kernel
+    looked at them (-3: a byte was missing)."""
+    b = _binding()
+    st = make_store(wlm.CFG1.small(n=512, seed=4))
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    for _ in range(3):
+        st.workspace.random_(0, 255, generator=gen)      # what the ring reads lies in there; nothing else is called on this handle
+        st.selftest_timeout(2)
+        torch.cuda.synchronize()
+        assert st.poll_status() == -6 and st.poll_status() == 0
+    with pytest.raises(b.KveError):
+        st.selftest_timeout(3)
+
+
 def test_config2_full_size():
     """Llama-2-7B-shaped layer at the size bench.py times (B 8, H 32, n 4096, MLP aggregator, d_g 256)."""
     st, pb, aw, lw = full_check(wlm.CFG2, "summary")
