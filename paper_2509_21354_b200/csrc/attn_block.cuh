@@ -99,13 +99,14 @@ __device__ __forceinline__ int first_pages(const BlockArgs& a, int s, int split,
 }
 
 // Producer warp: fetches the CTA's tiles with 2-D tensor copies into the ring `ring` (STAGES stages), arming full[stage] with the
-// byte count and waiting (bounded) on empty[stage] before a stage is reused; comes back when the copies have landed.  Page ids are looked up 32 granules at a time, a
+// byte count and waiting (bounded) on empty[stage] before a stage is reused.  Returns the tiles issued; their
+// copies may still be under way, and a CTA of which anybody gives up a wait has to see them land (ring_drain) before it leaves.  Page ids are looked up 32 granules at a time, a
 // batch ahead, and looked at only when a copy needs them: a look-up is a trip to L2, and one per tile in the producer's way made 128
 // sequences x 1084 rows 18.5 us, 18.1 so (64 x 4099 35.2 and 34.6).  What a lane fetches for a tile: up to two boxes (K and V each, both 64-column halves):
 //   page tiles:    lane j < granules: hp rows of a page to tile row j * hp
 //   summary tiles: lane j < ceil(valid / 16): 16 kept summary rows (compacted by kvE_compact)
 template <int STAGES>
-__device__ __forceinline__ void block_producer(const BlockArgs& a, const BlockGeom& gm, int s, int lane,
+__device__ __forceinline__ int block_producer(const BlockArgs& a, const BlockGeom& gm, int s, int lane,
                                                const CUtensorMap* tmK, const CUtensorMap* tmV, const CUtensorMap* tmKs,
                                                const CUtensorMap* tmVs, int first, unsigned char* ring, uint64_t* full,
                                                uint64_t* empty) {
@@ -165,7 +166,7 @@ __device__ __forceinline__ void block_producer(const BlockArgs& a, const BlockGe
       tma_load_2d(vdst + BK_KBLOCK_BYTES, mv, 64, src, &full[stage]);
     }
   }
-  ring_drain<STAGES>(full, i);      // whoever waits for these tiles may have given up
+  return i;
 }
 
 // normalises one query row's columns 4 c4 .. +3 and writes them (bf16) and, from c4 == 0, the row's lse

@@ -55,7 +55,7 @@ kve_decode_attn_block_warp_kernel(const __grid_constant__ CUtensorMap tmK, const
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + BW_OFF_BAR);
   uint64_t* empty = full + BW_STAGES;
   int* flag = reinterpret_cast<int*>(empty + BW_STAGES);
-  volatile int* gave_up = flag + 1;      // a consumer's wait ran out
+  volatile int* issued = flag + 1;       // tiles that the producer has issued when it is through, -1 before
 
   pdl_launch_dependents();
   const LayerView& v = a.v;
@@ -77,7 +77,7 @@ kve_decode_attn_block_warp_kernel(const __grid_constant__ CUtensorMap tmK, const
       mbar_init(&empty[i], BW_GWARPS);
     }
     mbar_fence_init();
-    *gave_up = 0;
+    *issued = -1;
   }
   __syncthreads();
 
@@ -90,7 +90,10 @@ kve_decode_attn_block_warp_kernel(const __grid_constant__ CUtensorMap tmK, const
     const BlockGeom gm = block_geometry(a, s, split);
     // the sequence has outgrown what this launch was sized for (a replayed launch): rows would be dropped
     if (gm.outgrown && split == 0 && lane == 0) set_status(v.status, ERR_CAPACITY);
-    if (split < gm.n_splits) block_producer<BW_STAGES>(a, gm, s, lane, &tmK, &tmV, &tmKs, &tmVs, first, ring, full, empty);
+    if (split < gm.n_splits) {
+      const int n = block_producer<BW_STAGES>(a, gm, s, lane, &tmK, &tmV, &tmKs, &tmVs, first, ring, full, empty);
+      if (lane == 0) *issued = n;
+    }
     return;
   }
 
@@ -140,10 +143,11 @@ kve_decode_attn_block_warp_kernel(const __grid_constant__ CUtensorMap tmK, const
   for (int i = group; i < gm.n_tiles; i += 2) {
     const int stage = i % BW_STAGES;
     if (!__all_sync(0xffffffffu, mbar_wait_bounded(&full[stage], (uint32_t)((i / BW_STAGES) & 1)))) {
-      if (lane == 0) {
-        set_status(v.status, ERR_TIMEOUT);
-        *gave_up = 1;
-      }
+      // copies into the ring may be under way: this warp meets the others, which use the ring for something else then, when they have landed
+      // (the producer comes to an end, too, if it waits for us)
+      if (lane == 0) set_status(v.status, ERR_TIMEOUT);
+      for (int k = 0; k < (1 << 20) && *issued < 0; ++k) __nanosleep(2048);
+      ring_drain<BW_STAGES>(full, *issued);
       break;
     }
     const int row0 = gm.r_begin + i * BK_TILE;
@@ -251,11 +255,10 @@ kve_decode_attn_block_warp_kernel(const __grid_constant__ CUtensorMap tmK, const
 
   // ---- the eight states (m_ref, l, O) meet in shared memory: [warp][row][BW_XP] from the start of the ring ----
   float* xch = reinterpret_cast<float*>(smem);
-  consumers_sync();      // every tile has been read, or somebody has given up: copies may be under way then, and the ring is left alone
-  const bool complete = *gave_up == 0;
+  consumers_sync();      // every tile has been read, or a warp has given up and seen the copies land
   float* mine = xch + warp * 32 * BW_XP;
 #pragma unroll
-  for (int mt = 0; mt < MT && complete; ++mt)
+  for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
       float l = l_run[mt][e];
@@ -270,15 +273,15 @@ kve_decode_attn_block_warp_kernel(const __grid_constant__ CUtensorMap tmK, const
   const bool direct = gm.n_splits == 1;
   for (int r = warp; r < a.R; r += BW_CWARPS) {
     float2 ml[BW_CWARPS];
-    float mC = -INFINITY, lC = 0.f;      // (what a CTA that gave up has to say of its rows)
+    float mC = -INFINITY, lC = 0.f;
 #pragma unroll
-    for (int w = 0; w < BW_CWARPS && complete; ++w) {
+    for (int w = 0; w < BW_CWARPS; ++w) {
       ml[w] = *reinterpret_cast<const float2*>(xch + (w * 32 + r) * BW_XP + 128);
       mC = fmaxf(mC, ml[w].x);
     }
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int w = 0; w < BW_CWARPS && complete; ++w) {
+    for (int w = 0; w < BW_CWARPS; ++w) {
       const float f = (ml[w].x == -INFINITY) ? 0.f : exp2f(ml[w].x - mC);
       lC = fmaf(ml[w].y, f, lC);
       const float4 o = *reinterpret_cast<const float4*>(xch + (w * 32 + r) * BW_XP + lane * 4);
