@@ -66,12 +66,15 @@ static_assert(GX_TMEM_ACC + 4 * GX_N == GX_TMEM_COLS, "tensor memory");
 // two warpgroups of the recurrence and a third with the projectors and the score warp (a warpgroup, because registers move
 // between whole warpgroups: with 9 warps of equal shares the recurrence would have 168 registers)
 constexpr int GATE_THREADS = RNN_THREADS + 128;
-// registers per thread of the recurrence and of the third warpgroup, which share out those of the launch
+// registers per thread of the recurrence and of the third warpgroup, which share out those of the launch.  As few as none of them spills:
+// what a launch leaves of an SM's registers is where the means of kvE_refresh's second range run (three planes at d_g = 256 with 232 and 40
+// left room for none of their CTAs: kvE_refresh of 512 sequences x 121 chunks of 128, MLP, 1041 us, 926 so)
 template <int DG, int PL>
-constexpr int RNN_REGS = DG == 256 ? (PL == 3 ? 232 : 208) : (DG == 128 ? 184 : 136);
-constexpr int PROJ_REGS = 40;
+constexpr int RNN_REGS = DG == 256 ? (PL == 3 ? 224 : 208) : (DG == 128 ? 184 : 136);
 template <int DG, int PL>
-constexpr int GATE_REGS = (2 * RNN_REGS<DG, PL> + PROJ_REGS) / 3;
+constexpr int PROJ_REGS = DG == 256 && PL == 3 ? 32 : 40;
+template <int DG, int PL>
+constexpr int GATE_REGS = (2 * RNN_REGS<DG, PL> + PROJ_REGS<DG, PL>) / 3;
 
 // Optional cycle budget of one recurrence step (build with -DKVE_RNN_STAMPS, see rnn_stamps.py): warp 0 of CTA 0 adds
 // up, over all steps and groups, the clock64 cycles between five points of a step - 0: waiting for the peers' h,
@@ -126,7 +129,8 @@ __global__ void __cluster_dims__(CL, 1, 1) __maxnreg__((GATE_REGS<DG, PL>))
   constexpr int SENDS = ((CL - 1) * PL * NS + 31) / 32;         // 16-byte messages to the peers per lane, step and group
   static_assert(HU == 8 * RNN_WARPS && KT % 2 == 0, "one pair of m16 tiles (8 units x 4 gates) per warp");
   // what the warpgroups ask for is exactly what the launch has, or the last one to ask would wait for good
-  static_assert(3 * GATE_REGS<DG, PL> == 2 * RNN_REGS<DG, PL> + PROJ_REGS && GATE_REGS<DG, PL> % 8 == 0 && RNN_REGS<DG, PL> % 8 == 0, "register split");
+  static_assert(3 * GATE_REGS<DG, PL> == 2 * RNN_REGS<DG, PL> + PROJ_REGS<DG, PL> && GATE_REGS<DG, PL> % 8 == 0 && RNN_REGS<DG, PL> % 8 == 0, "register split");
+  static_assert(GATE_THREADS * GATE_REGS<DG, PL> + 2 * MEAN_BESIDE_REGS <= 65536, "two CTAs of kve_chunk_mean_beside_kernel fit beside this one");
   static_assert(OFF_BARS % 16 == 0, "16-byte pieces");
 
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -178,7 +182,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __maxnreg__((GATE_REGS<DG, PL>))
     }
   };
   if (warp >= RNN_WARPS) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(PROJ_REGS));
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"((PROJ_REGS<DG, PL>)));
     // ================= projector warps =================
     // Pre-activations W_ih x_t a batch of GX_ROUNDS rounds ahead of the recurrence.  Each of the two issues the MMAs of one tile: every
     // issue holds up the other warps of its scheduler for some 45 cycles, wherever in the round it falls, and this way two schedulers

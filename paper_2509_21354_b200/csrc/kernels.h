@@ -76,6 +76,7 @@ cudaError_t launch_append_next(const LayerView& v, const void* k_new, const void
 // else the launch does nothing (a trigger that is replayed from a CUDA graph)
 // list_cut >= 0 (here, launch_chunk_token_mlp, launch_gate_rnn): the keep list covers no more than that many chunks from now on
 cudaError_t launch_chunk_mean(const LayerView& v, int t0, int t1, bool final_output, bool pool_max, cudaStream_t st, int dev_window, int list_cut);
+constexpr int MEAN_BESIDE_REGS = 64 * 32;      // registers of one of its CTAs
 cudaError_t launch_chunk_mean_beside(const LayerView& v, int t0, int t1, bool final_output, bool pool_max, cudaStream_t st);
 cudaError_t launch_chunk_mlp(const LayerView& v, int t0, int t1, const MlpWeights& w, int d_sum, cudaStream_t st, int dev_window);
 // the MLP's second layer on pooled activations hid [2][S * (t1 - t0)][d_sum]: Kbar = W2 hid + b2 (d_sum 128 or 256)

@@ -211,7 +211,7 @@ cudaError_t launch_chunk_mean(const LayerView& v, int t0, int t1, bool final_out
 }
 
 // ---- the same mean for a launch that runs beside the gate recurrence -----------------------------------------------
-// The recurrence leaves an SM a tenth of its registers and two thirds of its shared memory (two CTAs of this kernel), so the rows on their way wait there: a
+// The recurrence leaves an SM 4 K to 25 K of its registers and about two thirds of its shared memory (two CTAs of this kernel), so the rows on their way wait there: a
 // warp's pages come in bulk copies of 16 rows, eight of them in flight, and are added up row by row as above (the same rounding).
 // A CTA takes several units in a row, so that the copies of the next one are under way while the last is added up.
 // 4.1 TB/s beside the recurrence of 512 sequences, which takes 22 % longer meanwhile (pages of 128 tokens; the kernel above, its
@@ -224,7 +224,7 @@ constexpr int MB_SMEM_BAR = MEAN_WARPS * MB_STAGES * MB_STAGE_BYTES;
 constexpr int MB_SMEM_BYTES = MB_SMEM_BAR + MEAN_WARPS * MB_STAGES * 8;
 
 template <bool POOL_MAX>
-__global__ void __launch_bounds__(MEAN_WARPS * 32) kve_chunk_mean_beside_kernel(LayerView v, int t0, int n_range, FastDiv by_range, int n_units,
+__global__ void __launch_bounds__(MEAN_WARPS * 32, 65536 / MEAN_BESIDE_REGS) kve_chunk_mean_beside_kernel(LayerView v, int t0, int n_range, FastDiv by_range, int n_units,
                                                                                int units_per_cta, int final_output) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   pdl_launch_dependents();

@@ -1460,7 +1460,7 @@ def test_token_mlp_second_layer_is_no_less_precise_than_fp32_loops(d_sum):
 
 
 @pytest.mark.parametrize("agg,d_g,B,C,n", [("mean", 128, 16, 64, 4300), ("max", 256, 16, 40, 4100), ("mlp", 256, 16, 136, 8300), ("mean", 64, 4, 7, 9000)])
-def test_refresh_with_means_beside_the_recurrence_equals_the_stepwise_calls(agg, d_g, B, C, n):
+def test_refresh_with_means_beside_the_recurrence_equals_the_stepwise_calls(agg, d_g, B, C, n, planes=2):
     """Sizes at which kvE_refresh takes two ranges, the means of the second beside the recurrence over the first: pages of whole and of
     broken pieces of 16 rows, one and several to a CTA, both group counts; bit for bit what the three calls give, again when
     repeated, and a bad page id in the second range is reported and nothing of it written."""
@@ -1472,6 +1472,7 @@ def test_refresh_with_means_beside_the_recurrence_equals_the_stepwise_calls(agg,
     st.k_pages.normal_(generator=torch.Generator(device="cuda").manual_seed(1))
     st.v_pages.normal_(generator=torch.Generator(device="cuda").manual_seed(2))
     st.set_len(0, n)
+    st.set_gate_planes(planes)
     N = wl.n_stale_chunks()
     state = lambda: [t.clone() for t in (st.ksum_f32, st.vsum_f32, st.ksum_bf16, st.vsum_bf16, st.scores, st.keep_idx, st.keep_cnt, st.lstm_h, st.lstm_c)]
     st.summarize_chunks(0, 0, N, aw)
@@ -1504,6 +1505,12 @@ def test_refresh_with_means_beside_the_recurrence_equals_the_stepwise_calls(agg,
         torch.cuda.synchronize()
         assert st.poll_status() == -3
         assert bool((st.ksum_f32[0, 3, N - 1] == 7.0).all()) and torch.equal(st.ksum_f32[0, 4:], want[0][0, 4:])
+
+
+@pytest.mark.parametrize("agg,d_g,B,C,n", [("mlp", 256, 16, 136, 8300), ("mean", 256, 8, 64, 8000), ("max", 128, 16, 40, 4100)])
+def test_refresh_with_means_beside_the_recurrence_of_three_planes(agg, d_g, B, C, n):
+    """... with exact products in the recurrence, whose CTAs are larger: one and two groups of sequences to a cluster"""
+    test_refresh_with_means_beside_the_recurrence_equals_the_stepwise_calls(agg, d_g, B, C, n, planes=3)
 
 
 def test_decode_step_call_checks_its_tensors_and_takes_a_stream():
