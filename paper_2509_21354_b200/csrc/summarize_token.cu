@@ -22,7 +22,8 @@
 //      from tensor memory per 128 activations, no sums that meet in shared memory.  (All sixteen warps on every tile, 64 or 32 tokens a
 //      thread: 256 sequences x 56 chunks x 64 tokens x 256 units 254 us with the second layer, 238 so; 128 units 160 and 145 us; 64 x 30 x 128
 //      tokens 82 and 75 us.)  Items (chunks or groups of chunks) go through the accumulators in turn, so that the slices of a long chunk
-//      stay with the same threads.
+//      stay with the same threads.  A CTA with few items has all sixteen warps on every tile all the same (SHARED): the bits are those of the other
+//      way, the sums of 32 tokens are added up in the same order.
 //    * The exponentials of eight tokens are taken beside the polynomial of the next eight.
 //    * The pooled activations (1/C) sum_j gelu(...) go to a scratch row per (side, sequence, chunk).
 //    Bound by the activation arithmetic: 20 issue slots per pair of activations (18.6 cycles of the fp32 pipe, 16 of the exponentials'), 65 %
@@ -49,7 +50,8 @@ constexpr int TM_LAG = 2;                                    // tiles whose copi
 constexpr int TM_SMEM_X = TM_SMEM_W1 + 2 * TM_MAX_DSUM * umma::KBLOCK_ROW_BYTES;   // 4 buffers x 2 K-blocks: 128 KB
 constexpr int TM_TMEM_COLS = 512;                           // accumulators: one slab x 128 columns (four) or two (two)
 constexpr int TM_MAX_ACC = TM_TMEM_COLS / TM_N;
-constexpr int TM_SMEM_BAR = TM_SMEM_X + TM_XBUFS * 2 * TM_KB_BYTES;
+constexpr int TM_SMEM_POOL = TM_SMEM_X + TM_XBUFS * 2 * TM_KB_BYTES;          // [2 items][4 groups of 32 tokens][d_sum] sums
+constexpr int TM_SMEM_BAR = TM_SMEM_POOL + 2 * 4 * TM_MAX_DSUM * 4;
 constexpr int TM_SMEM_BYTES = TM_SMEM_BAR + (2 * TM_XBUFS + 2 * TM_MAX_ACC) * 8 + 16 + 1024;      // + slack to reach a 1024-byte boundary
 static_assert(TM_SMEM_BYTES > 116 * 1024, "one CTA per SM: each allocates all of tensor memory");
 
@@ -65,24 +67,89 @@ struct TokenMlpArgs {
   float* hid;                // [2][n_units][d_sum] pooled activations (side, unit = s * n_range + (t - t0))
 };
 
-// The order in which a CTA goes through its tiles: as many items side by side as there are accumulators, slice by slice.
-template <int ACCS>
+// The order in which a CTA goes through its tiles.  Items side by side, as many as there are accumulators, slice by slice; or (SHARED) one item
+// after the other, the accumulators in turn.
+template <int ACCS, bool SHARED>
 struct TileWalk {
   int my_items, tiles_per_item;      // items of this CTA: blockIdx.x + k gridDim.x
-  int k0 = 0, slice = 0, acc = 0;    // this tile: slice `slice` of item k0 + acc, in accumulator `acc`
+  int k0 = 0, slice = 0, acc = 0;    // this tile: slice `slice` of item k0 + acc (SHARED: k0), in accumulator `acc`
+  int turns = 0;                     // SHARED: completed rounds through the accumulators
   __device__ __forceinline__ bool done() const { return k0 >= my_items; }
-  __device__ __forceinline__ int item() const { return (int)blockIdx.x + (k0 + acc) * (int)gridDim.x; }
-  __device__ __forceinline__ int turn() const { return k0 / ACCS * tiles_per_item + slice; }      // of the accumulator: 0, 1, ..
+  __device__ __forceinline__ int item() const { return (int)blockIdx.x + (SHARED ? k0 : k0 + acc) * (int)gridDim.x; }
+  __device__ __forceinline__ int turn() const { return SHARED ? turns : k0 / ACCS * tiles_per_item + slice; }      // of the accumulator: 0, 1, ..
   __device__ __forceinline__ void next() {
-    if (++acc < ACCS && k0 + acc < my_items) return;
-    acc = 0;
-    if (++slice < tiles_per_item) return;
-    slice = 0;
-    k0 += ACCS;
+    if constexpr (SHARED) {
+      if (++acc == ACCS) { acc = 0; ++turns; }
+      if (++slice < tiles_per_item) return;
+      slice = 0;
+      ++k0;
+    } else {
+      if (++acc < ACCS && k0 + acc < my_items) return;
+      acc = 0;
+      if (++slice < tiles_per_item) return;
+      slice = 0;
+      k0 += ACCS;
+    }
   }
 };
 
-template <int DSUM>
+// The activations of GROUPS x 32 tokens (columns from `cols` on) of a thread's hidden unit, added to `sum` 32 by 32; frees the accumulator.
+template <int GROUPS>
+__device__ __forceinline__ void pool_tile(uint32_t cols, float b1, float (&sum)[GROUPS], uint64_t* acc_free) {
+  constexpr float G6[7] = KVE_GELU_TAIL6;
+  umma::fence_after_sync();
+  uint32_t h[2][16];                              // 16 columns in work, 16 on their way
+  umma::tmem_ld16_nowait(cols, h[0]);
+#pragma unroll
+  for (int g = 0; g < GROUPS; ++g) {
+    // 32 tokens, eight at a time; the exponentials of the block before go out between the polynomial steps of this one
+    float2 relu_sum = make_float2(0.f, 0.f), tail_sum = make_float2(0.f, 0.f), abs_before[4], p_before[4];
+#pragma unroll
+    for (int blk = 0; blk <= 4; ++blk) {
+      float2 abs_x[4], p[4];
+      if (blk < 4) {
+        const int q = blk >> 1;
+        if (blk % 2 == 0) {
+          umma::tmem_ld_wait16(h[q]);
+          if (blk == 0 || g < GROUPS - 1) umma::tmem_ld16_nowait(cols + (uint32_t)(g * 32 + (q + 1) * 16), h[q ^ 1]);
+          else {
+            umma::fence_before_sync();
+            __syncwarp();
+            if ((threadIdx.x & 31) == 0) mbar_arrive(acc_free);
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int e = (blk & 1) * 8 + 2 * i;
+          const float2 x = add2(make_float2(__uint_as_float(h[q][e]), __uint_as_float(h[q][e + 1])), make_float2(b1, b1));
+          abs_x[i] = make_float2(fminf(fabsf(x.x), 6.f), fminf(fabsf(x.y), 6.f));
+          relu_sum = add2(relu_sum, make_float2(relu_nan(x.x), relu_nan(x.y)));
+          p[i] = make_float2(G6[6], G6[6]);
+        }
+      }
+      float2 tail[4];
+#pragma unroll
+      for (int y = 0; y < 8; ++y) {      // an exponential of the block before, three steps of this one
+        if (blk > 0) {
+          if (y & 1) tail[y >> 1].y = ex2_fast(p_before[y >> 1].y);
+          else tail[y >> 1].x = ex2_fast(p_before[y >> 1].x);
+        }
+        if (blk < 4)
+#pragma unroll
+          for (int z = 3 * y; z < 3 * y + 3; ++z) p[z & 3] = fma2(p[z & 3], abs_x[z & 3], make_float2(G6[5 - z / 4], G6[5 - z / 4]));
+      }
+      if (blk > 0)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) tail_sum = fma2(abs_before[i], tail[i], tail_sum);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) { abs_before[i] = abs_x[i]; p_before[i] = p[i]; }
+    }
+    const float got = (relu_sum.x + relu_sum.y) - (tail_sum.x + tail_sum.y);
+    sum[g] += got;
+  }
+}
+
+template <int DSUM, bool SHARED>
 __global__ void __launch_bounds__(TM_THREADS, 1) kve_token_mlp_pool_kernel(TokenMlpArgs a) {
   constexpr int SLABS = DSUM / TM_SLAB;
   constexpr int ACCS = TM_TMEM_COLS / (TM_N * SLABS);          // accumulators, each with its own epilogue warps
@@ -117,7 +184,7 @@ __global__ void __launch_bounds__(TM_THREADS, 1) kve_token_mlp_pool_kernel(Token
     }
     for (int i = 0; i < ACCS; ++i) {
       mbar_init(&acc_full[i], 1);
-      mbar_init(&acc_free[i], ACC_WARPS);
+      mbar_init(&acc_free[i], SHARED ? TM_EPI_WARPS : ACC_WARPS);
     }
     mbar_fence_init();
   }
@@ -133,7 +200,7 @@ __global__ void __launch_bounds__(TM_THREADS, 1) kve_token_mlp_pool_kernel(Token
   // A CTA walks whole items (a chunk longer than a tile keeps all its 128-token slices on one CTA, in a row)
   const int my_items = a.n_items > (int)blockIdx.x ? (a.n_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
   const int n_tiles = my_items * a.tiles_per_item;      // of this CTA
-  TileWalk<ACCS> walk{my_items, a.tiles_per_item};
+  TileWalk<ACCS, SHARED> walk{my_items, a.tiles_per_item};
   const int chunk_shift = v.C >= TM_N ? 7 : (v.C == 64 ? 6 : 5);      // row r of a tile: chunk r >> chunk_shift
 
   if (warp >= TM_EPI_WARPS && warp < TM_MMA_WARP) {
@@ -212,88 +279,81 @@ __global__ void __launch_bounds__(TM_THREADS, 1) kve_token_mlp_pool_kernel(Token
     }
   } else {
     // ================= epilogue warps =================
-    // accumulator warp / ACC_WARPS, this thread's hidden unit: tensor-memory lane 32 (warp & 3) + lane of slab `slab`; all 128 tokens of
-    // a tile
+    // this thread's hidden unit: tensor-memory lane 32 (warp & 3) + lane of slab `slab`.  All 128 tokens of the tiles in accumulator
+    // warp / ACC_WARPS, or (SHARED) that share of the tokens of every tile
     const int buf = warp / ACC_WARPS, lg = warp & 3, slab = SLABS == 2 ? (warp >> 2) & 1 : 0;
     const int unit = slab * TM_SLAB + lg * 32 + lane;
     const float b1 = (side ? a.w.b1V : a.w.b1K)[unit];
-    const uint32_t cols = tmem_d + (uint32_t)((buf * SLABS + slab) * TM_N) + ((uint32_t)(lg * 32) << 16);
+    const uint32_t lanes = tmem_d + ((uint32_t)(lg * 32) << 16);
     const float inv_c = 1.f / (float)v.C;
-    float* hid = a.hid + (long long)side * a.n_units * DSUM + unit;
-    constexpr float G6[7] = KVE_GELU_TAIL6;
-    int turn = 0;
-    for (int k = buf; k < my_items; k += ACCS) {
-      float sum[4] = {0.f, 0.f, 0.f, 0.f};              // per 32 tokens (of all slices of a long chunk)
-      bool alive = true;
-      for (int slice = 0; slice < a.tiles_per_item && alive; ++slice, ++turn) {
-        alive = __all_sync(0xffffffffu, mbar_wait_bounded(&acc_full[buf], (uint32_t)(turn & 1)));
-        if (!alive) {
-          if (lane == 0) set_status(v.status, ERR_TIMEOUT);
-          break;
-        }
-        umma::fence_after_sync();
-        uint32_t h[2][16];                              // 16 columns in work, 16 on their way
-        umma::tmem_ld16_nowait(cols, h[0]);
+    if constexpr (SHARED) {
+      constexpr int GROUPS = TM_N / 32 / ACCS;
+      float* pool = reinterpret_cast<float*>(smem + TM_SMEM_POOL);      // [2][4][DSUM]: the sums of 32 tokens each of an item
+      float* hid = a.hid + (long long)side * a.n_units * DSUM;
+      const int unit_shift = a.units_per_item == 4 ? 0 : (a.units_per_item == 2 ? 1 : 2), unit_groups = 1 << unit_shift;      // sums that make up a chunk
+      bool alive = true;      // a warp whose wait ran out goes on without: the others meet it at the barrier below
+      int acc = 0, turn = 0;
+      for (int k = 0; k < my_items; ++k) {
+        float sum[GROUPS];
 #pragma unroll
-        for (int g = 0; g < 4; ++g) {
-          // 32 tokens, eight at a time; the exponentials of the block before go out between the polynomial steps of this one
-          float2 relu_sum = make_float2(0.f, 0.f), tail_sum = make_float2(0.f, 0.f), abs_before[4], p_before[4];
-#pragma unroll
-          for (int blk = 0; blk <= 4; ++blk) {
-            float2 abs_x[4], p[4];
-            if (blk < 4) {
-              const int q = blk >> 1;
-              if (blk % 2 == 0) {
-                umma::tmem_ld_wait16(h[q]);
-                if (blk == 0 || g < 3) umma::tmem_ld16_nowait(cols + (uint32_t)(g * 32 + (q + 1) * 16), h[q ^ 1]);
-                else {
-                  umma::fence_before_sync();
-                  __syncwarp();
-                  if (lane == 0) mbar_arrive(&acc_free[buf]);
-                }
-              }
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                const int e = (blk & 1) * 8 + 2 * i;
-                const float2 x = add2(make_float2(__uint_as_float(h[q][e]), __uint_as_float(h[q][e + 1])), make_float2(b1, b1));
-                abs_x[i] = make_float2(fminf(fabsf(x.x), 6.f), fminf(fabsf(x.y), 6.f));
-                relu_sum = add2(relu_sum, make_float2(relu_nan(x.x), relu_nan(x.y)));
-                p[i] = make_float2(G6[6], G6[6]);
-              }
-            }
-            float2 tail[4];
-#pragma unroll
-            for (int y = 0; y < 8; ++y) {      // an exponential of the block before, three steps of this one
-              if (blk > 0) {
-                if (y & 1) tail[y >> 1].y = ex2_fast(p_before[y >> 1].y);
-                else tail[y >> 1].x = ex2_fast(p_before[y >> 1].x);
-              }
-              if (blk < 4)
-#pragma unroll
-                for (int z = 3 * y; z < 3 * y + 3; ++z) p[z & 3] = fma2(p[z & 3], abs_x[z & 3], make_float2(G6[5 - z / 4], G6[5 - z / 4]));
-            }
-            if (blk > 0)
-#pragma unroll
-              for (int i = 0; i < 4; ++i) tail_sum = fma2(abs_before[i], tail[i], tail_sum);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) { abs_before[i] = abs_x[i]; p_before[i] = p[i]; }
+        for (int g = 0; g < GROUPS; ++g) sum[g] = 0.f;
+        for (int slice = 0; slice < a.tiles_per_item; ++slice) {
+          if (alive && !__all_sync(0xffffffffu, mbar_wait_bounded(&acc_full[acc], (uint32_t)(turn & 1)))) {
+            alive = false;
+            if (lane == 0) set_status(v.status, ERR_TIMEOUT);
           }
-          const float got = (relu_sum.x + relu_sum.y) - (tail_sum.x + tail_sum.y);
-          sum[g] += got;
+          if (alive) pool_tile<GROUPS>(lanes + (uint32_t)((acc * SLABS + slab) * TM_N + buf * GROUPS * 32), b1, sum, &acc_free[acc]);
+          if (++acc == ACCS) { acc = 0; ++turn; }
+        }
+        const int first = ((int)blockIdx.x + k * (int)gridDim.x) * a.units_per_item;
+        if (unit_groups <= GROUPS) {      // whole chunks
+#pragma unroll
+          for (int g = 0; g < GROUPS; ++g) {
+            if (g & (unit_groups - 1)) continue;
+            const int u = first + ((buf * GROUPS + g) >> unit_shift);
+            if (u < a.n_units) hid[(long long)u * DSUM + unit] = (unit_groups == 2 ? sum[g] + sum[(g + 1) % GROUPS] : sum[g]) * inv_c;
+          }
+          continue;
+        }
+        float* pl = pool + (k & 1) * 4 * DSUM;
+#pragma unroll
+        for (int g = 0; g < GROUPS; ++g) pl[(buf * GROUPS + g) * DSUM + unit] = sum[g];
+        asm volatile("bar.sync 1, %0;" ::"n"(TM_EPI_WARPS * 32) : "memory");      // the other half keeps the next item apart
+        for (int i = tid; i < a.units_per_item * DSUM; i += TM_EPI_WARPS * 32) {
+          const int x = i / DSUM, col = i % DSUM;
+          float total = pl[(x << unit_shift) * DSUM + col];
+          for (int g = 1; g < unit_groups; ++g) total += pl[((x << unit_shift) + g) * DSUM + col];
+          if (first + x < a.n_units) hid[(long long)(first + x) * DSUM + col] = total * inv_c;
         }
       }
-      if (!alive) break;
-      // the chunk(s) of this item are complete
-      const int first = ((int)blockIdx.x + k * (int)gridDim.x) * a.units_per_item;
-      if (a.units_per_item == 1) {
-        hid[(long long)first * DSUM] = (((sum[0] + sum[1]) + sum[2]) + sum[3]) * inv_c;
-      } else if (a.units_per_item == 2) {
-        if (first < a.n_units) hid[(long long)first * DSUM] = (sum[0] + sum[1]) * inv_c;
-        if (first + 1 < a.n_units) hid[(long long)(first + 1) * DSUM] = (sum[2] + sum[3]) * inv_c;
-      } else {
-#pragma unroll
-        for (int x = 0; x < 4; ++x)
-          if (first + x < a.n_units) hid[(long long)(first + x) * DSUM] = sum[x] * inv_c;
+    } else {
+      const uint32_t cols = lanes + (uint32_t)((buf * SLABS + slab) * TM_N);
+      float* hid = a.hid + (long long)side * a.n_units * DSUM + unit;
+      int turn = 0;
+      for (int k = buf; k < my_items; k += ACCS) {
+        float sum[4] = {0.f, 0.f, 0.f, 0.f};              // per 32 tokens (of all slices of a long chunk)
+        bool alive = true;
+        for (int slice = 0; slice < a.tiles_per_item && alive; ++slice, ++turn) {
+          alive = __all_sync(0xffffffffu, mbar_wait_bounded(&acc_full[buf], (uint32_t)(turn & 1)));
+          if (!alive) {
+            if (lane == 0) set_status(v.status, ERR_TIMEOUT);
+            break;
+          }
+          pool_tile<4>(cols, b1, sum, &acc_free[buf]);
+        }
+        if (!alive) break;
+        // the chunk(s) of this item are complete
+        const int first = ((int)blockIdx.x + k * (int)gridDim.x) * a.units_per_item;
+        if (a.units_per_item == 1) {
+          hid[(long long)first * DSUM] = (((sum[0] + sum[1]) + sum[2]) + sum[3]) * inv_c;
+        } else if (a.units_per_item == 2) {
+          if (first < a.n_units) hid[(long long)first * DSUM] = (sum[0] + sum[1]) * inv_c;
+          if (first + 1 < a.n_units) hid[(long long)(first + 1) * DSUM] = (sum[2] + sum[3]) * inv_c;
+        } else {
+  #pragma unroll
+          for (int x = 0; x < 4; ++x)
+            if (first + x < a.n_units) hid[(long long)(first + x) * DSUM] = sum[x] * inv_c;
+        }
       }
     }
   }
@@ -308,11 +368,11 @@ bool token_mlp_supported(int C, int d_sum) {
   return C <= 128 ? (128 % C == 0) : (C % 128 == 0);
 }
 
-template <int DSUM>
+template <int DSUM, bool SHARED>
 static cudaError_t launch_pool(const TokenMlpArgs& a, dim3 grid, cudaStream_t st) {
   static DeviceFlags opted;
-  const cudaError_t e = smem_opt_in(opted, kve_token_mlp_pool_kernel<DSUM>, TM_SMEM_BYTES);
-  return e == cudaSuccess ? launch_pdl(kve_token_mlp_pool_kernel<DSUM>, grid, dim3(TM_THREADS), TM_SMEM_BYTES, st, a) : e;
+  const cudaError_t e = smem_opt_in(opted, kve_token_mlp_pool_kernel<DSUM, SHARED>, TM_SMEM_BYTES);
+  return e == cudaSuccess ? launch_pdl(kve_token_mlp_pool_kernel<DSUM, SHARED>, grid, dim3(TM_THREADS), TM_SMEM_BYTES, st, a) : e;
 }
 
 cudaError_t launch_chunk_token_mlp(const LayerView& v, int t0, int t1, const MlpWeights& w, int d_sum, float* hid, int list_cut, cudaStream_t st) {
@@ -332,7 +392,15 @@ cudaError_t launch_chunk_token_mlp(const LayerView& v, int t0, int t1, const Mlp
   if (per_side > a.n_items) per_side = a.n_items;
   if (per_side < 1) per_side = 1;
   const dim3 grid((unsigned)per_side, 2);
-  const cudaError_t e = d_sum == 256 ? launch_pool<256>(a, grid, st) : launch_pool<128>(a, grid, st);
+  // All epilogue warps on every tile where a CTA has few of them: with one item the warps of one accumulator would have all the work (74 units of
+  // 128 tokens, d_sum 128: 12.1 us a call, 11.6 so; of 384 tokens 16.7 and 14.8), with many the sums that meet in shared memory cost more than
+  // an uneven end.  Lines where both meet, items a CTA: 3 with chunks of 32 (8 x 75: 16.9 and 16.5 us), where nothing has to meet; d_sum 128: 2 (148 x
+  // 64 tokens 15.9 and 15.7; 175 x 64 16.8 and 16.9); d_sum 256, where a thread has 64 tokens of a tile: 5 with chunks of 64 (600 x 64 26.3 and
+  // 26.1; 800 x 64 28.8 and 28.9), 1 with chunks of 128 (140 x 128 19.6 and 19.7), 3 with longer ones (200 x 384 36.4 and 35.0; 260 x 384 41.3 and 41.8).
+  const int shared_items = v.C == 32 ? 3 : (d_sum == 128 ? 2 : (v.C == 64 ? 5 : (v.C > TM_N ? 3 : 1)));
+  const bool shared = (a.n_items + per_side - 1) / per_side <= shared_items;
+  const cudaError_t e = d_sum == 256 ? (shared ? launch_pool<256, true>(a, grid, st) : launch_pool<256, false>(a, grid, st))
+                                     : (shared ? launch_pool<128, true>(a, grid, st) : launch_pool<128, false>(a, grid, st));
   return e == cudaSuccess ? launch_pooled_out(v, t0, t1, w, d_sum, hid, st) : e;
 }
 

@@ -1137,6 +1137,35 @@ def test_token_mlp_with_several_items_per_cta(C, S, d_sum):
             assert (got[0, s0:s0 + 8, :Nc].double() - want).abs().max() <= 2e-5 * max(1.0, float(want.abs().max()))
 
 
+@pytest.mark.parametrize("C", [32, 64, 128, 256, 384])
+@pytest.mark.parametrize("d_sum", [128, 256])
+def test_token_mlp_with_few_items_equals_many(C, d_sum):
+    # a call of up to five items per CTA has all warps on every tile, a longer one has accumulators of its own for every group of warps: chunk by
+    # chunk, in pieces of two and three and all at once, the same bits; 1 and 83 sequences fill a part of an item and of the CTAs
+    b = _binding()
+    for S, Nc in ((1, 5), (83, 3), (83, 28)):
+        wl = wlm.Workload("few", B=1, H=S, n=C * Nc + 32, C=C, W=32, d_g=64, agg="token_mlp", d_sum=d_sum, key_offset_std=0.5, seed=C + d_sum)
+        st = make_store(wl)
+        gen = torch.Generator(device="cuda").manual_seed(C)
+        for pages in (st.k_pages, st.v_pages):
+            pages.normal_(generator=gen)
+        st.set_len(0, wl.n)
+        aw = b.AggWeights(wlm.gen_mlp_weights(wl))
+        got = []
+        for step in (Nc, 1, 2, 3):
+            for t in (st.ksum_f32, st.vsum_f32):
+                t.fill_(float("nan"))
+            for t in range(0, Nc, step):
+                st.summarize_chunks(0, t, min(t + step, Nc), aw)
+            torch.cuda.synchronize()
+            assert st.poll_status() == 0
+            got.append((st.ksum_f32[:, :, :Nc].clone(), st.vsum_f32[:, :, :Nc].clone()))
+        assert torch.isfinite(got[0][0]).all()
+        for other in got[1:]:
+            assert torch.equal(other[0], got[0][0]) and torch.equal(other[1], got[0][1])
+        st.close()
+
+
 def test_token_mlp_aggregator_incremental_ranges_and_unsupported_geometry():
     b = _binding()
     wl = wlm.CFG2.small(B=1, H=5, n=64 * 11, C=64, W=128, agg="token_mlp", d_sum=256, seed=71)
