@@ -111,7 +111,7 @@ __device__ unsigned long long g_rnn_once[8];
 template <int DG, int NG, int PL>
 constexpr int RNN_SMEM_X = NG * 2 * (DG / 8) * PL * 8 * 8 * 2 + NG * 2 * RNN_WARPS * 64 * 4 + (2 * NG + 5) * 8 + 8;
 
-template <int DG, int CL, int NG, int PL>
+template <int DG, int CL, int NG, int PL, bool MANY>
 __global__ void __cluster_dims__(CL, 1, 1) __maxnreg__((GATE_REGS<DG, PL>))
     kve_gate_rnn_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, RnnArgs a) {
   constexpr int HU = DG / CL;            // hidden units owned by this CTA
@@ -149,7 +149,9 @@ __global__ void __cluster_dims__(CL, 1, 1) __maxnreg__((GATE_REGS<DG, PL>))
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);      // (the same in all lanes, for the compiler to see)
   const int g = lane >> 2, tig = lane & 3;
   const uint32_t rank = cluster_rank();
-  const int seq0 = (blockIdx.x / CL) * NS * NG;      // group gi owns sequences seq0 + 8 gi .. + 7
+  // A cluster takes a set of NS NG sequences, or (MANY) one set after the other: group gi owns sequences seq0 + 8 gi .. + 7
+  int seq0 = (blockIdx.x / CL) * NS * NG;
+  const int seq_step = MANY ? (int)(gridDim.x / CL) * NS * NG : 0;
   const int ug = (int)rank * HU + warp * 8 + g;                // this thread's hidden unit
 
   KVE_RNN_ONCE(0);
@@ -170,6 +172,14 @@ __global__ void __cluster_dims__(CL, 1, 1) __maxnreg__((GATE_REGS<DG, PL>))
   const uint32_t tmem = *tmem_slot;
 
   const int n_batches = (a.n_range + T - 1) / T;
+  // what the barriers have seen of earlier sets: batches of the projection, exchanges through buffer b of h (bit b: an odd number)
+  int batches_before = 0, exchanged = 0;
+  auto next_set = [&]() {      // false: that was the last one
+    if (!MANY || (seq0 += seq_step) >= a.S) return false;
+    batches_before += n_batches;
+    exchanged ^= ((a.n_range - 1) / 2 & 1) | (a.n_range / 2 & 1) << 1;
+    return true;
+  };
   // a warp's worth of partial sums from the products of a round: lane = (warp, sequence / 2), for both halves of the sequences
   auto put_scores = [&](int gi, int step) {
     const float* src = prod + (gi * 2 + (step & 1)) * PROD_BUF;
@@ -190,71 +200,73 @@ __global__ void __cluster_dims__(CL, 1, 1) __maxnreg__((GATE_REGS<DG, PL>))
     pdl_wait();      // the summaries come from earlier kernels
     __syncthreads();      // W_ih is in tensor memory, and xs, its staging area, is free
     umma::fence_after_sync();
-    cluster_arrive();      // the recurrence's first meeting, which this warp has nothing to wait for
-    bool ok = true;
-    int n_fetched = 0, n_begun = 0;
-    if ((warp == RNN_WARPS || warp == RNN_WARPS + 2) && lane == 0) {
-      const int tile = warp == RNN_WARPS ? 0 : 1;
-      asm volatile("fence.proxy.async.global;" ::: "memory");
-      for (int b = 0; b < n_batches && ok; ++b) {
-        const int buf = b & 1;
-        // the rows of all steps and sequences of the batch: a copy per K-block, zeros beyond the store (what it brings beyond the range
-        // or from another layer goes into columns that nobody reads)
-        if (tile == 0) {
-          mbar_arrive_expect_tx(x_full, GX_BYTES);
+    bool ok = true;      // (a CTA that has given up takes part in the meetings of the cluster until the last set)
+    do {
+      cluster_arrive();      // the recurrence's first meeting, which this warp has nothing to wait for
+      int n_fetched = 0, n_begun = 0;
+      if ((warp == RNN_WARPS || warp == RNN_WARPS + 2) && lane == 0 && ok) {
+        const int tile = warp == RNN_WARPS ? 0 : 1;
+        asm volatile("fence.proxy.async.global;" ::: "memory");
+        for (int b = 0; b < n_batches && ok; ++b) {
+          const int run = batches_before + b, buf = run & 1;
+          // the rows of all steps and sequences of the batch: a copy per K-block, zeros beyond the store (what it brings beyond the range
+          // or from another layer goes into columns that nobody reads)
+          if (tile == 0) {
+            mbar_arrive_expect_tx(x_full, GX_BYTES);
 #pragma unroll
-          for (int kb = 0; kb < GX_KB; ++kb)
-            tma_load_3d(smem_u32(xs) + kb * GX_KB_BYTES, kb < GX_KB / 2 ? &map_k : &map_v, (kb & 1) * umma::KBLOCK_ELEMS, a.seq_base + seq0, a.t0 + b * T, x_full);
-        }
-        n_fetched = b + 1;
-        ok = mbar_wait_bounded(x_full, (uint32_t)(b & 1)) && (b < 2 || mbar_wait_bounded(&x_read[buf], (uint32_t)(((b >> 1) - 1) & 1)));
-        if (!ok) break;
-        umma::fence_after_sync();
-        n_begun = b + 1;
-        const uint32_t acc = tmem + GX_TMEM_ACC + (uint32_t)((buf * 2 + tile) * GX_N);
-        // A K-block at a time, when warp 0 reports the right moment of a round (for the pace only: the wait gives up soon): behind its
-        // sends at d_g = 256, where the recurrence then waits for its peers (32 x 250 312 -> 303 us), behind its MMAs below (8 x 400 at
-        // d_g = 128 333 -> 321.5).  With two groups there is always somebody at work: a tile at a time (512 x 121 285 -> 277 us).
+            for (int kb = 0; kb < GX_KB; ++kb)
+              tma_load_3d(smem_u32(xs) + kb * GX_KB_BYTES, kb < GX_KB / 2 ? &map_k : &map_v, (kb & 1) * umma::KBLOCK_ELEMS, a.seq_base + seq0, a.t0 + b * T, x_full);
+          }
+          n_fetched = run + 1;
+          ok = mbar_wait_bounded(x_full, (uint32_t)(run & 1)) && (run < 2 || mbar_wait_bounded(&x_read[buf], (uint32_t)(((run >> 1) - 1) & 1)));
+          if (!ok) break;
+          umma::fence_after_sync();
+          n_begun = run + 1;
+          const uint32_t acc = tmem + GX_TMEM_ACC + (uint32_t)((buf * 2 + tile) * GX_N);
+          // A K-block at a time, when warp 0 reports the right moment of a round (for the pace only: the wait gives up soon): behind its
+          // sends at d_g = 256, where the recurrence then waits for its peers (32 x 250 312 -> 303 us), behind its MMAs below (8 x 400 at
+          // d_g = 128 333 -> 321.5).  With two groups there is always somebody at work: a tile at a time (512 x 121 285 -> 277 us).
 #pragma unroll 1
-        for (int kb = 0; kb < GX_KB; ++kb) {
-          const int due = NG == 1 ? (b - 1) * GX_ROUNDS + 1 + 2 * kb : (b - 1) * GX_ROUNDS + 2 + 3 * tile;
-          if (b > 0 && (NG == 1 || kb == 0))
-            for (int poll = 0; poll < 2048 && *rounds_done < due; ++poll) __nanosleep(30);
+          for (int kb = 0; kb < GX_KB; ++kb) {
+            const int due = NG == 1 ? (b - 1) * GX_ROUNDS + 1 + 2 * kb : (b - 1) * GX_ROUNDS + 2 + 3 * tile;
+            if (b > 0 && (NG == 1 || kb == 0))
+              for (int poll = 0; poll < 2048 && *rounds_done < due; ++poll) __nanosleep(30);
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
-            umma::mma_bf16_ts(acc, tmem + GX_TMEM_W + (uint32_t)(tile * D + kb * 32 + k * 8), umma::smem_desc(smem_u32(xs) + kb * GX_KB_BYTES + k * 32),
-                              umma::instr_desc_bf16(128, GX_N), (kb | k) != 0);
+            for (int k = 0; k < 4; ++k)
+              umma::mma_bf16_ts(acc, tmem + GX_TMEM_W + (uint32_t)(tile * D + kb * 32 + k * 8), umma::smem_desc(smem_u32(xs) + kb * GX_KB_BYTES + k * 32),
+                                umma::instr_desc_bf16(128, GX_N), (kb | k) != 0);
+          }
+          umma::commit(&x_done[buf]);
+          ok = mbar_wait_bounded(&x_done[buf], (uint32_t)((run >> 1) & 1));      // the rows may be overwritten
         }
-        umma::commit(&x_done[buf]);
-        ok = mbar_wait_bounded(&x_done[buf], (uint32_t)((b >> 1) & 1));      // the rows may be overwritten
-      }
-      if (!ok) {      // nothing is under way any more when the CTA leaves
-        set_status(a.status, ERR_TIMEOUT);
-        mbar_wait_bounded(x_full, (uint32_t)((n_fetched - 1) & 1));
-        if (n_begun > 0) mbar_wait_bounded(&x_done[(n_begun - 1) & 1], (uint32_t)(((n_begun - 1) >> 1) & 1));
-      }
-    }
-    if (warp == RNN_WARPS + 1) {
-      // ================= score warp =================
-      // Announces the bytes of every exchange, and adds up what the warps leave of w_s . h_t when it is through (eight units in pairs;
-      // the warps' sums go to memory).  Its arrival for the next exchange says that it has read what that one will overwrite.
-      for (int step = 0; step + 1 < a.n_range && ok; ++step) {
-        const int buf = (step + 1) & 1;
-        if (lane < NG) {
-          if (CL > 1) mbar_arrive_expect_tx(&hbar[2 * lane + buf], H_BYTES);
-          else mbar_arrive(&hbar[2 * lane + buf]);
+        if (!ok) {      // nothing is under way any more when the CTA leaves
+          set_status(a.status, ERR_TIMEOUT);
+          mbar_wait_bounded(x_full, (uint32_t)((n_fetched - 1) & 1));
+          if (n_begun > 0) mbar_wait_bounded(&x_done[(n_begun - 1) & 1], (uint32_t)(((n_begun - 1) >> 1) & 1));
         }
-        for (int gi = 0; gi < NG && ok; ++gi) {
-          ok = __all_sync(0xffffffffu, mbar_wait_cluster_bounded(&hbar[2 * gi + buf], (uint32_t)((step >> 1) & 1)));
-          if (ok) put_scores(gi, step);
-        }
-        __syncwarp();      // all lanes have read: an arrival orders only what its own lane has done
       }
-      if (!ok && lane == 0) set_status(a.status, ERR_TIMEOUT);
-    }
-    __syncwarp();
-    cluster_wait();
-    cluster_sync_all();
+      if (warp == RNN_WARPS + 1) {
+        // ================= score warp =================
+        // Announces the bytes of every exchange, and adds up what the warps leave of w_s . h_t when it is through (eight units in pairs;
+        // the warps' sums go to memory).  Its arrival for the next exchange says that it has read what that one will overwrite.
+        for (int step = 0; step + 1 < a.n_range && ok; ++step) {
+          const int buf = (step + 1) & 1;
+          if (lane < NG) {
+            if (CL > 1) mbar_arrive_expect_tx(&hbar[2 * lane + buf], H_BYTES);
+            else mbar_arrive(&hbar[2 * lane + buf]);
+          }
+          for (int gi = 0; gi < NG && ok; ++gi) {
+            ok = __all_sync(0xffffffffu, mbar_wait_cluster_bounded(&hbar[2 * gi + buf], (uint32_t)(((exchanged >> buf) + (step >> 1)) & 1)));
+            if (ok) put_scores(gi, step);
+          }
+          __syncwarp();      // all lanes have read: an arrival orders only what its own lane has done
+        }
+        if (!ok && lane == 0) set_status(a.status, ERR_TIMEOUT);
+      }
+      __syncwarp();
+      cluster_wait();
+      cluster_sync_all();
+    } while (next_set());
     return;
   }
 
@@ -334,223 +346,250 @@ __global__ void __cluster_dims__(CL, 1, 1) __maxnreg__((GATE_REGS<DG, PL>))
   umma::fence_smem_to_async();
   umma::fence_before_sync();
   __syncthreads();      // W_ih is in tensor memory: the projector may start
-  // ---- initial state: every CTA needs the full h of its sequences as planes in buffer 0 of each group -------------
-  for (int i = tid; i < NG * NS * (DG / 2); i += RNN_THREADS) {
-    const int js = i / (DG / 2), k2 = i % (DG / 2);      // js: sequence of the cluster, 0 .. 8 NG - 1
-    const int j = js % NS, s = seq0 + js;
-    float h0 = 0.f, h1 = 0.f;
-    if (!a.reset && s < a.S) {
-      const float2 hv = *reinterpret_cast<const float2*>(a.lstm_h + (long long)s * DG + k2 * 2);
-      h0 = hv.x; h1 = hv.y;
-    }
-    uint32_t p0[3], p1[3];      // the leading PL pieces are used
-    split3(h0, p0);
-    split3(h1, p1);
-#pragma unroll
-    for (int pl = 0; pl < PL; ++pl)
-      *reinterpret_cast<uint32_t*>(hs + js / NS * 2 * HS_BUF + (k2 >> 2) * KBLK + (pl * NS + j) * 8 + (k2 & 3) * 2) = p0[pl] | (p1[pl] << 16);
-  }
-  // state of the sequences 2 tig, 2 tig + 1 of every group
-  float2 c[NG], hlast[NG];
-#pragma unroll
-  for (int gi = 0; gi < NG; ++gi) {
-    const int s = seq0 + gi * NS + tig * 2;
-    const bool even = !a.reset && s < a.S, odd = !a.reset && s + 1 < a.S;
-    const long long at = (long long)s * DG + ug;
-    c[gi] = make_float2(even ? a.lstm_c[at] : 0.f, odd ? a.lstm_c[at + DG] : 0.f);
-    hlast[gi] = make_float2(even ? a.lstm_h[at] : 0.f, odd ? a.lstm_h[at + DG] : 0.f);
-  }
-
-  // message m of a warp goes to peer (rank + 1 + m / rows of a block): row m % rows of that CTA's buffers, as an address in the cluster window
-  uint32_t peer_hs[SENDS > 0 ? SENDS : 1];
-#pragma unroll
-  for (int x = 0; x < SENDS; ++x)
-    peer_hs[x] = map_to_rank(smem_u32(hs), (rank + 1 + (lane + 32 * x) / (PL * NS)) % CL) + (lane + 32 * x) % (PL * NS) * 16;
-
-  // barriers initialised and buffer 0 filled in every CTA before anyone sends
-  KVE_RNN_ONCE(3);
-  cluster_sync_all();
-  KVE_RNN_ONCE(4);
-
   bool alive = true;
-  KVE_RNN_MARK_BEGIN();
-  for (int batch = 0; batch < n_batches && alive; ++batch) {
-    // ---- the pre-activations of the next T steps' inputs
-    alive = __all_sync(0xffffffffu, mbar_wait_bounded(&x_done[batch & 1], (uint32_t)((batch >> 1) & 1)));
-    if (!alive) {
-      if (lane == 0) set_status(a.status, ERR_TIMEOUT);
-      break;
-    }
-    umma::fence_after_sync();
-    uint32_t acc_x = tmem_mine + GX_TMEM_ACC + (uint32_t)(((batch & 1) * 2 + (warp >> 2)) * GX_N);
-    const int step_end = min(batch * T + T, a.n_range);
-    for (int step = batch * T; step < step_end; ++step) {
-      const int buf = step & 1;
-      const bool send_h = step + 1 < a.n_range;
+  do {
+    if (MANY && tid == 0) *rounds_done = 0;
+    // ---- initial state: every CTA needs the full h of its sequences as planes in buffer 0 of each group -------------
+    for (int i = tid; i < NG * NS * (DG / 2); i += RNN_THREADS) {
+      const int js = i / (DG / 2), k2 = i % (DG / 2);      // js: sequence of the cluster, 0 .. 8 NG - 1
+      const int j = js % NS, s = seq0 + js;
+      float h0 = 0.f, h1 = 0.f;
+      if (!a.reset && s < a.S) {
+        const float2 hv = *reinterpret_cast<const float2*>(a.lstm_h + (long long)s * DG + k2 * 2);
+        h0 = hv.x; h1 = hv.y;
+      }
+      uint32_t p0[3], p1[3];      // the leading PL pieces are used
+      split3(h0, p0);
+      split3(h1, p1);
 #pragma unroll
-      for (int gi = 0; gi < NG; ++gi) {
-        uint16_t* hs_g = hs + gi * 2 * HS_BUF;
-        uint64_t* hbar_g = hbar + 2 * gi;
-        // pre-activations of the round's inputs, in the layout of the MMA accumulators
-        uint32_t pin[2][4];
-        auto ask_pin = [&]() {
-          umma::tmem_ld_frag_nowait(acc_x, pin[0]);
-          umma::tmem_ld_frag_nowait(acc_x + (16u << 16), pin[1]);
-          acc_x += 8;
-        };
-        if (!P_LATE) ask_pin();
-        KVE_RNN_MARK(2);
-        // ---- h_{t-1} from every CTA of the cluster (each buffer completes once per two steps) -----------------------------
-        if (step > 0) {
-          // (one poll usually waits long enough: it is the only thing in the way then)
-          const uint32_t parity = ((step - 1) >> 1) & 1;
-          if (!__all_sync(0xffffffffu, mbar_try_wait_cluster(&hbar_g[buf], parity))) {
-            alive = __all_sync(0xffffffffu, mbar_wait_cluster_bounded(&hbar_g[buf], parity));
-            if (!alive) {
-              if (lane == 0) set_status(a.status, ERR_TIMEOUT);
-              break;
+      for (int pl = 0; pl < PL; ++pl)
+        *reinterpret_cast<uint32_t*>(hs + js / NS * 2 * HS_BUF + (k2 >> 2) * KBLK + (pl * NS + j) * 8 + (k2 & 3) * 2) = p0[pl] | (p1[pl] << 16);
+    }
+    // state of the sequences 2 tig, 2 tig + 1 of every group
+    float2 c[NG], hlast[NG];
+#pragma unroll
+    for (int gi = 0; gi < NG; ++gi) {
+      const int s = seq0 + gi * NS + tig * 2;
+      const bool even = !a.reset && s < a.S, odd = !a.reset && s + 1 < a.S;
+      const long long at = (long long)s * DG + ug;
+      c[gi] = make_float2(even ? a.lstm_c[at] : 0.f, odd ? a.lstm_c[at + DG] : 0.f);
+      hlast[gi] = make_float2(even ? a.lstm_h[at] : 0.f, odd ? a.lstm_h[at + DG] : 0.f);
+    }
+
+    // message m of a warp goes to peer (rank + 1 + m / rows of a block): row m % rows of that CTA's buffers, as an address in the cluster window
+    uint32_t peer_hs[SENDS > 0 ? SENDS : 1];
+#pragma unroll
+    for (int x = 0; x < SENDS; ++x)
+      peer_hs[x] = map_to_rank(smem_u32(hs), (rank + 1 + (lane + 32 * x) / (PL * NS)) % CL) + (lane + 32 * x) % (PL * NS) * 16;
+
+    // barriers initialised and buffer 0 filled in every CTA before anyone sends
+    KVE_RNN_ONCE(3);
+    cluster_sync_all();
+    KVE_RNN_ONCE(4);
+
+    KVE_RNN_MARK_BEGIN();
+    for (int batch = 0; batch < n_batches && alive; ++batch) {
+      // ---- the pre-activations of the next T steps' inputs
+      const int run = batches_before + batch;
+      alive = __all_sync(0xffffffffu, mbar_wait_bounded(&x_done[run & 1], (uint32_t)((run >> 1) & 1)));
+      if (!alive) {
+        if (lane == 0) set_status(a.status, ERR_TIMEOUT);
+        break;
+      }
+      umma::fence_after_sync();
+      uint32_t acc_x = tmem_mine + GX_TMEM_ACC + (uint32_t)(((run & 1) * 2 + (warp >> 2)) * GX_N);
+      const int step_end = min(batch * T + T, a.n_range);
+      for (int step = batch * T; step < step_end; ++step) {
+        const int buf = step & 1;
+        const bool send_h = step + 1 < a.n_range;
+#pragma unroll
+        for (int gi = 0; gi < NG; ++gi) {
+          uint16_t* hs_g = hs + gi * 2 * HS_BUF;
+          uint64_t* hbar_g = hbar + 2 * gi;
+          // pre-activations of the round's inputs, in the layout of the MMA accumulators
+          uint32_t pin[2][4];
+          auto ask_pin = [&]() {
+            umma::tmem_ld_frag_nowait(acc_x, pin[0]);
+            umma::tmem_ld_frag_nowait(acc_x + (16u << 16), pin[1]);
+            acc_x += 8;
+          };
+          if (!P_LATE) ask_pin();
+          KVE_RNN_MARK(2);
+          // ---- h_{t-1} from every CTA of the cluster (each buffer completes once per two steps) -----------------------------
+          if (step > 0) {
+            // (one poll usually waits long enough: it is the only thing in the way then)
+            const uint32_t parity = ((exchanged >> buf) + ((step - 1) >> 1)) & 1;
+            if (!__all_sync(0xffffffffu, mbar_try_wait_cluster(&hbar_g[buf], parity))) {
+              alive = __all_sync(0xffffffffu, mbar_wait_cluster_bounded(&hbar_g[buf], parity));
+              if (!alive) {
+                if (lane == 0) set_status(a.status, ERR_TIMEOUT);
+                break;
+              }
             }
           }
-        }
-        KVE_RNN_MARK(0);
+          KVE_RNN_MARK(0);
 
-        // ---- W_hh h_{t-1} on the tensor cores: one accumulator set per plane ---------------------------------------------
-        float acc[PL][2][4];
+          // ---- W_hh h_{t-1} on the tensor cores: one accumulator set per plane ---------------------------------------------
+          float acc[PL][2][4];
 #pragma unroll
-        for (int pl = 0; pl < PL; ++pl)
+          for (int pl = 0; pl < PL; ++pl)
 #pragma unroll
-          for (int mt = 0; mt < 2; ++mt)
+            for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) acc[pl][mt][e] = 0.f;
-        // B fragments: one ldmatrix.x4 brings the 8 sequences x 32 k-values of a plane (two k tiles);
-        // lane l addresses row (l & 7) of the 8 x 8 block (l >> 3).
-        const uint32_t hb_lane = smem_u32(hs_g + buf * HS_BUF + (lane >> 3) * KBLK + (lane & 7) * 8);
-        uint32_t bf[2][PL][4];
-        auto load_b = [&](int kp) {
+              for (int e = 0; e < 4; ++e) acc[pl][mt][e] = 0.f;
+          // B fragments: one ldmatrix.x4 brings the 8 sequences x 32 k-values of a plane (two k tiles);
+          // lane l addresses row (l & 7) of the 8 x 8 block (l >> 3).
+          const uint32_t hb_lane = smem_u32(hs_g + buf * HS_BUF + (lane >> 3) * KBLK + (lane & 7) * 8);
+          uint32_t bf[2][PL][4];
+          auto load_b = [&](int kp) {
 #pragma unroll
-          for (int pl = 0; pl < PL; ++pl) ldmatrix_x4(bf[kp & 1][pl], hb_lane + (uint32_t)((kp * 4 * KBLK + pl * NS * 8) * 2));
-        };
-        load_b(0);
+            for (int pl = 0; pl < PL; ++pl) ldmatrix_x4(bf[kp & 1][pl], hb_lane + (uint32_t)((kp * 4 * KBLK + pl * NS * 8) * 2));
+          };
+          load_b(0);
 #pragma unroll
-        for (int kp = 0; kp < KT / 2; ++kp) {
-          if (kp + 1 < KT / 2) load_b(kp + 1);      // a pair of k tiles ahead
+          for (int kp = 0; kp < KT / 2; ++kp) {
+            if (kp + 1 < KT / 2) load_b(kp + 1);      // a pair of k tiles ahead
 #pragma unroll
-          for (int half = 0; half < 2; ++half)
+            for (int half = 0; half < 2; ++half)
 #pragma unroll
-            for (int pl = 0; pl < PL; ++pl)
+              for (int pl = 0; pl < PL; ++pl)
 #pragma unroll
-              for (int mt = 0; mt < 2; ++mt) mma_bf16_16816(acc[pl][mt], A[kp][mt][half], bf[kp & 1][pl][2 * half], bf[kp & 1][pl][2 * half + 1]);
-        }
-        if (!PACE_BY_SENDS && tid == 0) *rounds_done = step * NG + gi + 1;
-        KVE_RNN_MARK(1);
+                for (int mt = 0; mt < 2; ++mt) mma_bf16_16816(acc[pl][mt], A[kp][mt][half], bf[kp & 1][pl][2 * half], bf[kp & 1][pl][2 * half + 1]);
+          }
+          if (!PACE_BY_SENDS && tid == 0) *rounds_done = step * NG + gi + 1;
+          KVE_RNN_MARK(1);
 
-        // (the vote is a scheduling fence: without it the compiler draws what follows into the MMA chain, 10 % of a step)
-        if (!__all_sync(0xffffffffu, alive)) break;
-        if (P_LATE) ask_pin();
-        umma::tmem_ld_wait_frags(pin[0], pin[1]);
-        // ---- cell update (thread-local), planes of h_t into this CTA's buffer ---------------------
-        float2 pre[4];       // both sequences: 0 = i, 1 = f (tile 0, rows g / g+8), 2 = g, 3 = o (tile 1)
+          // (the vote is a scheduling fence: without it the compiler draws what follows into the MMA chain, 10 % of a step)
+          if (!__all_sync(0xffffffffu, alive)) break;
+          if (P_LATE) ask_pin();
+          umma::tmem_ld_wait_frags(pin[0], pin[1]);
+          // ---- cell update (thread-local), planes of h_t into this CTA's buffer ---------------------
+          float2 pre[4];       // both sequences: 0 = i, 1 = f (tile 0, rows g / g+8), 2 = g, 3 = o (tile 1)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int mt = q >> 1, ai = (q & 1) * 2;
-          float2 sum = make_float2(acc[PL - 1][mt][ai], acc[PL - 1][mt][ai + 1]);      // smallest plane first
+          for (int q = 0; q < 4; ++q) {
+            const int mt = q >> 1, ai = (q & 1) * 2;
+            float2 sum = make_float2(acc[PL - 1][mt][ai], acc[PL - 1][mt][ai + 1]);      // smallest plane first
 #pragma unroll
-          for (int pl = PL - 2; pl >= 0; --pl) sum = add2(sum, make_float2(acc[pl][mt][ai], acc[pl][mt][ai + 1]));
-          pre[q] = add2(sum, add2(make_float2(__uint_as_float(pin[mt][ai]), __uint_as_float(pin[mt][ai + 1])), make_float2(bias[q], bias[q])));
-        }
-        const float2 hv = lstm_cell_pair(pre, c[gi]);
-        hlast[gi] = hv;
-        KVE_RNN_MARK(3);
-        // products of the score: nothing of the chain waits for their sum
-        {
-          float* mine = prod + (gi * 2 + buf) * PROD_BUF + (warp * 2 * 4 + tig) * 8 + g;
-          mine[0] = w_score * hv.x;
-          mine[4 * 8] = w_score * hv.y;
-        }
-        // ---- the warp's k-block (8 units: [plane][sequence][8], contiguous) to every CTA of the cluster ----
-        if (send_h) {
-          const uint32_t off = (uint32_t)(((gi * 2 + (buf ^ 1)) * HS_BUF + ((int)rank * RNN_WARPS + warp) * KBLK) * 2);
-          // lanes g and g ^ 1 hold neighbouring units: an even g takes both units of sequence 2 tig, an odd one those of 2 tig + 1, and
-          // a warp's store instruction is a whole plane of the block: 128 bytes in a row
-          const bool odd = (g & 1) != 0;
-          unsigned char* mine = reinterpret_cast<unsigned char*>(hs) + off + (tig * 2 + (g & 1)) * 16 + (g >> 1) * 4;
-          uint32_t pl[3];      // planes of both sequences, the even one below
-          split3_pair(hv.x, hv.y, pl);
-          const uint32_t h0 = __byte_perm(pl[0], pl[1], 0x5410), h1 = __byte_perm(pl[0], pl[1], 0x7632);      // two planes of a sequence
-          const uint32_t keep = odd ? h1 : h0, got = __shfl_xor_sync(0xffffffffu, odd ? h0 : h1, 4);
-          *reinterpret_cast<uint32_t*>(mine) = __byte_perm(odd ? got : keep, odd ? keep : got, 0x5410);
-          *reinterpret_cast<uint32_t*>(mine + NS * 16) = __byte_perm(odd ? got : keep, odd ? keep : got, 0x7632);
-          if constexpr (PL == 3) {
-            const uint32_t got2 = __shfl_xor_sync(0xffffffffu, pl[2], 4);
-            *reinterpret_cast<uint32_t*>(mine + 2 * NS * 16) = __byte_perm(odd ? got2 : pl[2], odd ? pl[2] : got2, odd ? 0x7632 : 0x5410);
+            for (int pl = PL - 2; pl >= 0; --pl) sum = add2(sum, make_float2(acc[pl][mt][ai], acc[pl][mt][ai + 1]));
+            pre[q] = add2(sum, add2(make_float2(__uint_as_float(pin[mt][ai]), __uint_as_float(pin[mt][ai + 1])), make_float2(bias[q], bias[q])));
           }
-          __syncwarp();
-          // peers: 16-byte rows out of the own block, each counted in bytes on the receiver's barrier; lane l sends message l, l + 32 ..
-#pragma unroll
-          for (int x = 0; x < SENDS; ++x) {
-            const uint4 row = *reinterpret_cast<const uint4*>(reinterpret_cast<const unsigned char*>(hs) + off + (lane + 32 * x) % (PL * NS) * 16);
-            if (x * 32 + lane < (CL - 1) * PL * NS)
-              st_async_cluster(peer_hs[x] + off, row, peer_hs[x] - (lane + 32 * x) % (PL * NS) * 16 + OFF_BARS + (2 * gi + (buf ^ 1)) * 8);
+          const float2 hv = lstm_cell_pair(pre, c[gi]);
+          hlast[gi] = hv;
+          KVE_RNN_MARK(3);
+          // products of the score: nothing of the chain waits for their sum
+          {
+            float* mine = prod + (gi * 2 + buf) * PROD_BUF + (warp * 2 * 4 + tig) * 8 + g;
+            mine[0] = w_score * hv.x;
+            mine[4 * 8] = w_score * hv.y;
           }
-          if (lane == 0) mbar_arrive(&hbar_g[buf ^ 1]);     // release: this warp's own pieces are in place
-        }
-        if (PACE_BY_SENDS && tid == 0) *rounds_done = step + 1;
-        KVE_RNN_MARK(4);
+          // ---- the warp's k-block (8 units: [plane][sequence][8], contiguous) to every CTA of the cluster ----
+          if (send_h) {
+            const uint32_t off = (uint32_t)(((gi * 2 + (buf ^ 1)) * HS_BUF + ((int)rank * RNN_WARPS + warp) * KBLK) * 2);
+            // lanes g and g ^ 1 hold neighbouring units: an even g takes both units of sequence 2 tig, an odd one those of 2 tig + 1, and
+            // a warp's store instruction is a whole plane of the block: 128 bytes in a row
+            const bool odd = (g & 1) != 0;
+            unsigned char* mine = reinterpret_cast<unsigned char*>(hs) + off + (tig * 2 + (g & 1)) * 16 + (g >> 1) * 4;
+            uint32_t pl[3];      // planes of both sequences, the even one below
+            split3_pair(hv.x, hv.y, pl);
+            const uint32_t h0 = __byte_perm(pl[0], pl[1], 0x5410), h1 = __byte_perm(pl[0], pl[1], 0x7632);      // two planes of a sequence
+            const uint32_t keep = odd ? h1 : h0, got = __shfl_xor_sync(0xffffffffu, odd ? h0 : h1, 4);
+            *reinterpret_cast<uint32_t*>(mine) = __byte_perm(odd ? got : keep, odd ? keep : got, 0x5410);
+            *reinterpret_cast<uint32_t*>(mine + NS * 16) = __byte_perm(odd ? got : keep, odd ? keep : got, 0x7632);
+            if constexpr (PL == 3) {
+              const uint32_t got2 = __shfl_xor_sync(0xffffffffu, pl[2], 4);
+              *reinterpret_cast<uint32_t*>(mine + 2 * NS * 16) = __byte_perm(odd ? got2 : pl[2], odd ? pl[2] : got2, odd ? 0x7632 : 0x5410);
+            }
+            __syncwarp();
+            // peers: 16-byte rows out of the own block, each counted in bytes on the receiver's barrier; lane l sends message l, l + 32 ..
+#pragma unroll
+            for (int x = 0; x < SENDS; ++x) {
+              const uint4 row = *reinterpret_cast<const uint4*>(reinterpret_cast<const unsigned char*>(hs) + off + (lane + 32 * x) % (PL * NS) * 16);
+              if (x * 32 + lane < (CL - 1) * PL * NS)
+                st_async_cluster(peer_hs[x] + off, row, peer_hs[x] - (lane + 32 * x) % (PL * NS) * 16 + OFF_BARS + (2 * gi + (buf ^ 1)) * 8);
+            }
+            if (lane == 0) mbar_arrive(&hbar_g[buf ^ 1]);     // release: this warp's own pieces are in place
+          }
+          if (PACE_BY_SENDS && tid == 0) *rounds_done = step + 1;
+          KVE_RNN_MARK(4);
 #ifdef KVE_RNN_STAMPS
-        if (blockIdx.x == 0 && tid == 0) atomicAdd(&g_rnn_cycles[5], 1ull);
+          if (blockIdx.x == 0 && tid == 0) atomicAdd(&g_rnn_cycles[5], 1ull);
 #endif
-        KVE_RNN_MARK(6);
+          KVE_RNN_MARK(6);
+        }
+        if (!alive) break;
       }
-      if (!alive) break;
+      umma::fence_before_sync();      // this warp's loads out of the accumulators come before what the projector writes there next
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&x_read[run & 1]);
     }
-    umma::fence_before_sync();      // this warp's loads out of the accumulators come before what the projector writes there next
-    __syncwarp();
-    if (lane == 0) mbar_arrive(&x_read[batch & 1]);
-  }
 
-  KVE_RNN_ONCE(5);
-  // ---- carried state out ---------------------------------------------------------------------------
+    KVE_RNN_ONCE(5);
+    // ---- carried state out ---------------------------------------------------------------------------
 #pragma unroll
-  for (int gi = 0; gi < NG; ++gi)
+    for (int gi = 0; gi < NG; ++gi)
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int s = seq0 + gi * NS + tig * 2 + e;
-      if (s < a.S && alive) {
-        a.lstm_c[(long long)s * DG + ug] = e ? c[gi].y : c[gi].x;
-        a.lstm_h[(long long)s * DG + ug] = e ? hlast[gi].y : hlast[gi].x;
+      for (int e = 0; e < 2; ++e) {
+        const int s = seq0 + gi * NS + tig * 2 + e;
+        if (s < a.S && alive) {
+          a.lstm_c[(long long)s * DG + ug] = e ? c[gi].y : c[gi].x;
+          a.lstm_h[(long long)s * DG + ug] = e ? hlast[gi].y : hlast[gi].x;
+        }
       }
-    }
-  // (the last step's products, which no exchange follows)
-  asm volatile("bar.sync 1, %0;" ::"n"(RNN_THREADS) : "memory");
-  if (warp < NG && alive) put_scores(warp, a.n_range - 1);
-  // nobody leaves while a peer may still be sending into its shared memory; the partial sums of all CTAs are in place behind it
-  cluster_sync_all();
-  KVE_RNN_ONCE(6);
-  if (warp == 0) umma::tmem_dealloc(tmem, GX_TMEM_COLS);
-  // ---- score head: s_t = sigmoid(w_s . h_t + b_s); a row's d_g / 8 partial sums lie side by side and are added in order -----------
-  const int n_seq = min(NS * NG, a.S - seq0);
-  for (int i = (int)rank * RNN_THREADS + tid; i < n_seq * a.n_range; i += CL * RNN_THREADS) {
-    const float4* src = reinterpret_cast<const float4*>(a.H + ((long long)seq0 * a.n_range + i) * (DG / 8));
-    float sum = 0.f;
+    // (the last step's products, which no exchange follows)
+    asm volatile("bar.sync 1, %0;" ::"n"(RNN_THREADS) : "memory");
+    if (warp < NG && alive) put_scores(warp, a.n_range - 1);
+    // nobody leaves while a peer may still be sending into its shared memory; the partial sums of all CTAs are in place behind it
+    cluster_sync_all();
+    KVE_RNN_ONCE(6);
+    if (!MANY && warp == 0) umma::tmem_dealloc(tmem, GX_TMEM_COLS);
+    // ---- score head: s_t = sigmoid(w_s . h_t + b_s); a row's d_g / 8 partial sums lie side by side and are added in order -----------
+    const int n_seq = min(NS * NG, a.S - seq0);
+    for (int i = (int)rank * RNN_THREADS + tid; i < n_seq * a.n_range; i += CL * RNN_THREADS) {
+      const float4* src = reinterpret_cast<const float4*>(a.H + ((long long)seq0 * a.n_range + i) * (DG / 8));
+      float sum = 0.f;
 #pragma unroll
-    for (int q = 0; q < DG / 32; ++q) {
-      const float4 x = __ldcg(src + q);
-      sum += x.x; sum += x.y; sum += x.z; sum += x.w;
+      for (int q = 0; q < DG / 32; ++q) {
+        const float4 x = __ldcg(src + q);
+        sum += x.x; sum += x.y; sum += x.z; sum += x.w;
+      }
+      const int s = i / a.n_range;
+      a.scores[(long long)(seq0 + s) * a.max_chunks + a.t0 + (i - s * a.n_range)] = 1.f / (1.f + expf(-(sum + a.b_s)));
     }
-    const int s = i / a.n_range;
-    a.scores[(long long)(seq0 + s) * a.max_chunks + a.t0 + (i - s * a.n_range)] = 1.f / (1.f + expf(-(sum + a.b_s)));
-  }
+  } while (next_set());
+  if (MANY && warp == 0) umma::tmem_dealloc(tmem, GX_TMEM_COLS);
 }
 
-template <int DG, int CL, int NG, int PL>
+// Clusters that the current device holds at a time
+template <int DG, int CL, int NG, int PL, bool MANY>
+static cudaError_t resident_clusters(cudaLaunchConfig_t cfg, int* most) {
+  static std::atomic<int> known[MAX_DEVICES];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= MAX_DEVICES) return cudaErrorInvalidDevice;
+  *most = known[dev].load(std::memory_order_acquire);
+  if (*most > 0) return cudaSuccess;
+  cudaLaunchAttribute shape[1];
+  shape[0].id = cudaLaunchAttributeClusterDimension;
+  shape[0].val.clusterDim.x = CL;
+  shape[0].val.clusterDim.y = shape[0].val.clusterDim.z = 1;
+  cfg.attrs = shape;
+  cfg.numAttrs = 1;
+  e = cudaOccupancyMaxActiveClusters(most, kve_gate_rnn_kernel<DG, CL, NG, PL, MANY>, &cfg);
+  if (e == cudaSuccess && *most < 1) e = cudaErrorInvalidConfiguration;
+  if (e == cudaSuccess) known[dev].store(*most, std::memory_order_release);
+  return e;
+}
+
+template <int DG, int CL, int NG, int PL, bool MANY = false>
 static cudaError_t launch_rnn_t(const RnnArgs& a, const CUtensorMap* maps, cudaStream_t st) {
   constexpr int smem = RNN_SMEM_X<DG, NG, PL> + GX_BYTES + 1024;      // + slack to reach a 1024-byte boundary
   static DeviceFlags opted;
   {
-    cudaError_t e = smem_opt_in(opted, kve_gate_rnn_kernel<DG, CL, NG, PL>, smem);
+    cudaError_t e = smem_opt_in(opted, kve_gate_rnn_kernel<DG, CL, NG, PL, MANY>, smem);
     if (e != cudaSuccess) return e;
   }
-  const int clusters = (a.S + 8 * NG - 1) / (8 * NG);
+  int clusters = (a.S + 8 * NG - 1) / (8 * NG);
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -562,9 +601,17 @@ static cudaError_t launch_rnn_t(const RnnArgs& a, const CUtensorMap* maps, cudaS
   cfg.blockDim = dim3(GATE_THREADS);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
+  if (MANY) {      // as few sets one after the other as all clusters at a time need
+    int most = 0;
+    const cudaError_t e = resident_clusters<DG, CL, NG, PL, MANY>(cfg, &most);
+    if (e != cudaSuccess) return e;
+    const int sets = (clusters + most - 1) / most;
+    clusters = (clusters + sets - 1) / sets;
+    cfg.gridDim = dim3(clusters * CL);
+  }
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, kve_gate_rnn_kernel<DG, CL, NG, PL>, maps[0], maps[1], a);
+  return cudaLaunchKernelEx(&cfg, kve_gate_rnn_kernel<DG, CL, NG, PL, MANY>, maps[0], maps[1], a);
 }
 
 // CTAs of a cluster; two groups of 8 sequences per cluster once one group per cluster would need more than one wave of clusters
@@ -578,15 +625,20 @@ double gate_rnn_us_per_chunk(int S, int d_g, int planes) {
   return (two ? 2.28 : 1.22) * (planes == 3 ? 1.25 : 1.0) * ((clusters + wave - 1) / wave);
 }
 
-template <int PL>
-static cudaError_t launch_rnn_planes(const RnnArgs& a, const CUtensorMap* maps, int d_g, cudaStream_t st) {
-  const bool two = two_groups(a.S, d_g);
-  switch (d_g) {
-    case 256: return two ? launch_rnn_t<256, 4, 2, PL>(a, maps, st) : launch_rnn_t<256, 4, 1, PL>(a, maps, st);
-    case 128: return two ? launch_rnn_t<128, 2, 2, PL>(a, maps, st) : launch_rnn_t<128, 2, 1, PL>(a, maps, st);
-    case 64:  return two ? launch_rnn_t<64, 1, 2, PL>(a, maps, st) : launch_rnn_t<64, 1, 1, PL>(a, maps, st);
-    default:  return cudaErrorInvalidValue;
-  }
+// More sequences than the clusters of one wave hold, and few chunks: the clusters of one wave go through several sets of sequences, because what a
+// cluster does before its first round (weights into registers and tensor memory, 4 us) would be most of the launch.  us, a wave of new
+// clusters for every set -> one wave: 4096 sequences x 1 chunk at d_g = 64, 128, 256 14.0 -> 11.0, 31.2 -> 20.2, 76.4 -> 45.1; 1200 x 16 at d_g = 128
+// 59.9 -> 56.7, 2400 x 16 at d_g = 64 43.3 -> 43.0, 600 x 4 at d_g = 256 27.9 -> 26.6.  With more chunks the rounds of that instance, 5 % longer at d_g = 256
+// and 2 % at 64, outweigh it: 600 x 8 at d_g = 256 44.0 -> 44.7, 2400 x 28 at d_g = 64 68.3 -> 69.3.
+template <int DG>
+constexpr int MANY_CHUNKS = DG == 256 ? 4 : 16;
+
+template <int DG, int PL>
+static cudaError_t launch_rnn_planes(const RnnArgs& a, const CUtensorMap* maps, cudaStream_t st) {
+  constexpr int CL = DG / 64;
+  if (!two_groups(a.S, DG)) return launch_rnn_t<DG, CL, 1, PL>(a, maps, st);
+  const bool many = (a.S + 15) / 16 > sm_count() / CL && a.n_range <= MANY_CHUNKS<DG>;
+  return many ? launch_rnn_t<DG, CL, 2, PL, true>(a, maps, st) : launch_rnn_t<DG, CL, 2, PL>(a, maps, st);
 }
 
 cudaError_t encode_gate_maps(void* maps, const void* ksum, const void* vsum, long long n_seq, int max_chunks, int S, int d_g) {
@@ -614,7 +666,12 @@ cudaError_t launch_gate_rnn(const LayerView& v, const void* maps, int seq_base, 
   a.H = H; a.W_hh = W_hh; a.w_s = w_s; a.b_s = b_s;
   a.scores = v.scores; a.lstm_h = v.lstm_h; a.lstm_c = v.lstm_c; a.status = v.status;
   a.S = v.S; a.max_chunks = v.max_chunks; a.t0 = t0; a.n_range = t1 - t0; a.reset = reset_state ? 1 : 0;
-  return planes == 3 ? launch_rnn_planes<3>(a, tm, d_g, st) : launch_rnn_planes<2>(a, tm, d_g, st);
+  switch (d_g) {
+    case 256: return planes == 3 ? launch_rnn_planes<256, 3>(a, tm, st) : launch_rnn_planes<256, 2>(a, tm, st);
+    case 128: return planes == 3 ? launch_rnn_planes<128, 3>(a, tm, st) : launch_rnn_planes<128, 2>(a, tm, st);
+    case 64:  return planes == 3 ? launch_rnn_planes<64, 3>(a, tm, st) : launch_rnn_planes<64, 2>(a, tm, st);
+    default:  return cudaErrorInvalidValue;
+  }
 }
 
 }  // namespace kve

@@ -232,6 +232,34 @@ def test_long_gate_range_equals_short_ranges(d_g, S, planes, per_call):
         assert all(torch.equal(x, y) for x, y in zip(got[0], other))
 
 
+@pytest.mark.parametrize("d_g,S,planes", [(64, 2369, 2), (64, 5000, 3), (128, 1185, 3), (128, 3000, 2), (256, 593, 2), (256, 1800, 3)])
+def test_gate_of_many_sequences_and_few_chunks(d_g, S, planes):
+    # a cluster takes several sets of 16 sequences (two, three and four here, the last one partly empty) in calls of a few chunks, one set in longer
+    # calls: ranges of 1 to 16 chunks, even and odd, from scratch and behind a carried state, the same bits as the whole in one call
+    b = _binding()
+    Nc = 20
+    wl = wlm.Workload("many", B=1, H=S, n=Nc * 4 + 32, C=4, W=32, d_g=d_g, agg="mean", key_offset_std=0.5, seed=d_g + S)
+    st = make_store(wl)
+    gen = torch.Generator(device="cuda").manual_seed(S)
+    for pages in (st.k_pages, st.v_pages):
+        pages.normal_(generator=gen)
+    st.set_len(0, wl.n)
+    st.set_gate_planes(planes)
+    lw = b.LstmWeights(wlm.gen_lstm_weights(wl))
+    st.summarize_chunks(0, 0, Nc, None)
+    got = []
+    for cuts in ((0, 20), (0, 1, 2, 3, 4, 20), (0, 2, 5, 9, 11, 14, 18, 20), (0, 5, 12, 20), (0, 16, 20), (0, 4, 20)):
+        st.scores.fill_(float("nan"))
+        for t0, t1 in zip(cuts, cuts[1:]):
+            st.gate(0, t0, t1, lw)
+        torch.cuda.synchronize()
+        assert st.poll_status() == 0
+        got.append([x.clone() for x in (st.scores[0, :, :Nc], st.lstm_h, st.lstm_c)])
+    assert torch.isfinite(got[0][0]).all()
+    for other in got[1:]:
+        assert all(torch.equal(x, y) for x, y in zip(got[0], other))
+
+
 def test_chunk_of_one_identity_keep_all_is_dense():
     # C = 1 with identity aggregation and tau = 0: the summary path reproduces dense attention
     b = _binding()
