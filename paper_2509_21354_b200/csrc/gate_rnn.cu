@@ -70,9 +70,9 @@ constexpr int GATE_THREADS = RNN_THREADS + 128;
 // what a launch leaves of an SM's registers is where the means of kvE_refresh's second range run (three planes at d_g = 256 with 232 and 40
 // left room for none of their CTAs: kvE_refresh of 512 sequences x 121 chunks of 128, MLP, 1041 us, 926 so)
 template <int DG, int PL>
-constexpr int RNN_REGS = DG == 256 ? (PL == 3 ? 224 : 208) : (DG == 128 ? 184 : 136);
+constexpr int RNN_REGS = DG == 256 ? (PL == 3 ? 224 : 208) : (DG == 128 ? (PL == 3 ? 192 : 184) : 136);
 template <int DG, int PL>
-constexpr int PROJ_REGS = DG == 256 && PL == 3 ? 32 : 40;
+constexpr int PROJ_REGS = DG == 256 && PL == 3 ? 32 : (DG == 128 && PL == 3 ? 48 : 40);
 template <int DG, int PL>
 constexpr int GATE_REGS = (2 * RNN_REGS<DG, PL> + PROJ_REGS<DG, PL>) / 3;
 
