@@ -333,24 +333,6 @@ int kvE_create(const kvE_config* cfg, const kvE_buffers* buf, kvE_store** out) {
   st->off_kept_k = k.off_kept_k; st->off_kept_v = k.off_kept_v; st->off_listed = k.off_listed; st->ws_needed = k.total;
   st->attn_grid_max = attn_grid_cap();
   if ((size_t)st->attn_grid_max > ATTN_GRID_LIMIT) st->attn_grid_max = (int)ATTN_GRID_LIMIT;
-  if (encode_gate_maps(st->gate_maps, buf->ksum_bf16, buf->vsum_bf16, (long long)cfg->n_layers * st->S, st->max_chunks, st->S, cfg->d_g) != cudaSuccess) {
-    delete st;
-    return KVE_ERR_CUDA;
-  }
-  if (cfg->max_query_tokens > 0) {
-    st->block_hp = attn_block_hp(cfg->C);
-    st->block_split_cap = block_split_cap(st->S);
-    // maps over the page pools and over the compacted kept summary rows (all layers) in the workspace
-    char* ws0 = static_cast<char*>(buf->workspace);
-    const cudaError_t em = encode_attn_block_maps(st->block_maps, buf->k_pages, buf->v_pages, (long long)buf->n_pages * cfg->C,
-                                                  st->block_hp, ws0 + k.off_kept_k, ws0 + k.off_kept_v,
-                                                  (long long)cfg->n_layers * st->S * st->max_chunks);
-    if (em != cudaSuccess) {
-      delete st;
-      return KVE_ERR_CUDA;
-    }
-    st->block_ready = true;
-  }
   st->layers.assign(cfg->n_layers, LayerState());
   // partial records, tickets ... and the kept-row buffers (a box of the query-block kernel may reach past a sequence's
   // kept count: what it finds there must be finite)
@@ -359,6 +341,17 @@ int kvE_create(const kvE_config* cfg, const kvE_buffers* buf, kvE_store** out) {
   if (e == cudaSuccess) e = cudaMemset(buf->seq_len, 0, sizeof(int32_t) * (size_t)cfg->n_layers * cfg->B);
   if (e == cudaSuccess) e = cudaMemset(buf->keep_cnt, 0, sizeof(int32_t) * (size_t)cfg->n_layers * st->S);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  // tensor maps over the bf16 summaries; over the page pools and the compacted kept summary rows (all layers) in the workspace.  The driver
+  // refuses to encode them for a thread without a context: one whose first CUDA call this is has one since the calls above
+  if (e == cudaSuccess) e = encode_gate_maps(st->gate_maps, buf->ksum_bf16, buf->vsum_bf16, (long long)cfg->n_layers * st->S, st->max_chunks, st->S, cfg->d_g);
+  if (e == cudaSuccess && cfg->max_query_tokens > 0) {
+    st->block_hp = attn_block_hp(cfg->C);
+    st->block_split_cap = block_split_cap(st->S);
+    char* ws0 = static_cast<char*>(buf->workspace);
+    e = encode_attn_block_maps(st->block_maps, buf->k_pages, buf->v_pages, (long long)buf->n_pages * cfg->C, st->block_hp, ws0 + k.off_kept_k,
+                               ws0 + k.off_kept_v, (long long)cfg->n_layers * st->S * st->max_chunks);
+    st->block_ready = e == cudaSuccess;
+  }
   if (e != cudaSuccess) {
     release_host_objects(st);
     delete st;

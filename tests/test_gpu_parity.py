@@ -159,6 +159,35 @@ def test_gate_sizes_and_chunk_sizes(d_g, C):
     full_check(wl, "summary")
 
 
+@pytest.mark.parametrize("max_query_tokens", [0, 4])
+def test_handles_are_made_by_threads_that_have_not_called_before(max_query_tokens):
+    """kvE_create as the first CUDA call of a thread, several threads at once; the handles work"""
+    import ctypes as C
+    import threading
+    b = _binding()
+    wl = wlm.CFG1.small(n=512, seed=6)
+    pb = hz.Problem(wl)
+    stores = [b.Store(B=wl.B, H=wl.H, C_=wl.C, W=wl.W, max_tokens=wl.max_tokens, d_g=wl.d_g, agg=wl.agg, max_query_tokens=max_query_tokens) for _ in range(6)]
+    codes = {}
+    for st in stores:
+        st.lib.kvE_destroy(st.handle)
+        st.handle = C.c_void_p()
+
+    def make(i):
+        codes[i] = stores[i].lib.kvE_create(C.byref(stores[i].cfg), C.byref(stores[i].buf), C.byref(stores[i].handle))
+
+    threads = [threading.Thread(target=make, args=(i,)) for i in range(len(stores))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert codes == {i: 0 for i in range(len(stores))}
+    for st in stores[::5]:
+        load_kv(st, 0, pb.K, pb.V)
+        run_gpu_pipeline(st, pb, 0, None, b.LstmWeights(pb.lstm))
+        check_gate_and_keep(st, pb)
+
+
 @pytest.mark.parametrize("d_g,B,H", [(64, 37, 33), (256, 9, 35)])
 def test_two_sequence_groups_per_cluster(d_g, B, H):
     # more sequences than one group of 8 per cluster places in one wave: every cluster walks two groups;
