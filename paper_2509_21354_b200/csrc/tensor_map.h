@@ -3,6 +3,8 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
+
 namespace kve {
 
 // `rank` dimensions, innermost first; strides in bytes of the dimensions above the innermost; elements beyond the array read as zero
@@ -10,15 +12,16 @@ inline cudaError_t encode_bf16_map(CUtensorMap* tm, const void* base, int rank, 
   typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                                const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-  static EncodeFn encode = nullptr;
-  if (!encode) {
-    void* fn = nullptr;
+  static std::atomic<void*> found{nullptr};      // handles may be made by several threads at once
+  void* fn = found.load(std::memory_order_acquire);
+  if (!fn) {
     cudaDriverEntryPointQueryResult qres;
     cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres);
     if (e != cudaSuccess) return e;
     if (qres != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
-    encode = reinterpret_cast<EncodeFn>(fn);
+    found.store(fn, std::memory_order_release);
   }
+  const EncodeFn encode = reinterpret_cast<EncodeFn>(fn);
   const cuuint32_t estr[3] = {1u, 1u, 1u};
   const CUresult r = encode(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), dims, strides, box, estr,
                             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
