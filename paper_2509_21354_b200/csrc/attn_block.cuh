@@ -105,7 +105,11 @@ __device__ __forceinline__ int first_pages(const BlockArgs& a, int s, int split,
 // sequences x 1084 rows 18.5 us, 18.1 so (64 x 4099 35.2 and 34.6).  What a lane fetches for a tile: up to two boxes (K and V each, both 64-column halves):
 //   page tiles:    lane j < granules: hp rows of a page to tile row j * hp
 //   summary tiles: lane j < ceil(valid / 16): 16 kept summary rows (compacted by kvE_compact)
-template <int STAGES>
+// FILL_PAUSE_NS: pause between the tiles of the first filling of the ring.  Asked for all at once they land at about the same time, and the first
+// lands late: where a tile takes longer to work on than to fetch (the tcgen05 kernel: five hand-overs) that is the launch's start.  128 rows x 256
+// sequences x 300 rows 26.7 us without, 25.7 with 250 ns, 25.6 with 500; 64 rows x 128 x 1084 22.2, 21.6, 21.7; the kernel on
+// warp MMAs, which keeps up with the copies, loses (28 rows x 128 x 1084 16.5 and 16.9).
+template <int STAGES, int FILL_PAUSE_NS>
 __device__ __forceinline__ int block_producer(const BlockArgs& a, const BlockGeom& gm, int s, int lane,
                                                const CUtensorMap* tmK, const CUtensorMap* tmV, const CUtensorMap* tmKs,
                                                const CUtensorMap* tmVs, int first, unsigned char* ring, uint64_t* full,
@@ -165,6 +169,7 @@ __device__ __forceinline__ int block_producer(const BlockArgs& a, const BlockGeo
       tma_load_2d(vdst, mv, 0, src, &full[stage]);
       tma_load_2d(vdst + BK_KBLOCK_BYTES, mv, 64, src, &full[stage]);
     }
+    if (FILL_PAUSE_NS > 0 && i < STAGES - 1) __nanosleep(FILL_PAUSE_NS);
   }
   return i;
 }

@@ -155,7 +155,7 @@ kve_decode_attn_block_tc_kernel(const __grid_constant__ CUtensorMap tmK, const _
 
   if (warp == 0) {
     // ================= producer warp =================
-    const int issued = block_producer<TC_STAGES>(a, gm, s, lane, &tmK, &tmV, &tmKs, &tmVs, first, ring, full, empty);
+    const int issued = block_producer<TC_STAGES, 250>(a, gm, s, lane, &tmK, &tmV, &tmKs, &tmVs, first, ring, full, empty);
     if (issued < gm.n_tiles) ring_drain<TC_STAGES>(full, issued);
   } else if (warp == 1) {
     // ================= MMA issue (one thread) =================

@@ -91,7 +91,7 @@ kve_decode_attn_block_warp_kernel(const __grid_constant__ CUtensorMap tmK, const
     // the sequence has outgrown what this launch was sized for (a replayed launch): rows would be dropped
     if (gm.outgrown && split == 0 && lane == 0) set_status(v.status, ERR_CAPACITY);
     if (split < gm.n_splits) {
-      const int n = block_producer<BW_STAGES>(a, gm, s, lane, &tmK, &tmV, &tmKs, &tmVs, first, ring, full, empty);
+      const int n = block_producer<BW_STAGES, 0>(a, gm, s, lane, &tmK, &tmV, &tmKs, &tmVs, first, ring, full, empty);
       if (lane == 0) *issued = n;
     }
     return;
