@@ -22,35 +22,18 @@ __device__ __forceinline__ float relu_nan(float x) {
   return y;
 }
 
-// coefficients of -g at degree 6, lowest first
+// coefficients of -g at degree 6, lowest first (the per-token MLP, which has the steps of several values side by side)
 #define KVE_GELU_TAIL6 {-0.999993061f, -1.1512017f, -0.458770975f, -0.0534121019f, 0.00808071511f, -0.00076921928f, 3.30927681e-05f}
 
-// relu: max(x, 0); a: |x|, at most 6; result: the tail Q(a).  x Phi(x) = relu - a * Q
-template <int DEGREE>
-__device__ __forceinline__ float2 gelu_tail2(float2 x, float2& relu, float2& a) {
-  static_assert(DEGREE == 6 || DEGREE == 8, "degrees fitted");
-  a = make_float2(fminf(fabsf(x.x), 6.f), fminf(fabsf(x.y), 6.f));
-  relu = make_float2(relu_nan(x.x), relu_nan(x.y));
-  constexpr float G6[7] = KVE_GELU_TAIL6;
+// x Phi(x) at degree 8
+__device__ __forceinline__ float2 gelu2(float2 x) {
   constexpr float G8[9] = {-0.999998868f, -1.15112329f, -0.459115446f, -0.0527141988f, 0.00733338343f, -0.00032334181f, -0.000114462782f,
                            2.50833236e-05f, -1.69040277e-06f};
-  float2 p;
-  if constexpr (DEGREE == 6) {
-    p = make_float2(G6[6], G6[6]);
+  const float2 a = make_float2(fminf(fabsf(x.x), 6.f), fminf(fabsf(x.y), 6.f)), relu = make_float2(relu_nan(x.x), relu_nan(x.y));
+  float2 p = make_float2(G8[8], G8[8]);
 #pragma unroll
-    for (int k = 5; k >= 0; --k) p = fma2(p, a, make_float2(G6[k], G6[k]));
-  } else {
-    p = make_float2(G8[8], G8[8]);
-#pragma unroll
-    for (int k = 7; k >= 0; --k) p = fma2(p, a, make_float2(G8[k], G8[k]));
-  }
-  return make_float2(ex2_fast(p.x), ex2_fast(p.y));
-}
-
-__device__ __forceinline__ float2 gelu2(float2 x) {
-  float2 relu, a;
-  const float2 q = gelu_tail2<8>(x, relu, a);
-  return fma2(make_float2(-a.x, -a.y), q, relu);
+  for (int k = 7; k >= 0; --k) p = fma2(p, a, make_float2(G8[k], G8[k]));
+  return fma2(make_float2(-a.x, -a.y), make_float2(ex2_fast(p.x), ex2_fast(p.y)), relu);
 }
 
 }  // namespace kve
