@@ -179,8 +179,8 @@ def algorithmic_bytes(wl, Nc, keep_mean, R, attend="summary"):
     by = {}
     by["chunk_mean"] = S * Nc * (2 * wl.C * 256 + 2 * 128 * 4)            # every stale K and V row once; fp32 means out
     by["chunk_mlp"] = S * Nc * 2 * (128 * 4 + 128 * 4 + 128 * 2)          # means in, fp32 + bf16 summaries out
-    by["gate_proj"] = S * Nc * (2 * 256 + 4 * d_g * 4)                    # as a kernel of its own: bf16 summaries in, fp32 P out
-    by["gate_rnn"] = S * Nc * (4 * d_g * 4 + 4)                           # P in, scores out
+    by["gate_rnn"] = S * Nc * (2 * 256 + 4)                               # bf16 summaries in, scores out
+    by["gate_proj"] = S * Nc * (2 * 256 + 4 * d_g * 4)                    # the gate's input projection if its result went through memory
     by["compact"] = S * (Nc * 4 + Nc * 4 + 4)
     rows_per_kept = wl.C if attend == "raw" else 1                          # a kept chunk: its C raw rows, or its one summary row
     by["attn_gated"] = S * (2 * (R + keep_mean * rows_per_kept) * 256 + 2 * 256)   # retained rows of K and V once (+ q, out)
@@ -563,7 +563,7 @@ def measure_config(rig, peaks, peak_kind, flush, headline=False):
     us_in, us_cold = kernel_times(rig, flush)
     by = algorithmic_bytes(wl, rig.Nc, rig.keep_mean, rig.R, rig.attend)
     by_kernel = {"append": wl.S * 4 * 256, "chunk_mean": by["chunk_mean"], "chunk_mlp": by["chunk_mlp"],
-                 "gate_rnn": wl.S * rig.Nc * (2 * 256 + 4), "compact": by["compact"],
+                 "gate_rnn": by["gate_rnn"], "compact": by["compact"],
                  "attn": by["attn_gated"], "attn_dense": by["attn_dense"]}
     fl = algorithmic_flops(wl, rig.Nc)
     fl["gate_rnn"] += fl.pop("gate_proj")      # one kernel: bf16 summaries in, scores out

@@ -17,6 +17,7 @@ def test_algorithmic_bytes_of_cfg2():
     raw = bench.algorithmic_bytes(wl, Nc, keep_mean=28.0, R=R, attend="raw")
     assert raw["attn_gated"] == 256 * (2 * (512 + 28 * 64) * 256 + 512)                    # kept chunks at full resolution
     assert by["gate_proj"] == units * (2 * 256 + 1024 * 4)
+    assert by["gate_rnn"] == units * (2 * 256 + 4) == 7_397_376                           # one kernel: summaries in, scores out
     assert by["compact"] == 256 * (56 * 8 + 4)
 
 
