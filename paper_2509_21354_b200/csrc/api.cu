@@ -608,14 +608,13 @@ int kvE_adopt_device_state(kvE_store* st, int layer, void* stream) {
 // steps that leaves HBM idle, the chunk mean a stream that leaves everything else idle: of two ranges, the means of the second
 // are taken while the recurrence goes through the first (kve_chunk_mean_beside_kernel).  With M and R the microseconds of
 // the means and of the recurrence alone, x = M / (M + 0.7 R) of the chunks first lets both end at about the same time; M (1 - x)
-// is then hidden, and the second launches of MLP and gate and the slower recurrence are paid.  Measured, one
-// range -> two (us a step): 512 sequences x 121 chunks of 128, MLP 1008 -> 937; 128 x 121 of 128, MLP 353 -> 328; 256 x 240
-// of 32, MLP 570 -> 539; 512 x 56 of 64, mean 320 -> 300; 256 x 120 of 64, mean 340 -> 311, MLP 382 -> 366; 128 x 127 of 128 at d_g = 128, mean
-// 279 -> 244; below the lines, with the projection still a kernel of its own: 256 x 56 of 64 with 28 us to hide, mean 194 -> 189, MLP 218 -> 226; 32 x 250 of
-// 64, mean, 33 us: 356 -> 364.  (The figures of the
-// recurrence are those of d_g = 256; at 64 and 128 it is faster, which makes x too small rather than too large.  The rule over 240 settings
-// - d_g 64, 128, 256; 8 to 1024 sequences of 4160 to 16512 tokens in chunks of 32 to 512; mean and MLP - and 28 with three planes: never more than
-// 2 % behind one range, up to 23 % ahead of it, 128 x 127 of 128 at d_g = 64.)
+// is then hidden, and the second launches of MLP and gate and the slower recurrence are paid.  Measured, one range -> two, us a kvE_refresh:
+// 512 sequences x 121 chunks of 128, MLP 956 -> 880, three planes 1024 -> 935; 128 x 121 of 128, MLP 326 -> 292; 256 x 240 of 32, MLP 543 -> 510; 256 x
+// 120 of 64, mean 320 -> 291, MLP 353 -> 331; 512 x 56 of 64, mean 284 -> 263; 128 x 127 of 128 at d_g = 128, mean 271 -> 230.
+// The lines were drawn when a second range cost a second projection GEMM.  Below them two ranges would be as fast or faster by now with the mean (256 x 56
+// of 64, 28 us to hide, 153.8 -> 149.3; 32 x 250 of 64 346 -> 329; 512 x 30 of 128 227 -> 213), with the MLP sometimes (512 x 56 of 64 319 -> 305; 256 x 56
+// of 64 173.0 -> 173.7; 128 x 61 of 64 136 -> 144).  Above them one range is behind in all of 60 settings (d_g 128, 256; 32 to 512 sequences; 2 and 3 planes).
+// (The figures of the recurrence are those of d_g = 256; at 64 and 128 it is faster, which makes x too small rather than too large.)
 constexpr double REFRESH_HIDE_US = 40, REFRESH_HIDE_MLP_US = 60;
 
 static int first_range(const kvE_store* st, int nc, const kvE_lstm_weights* lw) {

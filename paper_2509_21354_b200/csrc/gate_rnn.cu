@@ -29,7 +29,7 @@
 //    (a GEMM over all chunks, P = 254 MB on 512 sequences x 121 chunks written and read again) it took 70 us there, 25 us on 256 x 56, 11 us on
 //    8 x 28 at d_g = 128; here it adds what the issue of its MMAs (32 a batch, ~68 cycles each whatever the columns) takes away from the
 //    recurrence's warps: 3 us on 256 x 56 (77.5 us without them, 3 more if one warp issues all).  A chain of 300 chunks of 8 sequences pays more for that than the
-//    GEMM cost it (348 -> 358 us), all others gain.  Issued by the recurrence's own warps it cost another 2 to 4 us and, with the branches
+//    GEMM cost it (348 -> 354 us; 8 x 400 at d_g = 128 315 -> 323), all others gain.  Issued by the recurrence's own warps it cost another 2 to 4 us and, with the branches
 //    around it, 10 % of a round.
 //  * Exchange of h_t: a warp writes the planes of its 8 hidden units into its own CTA's double-buffered h planes (two units per
 //    4-byte word, after one shuffle), and sends them from there to every other CTA of the cluster in 16-byte asynchronous stores that
@@ -40,8 +40,8 @@
 //    warpgroup adds up its 8 units (d_g / 8 partial sums per (s, t) go to memory: an eighth of the bytes of h_t) and announces the bytes of
 //    the next exchange, and when the chain is through the cluster adds the partial sums up in a fixed order.  (Both by the recurrence's
 //    warps: 77 us on 60 sequences x 80 chunks at d_g = 128, 73.6 so.)
-//  Measured, the whole gate: 512 sequences x 121 chunks 318 -> 277 us, 256 x 56 87.6 -> 74.3 us, 32 x 250 298 -> 299.5 us, 8 x 28 at d_g = 128
-//  30.7 -> 27.0 us, 60 x 80 75.7 -> 69.1 us, 60 x 5 12.9 -> 8.9 us (before: projection and recurrence as two kernels, back to back).
+//  Measured, the whole gate: 512 sequences x 121 chunks 319 -> 264 us, 256 x 56 86.9 -> 73.4 us, 32 x 250 297.2 -> 296.2 us, 8 x 28 at d_g = 128
+//  30 to 32 -> 27.0 us, 60 x 80 74.2 -> 69.4 us, 60 x 5 12.2 -> 8.8 us (before: projection and recurrence as two kernels, back to back).
 //  Slower, with the kernels of that time: waiting for the CTA's own planes and the peers' apart, with the own units' MMAs in between (255 -> 261 us a step
 //  on 256 sequences), the two warps of a scheduler taking turns at the tensor cores (512 x 121 279 -> 317 us), and the sums of the even and the
 //  odd k tiles in accumulators of their own (286 -> 308 us).
@@ -338,7 +338,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __maxnreg__((GATE_REGS<DG, PL>))
   umma::tmem_st_wait();
 
   KVE_RNN_ONCE(1);
-  pdl_wait();      // W_hh is in place; the carried state and P come from earlier kernels
+  pdl_wait();      // the weights are in place; the carried state comes from earlier kernels
   // only now, when all earlier work is complete: a launch may run beside this kernel without waiting for anything (kvE_refresh)
   pdl_launch_dependents();
   if (a.list_cut >= 0 && blockIdx.x == 0 && tid == 0) *a.n_listed = a.list_cut;
@@ -618,7 +618,8 @@ static cudaError_t launch_rnn_t(const RnnArgs& a, const CUtensorMap* maps, cudaS
 static int cluster_ctas(int d_g) { return d_g / 64; }
 static bool two_groups(int S, int d_g) { return (S + 7) / 8 > sm_count() / cluster_ctas(d_g); }
 
-// Microseconds per chunk as measured (two planes of h, d_g = 256): 1.22 with one group of sequences per cluster, 2.28 with two
+// Microseconds per chunk (two planes of h, d_g = 256): 1.22 with one group of sequences per cluster, 2.28 with two, as measured when kvE_refresh's rule was
+// fitted to them (1.18 and 2.18 now)
 double gate_rnn_us_per_chunk(int S, int d_g, int planes) {
   const bool two = two_groups(S, d_g);
   const int clusters = (S + (two ? 15 : 7)) / (two ? 16 : 8), wave = sm_count() / cluster_ctas(d_g);

@@ -214,8 +214,9 @@ cudaError_t launch_chunk_mean(const LayerView& v, int t0, int t1, bool final_out
 // The recurrence leaves an SM 4 K to 25 K of its registers and about two thirds of its shared memory (two CTAs of this kernel), so the rows on their way wait there: a
 // warp's pages come in bulk copies of 16 rows, eight of them in flight, and are added up row by row as above (the same rounding).
 // A CTA takes several units in a row, so that the copies of the next one are under way while the last is added up.
-// 4.1 TB/s beside the recurrence of 512 sequences, which takes 22 % longer meanwhile (pages of 128 tokens; the kernel above, its
-// rows in registers: 3 TB/s).  Fewer rows in flight were slower for the whole step (eight pieces of 8 rows +1 %, four +9 %), asynchronous
+// 512 sequences, pages of 128 tokens: 92 chunks of the gate (203 us alone) and the means of 29 (142 us alone) take 272 us together; with three
+// planes 86 chunks (239 us) and 35 (172 us) 325 us.  (Beside the recurrence of before, without the projection: 4.1 TB/s, the recurrence 22 % longer; the
+// kernel above, its rows in registers: 3 TB/s.)  Fewer rows in flight were slower for the whole step (eight pieces of 8 rows +1 %, four +9 %), asynchronous
 // 16-byte copies +0.6 %; 256 rows per CTA +1 %, 512 +2 %, and a CTA per page +4 % with pages of 32 tokens.
 constexpr int MB_ROWS = 16, MB_STAGES = 8;
 constexpr int MB_CTA_ROWS = 128;                      // rows of K (or V) that a CTA takes, about
