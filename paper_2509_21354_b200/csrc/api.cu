@@ -613,7 +613,7 @@ int kvE_adopt_device_state(kvE_store* st, int layer, void* stream) {
 // 120 of 64, mean 320 -> 291, MLP 353 -> 331; 512 x 56 of 64, mean 284 -> 263; 128 x 127 of 128 at d_g = 128, mean 271 -> 230.
 // The lines were drawn when a second range cost a second projection GEMM.  Below them two ranges would be as fast or faster by now with the mean (256 x 56
 // of 64, 28 us to hide, 153.8 -> 149.3; 32 x 250 of 64 346 -> 329; 512 x 30 of 128 227 -> 213), with the MLP sometimes (512 x 56 of 64 319 -> 305; 256 x 56
-// of 64 173.0 -> 173.7; 128 x 61 of 64 136 -> 144).  Above them one range is behind in all of 60 settings (d_g 128, 256; 32 to 512 sequences; 2 and 3 planes).
+// of 64 173.0 -> 173.7; 128 x 61 of 64 136 -> 144).  Above them one range is behind in all of 46 settings (d_g 128, 256; 32 to 512 sequences; 2 and 3 planes).
 // (The figures of the recurrence are those of d_g = 256; at 64 and 128 it is faster, which makes x too small rather than too large.)
 constexpr double REFRESH_HIDE_US = 40, REFRESH_HIDE_MLP_US = 60;
 
